@@ -160,7 +160,7 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 164);
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -195,47 +195,48 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
   const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer (one lane per CTA)
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
-        const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
-        const GroupStatic g = p.gs[c.g];
-        const int row = c.row0 + (2 * c.mp + (int)rank) * kUmmaBM;     // this CTA's m-tile
-        const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
-        const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
-        const bool by_threads = MODE == 1 && !g.is_shared && p.use_gather == 2;   // the gather warps fill A
-        int k_blocks, b_half, b_row, j = 0;
-        if (MODE == 1) {
-          const int bn = g.is_shared ? p.bn_s : p.bn_r;
-          k_blocks = k_blocks_fixed;
-          b_half = bn * kUmmaBK * 2;
-          b_row = g.w_row0 + c.nt * bn;
-        } else {
-          k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK;
-          b_half = kU2BBytes;
-          b_row = c.nt * 256 + (int)rank * 128;
-          j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
-        }
-        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
-          const uint32_t s = it % kU2Stages, n = it / kU2Stages;
-          if (!mbar_wait(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
-          const uint32_t fb_local = full0 + 8 * s;
-          const uint32_t fb = mapa_shared(fb_local, 0);               // the leader's barrier
-          const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
+    // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
+    uint32_t it = 0;
+    bool ok = true;
+    for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
+      const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
+      const GroupStatic g = p.gs[c.g];
+      const int row = c.row0 + (2 * c.mp + (int)rank) * kUmmaBM;     // this CTA's m-tile
+      const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
+      const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
+      const bool by_threads = MODE == 1 && !g.is_shared && p.use_gather == 2;   // the gather warps fill A
+      int k_blocks, b_half, b_row, j = 0;
+      if (MODE == 1) {
+        const int bn = g.is_shared ? p.bn_s : p.bn_r;
+        k_blocks = k_blocks_fixed;
+        b_half = bn * kUmmaBK * 2;
+        b_row = g.w_row0 + c.nt * bn;
+      } else {
+        k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK;
+        b_half = kU2BBytes;
+        b_row = c.nt * 256 + (int)rank * 128;
+        j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
+      }
+      for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+        const uint32_t s = it % kU2Stages, n = it / kU2Stages;
+        if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
+        const uint32_t fb_local = full0 + 8 * s;
+        const uint32_t fb = mapa_shared(fb_local, 0);               // the leader's barrier
+        const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
+        if (elect_one()) {
           if (leader) mbar_expect_tx(fb_local, 2 * ((by_threads ? 0 : kU2ABytes) + b_half));
           if (!by_threads) tma2_load_2d(sa, ta, fb, kb * kUmmaBK, row);
           if (MODE == 1) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, (int)rank);   // plane 0 gate, 1 up
           else if (g.is_shared) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
           else tma2_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
         }
+        __syncwarp();
       }
-      if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);
     }
+    if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (leader && lane == 0) {
+    // ------------------------------------------------------------ MMA issuer (leader CTA only; whole warp, one lane issues)
+    if (leader) {
       uint32_t it = 0, tile_n = 0;
       bool ok = true;
       for (int t = pair_id; t < total_tiles && ok; t += n_pairs, ++tile_n) {
@@ -246,22 +247,26 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
         else { k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK; n_mma = 256; }
         const uint32_t idesc = umma2_idesc(n_mma);
         const uint32_t buf = tile_n & 1, use = tile_n >> 1;
-        if (!mbar_wait(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
+        if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * 256;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const uint32_t s = it % kU2Stages, n = it / kU2Stages;
-          if (!mbar_wait(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
+          if (!mbar_wait_warp(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
           if (MODE == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_after();
           const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kUmmaBK / 16; ++k)
-            umma2_bf16(d_tmem, umma_smem_desc(sa + k * 32), umma_smem_desc(sb + k * 32), idesc,
-                       (kb | k) != 0 ? 1u : 0u);
-          umma2_commit_both(empty0 + 8 * s);
+            for (int k = 0; k < kUmmaBK / 16; ++k)
+              umma2_bf16(d_tmem, umma_smem_desc(sa + k * 32), umma_smem_desc(sb + k * 32), idesc,
+                         (kb | k) != 0 ? 1u : 0u);
+            umma2_commit_both(empty0 + 8 * s);
+          }
+          __syncwarp();
         }
-        if (ok) umma2_commit_both(accf0 + 8 * buf);
+        if (ok && elect_one()) umma2_commit_both(accf0 + 8 * buf);
+        __syncwarp();
       }
     }
   } else if (MODE == 1 && warp == 10) {

@@ -142,7 +142,7 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);  // !SPLIT: [n_groups + 1], same bytes
   int32_t* inv_tables = reinterpret_cast<int32_t*>(bars_gen + kDecInvOff);     // [4 warps][NT]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // rows of a tile of group g and the number of its tiles
   auto tile_rows = [&](const GroupStatic& g) { return MODE == 4 ? (g.is_shared ? p.tile_rows_s : p.tile_rows_r) : 128; };
   auto group_tiles = [&](int g) {
@@ -242,7 +242,7 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
   };
   // every other role: wait for the table (bounded), then for the router's writes
   auto await_table = [&]() -> bool {
-    if (!mbar_wait(tbl_bar, 0, abort_flag, p.err, kErrWaitFull)) return false;
+    if (!mbar_wait_warp(tbl_bar, 0, abort_flag, p.err, kErrWaitFull)) return false;
     grid_dep_wait();
     total_units = tile_start[p.n_groups];
     tbl_seen = true;
@@ -305,10 +305,10 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
       const int k_end = SPLIT ? un.kb1 : ((MODE == 4 ? p.d : g.width) + kBK - 1) / kBK;
       for (int kb = un.kb0; kb < k_end; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
-        if (!mbar_wait(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
+        if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb = full0 + 8 * s;
         const uint32_t sw = base + s * kStageBytes, sx = sw + kWBytes;
-        if (lane == 0) {
+        if (elect_one()) {
           const int tr = tile_rows(g);
           mbar_expect_tx(fb, (MODE == 4 ? 2 : 1) * tr * 128 + (W8 ? 2 : 1) * p.tok_box_rows * 128);
           if (MODE == 4) tma_load_3d(sw, tw, fb, kb * kBK, g.w_row0 + nt * tr, 0);   // gate rows, then the up rows behind them
@@ -326,33 +326,32 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
     }
     if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int round = 0; ok; ++round) {
-        const bool fe = early && round == 0;
-        if (!fe && !tbl_seen && !await_table()) { ok = false; break; }
-        const int t = fe ? cta : snake_tile(round, cta, n_ctas, total_units);
-        if (t < 0) break;
-        const Unit un = fe ? early_unit : find_unit(t);
-        const int gi = un.gi;
-        const GroupStatic g = p.gs[gi];
-        const int n_mma = ((MODE == 4 ? group_rows(g.outer, fe).count : p.gr[gi].count) + 15) & ~15;   // columns, rounded to 16
-        // W8: one MMA covers both token planes (N = hi rows + lo rows, adjacent in the stage): the decode
-        // kernels are bound by the number of MMAs a tile takes (~115 cycles each at these small N), not by bytes
-        const uint32_t idesc = W8 ? umma_idesc_e4m3(2 * p.tok_box_rows) : umma_idesc(n_mma);
-        const uint32_t buf = round & 1, use = round >> 1;
-        if (!mbar_wait(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
+    // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
+    uint32_t it = 0;
+    bool ok = true;
+    for (int round = 0; ok; ++round) {
+      const bool fe = early && round == 0;
+      if (!fe && !tbl_seen && !await_table()) { ok = false; break; }
+      const int t = fe ? cta : snake_tile(round, cta, n_ctas, total_units);
+      if (t < 0) break;
+      const Unit un = fe ? early_unit : find_unit(t);
+      const int gi = un.gi;
+      const GroupStatic g = p.gs[gi];
+      const int n_mma = ((MODE == 4 ? group_rows(g.outer, fe).count : p.gr[gi].count) + 15) & ~15;   // columns, rounded to 16
+      // W8: one MMA covers both token planes (N = hi rows + lo rows, adjacent in the stage)
+      const uint32_t idesc = W8 ? umma_idesc_e4m3(2 * p.tok_box_rows) : umma_idesc(n_mma);
+      const uint32_t buf = round & 1, use = round >> 1;
+      if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + buf * kBufCols;
+      const uint32_t up_off = (uint32_t)tile_rows(g) * 128u;          // the up plane follows the tile's gate rows
+      const int k_end = SPLIT ? un.kb1 : ((MODE == 4 ? p.d : g.width) + kBK - 1) / kBK;
+      for (int kb = un.kb0; kb < k_end; ++kb, ++it) {
+        const uint32_t s = it % kStages, n = it / kStages;
+        const uint32_t sw = base + s * kStageBytes, sx = sw + kWBytes;
+        if (!mbar_wait_warp(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * kBufCols;
-        const uint32_t up_off = (uint32_t)tile_rows(g) * 128u;          // the up plane follows the tile's gate rows
-        const int k_end = SPLIT ? un.kb1 : ((MODE == 4 ? p.d : g.width) + kBK - 1) / kBK;
-        for (int kb = un.kb0; kb < k_end; ++kb, ++it) {
-          const uint32_t s = it % kStages, n = it / kStages;
-          const uint32_t sw = base + s * kStageBytes, sx = sw + kWBytes;
-          if (!mbar_wait(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
-          tc_fence_after();
+        if (elect_one()) {
           // four k steps of 32 bytes per 128-byte row: 16 bf16 or 32 E4M3 values each
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -369,8 +368,10 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
           }
           umma_commit(empty0 + 8 * s);
         }
-        if (ok) umma_commit(accf0 + 8 * buf);
+        __syncwarp();
       }
+      if (ok && elect_one()) umma_commit(accf0 + 8 * buf);
+      __syncwarp();
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..5)

@@ -93,6 +93,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
   }
 }
+// The same for a whole warp: every lane gets the same answer, so the warp stays converged.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               int32_t* err_word, int code) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err_word, code));
+}
+// One lane of a converged warp, always the same one.  tcgen05 and TMA instructions take their operands from
+// uniform registers: issued under a branch on the lane number they cost 72-95 cycles each whatever their size
+// (measured: back-to-back M = 128 MMAs), under elect.sync in a loop that the whole warp runs 39 cycles at
+// N <= 32, 48 at N = 64, 64 at N = 128 and 128 at N = 256, the rate of the tensor core itself.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// Warp index as a value the compiler knows to be uniform.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -354,7 +370,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 164);
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int n_groups = MODE == 3 ? p.n_outer : p.n_groups;
 
   if (threadIdx.x == 0) {
@@ -434,62 +450,68 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
       const int kb_lo = kz * k_blocks / ksplit, kb_hi = (kz + 1) * k_blocks / ksplit;      // this unit's k slice
       for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
-        if (!mbar_wait(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
+        if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb = full0 + 8 * s;
         const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
-        if (lane == 0) mbar_expect_tx(fb, (by_threads ? 0 : a_bytes) + b_bytes);
-        __syncwarp();
         if (gather) {
+          if (lane == 0) mbar_expect_tx(fb, a_bytes + b_bytes);
+          __syncwarp();
           if (lane < n_issue) tma_gather4(sa + lane * 512, ta, fb, kb * kUmmaBK, gr0, gr1, gr2, gr3);
-        } else if (lane == 0 && !by_threads) {
-          tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
+          __syncwarp();
         }
-        if (lane == 0) {
+        if (elect_one()) {
+          if (!gather) {
+            mbar_expect_tx(fb, (by_threads ? 0 : a_bytes) + b_bytes);
+            if (!by_threads) tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
+          }
           if (MODE == 1) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, 0);
           else if (MODE == 3) tma_load_3d(sb, tb, fb, kb * kUmmaBK, 0, c.g);
           else if (g.is_shared) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
           else tma_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
         }
+        __syncwarp();
       }
     }
     if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t it = 0, tile_n = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++tile_n) {
-        const int t = u / ksplit, kz = u - t * ksplit;
-        const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
-        int k_blocks, n_mma;
-        if (MODE == 1) {
-          const GroupStatic g = p.gs[c.g];
-          k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r);
-        } else if (MODE == 2) {
-          k_blocks = (p.gs[c.g].width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
-        } else {
-          k_blocks = k_blocks_fixed; n_mma = 2 * p.n_rp;
-        }
-        const uint32_t idesc = umma_idesc(n_mma);
-        const uint32_t buf = tile_n & 1, use = tile_n >> 1;
-        if (!mbar_wait(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
+    // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
+    uint32_t it = 0, tile_n = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++tile_n) {
+      const int t = u / ksplit, kz = u - t * ksplit;
+      const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
+      int k_blocks, n_mma;
+      if (MODE == 1) {
+        const GroupStatic g = p.gs[c.g];
+        k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r);
+      } else if (MODE == 2) {
+        k_blocks = (p.gs[c.g].width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
+      } else {
+        k_blocks = k_blocks_fixed; n_mma = 2 * p.n_rp;
+      }
+      const uint32_t idesc = umma_idesc(n_mma);
+      const uint32_t buf = tile_n & 1, use = tile_n >> 1;
+      if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + buf * 256;
+      const int kb_lo = kz * k_blocks / ksplit, kb_hi = (kz + 1) * k_blocks / ksplit;
+      for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
+        const uint32_t s = it % kStages, n = it / kStages;
+        if (!mbar_wait_warp(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
+        if (MODE == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // cp.async-written rows
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * 256;
-        const int kb_lo = kz * k_blocks / ksplit, kb_hi = (kz + 1) * k_blocks / ksplit;
-        for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
-          const uint32_t s = it % kStages, n = it / kStages;
-          if (!mbar_wait(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
-          if (MODE == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // cp.async-written rows
-          tc_fence_after();
-          const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
+        const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
+        if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < kUmmaBK / 16; ++k)
             umma_bf16(d_tmem, umma_smem_desc(sa + k * 32), umma_smem_desc(sb + k * 32), idesc,
                       (kb != kb_lo || k != 0) ? 1u : 0u);
           umma_commit(empty0 + 8 * s);         // stage reusable once these MMAs have read it
         }
-        if (ok) umma_commit(accf0 + 8 * buf);  // accumulator complete
+        __syncwarp();
       }
+      if (ok && elect_one()) umma_commit(accf0 + 8 * buf);  // accumulator complete
+      __syncwarp();
     }
   } else if (MODE == 1 && warp >= 6) {
     // ------------------------------------------------------------ A-row gather (mode 1, warps 6..9)
