@@ -21,6 +21,7 @@
 #include "permute.cuh"
 #include "profile.cuh"
 #include "router.cuh"
+#include "router_cluster.cuh"
 #include "router_mma.cuh"
 #include "simt_gemm.cuh"
 #include "umma2_gemm.cuh"
@@ -112,8 +113,7 @@ struct cmoe_layer {
   UmmaPlan umma;
   DecodePlan decode;
   Umma2Plan pair;
-  float* rsk_part = nullptr;    // split-K router partial sums [slices][64 rows][64]
-  int32_t* rsk_ticket = nullptr;
+  int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
   float* rt_part = nullptr;     // tcgen05 router: K-slice partial sums and tickets
   int32_t* rt_ticket = nullptr;
   float* dec_part = nullptr;    // decode GEMMs: K-slice partial sums, tickets per (tile, epilogue warp)
@@ -236,10 +236,9 @@ void carve_workspace(cmoe_layer* L, char* base) {
   L->perm_scratch = a.take<int32_t>(permute_scratch_bytes((int)R, (int)(G ? G : 1)) / 4);
   L->gr = a.take<GroupRows>(L->n_groups_total());
   L->err_word = a.take<int32_t>(1);
-  L->rsk_ticket = a.take<int32_t>(kRskMaxChunks + 1);
+  L->router_ticket = a.take<int32_t>(1);
   L->share = a.take<float>(G ? G : 1);
   L->target = a.take<float>(G ? G : 1);
-  L->rsk_part = a.take<float>((size_t)kRskMaxTotalRows * kRskMaxSlices * 64);
   L->x_perm = a.take<char>(P * d * esz);
   L->h_s = a.take<char>(R * L->shared_width() * esz);
   L->h_r = a.take<char>(P * L->m * esz);
@@ -411,24 +410,18 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                                                  L->b, ooff, L->n_outer, L->scores, L->keys,      \
                                                  L->topk_idx, L->topk_gate)
     if constexpr (std::is_same<T, bf16>::value) {
-      if (use_umma && R > kRskMaxTotalRows) {
+      if (use_umma && R > kRcMaxRows) {
         if (umma_router_forward(&L->umma, R, ooff, L->err_word, st) < 0)
           return arg_fail(CMOE_ERR_CUDA, L->umma.error);
-      } else if (R <= kRskMaxTotalRows && d <= kRskMaxSlices * kRskSliceK) {
-        // Row chunks, the grid's second dimension: 16 rows for a router with more than 8 columns, whose gate
-        // logic takes a warp per row (measured: 8B-shaped layer at 32 rows 97.9 -> 95.0 us, at 128 rows
-        // 118.9 -> 108.7 us); 64 rows with up to 8 columns, where the four-rows-per-warp form on 64-row chunks
-        // is 1 us faster.  The last chunk's block also permutes batches of up to 128 rows (7B-shaped layer at
-        // 128 rows 91.0 -> 88.9 us; at 256 rows the permutation kernels are as fast).
-        const int chunk_rows = n_r > 8 ? 16 : kRskMaxRows;
-        const int chunks = (R + chunk_rows - 1) / chunk_rows;
-        perm_fused = G <= kRskFuseGroups && R <= 2 * kRskMaxRows && (long long)R * n_k <= 4096;
-        const bool sub8 = n_r <= 8 && R > 16;                        // pays when a chunk's last block has more than 16 rows
-        (sub8 ? router_splitk_kernel<true> : router_splitk_kernel<false>)
-            <<<dim3((d + kRskSliceK - 1) / kRskSliceK, chunks), kRskThreads, 0, st>>>(
-            xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->rsk_part,
-            L->rsk_ticket, chunk_rows, L->scores, L->keys, L->topk_idx, L->topk_gate, perm_fused ? 1 : 0, G, L->counts,
-            L->offsets, L->row_token, L->row_of, po);
+      } else if (R <= kRcMaxRows) {
+        perm_fused = router_cluster_fuses(R, n_k, G);
+        RouterArgs ra{};
+        ra.x = xo; ra.n_rows = R; ra.d = d; ra.n_r = n_r; ra.n_rp = L->n_rp; ra.n_k = n_k;
+        ra.w_rep = (const bf16*)L->w_rep; ra.u = L->u; ra.b = L->b; ra.outer_off = ooff; ra.n_outer = L->n_outer;
+        ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
+        ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
+        ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
+        CU_TRY(router_cluster_launch(ra, L->hier, false, st));
       } else {
         router_mma_kernel<8, 1><<<(R + 15) / 16, 256, 0, st>>>(
             xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->scores,
@@ -1082,7 +1075,7 @@ int cmoe_layer_status(cmoe_layer* L, int32_t* device_error_word) {
   // Clear the error word and every ticket so that the next forward starts from a clean state.
   cudaStream_t st = L->last_stream;
   CU_TRY(cudaMemsetAsync(L->err_word, 0, 4, st));
-  CU_TRY(cudaMemsetAsync(L->rsk_ticket, 0, 4 * (kRskMaxChunks + 1), st));
+  CU_TRY(cudaMemsetAsync(L->router_ticket, 0, 4, st));
   if (L->dec_ticket) CU_TRY(cudaMemsetAsync(L->dec_ticket, 0, L->n_dec_ticket * 4, st));
   if (L->rt_ticket) CU_TRY(cudaMemsetAsync(L->rt_ticket, 0, L->n_rt_ticket * 4, st));
   CU_TRY(cudaStreamSynchronize(st));
