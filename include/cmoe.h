@@ -258,7 +258,8 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
 int cmoe_layer_set_gemm_path(cmoe_layer* layer, int32_t path);
 
 /* Launch chaining (on by default): on the bf16 tensor-core path every kernel of a forward
- * after the expert router is launched as a programmatic dependent of its predecessor, so it
+ * (of a plain layer: from the expert router on for up to 1024 rows, after it for more; of a
+ * hierarchical one: after it) is launched as a programmatic dependent of its predecessor, so it
  * may become resident (and fetch what does not depend on the predecessor) while the
  * predecessor drains, and waits on the device before touching anything the predecessor
  * produces.  Results are bit-identical either way; 0 restores ordinary stream-ordered

@@ -356,9 +356,10 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   cudaEvent_t* ev = (L->ev_ring && !gate_up_only) ? &L->ev[(size_t)(L->ev_count % L->ev_ring) * (CMOE_N_STAGES + 1)] : nullptr;
   auto mark = [&](int i) { if (ev) cudaEventRecord(ev[i], st); };
   mark(0);
-  // bf16 layers on the tensor path chain their kernels by programmatic dependent launch (every
-  // kernel after the expert router may become resident early and waits on the device for its
-  // predecessor); per-stage events and the prologue of a hierarchical layer (outer router, outer
+  // bf16 layers on the tensor path chain their kernels by programmatic dependent launch (a kernel
+  // may become resident early and waits on the device for its predecessor).  The small-batch router of a
+  // plain layer is chained to whatever precedes it in the stream, which it waits for in full (7B-shaped layer
+  // 1 / 16 / 300 rows 35.0 / 63.1 / 108.9 -> 33.6 / 61.4 / 104.8 us, even from 600 rows on); per-stage events and the prologue of a hierarchical layer (outer router, outer
   // permutation, row copy) use ordinary launches.
   const bool dep = use_umma && !ev && L->chain_launches;
 
@@ -396,7 +397,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   if (use_umma && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if (decode && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if (decode && L->fp8) {                          // E4M3 planes of the token rows: independent of the routing
-    if (decode_split_x(&L->umma, &L->decode, R, st, false) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
+    if (decode_split_x(&L->umma, &L->decode, R, st, dep && !L->hier) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
     ++launches;
   }
   GroupPlanOut po;                                // the permutation also writes every group's row range
@@ -421,7 +422,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
         ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
         ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
-        CU_TRY(router_cluster_launch(ra, L->hier, false, st));
+        CU_TRY(router_cluster_launch(ra, L->hier, dep && !L->hier, st));
       } else {
         router_mma_kernel<8, 1><<<(R + 15) / 16, 256, 0, st>>>(
             xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->scores,

@@ -170,8 +170,6 @@ __device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint
 template <int MAXT, int NB>
 __global__ void __cluster_dims__(kRcCluster, 1, 1) __launch_bounds__(kRcThreads, 2)
 router_cluster_kernel(const RouterArgs p) {
-  grid_dep_wait();
-  grid_dep_trigger();
   constexpr int kCols = MAXT * 8, kStride = kCols + 8;
   constexpr int kUnr = 16 / (MAXT * NB) >= 2 ? 2 : 1;                // k slices in flight per warp
   constexpr int kPartBytes = 8 * kRcRows * kStride * 4;
@@ -186,6 +184,29 @@ router_cluster_kernel(const RouterArgs p) {
   const int row_base = blockIdx.y * kRcRows;
   const int n_rows = min(kRcRows, p.n_rows - row_base);
   rc_cluster_arrive();                                               // the peers have started: waited for before the push
+  const int g = lane >> 2, t = lane & 3;
+  const int n2 = 2 * p.n_rp, n_tiles = n2 >> 3;
+  const int n_slices = (p.d + 31) >> 5, s0 = (int)rank * 8 + warp;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  uint4 w[kUnr][NB][MAXT];
+  // representative rows of expert list entries i0 .. i0 + NB - 1, k slices s, s + 64 ..
+  auto load_w = [&](int s, int i0, int nl) {
+#pragma unroll
+    for (int q = 0; q < kUnr; ++q) {
+      const int k = (s + 64 * q) * 32 + 8 * t;
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        const bool have = k < p.d && (NB == 1 || i0 + i < nl);
+        const bf16* wr = p.w_rep + ((size_t)(NB > 1 && have ? g_list[i0 + i] : 0) * n2 + g) * p.d + k;
+#pragma unroll
+        for (int nt = 0; nt < MAXT; ++nt)
+          w[q][i][nt] = (have && nt < n_tiles) ? __ldg(reinterpret_cast<const uint4*>(wr + (size_t)nt * 8 * p.d)) : zero;
+      }
+    }
+  };
+  if (NB == 1) load_w(s0, 0, 1);          // the layer's own rows: fetched while the preceding kernel of the stream drains
+  grid_dep_wait();
+  grid_dep_trigger();
   if (warp == 0) {
     const int go = (p.outer_off && lane < kRcRows) ? find_outer(p.outer_off, p.n_outer, row_base + min(lane, n_rows - 1)) : 0;
     const int prev = __shfl_up_sync(0xffffffffu, go, 1);
@@ -206,12 +227,9 @@ router_cluster_kernel(const RouterArgs p) {
     if (lane < p.n_r) { u_pre = __ldg(p.u + go_mine * p.n_r + lane); b_pre = __ldg(p.b + go_mine * p.n_r + lane); }
   }
   // ---- partial sums over this warp's k slices
-  const int g = lane >> 2, t = lane & 3;
-  const int n2 = 2 * p.n_rp, n_tiles = n2 >> 3;
   const int r_lo = min(g, n_rows - 1), r_hi = min(g + 8, n_rows - 1);
   const bf16* x_lo = p.x + (size_t)(row_base + r_lo) * p.d + 8 * t;
   const bf16* x_hi = p.x + (size_t)(row_base + r_hi) * p.d + 8 * t;
-  const int n_slices = (p.d + 31) >> 5, s0 = (int)rank * 8 + warp;
   const int nl = NB > 1 ? n_list : 1;
   for (int i0 = 0; i0 < nl; i0 += NB) {
     float acc[NB][MAXT][4];
@@ -222,23 +240,15 @@ router_cluster_kernel(const RouterArgs p) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[i][nt][q] = 0.0f;
     for (int s = s0; s < n_slices; s += 64 * kUnr) {
-      uint4 a_lo[kUnr], a_hi[kUnr], w[kUnr][NB][MAXT];
+      uint4 a_lo[kUnr], a_hi[kUnr];
 #pragma unroll
       for (int q = 0; q < kUnr; ++q) {
         const int k = (s + 64 * q) * 32;
         const bool in = k + 8 * t < p.d;
-        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
         a_lo[q] = in ? __ldg(reinterpret_cast<const uint4*>(x_lo + k)) : zero;
         a_hi[q] = in ? __ldg(reinterpret_cast<const uint4*>(x_hi + k)) : zero;
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-          const bool have = in && (NB == 1 || i0 + i < nl);
-          const bf16* wr = p.w_rep + ((size_t)(NB > 1 && have ? g_list[i0 + i] : 0) * n2 + g) * p.d + k + 8 * t;
-#pragma unroll
-          for (int nt = 0; nt < MAXT; ++nt)
-            w[q][i][nt] = (have && nt < n_tiles) ? __ldg(reinterpret_cast<const uint4*>(wr + (size_t)nt * 8 * p.d)) : zero;
-        }
       }
+      if (NB > 1 || s != s0) load_w(s, i0, nl);
 #pragma unroll
       for (int q = 0; q < kUnr; ++q)
 #pragma unroll
