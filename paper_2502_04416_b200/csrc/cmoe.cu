@@ -27,6 +27,7 @@
 #include "umma2_gemm.cuh"
 #include "umma_decode.cuh"
 #include "gemv.cuh"
+#include "stream.cuh"
 #include "umma_gemm.cuh"
 
 using namespace cmoe;
@@ -113,12 +114,13 @@ struct cmoe_layer {
   UmmaPlan umma;
   DecodePlan decode;
   Umma2Plan pair;
+  StreamPlan stream;
   int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
   float* rt_part = nullptr;     // tcgen05 router: K-slice partial sums and tickets
   int32_t* rt_ticket = nullptr;
   float* dec_part = nullptr;    // decode GEMMs: K-slice partial sums, tickets per (tile, epilogue warp)
   int32_t* dec_ticket = nullptr;
-  size_t n_dec_ticket = 0, n_rt_ticket = 0;    // lengths of the ticket arrays (zeroed again after a device timeout)
+  size_t n_dec_ticket = 0, n_rt_ticket = 0, n_stream_ticket = 0;    // lengths of the ticket arrays (zeroed again after a device timeout)
   float *share = nullptr, *target = nullptr;   // utilisation of the last step / bias-update targets
 
   cudaStream_t last_stream = nullptr;
@@ -263,6 +265,12 @@ void carve_workspace(cmoe_layer* L, char* base) {
     L->dec_ticket = a.take<int32_t>(L->n_dec_ticket);
     L->dec_part = a.take<float>((size_t)kDecMaxSlots * kDecSlotFloats);
   }
+  if (esz == 2 && !L->hier) {
+    L->n_stream_ticket = stream_tickets((int)d);
+    L->stream.ticket = a.take<int32_t>(L->n_stream_ticket);
+    L->stream.h = a.take<bf16>((size_t)kStreamMaxRows * L->cfg.d_ff);
+    L->stream.part = a.take<float>(stream_part_floats((int)T));
+  }
   if (esz == 2 && nr > 0) {
     L->n_rt_ticket = 4 * 256;
     L->rt_ticket = a.take<int32_t>(L->n_rt_ticket);
@@ -317,6 +325,8 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     if (L->umma_ok && !decode_plan_create(&L->umma, &L->decode)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     L->decode.part = L->dec_part; L->decode.ticket = L->dec_ticket;
     L->umma.rt_part = L->rt_part; L->umma.rt_ticket = L->rt_ticket;
+    if (L->umma_ok && stream_shape_ok(s, L->umma.n_sms) && !stream_plan_create(&L->umma, &L->stream))
+      return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     if (L->umma_ok && !umma2_plan_create(&L->umma, &L->pair)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   }
   CU_TRY(cudaStreamSynchronize(st));
@@ -392,9 +402,12 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                      L->fp8, &gemv_ring);
   // Weights-on-M streaming kernels: up to 64 rows; on bf16 weights (the FP8 token planes stop at 64) the wide
   // form takes up to 128 rows.  Path 2 keeps token-major tiles from 65 rows.
+  // Two to 64 rows of a plain bf16 layer: the weight streamers that end in the layer's output (automatic path only).  From 65
+  // rows on a token's bits do not depend on the batch size, which the folded gates of the streamers would break.
+  const bool stream = use_umma && !gemv && !L->fp8 && L->gemm_path == 0 && L->stream.built && R <= kStreamMaxRows;
   const int decode_rows = (!L->fp8 && L->gemm_path != 2) ? kDecWideRows : kDecMaxRows;
-  const bool decode = use_umma && !gemv && R <= decode_rows;
-  if (use_umma && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+  const bool decode = use_umma && !gemv && !stream && R <= decode_rows;
+  if (use_umma && !stream && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if (decode && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if (decode && L->fp8) {                          // E4M3 planes of the token rows: independent of the routing
     if (decode_split_x(&L->umma, &L->decode, R, st, dep && !L->hier) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
@@ -422,7 +435,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
         ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
         ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
-        CU_TRY(router_cluster_launch(ra, L->hier, dep && !L->hier, st));
+        CU_TRY(router_cluster_launch(ra, L->hier, dep && !L->hier, stream, st));
       } else {
         router_mma_kernel<8, 1><<<(R + 15) / 16, 256, 0, st>>>(
             xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->scores,
@@ -500,6 +513,21 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
       launches += n;
     }
     if (!gate_up_only) {                              // the second launch wrote `out`: nothing left to combine
+      mark(4);
+      mark(5);
+      if (ev) ++L->ev_count;
+      CU_TRY(cudaGetLastError());
+      L->launches = launches;
+      return CMOE_OK;
+    }
+  } else if (stream) {
+    if constexpr (std::is_same<T, bf16>::value) {
+      const int n = stream_forward(&L->umma, &L->stream, L->decode.wd_s, L->decode.wd_r, L->gr, xo, R, out,
+                                   gate_up_only ? (bf16*)L->h_s : L->stream.h, L->err_word, st, ev ? ev[3] : nullptr, dep, gate_up_only);
+      if (n < 0) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+      launches += n;
+    }
+    if (!gate_up_only) {
       mark(4);
       mark(5);
       if (ev) ++L->ev_count;
@@ -1078,6 +1106,7 @@ int cmoe_layer_status(cmoe_layer* L, int32_t* device_error_word) {
   CU_TRY(cudaMemsetAsync(L->err_word, 0, 4, st));
   CU_TRY(cudaMemsetAsync(L->router_ticket, 0, 4, st));
   if (L->dec_ticket) CU_TRY(cudaMemsetAsync(L->dec_ticket, 0, L->n_dec_ticket * 4, st));
+  if (L->n_stream_ticket) CU_TRY(cudaMemsetAsync(L->stream.ticket, 0, L->n_stream_ticket * 4, st));
   if (L->rt_ticket) CU_TRY(cudaMemsetAsync(L->rt_ticket, 0, L->n_rt_ticket * 4, st));
   CU_TRY(cudaStreamSynchronize(st));
   return CMOE_ERR_DEVICE_TIMEOUT;

@@ -37,6 +37,36 @@ inline cudaError_t launch_kernel(bool dependent, void (*kernel)(KP...), dim3 gri
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// An SM's split between L1 and shared memory is fixed while blocks run on it and by default just fits the kernel
+// that arrived first; kernels that are to share an SM with a chained successor ask for all of it: the ones with
+// dynamic shared memory for good, others per launch (launch_kernel_smem), since successors that live on L1 lose by it.
+template <typename K> inline cudaError_t allow_smem(K kernel, int bytes) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e == cudaSuccess
+      ? cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) : e;
+}
+template <typename... KP, typename... A>
+inline cudaError_t launch_kernel_smem(bool dependent, bool all_smem, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (dependent) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (all_smem) {
+    at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+// Swish(a) * u for the GEMM epilogues: branch-free, so that a thread's columns overlap.
+__device__ __forceinline__ float swiglu_fast(float a, float u) { return __fdividef(a, 1.0f + __expf(-a)) * u; }
+
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(bf16 v) { return __bfloat162float(v); }
 

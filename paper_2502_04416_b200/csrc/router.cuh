@@ -11,6 +11,7 @@ namespace cmoe {
 // Index of the outer expert whose row range [off[g], off[g+1]) holds row r.
 __device__ __forceinline__ int find_outer(const int32_t* __restrict__ off, int n_outer, int r) {
   int g = 0;
+#pragma unroll 4
   for (int i = 1; i < n_outer; ++i) g += (__ldg(off + i) <= r) ? 1 : 0;
   return g;
 }

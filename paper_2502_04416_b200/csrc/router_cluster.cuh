@@ -71,6 +71,7 @@ __device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float
   const float rank_key = (key != key) ? -INFINITY : key;               // NaN ranks last
   uint32_t bits = live ? ordered_bits(rank_key) : 0u;                  // every live key is above 0
   float my_gate = 0.0f;
+#pragma unroll 1
   for (int i = 0; i < n_k; ++i) {
     const uint32_t best = __reduce_max_sync(0xffffffffu, bits);
     const int who = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
@@ -104,11 +105,15 @@ __device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint
                                                  int32_t* count, int32_t* offs) {
   const int words = (p.n_rows + 31) >> 5, pairs = p.n_rows * p.n_k;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int i = threadIdx.x; i < p.n_groups * words; i += kRcThreads) mask[i] = 0;
   __syncthreads();
+#pragma unroll 1
   for (int row = threadIdx.x; row < p.n_rows; row += kRcThreads)
+#pragma unroll 1
     for (int j = 0; j < p.n_k; ++j) atomicOr(&mask[sel[row * p.n_k + j] * words + (row >> 5)], 1u << (row & 31));
   __syncthreads();
+#pragma unroll 1
   for (int g = warp; g < p.n_groups; g += kRcThreads / 32) {           // lane: word (at most kRcMaxRows / 32 = 32)
     const int c = lane < words ? __popc(mask[g * words + lane]) : 0;
     int incl = c;
@@ -145,6 +150,7 @@ __device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint
       }
     }
   } else if (p.po.gr) {
+#pragma unroll 1
     for (int g = threadIdx.x - 32; g < p.po.n_outer; g += kRcThreads - 32) {
       GroupRows r;
       r.row0 = p.po.outer_off ? p.po.outer_off[g] : 0;
@@ -153,9 +159,11 @@ __device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int row = threadIdx.x; row < p.n_rows; row += kRcThreads) {
     const int w = row >> 5;
     const uint32_t below = (1u << (row & 31)) - 1u;
+#pragma unroll 1
     for (int j = 0; j < p.n_k; ++j) {
       const int g = sel[row * p.n_k + j];
       const int pos = offs[g] + before[g * words + w] + __popc(mask[g * words + w] & below);
@@ -168,7 +176,7 @@ __device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint
 // MAXT: tiles of 8 router columns at most (2 N_r rounded up); NB: outer experts whose representative rows are held in
 // flight at once when a tile's rows belong to several (1 for a plain layer).
 template <int MAXT, int NB>
-__global__ void __cluster_dims__(kRcCluster, 1, 1) __launch_bounds__(kRcThreads, 2)
+__global__ void __cluster_dims__(kRcCluster, 1, 1) __launch_bounds__(kRcThreads, MAXT * NB <= 2 ? 3 : 2)
 router_cluster_kernel(const RouterArgs p) {
   constexpr int kCols = MAXT * 8, kStride = kCols + 8;
   constexpr int kUnr = 16 / (MAXT * NB) >= 2 ? 2 : 1;                // k slices in flight per warp
@@ -207,7 +215,7 @@ router_cluster_kernel(const RouterArgs p) {
   if (NB == 1) load_w(s0, 0, 1);          // the layer's own rows: fetched while the preceding kernel of the stream drains
   grid_dep_wait();
   grid_dep_trigger();
-  if (warp == 0) {
+  if (NB > 1 && warp == 0) {
     const int go = (p.outer_off && lane < kRcRows) ? find_outer(p.outer_off, p.n_outer, row_base + min(lane, n_rows - 1)) : 0;
     const int prev = __shfl_up_sync(0xffffffffu, go, 1);
     const bool first = lane == 0 || (lane < kRcRows && go != prev);  // rows are sorted by outer expert
@@ -231,6 +239,7 @@ router_cluster_kernel(const RouterArgs p) {
   const bf16* x_lo = p.x + (size_t)(row_base + r_lo) * p.d + 8 * t;
   const bf16* x_hi = p.x + (size_t)(row_base + r_hi) * p.d + 8 * t;
   const int nl = NB > 1 ? n_list : 1;
+#pragma unroll 1
   for (int i0 = 0; i0 < nl; i0 += NB) {
     float acc[NB][MAXT][4];
 #pragma unroll
@@ -239,6 +248,7 @@ router_cluster_kernel(const RouterArgs p) {
       for (int nt = 0; nt < MAXT; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[i][nt][q] = 0.0f;
+#pragma unroll 1
     for (int s = s0; s < n_slices; s += 64 * kUnr) {
       uint4 a_lo[kUnr], a_hi[kUnr];
 #pragma unroll
@@ -277,6 +287,7 @@ router_cluster_kernel(const RouterArgs p) {
   }
   __syncthreads();
   rc_cluster_wait();
+#pragma unroll 1
   for (int i = threadIdx.x; i < kRcRows * n2; i += kRcThreads) {     // this CTA's sums, each to the CTA of its row
     const int r = i / n2, c = i - r * n2;
     float s = 0.0f;
@@ -309,6 +320,7 @@ router_cluster_kernel(const RouterArgs p) {
   uint32_t* mask = reinterpret_cast<uint32_t*>(offs + kRcFuseGroups);
   uint16_t* before = reinterpret_cast<uint16_t*>(mask + kRcFuseGroups * (kRcMaxRows / 32));
   if (gridDim.y == 1) {
+#pragma unroll 1
     for (int i = threadIdx.x; i < n_rows * p.n_k; i += kRcThreads) sel[i] = (uint8_t)sel_recv[i];
   } else {
     if (threadIdx.x == 0) {                                           // the tile's selections are ordered before the ticket
@@ -320,6 +332,7 @@ router_cluster_kernel(const RouterArgs p) {
     __syncthreads();
     if (!is_last) return;
     const int pairs = p.n_rows * p.n_k;
+#pragma unroll 1
     for (int i0 = threadIdx.x; i0 < pairs; i0 += 8 * kRcThreads) {    // eight loads in flight per thread
       int v[8];
 #pragma unroll
@@ -337,17 +350,17 @@ inline bool router_cluster_fuses(int n_rows, int n_k, int n_groups) {
   return n_groups <= kRcFuseGroups && n_rows <= kRcMaxRows && (long long)n_rows * n_k <= kRcFusePairs;
 }
 
-inline cudaError_t router_cluster_launch(const RouterArgs& a, bool hier, bool dep, cudaStream_t st) {
+inline cudaError_t router_cluster_launch(const RouterArgs& a, bool hier, bool dep, bool all_smem, cudaStream_t st) {
   const dim3 grid(kRcCluster, (a.n_rows + kRcRows - 1) / kRcRows), block(kRcThreads);
   const int tiles = 2 * a.n_rp / 8;
   if (hier) {
-    if (tiles <= 2) return launch_kernel(dep, router_cluster_kernel<2, 4>, grid, block, 0, st, a);
-    if (tiles <= 4) return launch_kernel(dep, router_cluster_kernel<4, 2>, grid, block, 0, st, a);
-    return launch_kernel(dep, router_cluster_kernel<8, 2>, grid, block, 0, st, a);
+    if (tiles <= 2) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<2, 4>, grid, block, 0, st, a);
+    if (tiles <= 4) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<4, 2>, grid, block, 0, st, a);
+    return launch_kernel_smem(dep, all_smem, router_cluster_kernel<8, 2>, grid, block, 0, st, a);
   }
-  if (tiles <= 2) return launch_kernel(dep, router_cluster_kernel<2, 1>, grid, block, 0, st, a);
-  if (tiles <= 4) return launch_kernel(dep, router_cluster_kernel<4, 1>, grid, block, 0, st, a);
-  return launch_kernel(dep, router_cluster_kernel<8, 1>, grid, block, 0, st, a);
+  if (tiles <= 2) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<2, 1>, grid, block, 0, st, a);
+  if (tiles <= 4) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<4, 1>, grid, block, 0, st, a);
+  return launch_kernel_smem(dep, all_smem, router_cluster_kernel<8, 1>, grid, block, 0, st, a);
 }
 
 }  // namespace cmoe
