@@ -249,7 +249,7 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
  * rows each of the two GEMMs may run on CTA pairs: below 1024 rows when the experts are at least
  * 1024 neurons wide (a pair fetches a third less operand data per SM), from 1024 rows when the
  * padding of the expert groups to 256-row tiles is expected to stay small; batches of 65 to 128 rows stream the bf16 weights through the
- * decode-shaped kernels, weights on the MMA's M side; 2 to 64 rows of a plain layer without FP8 weights
+ * decode-shaped kernels, weights on the MMA's M side; 2 to 64 rows of a plain layer
  * run on two weight streamers with the gates folded into the hidden activations (rounded to bf16 once, after the
  * gate) and the sum over the experts inside the down projection; a single row of a plain layer
  * runs on the CUDA cores with plain-load weight streams, down projection and combine in one

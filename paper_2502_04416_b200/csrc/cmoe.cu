@@ -400,16 +400,18 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     gemv = use_umma && !L->hier && L->gemm_path == 0 &&
            gemv_plan((int)R, L->n_outer, L->n_groups_total(), n_k, n_r, d, L->shared_width(), L->m, L->cfg.n_shared > 0,
                      L->fp8, &gemv_ring);
-  // Weights-on-M streaming kernels: up to 64 rows; on bf16 weights (the FP8 token planes stop at 64) the wide
-  // form takes up to 128 rows.  Path 2 keeps token-major tiles from 65 rows.
   // Two to 64 rows of a plain bf16 layer: the weight streamers that end in the layer's output (automatic path only).  From 65
   // rows on a token's bits do not depend on the batch size, which the folded gates of the streamers would break.
-  const bool stream = use_umma && !gemv && !L->fp8 && L->gemm_path == 0 && L->stream.built && R <= kStreamMaxRows;
-  const int decode_rows = (!L->fp8 && L->gemm_path != 2) ? kDecWideRows : kDecMaxRows;
+  const bool stream = use_umma && !gemv && L->gemm_path == 0 && L->stream.built && L->fp8 == L->stream.fp8 &&
+                      R <= kStreamMaxRows;
+  // Weights-on-M streaming kernels: up to 64 rows; the wide form takes up to 128 rows, on the bf16 weights also where the
+  // layer holds FP8 codes (their token planes stop at 64 rows; 7B-shaped layer with FP8 weights, 100 rows: 83.2 ->
+  // 75.6 us against token-major tiles, 13B-shaped 138.8 -> 101.8).  Path 2 keeps token-major tiles from 65 rows.
+  const int decode_rows = L->gemm_path != 2 ? kDecWideRows : kDecMaxRows;
   const bool decode = use_umma && !gemv && !stream && R <= decode_rows;
   if (use_umma && !stream && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
-  if (decode && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
-  if (decode && L->fp8) {                          // E4M3 planes of the token rows: independent of the routing
+  if ((decode || (stream && L->fp8)) && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+  if ((decode || stream) && L->fp8 && R <= kDecMaxRows) {      // E4M3 planes of the token rows: independent of the routing
     if (decode_split_x(&L->umma, &L->decode, R, st, dep && !L->hier) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
     ++launches;
   }
@@ -522,7 +524,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     }
   } else if (stream) {
     if constexpr (std::is_same<T, bf16>::value) {
-      const int n = stream_forward(&L->umma, &L->stream, L->decode.wd_s, L->decode.wd_r, L->gr, xo, R, out,
+      const int n = stream_forward(&L->umma, &L->stream, L->fp8 ? L->decode.wd8_s : L->decode.wd_s,
+                                   L->fp8 ? L->decode.wd8_r : L->decode.wd_r, L->gr, xo, R, out,
                                    gate_up_only ? (bf16*)L->h_s : L->stream.h, L->err_word, st, ev ? ev[3] : nullptr, dep, gate_up_only);
       if (n < 0) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
       launches += n;
@@ -875,6 +878,8 @@ int cmoe_layer_quantise_fp8(cmoe_layer* L, void* stream) {
   f.w_gu8 = L->w_gu8; f.wd8 = L->wd8; f.scale_gu = L->scale_gu; f.scale_d = L->scale_d;
   f.xq_rows = kDecMaxRows;
   f.hr_rows = (size_t)kDecMaxRows * (L->cfg.top_k > 0 ? L->cfg.top_k : 1);
+  uint8_t* hq = nullptr;                             // the streamers' planes of Hd
+  float* hq_scale = nullptr;
   {
     Arena a;
     auto carve = [&](char* base) {
@@ -885,6 +890,10 @@ int cmoe_layer_quantise_fp8(cmoe_layer* L, void* stream) {
       f.x_scale = a.take<float>(f.xq_rows);
       f.hs_scale = a.take<float>(f.xq_rows);
       f.hr_scale = a.take<float>(f.hr_rows);
+      if (!L->hier) {
+        hq = a.take<uint8_t>(2 * (size_t)kStreamMaxRows * L->cfg.d_ff);
+        hq_scale = a.take<float>(kStreamMaxRows);
+      }
     };
     carve(nullptr);
     const size_t bytes = a.used + 256;
@@ -893,6 +902,10 @@ int cmoe_layer_quantise_fp8(cmoe_layer* L, void* stream) {
     carve(static_cast<char*>(L->fp8_tok));
   }
   if (!decode_plan_attach_fp8(&L->umma, &L->decode, f))
+    return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+  static_assert(kStreamMaxRows == kDecMaxRows, "the streamers read the planes of x that the decode kernels use");
+  if (L->stream.built && !stream_plan_attach_fp8(&L->umma, &L->stream, L->w_gu8, f.xq, f.x_scale, hq, hq_scale, L->scale_gu,
+                                                 L->scale_d))
     return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   L->fp8 = true;
   return CMOE_OK;

@@ -88,6 +88,8 @@ quantise_rows_fp8_kernel(const bf16* w, int rows, int cols, long long ld, uint8_
   }
 }
 
+constexpr int kSplitThreads = 256;         // threads per token row of the split
+
 // Splits bf16 rows into two E4M3 planes for the FP8 tensor-core path: with the row's power-of-two
 // scale 2^e (largest magnitude brought to at most 448), hi = E4M3(v / 2^e) and lo = E4M3(16 (v / 2^e - hi)).
 // A bf16 value has 8 significant bits, hi keeps the top 4 and the remainder is a multiple of the
@@ -95,26 +97,47 @@ quantise_rows_fp8_kernel(const bf16* w, int rows, int cols, long long ld, uint8_
 // (values under 2^-13 of the row's maximum): v = (hi + lo / 16) 2^e.  One block per row.
 __device__ __forceinline__ void split_row_e4m3(const bf16* __restrict__ row, int cols, uint8_t* __restrict__ h,
                                                uint8_t* __restrict__ l, float* __restrict__ scale_out) {
-  __shared__ float red[4];
+  constexpr int kKeep = 6;                   // chunks of 8 per thread held between the two passes
+  __shared__ float red[kSplitThreads / 32];
+  uint4 raw[kKeep];
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    const int c = 8 * (threadIdx.x + i * kSplitThreads);
+    raw[i] = c < cols ? __ldcg(reinterpret_cast<const uint4*>(row + c)) : make_uint4(0u, 0u, 0u, 0u);
+  }
   float amax = 0.0f;
-  for (int c = 8 * threadIdx.x; c < cols; c += 8 * 128) {
+  auto unpack = [](const uint4& r, float (&v)[8]) {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { v[2 * i] = __uint_as_float(w[i] << 16); v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+  };
+  auto take_max = [&](const uint4& r) {
     float v[8];
-    load8(row + c, v);
+    unpack(r, v);
 #pragma unroll
     for (int q = 0; q < 8; ++q) { const float a = fabsf(v[q]); amax = (a > amax) ? a : amax; }
-  }
+  };
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) take_max(raw[i]);
+#pragma unroll 1
+  for (int c = 8 * (threadIdx.x + kKeep * kSplitThreads); c < cols; c += 8 * kSplitThreads)
+    take_max(__ldcg(reinterpret_cast<const uint4*>(row + c)));
   amax = warp_max(amax);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
   __syncthreads();
-  const int e = pow2_scale_exponent(fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3])));
+#pragma unroll
+  for (int i = 0; i < kSplitThreads / 32; ++i) amax = fmaxf(amax, red[i]);
+  const int e = pow2_scale_exponent(amax);
   if (threadIdx.x == 0) *scale_out = ldexpf(1.0f, e);
-  for (int c = 8 * threadIdx.x; c < cols; c += 8 * 128) {
+  // 2^-e as two factors (2^-e itself may be out of range): every product is exact or far below the codes' range
+  const float f0 = ldexpf(1.0f, -(e / 2)), f1 = ldexpf(1.0f, -(e - e / 2));
+  auto convert = [&](const uint4& r, int c) {
     float v[8];
-    load8(row + c, v);
+    unpack(r, v);
     uint32_t hw[2], lw[2];
 #pragma unroll
     for (int q = 0; q < 8; q += 2) {
-      const float v0 = ldexpf(v[q], -e), v1 = ldexpf(v[q + 1], -e);
+      const float v0 = v[q] * f0 * f1, v1 = v[q + 1] * f0 * f1;
       const uint16_t hq = f32x2_to_e4m3x2(v0, v1);
       const float2 back = e4m3x2_to_f32x2(hq);
       const uint16_t lq = f32x2_to_e4m3x2((v0 - back.x) * 16.0f, (v1 - back.y) * 16.0f);
@@ -123,7 +146,15 @@ __device__ __forceinline__ void split_row_e4m3(const bf16* __restrict__ row, int
     }
     *reinterpret_cast<uint2*>(h + c) = make_uint2(hw[0], hw[1]);
     *reinterpret_cast<uint2*>(l + c) = make_uint2(lw[0], lw[1]);
+  };
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    const int c = 8 * (threadIdx.x + i * kSplitThreads);
+    if (c < cols) convert(raw[i], c);
   }
+#pragma unroll 1
+  for (int c = 8 * (threadIdx.x + kKeep * kSplitThreads); c < cols; c += 8 * kSplitThreads)
+    convert(__ldcg(reinterpret_cast<const uint4*>(row + c)), c);
 }
 
 // One segment of rows: src [rows, cols] bf16 (leading dimension ld) -> planes [2][plane_rows][cols], scales [rows].
@@ -137,7 +168,7 @@ struct SplitSegment {
 };
 
 // Blocks 0 .. a.rows-1 split the rows of segment a, the next b.rows blocks those of segment b (b.rows may be 0).
-__global__ void __launch_bounds__(128) split_rows_e4m3_kernel(const SplitSegment a, const SplitSegment b) {
+__global__ void __launch_bounds__(kSplitThreads) split_rows_e4m3_kernel(const SplitSegment a, const SplitSegment b) {
   grid_dep_wait();
   grid_dep_trigger();
   int r = blockIdx.x;

@@ -18,7 +18,14 @@
 // What the up kernel needs of the router is only the epilogue's gates when (nearly) every expert is expected to be active
 // (`dense`): then it streams from its first cycle, under the router's latency.  Otherwise the shared expert's tiles go
 // first and the routed ones follow once the router is done.  The down kernel fetches its first ring of weights before it
-// waits for the up kernel.  Registers and shared memory are sized so that the router, the up and the down kernel fit one SM
+// waits for the up kernel.
+//
+// W8 = true streams FP8 (E4M3) codes, half the bytes, into kind::f8f6f4 MMAs.  The token rows are E4M3 planes hi and lo (see
+// split_rows_e4m3_kernel), both multiplied by one MMA (N = 2 x token rows); the planes of x are written ahead of the router,
+// those of Hd by a split launch between the two kernels.  The scale of a down weight row differs from expert to expert, so the
+// down kernel accumulates one group at a time and its epilogue adds them up in registers.
+//
+// Registers and shared memory are sized so that the router, the up and the down kernel fit one SM
 // pairwise: otherwise the successor's CTAs start when the predecessor's end, and the streams pause in between.  Loops
 // whose trip count is not fixed are not unrolled: the weight streams push the code out of L2 between two forwards, and
 // every line of it that a short kernel needs is a miss to DRAM.
@@ -28,12 +35,14 @@
 // 77.8 / 82.6 -> 48.6 / 71.0 / 77.9, 13B-shaped 16 / 64 rows 79.4 / 97.4 -> 72.9 / 87.6.  In a forward of 16 rows (270 MB of
 // weights, 41 us at the copy rate) the up kernel streams for 31 us from its start under the router, its slowest CTA and the
 // hand-over cost 4, the down kernel streams for 13 and its sums take 4.  A single row stays on the CUDA-core kernels of
-// gemv.cuh (33.7 us against 46).  Fetching the down kernel's weights into L2 at the end of the up kernel was slower (it
+// gemv.cuh (33.7 us against 46).  FP8 weights: 7B-shaped 2 / 16 / 48 / 64 rows 44.4 / 48.6 / 56.0 / 58.1 -> 38.0 / 39.2 / 46.9 /
+// 49.8 us, 8B-shaped 8 / 32 / 64 rows 52.1 / 62.6 / 68.6 -> 47.8 / 50.2 / 56.5, 13B-shaped 16 / 48 rows 61.9 / 75.1 -> 49.6 / 58.5.  Fetching the down kernel's weights into L2 at the end of the up kernel was slower (it
 // delays the up kernel's last CTAs), equal runs of k blocks instead of tiles in the up kernel as well (the partial sums).
 #pragma once
 
 #include <cmath>
 
+#include "fp8.cuh"
 #include "umma_gemm.cuh"
 
 namespace cmoe {
@@ -51,6 +60,7 @@ struct StreamArgs {
   int n_rows, d, shared_w, m;
   int dense;                   // up: every routed expert is treated as active
   int tile_rows;               // up: neurons per tile (a multiple of 8)
+  int tok_rows;                // rows of the token boxes: n_rows rounded up to 16
   int stages;
   const int32_t* topk_idx;     // [rows][n_k] selected routed expert
   const float* topk_gate;
@@ -60,6 +70,11 @@ struct StreamArgs {
   float* part;                 // down: [2 * CTAs] slots of 128 x NT fp32
   int32_t* ticket;             // down: [tiles][8], zero between launches
   int32_t* err;
+  // FP8 weights: per-row power-of-two scales of the token planes (up: x rows; down: Hd rows) and of the weight rows
+  const float* tok_scale;
+  const float* scale_gu;       // [2][rows_w]: gate plane, then up plane, packed neuron order
+  const float* scale_d;        // [1 + n_r][d]: per group and output channel
+  long long rows_w;
 };
 
 __device__ __forceinline__ int atom_inc_acq_rel(int32_t* p) {
@@ -99,9 +114,9 @@ struct StreamCursor { int tile, a, kk; };
 // The down kernel's work: the k blocks of all tiles in one row, dealt to the first n_ctas CTAs in equal runs.
 struct StreamRun {
   int kb_s, kb_m, n_act, kb_tile, blocks, n_ctas;
-  __device__ __forceinline__ StreamRun(const StreamArgs& p, int n_active) {
-    kb_s = p.has_s ? (p.shared_w + kUmmaBK - 1) / kUmmaBK : 0;
-    kb_m = (p.m + kUmmaBK - 1) / kUmmaBK;
+  __device__ __forceinline__ StreamRun(const StreamArgs& p, int n_active, int bk) {
+    kb_s = p.has_s ? (p.shared_w + bk - 1) / bk : 0;
+    kb_m = (p.m + bk - 1) / bk;
     n_act = n_active;
     kb_tile = kb_s + n_act * kb_m;
     blocks = kb_tile * ((p.d + 127) / 128);
@@ -116,6 +131,10 @@ struct StreamRun {
     if (kb < kb_s) { c.a = -1; c.kk = kb; } else { c.a = (kb - kb_s) / kb_m; c.kk = kb - kb_s - c.a * kb_m; }
     return c;
   }
+  __device__ __forceinline__ int group_end(int tile_b0, int b) const {    // end of the group that block b of a tile belongs to
+    const int kb = b - tile_b0;
+    return tile_b0 + (kb < kb_s ? kb_s : kb_s + ((kb - kb_s) / kb_m + 1) * kb_m);
+  }
   __device__ __forceinline__ void advance(StreamCursor& c) const {
     if (++c.kk == (c.a < 0 ? kb_s : kb_m)) {
       c.kk = 0;
@@ -124,7 +143,7 @@ struct StreamRun {
   }
 };
 
-template <int NT>
+template <int NT, bool W8>
 __global__ void __maxnreg__(96)
 stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const StreamArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -140,8 +159,11 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
   float* gate_tables = reinterpret_cast<float*>(tail + kStreamTail);    // [8 warps][NT]
   const uint32_t ring = base + (kStreamTail + 8 * NT * 4 + 1023) / 1024 * 1024;
   const int h = p.tile_rows, stages = p.stages;
-  const uint32_t plane = h * 128, stage_bytes = 2 * plane + NT * 128;
-  constexpr int kTmemCols = 4 * NT < 32 ? 32 : 4 * NT;
+  const uint32_t plane = h * 128, stage_bytes = 2 * plane + (W8 ? 2 : 1) * p.tok_rows * 128;
+  constexpr int kBK = W8 ? 2 * kUmmaBK : kUmmaBK;              // k per stage: 128 bytes of a weight row
+  constexpr int kAcc = (W8 ? 2 : 1) * NT;                       // columns of one accumulator
+  constexpr int kBufs = 2 * 2 * kAcc > 256 ? 1 : 2;             // the down kernel's 256 columns have to fit as well
+  constexpr int kTmemCols = kBufs * 2 * kAcc < 32 ? 32 : kBufs * 2 * kAcc;
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -164,7 +186,7 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
   const uint32_t tmem_base = *tmem_slot;
 
   const int n_ctas = gridDim.x;
-  const int k_blocks = (p.d + kUmmaBK - 1) / kUmmaBK;
+  const int k_blocks = (p.d + kBK - 1) / kBK;
   const int tiles_s = p.has_s ? (p.shared_w + h - 1) / h : 0, tiles_m = (p.m + h - 1) / h;
   // group of a tile: -1 the shared expert, else a routed expert; first neuron inside the group; its weight row
   struct Tile { int j, n0, width, w_row0; };
@@ -204,8 +226,9 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
         if (elect_one()) {
           const uint32_t fb = full0 + 8 * rp.s, sw = ring + rp.s * stage_bytes;
           mbar_expect_tx(fb, stage_bytes);
-          tma_load_3d(sw, &tm_w, fb, kb * kUmmaBK, row, 0);          // gate rows, then the up rows behind them
-          tma_load_2d(sw + 2 * plane, &tm_x, fb, kb * kUmmaBK, 0);
+          tma_load_3d(sw, &tm_w, fb, kb * kBK, row, 0);              // gate rows, then the up rows behind them
+          if (W8) tma_load_3d(sw + 2 * plane, &tm_x, fb, kb * kBK, 0, 0);        // hi rows, then the lo rows
+          else tma_load_2d(sw + 2 * plane, &tm_x, fb, kb * kBK, 0);
         }
         __syncwarp();
       }
@@ -213,7 +236,7 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
     if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);             // let copies in flight land
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
-    const uint32_t idesc = umma_idesc((p.n_rows + 15) & ~15);
+    const uint32_t idesc = W8 ? umma_idesc_e4m3(2 * p.tok_rows) : umma_idesc(p.tok_rows);
     RingPos rp;
     uint32_t seg = 0;
     bool ok = true, listed = p.dense != 0;
@@ -226,10 +249,10 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
         total = tiles_s + *n_active * tiles_m;
         if (t >= total) break;
       }
-      const uint32_t buf = seg & 1, use = seg >> 1;
+      const uint32_t buf = seg % kBufs, use = seg / kBufs;
       if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t d_tmem = tmem_base + buf * 2 * NT;
+      const uint32_t d_tmem = tmem_base + buf * 2 * kAcc;
 #pragma unroll 1
       for (int kb = 0; kb < k_blocks; ++kb, rp.next(stages)) {
         if (!mbar_wait_warp(full0 + 8 * rp.s, rp.ph, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
@@ -240,8 +263,13 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
           for (int k = 0; k < 4; ++k) {
             const uint32_t acc = (kb != 0 || k != 0) ? 1u : 0u;
             const uint64_t x_desc = umma_smem_desc(sw + 2 * plane + k * 32);
-            umma_bf16(d_tmem, umma_smem_desc(sw + k * 32), x_desc, idesc, acc);
-            umma_bf16(d_tmem + NT, umma_smem_desc(sw + plane + k * 32), x_desc, idesc, acc);
+            if (W8) {
+              umma_e4m3(d_tmem, umma_smem_desc(sw + k * 32), x_desc, idesc, acc);
+              umma_e4m3(d_tmem + kAcc, umma_smem_desc(sw + plane + k * 32), x_desc, idesc, acc);
+            } else {
+              umma_bf16(d_tmem, umma_smem_desc(sw + k * 32), x_desc, idesc, acc);
+              umma_bf16(d_tmem + kAcc, umma_smem_desc(sw + plane + k * 32), x_desc, idesc, acc);
+            }
           }
           umma_commit(empty0 + 8 * rp.s);
         }
@@ -256,6 +284,9 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
     float* gate = gate_tables + (warp - 2) * NT;
     grid_dep_wait();                                  // the router's results are final: the down kernel may become
     grid_dep_trigger();                               // resident and list the active experts
+    float ts_lo = 1.0f, ts_hi = 1.0f;                 // W8: this lane's token scales
+    if (W8 && lane < p.n_rows) ts_lo = __ldcg(p.tok_scale + lane);
+    if (W8 && lane + 32 < p.n_rows) ts_hi = __ldcg(p.tok_scale + lane + 32);
     bool ok = true, listed = p.dense != 0;
     int total = listed ? tiles_s + *n_active * tiles_m : tiles_s;
     uint32_t seg = 0;
@@ -280,20 +311,38 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
         }
         __syncwarp();
       }
-      const uint32_t buf = seg & 1, use = seg >> 1;
-      if (!mbar_wait_warp(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t taddr = tmem_base + buf * 2 * NT + ((uint32_t)(quad * 32) << 16);
       const int r = quad * 32 + lane, nn = tl.n0 + r;
       const bool live = r < h && nn < tl.width;
+      float sc_a = 1.0f, sc_u = 1.0f;                 // W8: scales of this thread's weight rows
+      if (W8 && live) {
+        sc_a = __ldg(p.scale_gu + tl.w_row0 + nn);
+        sc_u = __ldg(p.scale_gu + p.rows_w + tl.w_row0 + nn);
+      }
       bf16* dst = p.h + tl.w_row0 + nn;
+      const uint32_t buf = seg % kBufs, use = seg / kBufs;
+      if (!mbar_wait_warp(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + buf * 2 * kAcc + ((uint32_t)(quad * 32) << 16);
       const bool routed = tl.j >= 0;
 #pragma unroll 1
       for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
         float a[8], u[8];
         tmem_ld8(taddr + c0, a);
-        tmem_ld8(taddr + NT + c0, u);
-        tmem_ld_wait();
+        tmem_ld8(taddr + kAcc + c0, u);
+        if constexpr (W8) {                           // (hi + lo / 16) x weight row scale x token scale
+          float al[8], ul[8];
+          tmem_ld8(taddr + p.tok_rows + c0, al);
+          tmem_ld8(taddr + kAcc + p.tok_rows + c0, ul);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float ts = __shfl_sync(0xffffffffu, c0 < 32 ? ts_lo : ts_hi, (c0 + q) & 31);
+            a[q] = fmaf(al[q], 0.0625f, a[q]) * (sc_a * ts);
+            u[q] = fmaf(ul[q], 0.0625f, u[q]) * (sc_u * ts);
+          }
+        } else {
+          tmem_ld_wait();
+        }
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           a[q] = swiglu_fast(a[q], u[q]);
@@ -321,7 +370,7 @@ stream_up_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
   }
 }
 
-template <int NT>
+template <int NT, bool W8>
 __global__ void __maxnreg__(104)
 stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_constant__ CUtensorMap tm_w_r,
                    const __grid_constant__ CUtensorMap tm_h_s, const __grid_constant__ CUtensorMap tm_h_r,
@@ -337,8 +386,11 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
   int* active = reinterpret_cast<int*>(tail + 192);             // [32]
   const uint32_t ring = base + 1024;
   const int stages = p.stages;
-  constexpr uint32_t kWBytes = 128 * 128, kStageBytes = kWBytes + NT * 128;
-  constexpr int kTmemCols = 2 * NT < 32 ? 32 : 2 * NT;
+  constexpr uint32_t kWBytes = 128 * 128;
+  const uint32_t stage_bytes = kWBytes + (W8 ? 2 : 1) * p.tok_rows * 128;
+  constexpr int kBK = W8 ? 2 * kUmmaBK : kUmmaBK;
+  constexpr int kAcc = (W8 ? 2 : 1) * NT;
+  constexpr int kTmemCols = 2 * kAcc < 32 ? 32 : 2 * kAcc;
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -362,20 +414,25 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   const int cta = blockIdx.x;
-  const StreamRun run(p, *n_active);
+  const StreamRun run(p, *n_active, kBK);
   const int kb_tile = run.kb_tile, lo = run.lo(cta), hi = run.lo(cta + 1);
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
     auto load_weights = [&](int s, const StreamCursor& c) {
-      const uint32_t fb = full0 + 8 * s, sw = ring + s * kStageBytes;
-      if (c.a < 0) tma_load_3d(sw, &tm_w_s, fb, c.kk * kUmmaBK, c.tile * 128, 0);
-      else tma_load_4d(sw, &tm_w_r, fb, c.kk * kUmmaBK, c.tile * 128, active[c.a], 0);
+      const uint32_t fb = full0 + 8 * s, sw = ring + s * stage_bytes;
+      if (c.a < 0) tma_load_3d(sw, &tm_w_s, fb, c.kk * kBK, c.tile * 128, 0);
+      else tma_load_4d(sw, &tm_w_r, fb, c.kk * kBK, c.tile * 128, active[c.a], 0);
     };
     auto load_tokens = [&](int s, const StreamCursor& c) {
-      const uint32_t fb = full0 + 8 * s, st = ring + s * kStageBytes + kWBytes;
-      if (c.a < 0) tma_load_2d(st, &tm_h_s, fb, c.kk * kUmmaBK, 0);
-      else tma_load_3d(st, &tm_h_r, fb, c.kk * kUmmaBK, active[c.a], 0);
+      const uint32_t fb = full0 + 8 * s, st = ring + s * stage_bytes + kWBytes;
+      if (W8) {                                       // hi rows, then the lo rows
+        if (c.a < 0) tma_load_3d(st, &tm_h_s, fb, c.kk * kBK, 0, 0);
+        else tma_load_4d(st, &tm_h_r, fb, c.kk * kBK, active[c.a], 0, 0);
+      } else {
+        if (c.a < 0) tma_load_2d(st, &tm_h_s, fb, c.kk * kBK, 0);
+        else tma_load_3d(st, &tm_h_r, fb, c.kk * kBK, active[c.a], 0);
+      }
     };
     bool ok = true;
     const int ahead = min(stages, hi - lo);
@@ -383,7 +440,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
       StreamCursor c = run.cursor(lo), c2 = c;
 #pragma unroll 1
       for (int i = 0; i < ahead; ++i, run.advance(c)) {                       // the first ring of weights needs nothing
-        if (elect_one()) { mbar_expect_tx(full0 + 8 * i, kStageBytes); load_weights(i, c); }
+        if (elect_one()) { mbar_expect_tx(full0 + 8 * i, stage_bytes); load_weights(i, c); }
         __syncwarp();
       }
       grid_dep_wait();                                                    // Hd is complete
@@ -398,7 +455,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
       for (int b = lo + ahead; b < hi; ++b, run.advance(c), rp.next(stages)) {
         if (!mbar_wait_warp(empty0 + 8 * rp.s, rp.ph ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         if (elect_one()) {
-          mbar_expect_tx(full0 + 8 * rp.s, kStageBytes);
+          mbar_expect_tx(full0 + 8 * rp.s, stage_bytes);
           load_weights(rp.s, c);
           load_tokens(rp.s, c);
         }
@@ -408,27 +465,30 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
     if (!ok) for (int i = 0; i < 200; ++i) __nanosleep(1000);             // let copies in flight land
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
-    const uint32_t idesc = umma_idesc((p.n_rows + 15) & ~15);
+    const uint32_t idesc = W8 ? umma_idesc_e4m3(2 * p.tok_rows) : umma_idesc(p.tok_rows);
     RingPos rp;
     uint32_t seg = 0;
     bool ok = true;
 #pragma unroll 1
     for (int b = lo; b < hi && ok; ++seg) {
-      const int end = min(hi, (b / kb_tile + 1) * kb_tile);
+      const int tile_b0 = b / kb_tile * kb_tile;
+      int end = min(hi, tile_b0 + kb_tile);
+      if (W8) end = min(end, run.group_end(tile_b0, b));          // scales differ from group to group: one accumulation each
       const uint32_t buf = seg & 1, use = seg >> 1;
       if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t d_tmem = tmem_base + buf * NT;
+      const uint32_t d_tmem = tmem_base + buf * kAcc;
       uint32_t acc = 0;
 #pragma unroll 1
       for (; b < end; ++b, rp.next(stages)) {
         if (!mbar_wait_warp(full0 + 8 * rp.s, rp.ph, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t sw = ring + rp.s * kStageBytes;
+        const uint32_t sw = ring + rp.s * stage_bytes;
         if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            umma_bf16(d_tmem, umma_smem_desc(sw + k * 32), umma_smem_desc(sw + kWBytes + k * 32), idesc, k == 0 ? acc : 1u);
+            (W8 ? umma_e4m3 : umma_bf16)(d_tmem, umma_smem_desc(sw + k * 32), umma_smem_desc(sw + kWBytes + k * 32), idesc,
+                                         k == 0 ? acc : 1u);
           umma_commit(empty0 + 8 * rp.s);
         }
         __syncwarp();
@@ -441,88 +501,118 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
     // ------------------------------------------------------------ epilogue (warps 2..9)
     const int quad = warp & 3, half = (warp - 2) >> 2;              // 8-column chunks half, half + 2, ...
     const int slot_q = quad * 32 + lane;
+    constexpr int kCh = NT / 16;                                    // this warp's chunks: columns 16 i + 8 half
     grid_dep_wait();                                                // also orders this kernel's stores to `out`
+    float ts_lo = 1.0f, ts_hi = 1.0f;                               // W8: this lane's token scales
+    if (W8 && lane < p.n_rows) ts_lo = __ldcg(p.tok_scale + lane);
+    if (W8 && lane + 32 < p.n_rows) ts_hi = __ldcg(p.tok_scale + lane + 32);
     bool ok = true;
     uint32_t seg = 0;
 #pragma unroll 1
-    for (int b = lo; b < hi && ok; ++seg) {
+    for (int b = lo; b < hi && ok;) {
       const int tile = b / kb_tile, tile_b0 = tile * kb_tile;
       const int end = min(hi, tile_b0 + kb_tile);
       const bool whole = b == tile_b0 && end == tile_b0 + kb_tile;
-      b = end;
       const int ch = tile * 128 + slot_q;
-      const uint32_t buf = seg & 1, use = seg >> 1;
+      float v[kCh][8];
+#pragma unroll
+      for (int i = 0; i < kCh; ++i)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[i][q] = 0.0f;
+#pragma unroll 1
+      for (; b < end; ++seg) {
+        float sc = 1.0f;                                            // W8: scale of this thread's channel in the group
+        if (W8) {
+          const int kb = b - tile_b0;
+          const int g = kb < run.kb_s ? 0 : 1 + active[(kb - run.kb_s) / run.kb_m];
+          if (ch < p.d) sc = __ldg(p.scale_d + (size_t)g * p.d + ch);
+        }
+        b = W8 ? min(end, run.group_end(tile_b0, b)) : end;
+        const uint32_t buf = seg & 1, use = seg >> 1;
+        if (!mbar_wait_warp(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + buf * kAcc + ((uint32_t)(quad * 32) << 16) + 8 * half;
+#pragma unroll
+        for (int i = 0; i < kCh; ++i)
+          if (16 * i + 8 * half < p.n_rows) {
+            float t[8];
+            tmem_ld8(taddr + 16 * i, t);
+            if constexpr (W8) {
+              float l[8];
+              tmem_ld8(taddr + p.tok_rows + 16 * i, l);
+              tmem_ld_wait();
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[i][q] = fmaf(fmaf(l[q], 0.0625f, t[q]), sc, v[i][q]);
+            } else {
+              tmem_ld_wait();
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[i][q] = t[q];
+            }
+          }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce0 + 8 * buf);
+      }
+      if (!ok) break;
+      auto store8 = [&](int c0, const float (&r)[8]) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float y = r[q];
+          if (W8) y *= __shfl_sync(0xffffffffu, c0 < 32 ? ts_lo : ts_hi, (c0 + q) & 31);
+          if (ch < p.d && c0 + q < p.n_rows) p.out[(size_t)(c0 + q) * p.d + ch] = __float2bfloat16_rn(y);
+        }
+      };
+      if (whole) {
+#pragma unroll
+        for (int i = 0; i < kCh; ++i)
+          if (16 * i + 8 * half < p.n_rows) store8(16 * i + 8 * half, v[i]);
+        continue;
+      }
       int32_t* tk = p.ticket + (size_t)tile * 8 + (warp - 2);
       const int first = run.cta_of(tile_b0), nz = run.cta_of(tile_b0 + kb_tile - 1) - first + 1, own = cta - first;
-      const uint32_t taddr = tmem_base + buf * NT + ((uint32_t)(quad * 32) << 16);
       // slot of the tile's contributor z: the first one's is its CTA's second, the others' their first; [column / 4][128][4]
       auto slot = [&](int z) {
         return reinterpret_cast<float4*>(p.part) + (size_t)(2 * (first + z) + (z == 0 ? 1 : 0)) * (32 * NT) + slot_q;
       };
-      auto store8 = [&](int c0, const float (&v)[8]) {
-        if (ch < p.d) {
+      float4* mine = slot(own) + 2 * half * 128;
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (c0 + q < p.n_rows) p.out[(size_t)(c0 + q) * p.d + ch] = __float2bfloat16_rn(v[q]);
+      for (int i = 0; i < kCh; ++i)
+        if (16 * i + 8 * half < p.n_rows) {
+          __stcg(mine + (size_t)(4 * i) * 128, make_float4(v[i][0], v[i][1], v[i][2], v[i][3]));
+          __stcg(mine + (size_t)(4 * i + 1) * 128, make_float4(v[i][4], v[i][5], v[i][6], v[i][7]));
         }
-      };
-      if (!mbar_wait_warp(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
-      tc_fence_after();
-      if (whole) {
-#pragma unroll 1
-        for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
-          float v[8];
-          tmem_ld8(taddr + c0, v);
-          tmem_ld_wait();
-          store8(c0, v);
-        }
-      } else {
-        float4* mine = slot(own);
-#pragma unroll 1
-        for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
-          float v[8];
-          tmem_ld8(taddr + c0, v);
-          tmem_ld_wait();
-          __stcg(mine + (size_t)(c0 / 4) * 128, make_float4(v[0], v[1], v[2], v[3]));
-          __stcg(mine + (size_t)(c0 / 4 + 1) * 128, make_float4(v[4], v[5], v[6], v[7]));
-        }
-        __threadfence();
-        __syncwarp();
-        int taken = 0;
-        if (lane == 0) taken = atom_inc_acq_rel(tk);
-        taken = __shfl_sync(0xffffffffu, taken, 0);
-        if (taken == nz - 1) {                                      // every contribution is in: add them in CTA order
-          __threadfence();
-#pragma unroll 1
-          for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
-            float v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = 0.0f;
-#pragma unroll 1
-            for (int z0 = 0; z0 < nz; z0 += 6) {                    // six in flight
-              float4 t[6][2];
-#pragma unroll
-              for (int z = 0; z < 6; ++z)
-                if (z0 + z < nz) {
-                  const float4* s = slot(z0 + z) + (size_t)(c0 / 4) * 128;
-                  t[z][0] = __ldcg(s);
-                  t[z][1] = __ldcg(s + 128);
-                }
-#pragma unroll
-              for (int z = 0; z < 6; ++z)
-                if (z0 + z < nz) {
-                  v[0] += t[z][0].x; v[1] += t[z][0].y; v[2] += t[z][0].z; v[3] += t[z][0].w;
-                  v[4] += t[z][1].x; v[5] += t[z][1].y; v[6] += t[z][1].z; v[7] += t[z][1].w;
-                }
-            }
-            store8(c0, v);
-          }
-          if (lane == 0) *tk = 0;                                   // ready for the next launch
-        }
-      }
-      tc_fence_before();
+      __threadfence();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acce0 + 8 * buf);
+      int taken = 0;
+      if (lane == 0) taken = atom_inc_acq_rel(tk);
+      taken = __shfl_sync(0xffffffffu, taken, 0);
+      if (taken != nz - 1) continue;
+      __threadfence();                                              // every contribution is in: add them in CTA order
+#pragma unroll 1
+      for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
+        float r[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) r[q] = 0.0f;
+#pragma unroll 1
+        for (int z0 = 0; z0 < nz; z0 += 6) {                        // six in flight
+          float4 t[6][2];
+#pragma unroll
+          for (int z = 0; z < 6; ++z)
+            if (z0 + z < nz) {
+              const float4* sl = slot(z0 + z) + (size_t)(c0 / 4) * 128;
+              t[z][0] = __ldcg(sl);
+              t[z][1] = __ldcg(sl + 128);
+            }
+#pragma unroll
+          for (int z = 0; z < 6; ++z)
+            if (z0 + z < nz) {
+              r[0] += t[z][0].x; r[1] += t[z][0].y; r[2] += t[z][0].z; r[3] += t[z][0].w;
+              r[4] += t[z][1].x; r[5] += t[z][1].y; r[6] += t[z][1].z; r[7] += t[z][1].w;
+            }
+        }
+        store8(c0, r);
+      }
+      if (lane == 0) *tk = 0;                                       // ready for the next launch
     }
   }
   tc_fence_before();
@@ -535,13 +625,18 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
 
 // ----------------------------------------------------------------------------- host
 struct StreamPlan {
-  bool built = false;
+  bool built = false, fp8 = false;
   bf16* h = nullptr;                // Hd [kStreamMaxRows][d_ff]
   float* part = nullptr;
   int32_t* ticket = nullptr;
   CUtensorMap w_gu[16];             // gate/up rows, boxes of 64 k x 8 (i + 1) rows x 2 planes
-  CUtensorMap h_s[3], h_r[3];       // Hd: shared columns; routed columns per expert; boxes of 16 << i rows
-  CUtensorMap x[3];                 // x of this forward
+  CUtensorMap h_s[4], h_r[4];       // Hd: shared columns; routed columns per expert; boxes of 16 (i + 1) rows
+  CUtensorMap x[4];                 // x of this forward
+  // FP8 weights (stream_plan_attach_fp8): codes of the gate/up rows, boxes of 128 k; E4M3 planes of x and of Hd
+  CUtensorMap w_gu8[16], xq[4], hq_s[4], hq_r[4];
+  uint8_t* hq = nullptr;            // [2][kStreamMaxRows][d_ff]
+  float* hq_scale = nullptr;        // [kStreamMaxRows]
+  const float *x_scale = nullptr, *scale_gu = nullptr, *scale_d = nullptr;
 };
 
 inline size_t stream_part_floats(int max_rows) {       // 2 slots per CTA, 128 rows x token columns
@@ -551,25 +646,29 @@ inline size_t stream_part_floats(int max_rows) {       // 2 slots per CTA, 128 r
 }
 inline size_t stream_tickets(int d) { return 8 * (size_t)((d + 127) / 128); }
 
-// Ring sizes.  Up to 64 token columns the two kernels (and the router) share an SM: 228 KB, 1 KB of it per block.
-inline int stream_up_stages(int h, int nt) {
-  const int budget = 118 * 1024, n = budget / (h * 256 + nt * 128);
+// Ring sizes: the two kernels (and the router) share an SM: 228 KB, 1 KB of it per block.  tok: bytes of a stage's token rows.
+// FP8 with 64 token rows (16 KB a stage) gives that up for tiles high enough to need one round (8B-shaped layer, 64
+// rows: 66.8 -> 56.5 us).
+inline int stream_up_stages(int h, int tok) {
+  const int n = (tok >= 16384 ? 136 : 120) * 1024 / (h * 256 + tok);
   return n > 8 ? 8 : n;
 }
-inline int stream_up_smem(int h, int nt, int stages) {
+inline int stream_up_smem(int h, int tok, int nt, int stages) {
   // a tile's MMAs read 128 rows per plane: the last stage's up plane may be read past the ring's end
-  const int ring = stages * (h * 256 + nt * 128), over = (stages - 1) * (h * 256 + nt * 128) + h * 128 + 128 * 128;
+  const int ring = stages * (h * 256 + tok), over = (stages - 1) * (h * 256 + tok) + h * 128 + 128 * 128;
   return 1024 + (kStreamTail + 32 * nt + 1023) / 1024 * 1024 + (ring > over ? ring : over);
 }
-inline int stream_down_stages(int nt) {
-  const int budget = 90 * 1024, n = budget / (16384 + nt * 128);
+inline int stream_down_stages(int tok) {
+  const int n = 98 * 1024 / (16384 + tok);
   return n > 8 ? 8 : n;
 }
-inline int stream_down_smem(int nt) { return 2048 + stream_down_stages(nt) * (16384 + nt * 128); }
+inline int stream_down_smem(int tok) { return 2048 + stream_down_stages(tok) * (16384 + tok); }
 
 template <int NT> inline cudaError_t stream_allow_smem() {
-  cudaError_t e = allow_smem(stream_up_kernel<NT>, 227 * 1024);
-  if (e == cudaSuccess) e = allow_smem(stream_down_kernel<NT>, 227 * 1024);
+  cudaError_t e = allow_smem(stream_up_kernel<NT, false>, 227 * 1024);
+  if (e == cudaSuccess) e = allow_smem(stream_down_kernel<NT, false>, 227 * 1024);
+  if (e == cudaSuccess) e = allow_smem(stream_up_kernel<NT, true>, 227 * 1024);
+  if (e == cudaSuccess) e = allow_smem(stream_down_kernel<NT, true>, 227 * 1024);
   return e;
 }
 
@@ -589,8 +688,8 @@ inline bool stream_plan_create(UmmaPlan* P, StreamPlan* S) {
     const cuuint32_t box[3] = {kUmmaBK, (cuuint32_t)(8 * (i + 1)), 2};
     ok = umma_encode(P, &S->w_gu[i], P->buf.w_gate_up, 3, dims, str, box, "gate/up weights (stream)");
   }
-  for (int i = 0; i < 3 && ok; ++i) {
-    const cuuint32_t rows = 16u << i;
+  for (int i = 0; i < 4 && ok; ++i) {
+    const cuuint32_t rows = 16u * (i + 1);
     if (P->has_s) {
       const cuuint64_t dims[2] = {(cuuint64_t)s.shared_width, (cuuint64_t)kStreamMaxRows};
       const cuuint64_t str[1] = {rows_w * 2};
@@ -618,6 +717,57 @@ inline bool stream_plan_create(UmmaPlan* P, StreamPlan* S) {
   return true;
 }
 
+// FP8 codes and token planes of a quantised layer, all owned by the caller: w_gu8 [2][d_ff][d], xq [2][kStreamMaxRows][d],
+// hq [2][kStreamMaxRows][d_ff]; d, m and the shared width are multiples of 16.
+inline bool stream_plan_attach_fp8(UmmaPlan* P, StreamPlan* S, const void* w_gu8, const uint8_t* xq, const float* x_scale,
+                                   uint8_t* hq, float* hq_scale, const float* scale_gu, const float* scale_d) {
+  const UmmaShape& s = P->shape;
+  const cuuint64_t d = s.d, rows_w = s.d_ff, plane_rows = kStreamMaxRows;
+  auto encode8 = [&](CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* str,
+                     const cuuint32_t* box, const char* what) {
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = P->encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, (cuuint32_t)rank, const_cast<void*>(base), dims, str,
+                                 box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+      snprintf(P->error, sizeof(P->error), "cuTensorMapEncodeTiled(%s) failed with CUresult %d", what, (int)r);
+      return false;
+    }
+    return true;
+  };
+  bool ok = true;
+  for (int i = 0; i < 16 && ok; ++i) {
+    const cuuint64_t dims[3] = {d, rows_w, 2}, str[2] = {d, rows_w * d};
+    const cuuint32_t box[3] = {2 * kUmmaBK, (cuuint32_t)(8 * (i + 1)), 2};
+    ok = encode8(&S->w_gu8[i], w_gu8, 3, dims, str, box, "FP8 gate/up weights (stream)");
+  }
+  for (int i = 0; i < 4 && ok; ++i) {
+    const cuuint32_t rows = 16u * (i + 1);
+    {
+      const cuuint64_t dims[3] = {d, plane_rows, 2}, str[2] = {d, plane_rows * d};
+      const cuuint32_t box[3] = {2 * kUmmaBK, rows, 2};
+      ok = encode8(&S->xq[i], xq, 3, dims, str, box, "E4M3 planes of x (stream)");
+    }
+    if (ok && P->has_s) {
+      const cuuint64_t dims[3] = {(cuuint64_t)s.shared_width, plane_rows, 2}, str[2] = {rows_w, plane_rows * rows_w};
+      const cuuint32_t box[3] = {2 * kUmmaBK, rows, 2};
+      ok = encode8(&S->hq_s[i], hq, 3, dims, str, box, "E4M3 planes of Hd shared");
+    }
+    if (ok && P->has_r) {
+      const cuuint64_t dims[4] = {(cuuint64_t)s.m, (cuuint64_t)s.n_r, plane_rows, 2};
+      const cuuint64_t str[3] = {(cuuint64_t)s.m, rows_w, plane_rows * rows_w};
+      const cuuint32_t box[4] = {2 * kUmmaBK, 1, rows, 2};
+      ok = encode8(&S->hq_r[i], hq + s.shared_width, 4, dims, str, box, "E4M3 planes of Hd routed");
+    }
+    if (!P->has_s) S->hq_s[i] = S->hq_r[i];
+    if (!P->has_r) S->hq_r[i] = S->hq_s[i];
+  }
+  if (!ok) return false;
+  S->hq = hq; S->hq_scale = hq_scale; S->x_scale = x_scale; S->scale_gu = scale_gu; S->scale_d = scale_d;
+  S->fp8 = true;
+  return true;
+}
+
 // Experts expected to be active, and whether to treat all as active: when the weights streamed in vain are expected to
 // take less time than the part of the router's latency that is hidden in return (about 4 us, 24 MB of the stream).
 inline double stream_expected_active(const UmmaShape& s, int n_rows) {
@@ -634,66 +784,79 @@ inline int stream_likely_active(const UmmaShape& s, int n_rows, double active) {
   if (hi > s.n_r) hi = s.n_r;
   return (long long)hi > (long long)n_rows * s.n_k ? n_rows * s.n_k : hi;
 }
-inline bool stream_dense(const UmmaShape& s, double active) { return (s.n_r - active) * s.m * 4.0 * s.d < 24e6; }
+inline bool stream_dense(const UmmaShape& s, double active, bool w8) {
+  return (s.n_r - active) * s.m * (w8 ? 2.0 : 4.0) * s.d < 24e6;
+}
 
 // Neurons per tile: the height whose rounds over the SMs take the least time for the expected tiles.  A round is bound by
 // its weight bytes, the token rows that go with each block (from L2, counted a third) and the MMAs of a block (at least the
 // time of some 8 KB of the stream).
-inline int stream_pick_rows(const UmmaShape& s, int active, int nt, int n_sms) {
+inline int stream_pick_rows(const UmmaShape& s, int active, int tok, int n_sms) {
   int best = 64;
   double best_cost = 1e30;
   for (int h = 128; h >= 16; h -= 8) {
-    if (stream_up_stages(h, nt) < 3) continue;
+    if (stream_up_stages(h, tok) < 3) continue;
     const int tiles = (s.shared_width + h - 1) / h + active * ((s.m + h - 1) / h);
     const int rounds = tiles > 0 ? (tiles + n_sms - 1) / n_sms : 1;
-    const double bytes = h * 256.0 + nt * 128.0 / 3;
+    const double bytes = h * 256.0 + tok / 3.0;
     const double cost = rounds * (bytes < 8192 ? 8192 : bytes);
     if (cost < best_cost * 0.999) { best_cost = cost; best = h; }
   }
   return best;
 }
 
-template <int NT>
+template <int NT, bool W8>
 inline void stream_launch(const UmmaPlan* P, const StreamPlan* S, const CUtensorMap& wd_s, const CUtensorMap& wd_r, int bi,
                           StreamArgs a, cudaStream_t st, cudaEvent_t mid, bool dep, bool gate_up_only) {
-  a.stages = stream_up_stages(a.tile_rows, NT);
-  launch_kernel(dep, stream_up_kernel<NT>, dim3(P->n_sms), dim3(kStreamThreads), stream_up_smem(a.tile_rows, NT, a.stages), st,
-                S->w_gu[a.tile_rows / 8 - 1], S->x[bi], a);
+  const int tok = (W8 ? 2 : 1) * a.tok_rows * 128, wi = a.tile_rows / 8 - 1;
+  a.stages = stream_up_stages(a.tile_rows, tok);
+  launch_kernel(dep, stream_up_kernel<NT, W8>, dim3(P->n_sms), dim3(kStreamThreads),
+                stream_up_smem(a.tile_rows, tok, NT, a.stages), st, W8 ? S->w_gu8[wi] : S->w_gu[wi], W8 ? S->xq[bi] : S->x[bi], a);
   if (mid) cudaEventRecord(mid, st);
   if (gate_up_only) return;
-  a.stages = stream_down_stages(NT);
-  launch_kernel(dep, stream_down_kernel<NT>, dim3(P->n_sms), dim3(kStreamThreads), stream_down_smem(NT), st, wd_s, wd_r,
-                S->h_s[bi], S->h_r[bi], a);
+  if (W8) {                                       // E4M3 planes of Hd
+    const SplitSegment hd{S->h, a.n_rows, a.ld_h, (long long)a.ld_h, S->hq, (long long)kStreamMaxRows, S->hq_scale};
+    launch_kernel(dep, split_rows_e4m3_kernel, dim3(a.n_rows), dim3(kSplitThreads), 0, st, hd, SplitSegment{});
+    a.tok_scale = S->hq_scale;
+  }
+  a.stages = stream_down_stages(tok);
+  launch_kernel(dep, stream_down_kernel<NT, W8>, dim3(P->n_sms), dim3(kStreamThreads), stream_down_smem(tok), st, wd_s, wd_r,
+                W8 ? S->hq_s[bi] : S->h_s[bi], W8 ? S->hq_r[bi] : S->h_r[bi], a);
 }
 
 // Both streamers for n_rows <= kStreamMaxRows rows of x; `h`: where the up kernel writes (Hd, or H of an all-shared
-// layer when only the gate/up part is wanted).  Returns the number of launches or -1.
+// layer when only the gate/up part is wanted).  FP8 layers: the planes of x have been written.  Returns the number of
+// launches or -1.
 inline int stream_forward(UmmaPlan* P, StreamPlan* S, const CUtensorMap& wd_s, const CUtensorMap& wd_r, const GroupRows* gr,
                           const void* x, int n_rows, bf16* out, bf16* h, int32_t* err_word, cudaStream_t st,
                           cudaEvent_t mid, bool dep, bool gate_up_only) {
   const UmmaShape& s = P->shape;
-  const int bi = n_rows <= 16 ? 0 : (n_rows <= 32 ? 1 : 2);
-  if (!umma_encode_rows(P, &S->x[bi], x, (size_t)n_rows, (size_t)s.d, 16 << bi, "x (stream)")) return -1;
+  const int bi = (n_rows + 15) / 16 - 1;
+  const bool w8 = S->fp8;
+  if (!w8 && !umma_encode_rows(P, &S->x[bi], x, (size_t)n_rows, (size_t)s.d, 16 * (bi + 1), "x (stream)")) return -1;
   const double active = P->has_r ? stream_expected_active(s, n_rows) : 0.0;
   StreamArgs a{};
   a.gr = gr; a.has_s = P->has_s; a.n_r = P->has_r ? s.n_r : 0; a.n_k = s.n_k;
   a.n_rows = n_rows; a.d = s.d; a.shared_w = s.shared_width; a.m = s.m;
-  a.dense = !P->has_r || stream_dense(s, active);
-  a.tile_rows = stream_pick_rows(s, a.dense && P->has_r ? s.n_r : stream_likely_active(s, n_rows, active), 16 << bi, P->n_sms);
+  a.dense = !P->has_r || stream_dense(s, active, w8);
+  a.tok_rows = 16 * (bi + 1);
+  a.tile_rows = stream_pick_rows(s, a.dense && P->has_r ? s.n_r : stream_likely_active(s, n_rows, active),
+                                 (w8 ? 2 : 1) * a.tok_rows * 128, P->n_sms);
   a.topk_idx = P->buf.topk_idx; a.topk_gate = P->buf.topk_gate;
   a.h = h; a.ld_h = s.d_ff; a.out = out;
   a.part = S->part; a.ticket = S->ticket; a.err = err_word;
-  switch (bi) {
-    case 0: stream_launch<16>(P, S, wd_s, wd_r, bi, a, st, mid, dep, gate_up_only); break;
-    case 1: stream_launch<32>(P, S, wd_s, wd_r, bi, a, st, mid, dep, gate_up_only); break;
-    default: stream_launch<64>(P, S, wd_s, wd_r, bi, a, st, mid, dep, gate_up_only); break;
-  }
+  a.tok_scale = S->x_scale; a.scale_gu = S->scale_gu; a.scale_d = S->scale_d; a.rows_w = s.d_ff;
+#define CMOE_STREAM(NT) (w8 ? stream_launch<NT, true> : stream_launch<NT, false>)(P, S, wd_s, wd_r, bi, a, st, mid, dep, gate_up_only)
+  if (bi == 0) CMOE_STREAM(16);
+  else if (bi == 1) CMOE_STREAM(32);
+  else CMOE_STREAM(64);
+#undef CMOE_STREAM
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "stream launch: %s", cudaGetErrorString(e));
     return -1;
   }
-  return gate_up_only ? 1 : 2;
+  return gate_up_only ? 1 : 2 + (w8 ? 1 : 0);
 }
 
 }  // namespace cmoe

@@ -723,7 +723,7 @@ inline bool decode_bind_x(UmmaPlan* P, DecodePlan* D, const void* x_rows, int n_
 inline int decode_split_x(UmmaPlan* P, DecodePlan* D, int n_rows, cudaStream_t st, bool dep) {
   SplitSegment a{(const bf16*)D->x_ptr, n_rows, P->shape.d, (long long)P->shape.d, D->xq, (long long)D->xq_rows, D->x_scale};
   SplitSegment none{nullptr, 0, 0, 0, nullptr, 0, nullptr};
-  launch_kernel(dep, split_rows_e4m3_kernel, dim3(n_rows), dim3(128), 0, st, a, none);
+  launch_kernel(dep, split_rows_e4m3_kernel, dim3(n_rows), dim3(kSplitThreads), 0, st, a, none);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -779,7 +779,7 @@ inline int decode_forward(UmmaPlan* P, DecodePlan* D, const GroupRows* gr, int n
     SplitSegment hs{(const bf16*)P->buf.h_s, rows_s, s.shared_width, (long long)s.shared_width, D->hq_s,
                     (long long)D->xq_rows, D->hs_scale};
     SplitSegment hr{(const bf16*)P->buf.h_r, rows_r, s.m, (long long)s.m, D->hq_r, (long long)D->hr_rows, D->hr_scale};
-    launch_kernel(dep, split_rows_e4m3_kernel, dim3(rows_s + rows_r), dim3(128), 0, st, hs, hr);
+    launch_kernel(dep, split_rows_e4m3_kernel, dim3(rows_s + rows_r), dim3(kSplitThreads), 0, st, hs, hr);
     extra = 1;
     a.tok_scale_s = D->hs_scale; a.tok_scale_r = D->hr_scale;
     decode_launch<5, true, kDecMaxRows>(dep, split2, sms, st, D->wd8_s, D->wd8_r, D->hqs_map[bi], D->hqr_map[bi], a);
