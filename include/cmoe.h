@@ -265,7 +265,7 @@ int cmoe_layer_set_gemm_path(cmoe_layer* layer, int32_t path);
  * may become resident (and fetch what does not depend on the predecessor) while the
  * predecessor drains, and waits on the device before touching anything the predecessor
  * produces.  Results are bit-identical either way; 0 restores ordinary stream-ordered
- * launches.  Has no effect on fp32 layers or while per-stage timing is enabled, and the
+ * launches.  Has no effect while per-stage timing is enabled, and the
  * prologue of a hierarchical layer (top-level router, its permutation, the row copy) always
  * uses ordinary launches.  Error: INVALID_ARG (null layer). */
 int cmoe_layer_set_launch_chaining(cmoe_layer* layer, int32_t on);

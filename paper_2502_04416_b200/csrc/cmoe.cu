@@ -371,7 +371,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   // plain layer is chained to whatever precedes it in the stream, which it waits for in full (7B-shaped layer
   // 1 / 16 / 300 rows 35.0 / 63.1 / 108.9 -> 33.6 / 61.4 / 104.8 us, even from 600 rows on); per-stage events and the prologue of a hierarchical layer (outer router, outer
   // permutation, row copy) use ordinary launches.
-  const bool dep = use_umma && !ev && L->chain_launches;
+  const bool dep = !ev && L->chain_launches;
 
   if (L->hier) {
     if constexpr (std::is_same<T, bf16>::value) {
@@ -421,10 +421,12 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   if (n_r > 0) {
     const int warps = (R + 1) / 2, blocks = (warps + 7) / 8;
     const int32_t* ooff = L->hier ? L->outer_off : nullptr;
-#define CMOE_ROUTER(NACC)                                                                         \
-  router_kernel<T, NACC><<<blocks, 256, 0, st>>>(xo, R, d, n_r, L->n_rp, n_k, (const T*)L->w_rep, L->u,   \
-                                                 L->b, ooff, L->n_outer, L->scores, L->keys,      \
-                                                 L->topk_idx, L->topk_gate)
+    // fp32: a warp per row while that leaves SMs idle (4 warps on each), two rows per warp beyond
+#define CMOE_ROUTER(NACC)                                                                                  \
+  launch_kernel(dep && !L->hier, R <= 592 ? router_row_kernel<T, NACC> : router_kernel<T, NACC>,           \
+                dim3(R <= 592 ? (R + 3) / 4 : blocks), dim3(R <= 592 ? 128 : 256), 0, st, xo, R, d, n_r, L->n_rp, n_k,  \
+                (const T*)L->w_rep, (const float*)L->u, (const float*)L->b, ooff, L->n_outer, L->scores, L->keys,       \
+                L->topk_idx, L->topk_gate)
     if constexpr (std::is_same<T, bf16>::value) {
       if (use_umma && R > kRcMaxRows) {
         if (umma_router_forward(&L->umma, R, ooff, L->err_word, st) < 0)
@@ -492,7 +494,11 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     }
   }
   const int gather_mode = P <= kTmaGatherMaxRows ? 1 : 2;
-  if (P > 0 && !use_umma) {
+  // SIMT path: small tiles (which gather their rows themselves) while 64 x 64 tiles would not give every SM a few
+  const long long simt_tiles = (long long)((R + kSimtTile - 1) / kSimtTile) * ((L->shared_width() + kSimtTile - 1) / kSimtTile) +
+                               ((long long)P / kSimtTile + G) * ((L->m + kSimtTile - 1) / kSimtTile);
+  const bool simt_small = !use_umma && simt_tiles <= 4 * 148;
+  if (P > 0 && !use_umma && !simt_small) {
     gather_rows_kernel<<<P, 256, 0, st>>>((const uint4*)xo, L->row_token, P, row_vec, (uint4*)L->x_perm);
     ++launches;
   }
@@ -564,15 +570,18 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     a.a_shared = xo; a.a_routed = (const T*)L->x_perm;
     a.w_gate = (const T*)L->wg_p; a.w_up = (const T*)L->wu_p;
     a.c_shared = (T*)L->h_s; a.c_routed = (T*)L->h_r;
-    dim3 g1((R + kSimtTile - 1) / kSimtTile, (max_w + kSimtTile - 1) / kSimtTile, L->n_groups_total());
-    simt_gemm1_kernel<T><<<g1, 256, 0, st>>>(a);
+    a.row_token = L->row_token;
+    const int tm = simt_small ? kSimtSmallM : kSimtTile, tn = simt_small ? kSimtSmallN : kSimtTile;
+    const int threads = simt_small ? kSimtSmallThreads : 256;
+    const dim3 g1((R + tm - 1) / tm, (max_w + tn - 1) / tn, L->n_groups_total());
+    launch_kernel(dep, simt_small ? simt_small_kernel<T, false> : simt_gemm1_kernel<T>, g1, dim3(threads), 0, st, a);
     mark(3);
     if (gate_up_only) { L->launches = launches + 1; CU_TRY(cudaGetLastError()); return CMOE_OK; }
     a.a_shared = (const T*)L->h_s; a.a_routed = (const T*)L->h_r;
     a.w_gate = (const T*)L->wd_p; a.w_up = nullptr;
     a.c_shared = (T*)L->y_s; a.c_routed = (T*)L->y_r;
-    dim3 g2((R + kSimtTile - 1) / kSimtTile, (d + kSimtTile - 1) / kSimtTile, L->n_groups_total());
-    simt_gemm2_kernel<T><<<g2, 256, 0, st>>>(a);
+    const dim3 g2((R + tm - 1) / tm, (d + tn - 1) / tn, L->n_groups_total());
+    launch_kernel(dep, simt_small ? simt_small_kernel<T, true> : simt_gemm2_kernel<T>, g2, dim3(threads), 0, st, a);
     launches += 2;
   }
 

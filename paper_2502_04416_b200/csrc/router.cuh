@@ -95,6 +95,111 @@ __device__ __forceinline__ void gate_row_sub(int sub, bool live_row, int n_r, in
   }
 }
 
+// A float's bits mapped so that unsigned order is numeric order (-0 counts as +0).
+__device__ __forceinline__ uint32_t ordered_bits(float v) {
+  const uint32_t b = __float_as_uint(v + 0.0f);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+
+// gate_row with u and b already in registers and the arg-max by one warp-wide integer reduction and a ballot (the
+// same order: larger key first, equal keys by index).  Lane i < n_k returns its selection in `sel`.
+__device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float a, float v, float u, float b, int group_base,
+                                               float* __restrict__ scores_row, float* __restrict__ keys_row,
+                                               int32_t* __restrict__ idx_row, float* __restrict__ gates_row, int& sel) {
+  const bool live = lane < n_r;
+  const float s = live ? silu_accurate(a) * v : -INFINITY;            // Eq. router
+  const float s_max = warp_max(s);
+  const float e = live ? expf(s - s_max) : 0.0f;
+  const float s_prime = e / warp_sum(e);                               // Softmax over all N_r
+  const float key = live ? s_prime + b : -INFINITY;
+  if (live) { scores_row[lane] = s; keys_row[lane] = key; }
+  const float gate = 1.0f + s_prime * u;                               // 1 + s'_i u_i
+  const float rank_key = (key != key) ? -INFINITY : key;               // NaN ranks last
+  uint32_t bits = live ? ordered_bits(rank_key) : 0u;                  // every live key is above 0
+  float my_gate = 0.0f;
+#pragma unroll 1
+  for (int i = 0; i < n_k; ++i) {
+    const uint32_t best = __reduce_max_sync(0xffffffffu, bits);
+    const int who = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
+    const float g = __shfl_sync(0xffffffffu, gate, who);
+    if (lane == who) bits = 0u;
+    if (lane == i) { sel = group_base + who; my_gate = g; }
+  }
+  if (lane < n_k) { idx_row[lane] = sel; gates_row[lane] = my_gate; }
+}
+
+// One row per warp, for batches that leave SMs idle otherwise (bound by latency).  The column sums meet by a reduce-scatter over the lanes (each step halves
+// the columns a lane still carries): the pairs of lanes are those of warp_sum, so every sum has the same bits.
+template <typename T, int NACC>
+__global__ void __launch_bounds__(128)
+router_row_kernel(const T* __restrict__ xo, int n_rows, int d, int n_r, int n_rp, int n_k,
+                  const T* __restrict__ w_rep, const float* __restrict__ u, const float* __restrict__ b,
+                  const int32_t* __restrict__ outer_off, int n_outer,
+                  float* __restrict__ scores, float* __restrict__ keys,
+                  int32_t* __restrict__ topk_idx, float* __restrict__ topk_gate) {
+  grid_dep_wait();
+  grid_dep_trigger();
+  const int lane = threadIdx.x & 31;
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (row >= n_rows) return;
+  const int go = outer_off ? find_outer(outer_off, n_outer, row) : 0;
+  const int n2 = 2 * n_rp;
+  const T* xr = xo + (size_t)row * d;
+  const T* w = w_rep + (size_t)go * n2 * d;
+  const float u_pre = lane < n_r ? __ldcg(u + go * n_r + lane) : 0.0f, b_pre = lane < n_r ? __ldcg(b + go * n_r + lane) : 0.0f;
+  float acc[NACC];
+#pragma unroll
+  for (int j = 0; j < NACC; ++j) acc[j] = 0.0f;
+#pragma unroll 1
+  for (int k = lane * 8; k < d; k += 256) {
+    float xa[8];
+    load8(xr + k, xa);
+#pragma unroll
+    for (int j = 0; j < NACC; ++j)
+      if (j < n2) {
+        float wa[8];
+        load8(w + (size_t)j * d + k, wa);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[j] = fmaf(wa[q], xa[q], acc[j]);
+      }
+  }
+  // after the steps with a column to give away, lane l carries column l * NACC / 32 (NACC = 64: two columns, j and j + 32)
+  constexpr int kSets = NACC > 32 ? NACC / 32 : 1, kCols = NACC / kSets;
+  float col[kSets];
+#pragma unroll
+  for (int s = 0; s < kSets; ++s) {
+    float* v = acc + s * kCols;
+    int n = kCols;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if (n > 1) {
+        n >>= 1;
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < kCols / 2; ++j)
+          if (j < n) {
+            const float give = up ? v[j] : v[j + n], keep = up ? v[j + n] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      }
+    }
+    col[s] = v[0];
+  }
+  constexpr int kPer = 32 / kCols;                // lanes that carry the same column
+  const int cv = n_rp + lane;                     // column of expert `lane`'s up sum
+  const float a = __shfl_sync(0xffffffffu, col[0], (lane * kPer) & 31);
+  float v = __shfl_sync(0xffffffffu, col[0], (cv * kPer) & 31);
+  if (kSets > 1) {
+    const float v1 = __shfl_sync(0xffffffffu, col[kSets - 1], cv & 31);
+    if (cv >= 32) v = v1;
+  }
+  int sel = 0;
+  gate_row_redux(lane, n_r, n_k, a, v, u_pre, b_pre, go * n_r, scores + (size_t)row * n_r, keys + (size_t)row * n_r,
+                 topk_idx + (size_t)row * n_k, topk_gate + (size_t)row * n_k, sel);
+}
+
 template <typename T, int NACC>
 __global__ void __launch_bounds__(256)
 router_kernel(const T* __restrict__ xo, int n_rows, int d, int n_r, int n_rp, int n_k,
@@ -102,6 +207,8 @@ router_kernel(const T* __restrict__ xo, int n_rows, int d, int n_r, int n_rp, in
               const int32_t* __restrict__ outer_off, int n_outer,
               float* __restrict__ scores, float* __restrict__ keys,
               int32_t* __restrict__ topk_idx, float* __restrict__ topk_gate) {
+  grid_dep_wait();
+  grid_dep_trigger();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int r0 = warp * 2;

@@ -28,11 +28,7 @@ constexpr int kRcThreads = 256;
 constexpr int kRcCluster = 8;
 constexpr int kRcRows = 16;                 // rows of a cluster's tile
 constexpr int kRcMaxRows = 1024;            // rows of a batch this kernel takes
-constexpr int kRcFuseGroups = 64;           // routed groups up to which the permutation runs in the same launch
-// ... and selections (fused against the permutation kernels: 8B-shaped 700 rows x 4: 129.5 against 131.4 us, 7B-shaped 1000 x 2:
-// 179.3 against 184.6, 8B-shaped 1000 x 4: 174.9 against 170.3)
-constexpr int kRcFusePairs = 3072;
-constexpr int kRcPermBytes = kRcFusePairs + kRcFuseGroups * (kRcMaxRows / 32) * 6 + kRcFuseGroups * 8;
+static_assert(kRcMaxRows <= kMaskRows && kRcThreads == kMaskThreads, "the fused permutation is permute_by_masks");
 
 __device__ __forceinline__ void rc_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void rc_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -47,39 +43,6 @@ __device__ __forceinline__ void rc_push(uint32_t addr, float v) {
 }
 __device__ __forceinline__ void rc_push(uint32_t addr, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
-// A float's bits mapped so that unsigned order is numeric order (-0 counts as +0).
-__device__ __forceinline__ uint32_t ordered_bits(float v) {
-  const uint32_t b = __float_as_uint(v + 0.0f);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-// gate_row with u and b already in registers and the arg-max by one warp-wide integer reduction and a ballot (the
-// same order: larger key first, equal keys by index).  Lane i < n_k returns its selection in `sel`.
-__device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float a, float v, float u, float b, int group_base,
-                                               float* __restrict__ scores_row, float* __restrict__ keys_row,
-                                               int32_t* __restrict__ idx_row, float* __restrict__ gates_row, int& sel) {
-  const bool live = lane < n_r;
-  const float s = live ? silu_accurate(a) * v : -INFINITY;            // Eq. router
-  const float s_max = warp_max(s);
-  const float e = live ? expf(s - s_max) : 0.0f;
-  const float s_prime = e / warp_sum(e);                               // Softmax over all N_r
-  const float key = live ? s_prime + b : -INFINITY;
-  if (live) { scores_row[lane] = s; keys_row[lane] = key; }
-  const float gate = 1.0f + s_prime * u;                               // 1 + s'_i u_i
-  const float rank_key = (key != key) ? -INFINITY : key;               // NaN ranks last
-  uint32_t bits = live ? ordered_bits(rank_key) : 0u;                  // every live key is above 0
-  float my_gate = 0.0f;
-#pragma unroll 1
-  for (int i = 0; i < n_k; ++i) {
-    const uint32_t best = __reduce_max_sync(0xffffffffu, bits);
-    const int who = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
-    const float g = __shfl_sync(0xffffffffu, gate, who);
-    if (lane == who) bits = 0u;
-    if (lane == i) { sel = group_base + who; my_gate = g; }
-  }
-  if (lane < n_k) { idx_row[lane] = sel; gates_row[lane] = my_gate; }
 }
 
 struct RouterArgs {
@@ -98,81 +61,6 @@ struct RouterArgs {
   GroupPlanOut po;
 };
 
-// Histogram, scan and stable permutation of at most kRcFusePairs selections over at most kRcFuseGroups groups, by one
-// block.  sel[i]: selection of pair i = row * n_k + j, already in shared memory.  mask[g][w]: which of the rows
-// 32 w .. 32 w + 31 selected group g; before[g][w]: how many rows ahead of those did.
-__device__ __forceinline__ void permute_by_masks(const RouterArgs& p, const uint8_t* sel, uint32_t* mask, uint16_t* before,
-                                                 int32_t* count, int32_t* offs) {
-  const int words = (p.n_rows + 31) >> 5, pairs = p.n_rows * p.n_k;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll 1
-  for (int i = threadIdx.x; i < p.n_groups * words; i += kRcThreads) mask[i] = 0;
-  __syncthreads();
-#pragma unroll 1
-  for (int row = threadIdx.x; row < p.n_rows; row += kRcThreads)
-#pragma unroll 1
-    for (int j = 0; j < p.n_k; ++j) atomicOr(&mask[sel[row * p.n_k + j] * words + (row >> 5)], 1u << (row & 31));
-  __syncthreads();
-#pragma unroll 1
-  for (int g = warp; g < p.n_groups; g += kRcThreads / 32) {           // lane: word (at most kRcMaxRows / 32 = 32)
-    const int c = lane < words ? __popc(mask[g * words + lane]) : 0;
-    int incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    if (lane < words) before[g * words + lane] = (uint16_t)(incl - c);
-    if (lane == 31) count[g] = incl;
-  }
-  __syncthreads();
-  if (warp == 0) {                                                     // lane l: groups 2l and 2l + 1
-    int c[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) c[q] = 2 * lane + q < p.n_groups ? count[2 * lane + q] : 0;
-    int incl = c[0] + c[1];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    int run = incl - c[0] - c[1];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int g = 2 * lane + q;
-      if (g < p.n_groups) {
-        offs[g] = run;
-        p.counts[g] = c[q];
-        p.offsets[g] = run;
-        if (p.po.gr) { GroupRows r; r.row0 = run; r.count = c[q]; p.po.gr[p.po.n_outer + g] = r; }
-        run += c[q];
-        if (g == p.n_groups - 1) p.offsets[p.n_groups] = run;
-      }
-    }
-  } else if (p.po.gr) {
-#pragma unroll 1
-    for (int g = threadIdx.x - 32; g < p.po.n_outer; g += kRcThreads - 32) {
-      GroupRows r;
-      r.row0 = p.po.outer_off ? p.po.outer_off[g] : 0;
-      r.count = p.po.outer_off ? p.po.outer_off[g + 1] - r.row0 : p.po.n_tokens;
-      p.po.gr[g] = r;
-    }
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int row = threadIdx.x; row < p.n_rows; row += kRcThreads) {
-    const int w = row >> 5;
-    const uint32_t below = (1u << (row & 31)) - 1u;
-#pragma unroll 1
-    for (int j = 0; j < p.n_k; ++j) {
-      const int g = sel[row * p.n_k + j];
-      const int pos = offs[g] + before[g * words + w] + __popc(mask[g * words + w] & below);
-      p.row_token[pos] = row;
-      p.row_of[row * p.n_k + j] = pos;
-    }
-  }
-}
-
 // MAXT: tiles of 8 router columns at most (2 N_r rounded up); NB: outer experts whose representative rows are held in
 // flight at once when a tile's rows belong to several (1 for a plain layer).
 template <int MAXT, int NB>
@@ -181,7 +69,7 @@ router_cluster_kernel(const RouterArgs p) {
   constexpr int kCols = MAXT * 8, kStride = kCols + 8;
   constexpr int kUnr = 16 / (MAXT * NB) >= 2 ? 2 : 1;                // k slices in flight per warp
   constexpr int kPartBytes = 8 * kRcRows * kStride * 4;
-  __shared__ __align__(16) uint8_t scratch[kPartBytes > kRcPermBytes ? kPartBytes : kRcPermBytes];
+  __shared__ __align__(16) uint8_t scratch[kPartBytes > kMaskBytes ? kPartBytes : kMaskBytes];
   float (*part)[kRcRows][kStride] = reinterpret_cast<float (*)[kRcRows][kStride]>(scratch);   // [warp]
   __shared__ float recv[kRcCluster][2][kCols];                       // [source CTA][row 2 rank + i][column]
   __shared__ int sel_recv[kRcRows * kMaxTopK];                       // rank 0: the tile's selections
@@ -232,7 +120,7 @@ router_cluster_kernel(const RouterArgs p) {
   int go_mine = 0;
   if (gate_warp) {
     if (NB > 1) go_mine = row_group[my_row];
-    if (lane < p.n_r) { u_pre = __ldg(p.u + go_mine * p.n_r + lane); b_pre = __ldg(p.b + go_mine * p.n_r + lane); }
+    if (lane < p.n_r) { u_pre = __ldcg(p.u + go_mine * p.n_r + lane); b_pre = __ldcg(p.b + go_mine * p.n_r + lane); }
   }
   // ---- partial sums over this warp's k slices
   const int r_lo = min(g, n_rows - 1), r_hi = min(g + 8, n_rows - 1);
@@ -255,8 +143,8 @@ router_cluster_kernel(const RouterArgs p) {
       for (int q = 0; q < kUnr; ++q) {
         const int k = (s + 64 * q) * 32;
         const bool in = k + 8 * t < p.d;
-        a_lo[q] = in ? __ldg(reinterpret_cast<const uint4*>(x_lo + k)) : zero;
-        a_hi[q] = in ? __ldg(reinterpret_cast<const uint4*>(x_hi + k)) : zero;
+        a_lo[q] = in ? ld_dep16(x_lo + k) : zero;
+        a_hi[q] = in ? ld_dep16(x_hi + k) : zero;
       }
       if (NB > 1 || s != s0) load_w(s, i0, nl);
 #pragma unroll
@@ -314,11 +202,7 @@ router_cluster_kernel(const RouterArgs p) {
   rc_cluster_wait();
   if (rank != 0) return;
   // ---- permutation
-  uint8_t* sel = scratch;                                             // [n_rows * n_k <= kRcFusePairs]
-  int32_t* count = reinterpret_cast<int32_t*>(sel + kRcFusePairs);     // [n_groups], then the exclusive scan
-  int32_t* offs = count + kRcFuseGroups;
-  uint32_t* mask = reinterpret_cast<uint32_t*>(offs + kRcFuseGroups);
-  uint16_t* before = reinterpret_cast<uint16_t*>(mask + kRcFuseGroups * (kRcMaxRows / 32));
+  uint8_t* sel = scratch;                                             // [n_rows * n_k <= kMaskPairs]
   if (gridDim.y == 1) {
 #pragma unroll 1
     for (int i = threadIdx.x; i < n_rows * p.n_k; i += kRcThreads) sel[i] = (uint8_t)sel_recv[i];
@@ -343,11 +227,11 @@ router_cluster_kernel(const RouterArgs p) {
     }
   }
   __syncthreads();
-  permute_by_masks(p, sel, mask, before, count, offs);
+  permute_by_masks(PermuteOut{p.n_rows, p.n_k, p.n_groups, p.counts, p.offsets, p.row_token, p.row_of, p.po}, scratch);
 }
 
 inline bool router_cluster_fuses(int n_rows, int n_k, int n_groups) {
-  return n_groups <= kRcFuseGroups && n_rows <= kRcMaxRows && (long long)n_rows * n_k <= kRcFusePairs;
+  return n_rows <= kRcMaxRows && permute_masks_fit(n_rows, n_k, n_groups);
 }
 
 inline cudaError_t router_cluster_launch(const RouterArgs& a, bool hier, bool dep, bool all_smem, cudaStream_t st) {

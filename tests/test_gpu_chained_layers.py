@@ -1,0 +1,54 @@
+"""-m gpu: forwards enqueued back to back without synchronising, each reading what the one before it wrote (a stack of
+layers), against the same calls with a synchronisation after each.  Launch chaining lets a forward's first kernel become
+resident while the preceding layer's last kernel still runs."""
+import numpy as np
+import pytest
+
+from paper_2502_04416_b200 import workloads as wl
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _stack(dtype, fp8, tokens, n_layers=3, d=512, m=176):
+    shape = wl.LayerShape(d, m * 8, 8, 2, 2, dtype)
+    rng = np.random.Generator(np.random.PCG64(3))
+    layers = []
+    for _ in range(n_layers):
+        lay = wl.draw_layer(rng, shape)
+        for w in (lay.w_gate, lay.w_up, lay.w_down):       # a layer's output is of its input's size
+            w *= 2.0
+        layers.append(parity.gpu_layer(lay, tokens))
+        if fp8:
+            layers[-1].quantise_fp8()
+    return layers, wl.draw_tokens(rng, tokens, shape)
+
+
+@pytest.mark.parametrize("dtype,fp8,tokens", [("bf16", False, t) for t in (1, 2, 16, 64, 100, 300, 1100)] +
+                         [("bf16", True, t) for t in (1, 16, 64)] + [("fp32", False, t) for t in (1, 64, 700)])
+def test_layer_stack_matches_synchronised_calls(dtype, fp8, tokens):
+    import torch
+    layers, x = _stack(dtype, fp8, tokens)
+    xs = [parity.to_device(x, dtype)]
+    xs += [torch.roll(xs[0], k, 1).contiguous() for k in (1, 2, 3)]
+    bufs = [torch.empty_like(xs[0]) for _ in range(3)]
+
+    def step(k, sync):
+        src = xs[k]
+        for layer, dst in zip(layers, bufs):
+            layer.forward(src, dst)
+            if sync:
+                torch.cuda.synchronize()
+            src = dst
+        return src.clone()
+
+    want = [step(k, True) for k in range(4)]
+    assert not torch.equal(want[0], want[1])
+    for _ in range(5):
+        got = [step(k, False) for k in range(4)]
+        torch.cuda.synchronize()
+        for g, w in zip(got, want):
+            assert torch.equal(g, w)
+    for layer in layers:
+        assert layer.status() == 0
+        layer.destroy()
