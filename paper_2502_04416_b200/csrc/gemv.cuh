@@ -206,7 +206,7 @@ gemv_gate_up_kernel(const GemvArgs p) {
       float g[TT], u[TT];
       neuron((size_t)(g0.w_row0 + n), xr, g, u);
 #pragma unroll
-      for (int j = 0; j < TT; ++j) early_h[i][j] = g[j] / (1.0f + __expf(-g[j])) * u[j];
+      for (int j = 0; j < TT; ++j) early_h[i][j] = swiglu_fast(g[j], u[j]);
     }
   }
   grid_dep_wait();
@@ -239,7 +239,7 @@ gemv_gate_up_kernel(const GemvArgs p) {
       for (int j = 0; j < TT; ++j)
         if (j < count) {
           bf16* dst = L.is_shared[lo] ? p.h_s + (size_t)(L.row0[lo] + j) * p.ld_h_s : p.h_r + (size_t)(L.row0[lo] + j) * p.ld_h_r;
-          dst[n] = __float2bfloat16_rn(g[j] / (1.0f + __expf(-g[j])) * u[j]);
+          dst[n] = __float2bfloat16_rn(swiglu_fast(g[j], u[j]));
         }
     }
   }

@@ -359,7 +359,7 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
           if (row_ok) {
             float h16[16];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) h16[q] = gt[q] / (1.0f + __expf(-gt[q])) * up[q];
+            for (int q = 0; q < 16; ++q) h16[q] = swiglu_fast(gt[q], up[q]);
             if (wide && c0 + 16 <= n_valid) {
               store16(dst + c0, h16);
             } else {

@@ -432,7 +432,7 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
           const int pos = lookup ? inv[c] : c;
           if (pos >= 0) {
             if constexpr (W8) { const float ts = __ldg(tok_scale + c); a *= sc_a * ts; b *= sc_b * ts; }
-            const float v = MODE == 4 ? a / (1.0f + __expf(-a)) * b : a;
+            const float v = MODE == 4 ? swiglu_fast(a, b) : a;
             dst[(size_t)pos * ld] = __float2bfloat16_rn(v);
           }
         }
