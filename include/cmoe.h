@@ -246,8 +246,8 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
 
 /* Choose the expert-GEMM implementation: 0 = automatic (tensor-core path when the
  * dtype is bf16 and the shape allows, else the plain SIMT path; for batches of at least 256
- * rows each of the two GEMMs may run on CTA pairs: below 1024 rows when the experts are at least
- * 1024 neurons wide (a pair fetches a third less operand data per SM), from 1024 rows when the
+ * rows each of the two GEMMs may run on CTA pairs: the gate/up GEMM below 2048 rows when the expected tiles
+ * keep the busiest SM for less time that way, both from 2048 rows on when the
  * padding of the expert groups to 256-row tiles is expected to stay small; batches of 65 to 128 rows stream the bf16 weights through the
  * decode-shaped kernels, weights on the MMA's M side; 2 to 64 rows of a plain layer
  * run on two weight streamers with the gates folded into the hidden activations (rounded to bf16 once, after the

@@ -53,8 +53,6 @@ int arg_fail(int code, const char* what) {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-constexpr int kPairMinRows = 256;        // outer rows from which the expert GEMMs may run on CTA pairs
-constexpr int kTmaGatherMaxRows = 512;   // routed rows up to which gather4 replaces the permuted copy of x
 
 // Bump allocator over one device allocation (base == nullptr: measure only).
 struct Arena {
@@ -314,7 +312,6 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     UmmaBuffers ub;
     ub.w_gate_up = L->w_gu; ub.w_down = L->wd_p; ub.w_rep = L->w_rep;
     ub.x_fixed = L->hier ? L->xo : nullptr;
-    ub.x_perm = L->x_perm;
     ub.h_s = L->h_s; ub.h_r = L->h_r; ub.y_s = L->y_s; ub.y_r = L->y_r;
     ub.gs_dev = L->gs; ub.u = L->u; ub.b = L->b;
     ub.scores = L->scores; ub.keys = L->keys; ub.topk_idx = L->topk_idx; ub.topk_gate = L->topk_gate;
@@ -462,38 +459,9 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                                           L->counts, L->offsets, L->gr);
     ++launches;
   }
-  // The tensor path gathers routed rows inside the gate/up GEMM (decode: not at all; a few rows:
-  // TMA gather4; otherwise cp.async by dedicated warps); only the SIMT path reads a permuted copy of x.
-  // CTA pairs (cta_group::2, 256-row tiles) move a third less operand data per flop but round every
-  // group up to an even number of 128-row tiles.  Path 3 forces them; the automatic choice takes them
-  // per GEMM when the padding expected for evenly loaded experts stays small (thresholds measured on
-  // the paper-shaped workloads: the down GEMM gains more from pairs than the gate/up GEMM, except
-  // when its K extent, the expert width, is only a few k blocks).
-  int pair_mask = 0;                               // bit 0: gate/up on pairs, bit 1: down on pairs
-  if (use_umma && !decode && R >= kPairMinRows) {
-    if (L->gemm_path == 3) {
-      pair_mask = 3;
-    } else if (L->gemm_path == 0) {
-      auto pad = [](double rows) {                 // tile slots on pairs / tiles on single CTAs
-        const int mt = (int)((rows + 127) / 128);
-        return mt > 0 ? (double)(2 * ((mt + 1) / 2)) / mt : 1.0;
-      };
-      const double rows_s = (double)R / L->n_outer, rows_r = G > 0 ? (double)P / G : 0.0;
-      const double w_s = (double)R * L->cfg.n_shared, w_r = (double)P;
-      const double ratio = (w_s + w_r) > 0 ? (pad(rows_s) * w_s + pad(rows_r) * w_r) / (w_s + w_r) : 1.0;
-      if (R < 1024 && !L->hier) {
-        // A few tiles per SM: operand fetch per SM is the limit, and a pair halves the weight bytes a CTA fetches,
-        // but every routed group is padded to 256 rows.  Measured at 256-768 rows: pairs win with wide experts
-        // (1376 neurons: 114 vs 126 us at 256 rows, 120 vs 127 at 512), single-CTA tiles with narrow ones (864:
-        // 134 vs 162 us at 256 rows, 165 vs 174 at 384; 448: 113 vs 127 at 256, 151 vs 167 at 768).
-        pair_mask = L->m >= 1024 ? 3 : 0;
-      } else {
-        if (ratio <= 1.03) pair_mask |= 1;
-        if (ratio <= 1.08 && L->m >= 512) pair_mask |= 2;
-      }
-    }
-  }
-  const int gather_mode = P <= kTmaGatherMaxRows ? 1 : 2;
+  // The tensor path gathers routed rows inside the gate/up GEMM; only large SIMT tiles read a permuted copy of x.
+  const int pair_mask = use_umma && !gemv && !stream && !decode
+      ? umma_pick_pairs(&L->umma, L->pair.grid, R, P, G, L->gemm_path) : 0;
   // SIMT path: small tiles (which gather their rows themselves) while 64 x 64 tiles would not give every SM a few
   const long long simt_tiles = (long long)((R + kSimtTile - 1) / kSimtTile) * ((L->shared_width() + kSimtTile - 1) / kSimtTile) +
                                ((long long)P / kSimtTile + G) * ((L->m + kSimtTile - 1) / kSimtTile);
@@ -555,8 +523,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
       for (int bit = 1; bit <= 2 && n >= 0; bit <<= 1) {          // gate/up, then down, each on its chosen tile shape
         if (!(todo & bit)) continue;
         const int k = (pair_mask & bit)
-            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, 2, xo, L->err_word, st, mid, dep, bit)
-            : umma_forward(&L->umma, L->gr, gather_mode, xo, L->err_word, st, mid, dep, bit);
+            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit)
+            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit);
         n = k < 0 ? -1 : n + k;
       }
     }

@@ -27,6 +27,8 @@
 //                four epilogue warps of each CTA, the peer's arriving remotely).
 #pragma once
 
+#include <cmath>
+
 #include "umma_decode.cuh"
 #include "umma_gemm.cuh"
 
@@ -204,7 +206,7 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
       const int row = c.row0 + (2 * c.mp + (int)rank) * kUmmaBM;     // this CTA's m-tile
       const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
       const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
-      const bool by_threads = MODE == 1 && !g.is_shared && p.use_gather == 2;   // the gather warps fill A
+      const bool by_threads = MODE == 1 && !g.is_shared;   // the gather warps fill A
       int k_blocks, b_half, b_row, j = 0;
       if (MODE == 1) {
         const int bn = g.is_shared ? p.bn_s : p.bn_r;
@@ -297,15 +299,14 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
     for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
       const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
       const GroupStatic g = p.gs[c.g];
-      const bool mine = !g.is_shared && p.use_gather == 2;
+      const bool mine = !g.is_shared;
       const bf16* src_row[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         src_row[i] = nullptr;
-        if (mine) {                                   // rows past the group repeat its last row
-          const int r = c.row0 + min((2 * c.mp + (int)rank) * kUmmaBM + i * 16 + r_sub, c.count - 1);
-          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + r) * p.d;
-        }
+        const int r = (2 * c.mp + (int)rank) * kUmmaBM + i * 16 + r_sub;
+        if (mine && r < c.count)                      // rows past the group are left as they are: nothing of them is stored
+          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + c.row0 + r) * p.d;
       }
       for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
         const uint32_t s = it % kU2Stages, n = it / kU2Stages;
@@ -319,7 +320,8 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int r = i * 16 + r_sub;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+            if (src_row[i])
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
                          ::"r"(sa + r * 128 + ((ch ^ (r & 7)) << 4)), "l"(src_row[i] + k_src), "r"(bytes)
                          : "memory");
           }
@@ -460,23 +462,20 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
   return true;
 }
 
-// Gate/up and down GEMM on CTA pairs.  gather_mode 2: routed rows are gathered from x_rows inside
-// the gate/up kernel; 0: they come from the permuted copy of x by TMA.
+// Gate/up and down GEMM on CTA pairs; routed rows are gathered from x_rows inside the gate/up kernel.
 // `D` supplies the 128-channel W_down maps (shared with the decode path).  Requires
 // umma_bind_x for this forward.  which: bit 0 the gate/up GEMM, bit 1 the down GEMM.  Returns launches or -1.
-inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRows* gr, int gather_mode,
-                         const void* x_rows, int32_t* err_word, cudaStream_t st, cudaEvent_t mid, bool dep = false,
-                         int which = 3) {
+inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRows* gr, const void* x_rows, int32_t* err_word, cudaStream_t st, cudaEvent_t mid, bool dep,
+                         int which) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   const int grid = Q->grid;
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
-  a.use_gather = gather_mode;
   a.x_rows_ptr = (const bf16*)x_rows;
   a.band_mt = umma_band_tiles(s.d);
   if (which & 1)
     launch_kernel(dep, umma2_grouped_kernel<1>, dim3(grid), dim3(kU2Threads1), kU2SmemBytes, st,
-                  P->x_rows, P->has_r ? P->x_perm : P->x_rows, Q->b1_s, Q->b1_r, a);
+                  P->x_rows, P->x_rows, Q->b1_s, Q->b1_r, a);
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
@@ -489,6 +488,69 @@ inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRo
     return -1;
   }
   return (which & 1) + ((which >> 1) & 1);
+}
+
+// ----------------------------------------------------------------------------- tile shapes
+constexpr int kPairMinRows = 256;        // outer rows from which the expert GEMMs may run on CTA pairs
+
+// Expected number of `rows`-row tiles of a group whose rows are binomial with this mean and deviation.
+inline double umma_expected_tiles(double mean, double dev, int rows) {
+  double n = 0.0;
+  for (int j = 0; j * rows < mean + 5.0 * dev + 1.0; ++j) {
+    const double z = dev > 1e-3 ? (j * rows + 0.5 - mean) / dev : (j * rows + 0.5 > mean ? 9.0 : -9.0);
+    n += 0.5 * erfc(z * 0.70710678);
+  }
+  return n;
+}
+
+// Busiest CTA (or pair) of n_slots when n_s tiles of cost c_s and then n_r tiles of cost c_r are dealt round-robin.
+inline double umma_busiest(int n_s, double c_s, int n_r, double c_r, int n_slots) {
+  double worst = 0.0;
+  for (int i = 0; i < n_slots; ++i) {
+    const int s = n_s > i ? (n_s - 1 - i) / n_slots + 1 : 0, all = n_s + n_r > i ? (n_s + n_r - 1 - i) / n_slots + 1 : 0;
+    const double load = s * c_s + (all - s) * c_r;
+    worst = load > worst ? load : worst;
+  }
+  return worst;
+}
+
+// Which of the two GEMMs run on CTA pairs (bit 0: gate/up, bit 1: down) for R outer rows and n_sel selections over
+// n_routed groups (even load assumed).  Both are persistent kernels whose tiles are dealt round-robin.
+//   Below kPairLargeRows: a few rounds, so what counts for gate/up is the busiest SM.  Per 64-wide k block a 128 x 256 tile
+// takes 425 ns on a single CTA (the operands' round trip through four stages) and a 256 x 256 tile 320 ns on a pair
+// (on-device timelines, 7B-shaped layer, 512 rows).  Single against pairs: 7B-shaped 300 / 512 / 1000 rows 78 / 124 / 173
+// against 98 / 110 / 159 us, 8B-shaped 300 / 700 / 1000 rows 116 / 132 / 171 against 104 / 141 / 164.  The load is taken
+// once as expected and once with a fifth more tiles, for skewed routing.  The down GEMM stays on single CTAs (8B-shaped
+// 300 rows 104 against 118 us, hierarchical 300 rows 545 against 614, 7B-shaped 512 rows 110 against 108).
+//   From there on the part runs at its power limit and padding costs energy: pairs when rounding the groups up to an
+// even number of 128-row tiles adds at most 3 % (gate/up) or 8 % (down, not for K extents of a few k blocks).
+constexpr int kPairLargeRows = 2048;
+inline int umma_pick_pairs(const UmmaPlan* P, int pair_grid, int R, int n_sel, int n_routed, int gemm_path) {
+  if (gemm_path == 2 || R < kPairMinRows) return 0;
+  if (gemm_path == 3) return 3;
+  const UmmaShape& s = P->shape;
+  const double rows_s = (double)R / s.n_outer, mean = n_routed > 0 ? (double)n_sel / n_routed : 0.0;
+  if (R >= kPairLargeRows) {
+    auto pad = [](double rows) {                 // tile slots on pairs / tiles on single CTAs
+      const int mt = (int)((rows + 127) / 128);
+      return mt > 0 ? (double)(2 * ((mt + 1) / 2)) / mt : 1.0;
+    };
+    const double w_s = (double)R * s.shared_width, w_r = (double)n_sel * s.m;
+    const double ratio = w_s + w_r > 0 ? (pad(rows_s) * w_s + pad(mean) * w_r) / (w_s + w_r) : 1.0;
+    return (ratio <= 1.03 ? 1 : 0) | (ratio <= 1.08 && s.m >= 512 ? 2 : 0);
+  }
+  const double dev = rows_s > 0 ? sqrt(mean * (1.0 - (mean < rows_s ? mean / rows_s : 1.0))) : 0.0;
+  double cost[2];
+  for (int pair = 0; pair < 2; ++pair) {
+    const int rows = pair ? 256 : 128;
+    const int n_s = !P->has_s ? 0 : (int)(s.n_outer * umma_expected_tiles(rows_s, s.n_outer > 1 ? sqrt(rows_s) : 0.0, rows) *
+                                              ((s.shared_width + P->bn_s - 1) / P->bn_s) + 0.5);
+    const double n_r = !P->has_r ? 0.0 : n_routed * umma_expected_tiles(mean, dev, rows) * ((s.m + P->bn_r - 1) / P->bn_r);
+    const int slots = pair ? pair_grid / 2 : P->n_sms;
+    cost[pair] = (pair ? 320.0 : 425.0) * (umma_busiest(n_s, 1.0, (int)(n_r + 0.5), 1.0, slots) +
+                                           umma_busiest(n_s, 1.0, (int)(1.2 * n_r + 0.5), 1.0, slots));
+  }
+  return cost[1] < 0.97 * cost[0] ? 1 : 0;
 }
 
 }  // namespace cmoe

@@ -8,10 +8,9 @@
 //                 Routed groups gather their rows straight from x, so no permuted copy of
 //                 x is ever written: four extra warps (one thread per tile row) issue
 //                 16-byte cp.async copies into the 128-byte-swizzled layout the MMA expects
-//                 and arrive on the stage's barrier when their copies land.  (TMA
-//                 tile::gather4 does the same with one copy per 4 rows; it is correct but a
-//                 full tile needs 32 copies per stage, which the TMA unit issues ~3x slower
-//                 than one tiled box, so it is kept only for batches of a few rows.)
+//                 and arrive on the stage's barrier when their copies land.  TMA tile::gather4
+//                 does the same with one copy per 4 rows and is slower for every batch: 7B-shaped
+//                 layer 200 / 256 rows 94.2 / 106.2 us against 78.2 / 78.1.
 //       B tile  : bn gate rows + bn up rows of the group's neurons x 64 k (one 3-D TMA box)
 //       D (TMEM): 128 lanes x 2*bn fp32 columns; epilogue fuses SiLU(gate)*up -> bf16 H
 //   MODE 2, down GEMM: Y[r, c] = sum_n H[r, n] Wd[c, n]
@@ -126,14 +125,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm,
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
-// Four rows r0..r3 of a 2-D tensor (box: 64 columns x 1 row) to four consecutive 128-byte rows.
-__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int r0,
-                                            int r1, int r2, int r3) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
-}
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_slot, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_slot), "r"(cols)
                : "memory");
@@ -231,7 +222,6 @@ struct UmmaArgs {
   int ld_out_s, ld_out_r;
   const int32_t* row_token;   // mode 1: outer row held by each routed row (gather source)
   int band_mt;                // row tiles per band of the tile order (see umma_decode)
-  int use_gather;             // mode 1, routed A rows: 0 permuted copy by TMA, 1 TMA gather4 from x, 2 cp.async from x
   const bf16* x_rows_ptr;     // mode 1: the outer rows of x (source of the cp.async gather)
   int32_t* err;
   // mode 3 (router)
@@ -416,28 +406,15 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
       GroupStatic g;
       if (MODE != 3) g = p.gs[c.g]; else { g.is_shared = 1; g.outer = c.g; g.width = 0; g.w_row0 = 0; }
       const int row = c.row0 + c.mt * kUmmaBM;
-      const bool gather = MODE == 1 && !g.is_shared && p.use_gather == 1;
-      const bool by_threads = MODE == 1 && !g.is_shared && p.use_gather == 2;   // the gather warps fill A
+      const bool by_threads = MODE == 1 && !g.is_shared;              // the gather warps fill A
       const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
       const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
       int k_blocks, b_bytes, b_row = 0, j = 0;
-      int a_bytes = kUmmaABytes, n_issue = 0;
-      int gr0 = 0, gr1 = 0, gr2 = 0, gr3 = 0;
       if (MODE == 1) {
         const int bn = g.is_shared ? p.bn_s : p.bn_r;
         k_blocks = k_blocks_fixed;
         b_bytes = 2 * bn * kUmmaBK * 2;
         b_row = g.w_row0 + c.nt * bn;
-        if (gather) {                          // this lane's four rows; rows past the group repeat its last row
-          n_issue = (min(kUmmaBM, c.count - c.mt * kUmmaBM) + 3) >> 2;    // copies that carry valid rows
-          a_bytes = n_issue * 512;
-          const int last = c.row0 + c.count - 1;
-          const int r = row + 4 * lane;
-          gr0 = __ldg(p.row_token + min(r, last));
-          gr1 = __ldg(p.row_token + min(r + 1, last));
-          gr2 = __ldg(p.row_token + min(r + 2, last));
-          gr3 = __ldg(p.row_token + min(r + 3, last));
-        }
       } else if (MODE == 2) {
         k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK;
         b_bytes = kUmmaBBytes;
@@ -453,17 +430,9 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
         if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb = full0 + 8 * s;
         const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
-        if (gather) {
-          if (lane == 0) mbar_expect_tx(fb, a_bytes + b_bytes);
-          __syncwarp();
-          if (lane < n_issue) tma_gather4(sa + lane * 512, ta, fb, kb * kUmmaBK, gr0, gr1, gr2, gr3);
-          __syncwarp();
-        }
         if (elect_one()) {
-          if (!gather) {
-            mbar_expect_tx(fb, (by_threads ? 0 : a_bytes) + b_bytes);
-            if (!by_threads) tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
-          }
+          mbar_expect_tx(fb, (by_threads ? 0 : kUmmaABytes) + b_bytes);
+          if (!by_threads) tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
           if (MODE == 1) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, 0);
           else if (MODE == 3) tma_load_3d(sb, tb, fb, kb * kUmmaBK, 0, c.g);
           else if (g.is_shared) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
@@ -515,7 +484,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     }
   } else if (MODE == 1 && warp >= 6) {
     // ------------------------------------------------------------ A-row gather (mode 1, warps 6..9)
-    // For routed groups (use_gather == 2) the 128 threads copy the tile's 128 rows x 128 bytes of
+    // For routed groups the 128 threads copy the tile's 128 rows x 128 bytes of
     // this k block from x: eight consecutive threads cover one row (coalesced 128-byte reads), 16
     // rows per pass, 8 passes; 16-byte chunk c of row r goes to the swizzled chunk c ^ (r & 7).
     // Otherwise the threads only arrive.
@@ -526,15 +495,14 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
       const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
       const GroupStatic g = p.gs[c.g];
-      const bool mine = !g.is_shared && p.use_gather == 2;
+      const bool mine = !g.is_shared;
       const bf16* src_row[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         src_row[i] = nullptr;
-        if (mine) {                                   // rows past the group repeat its last row
-          const int r = c.row0 + min(c.mt * kUmmaBM + i * 16 + r_sub, c.count - 1);
-          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + r) * p.d;
-        }
+        const int r = c.mt * kUmmaBM + i * 16 + r_sub;
+        if (mine && r < c.count)                      // rows past the group are left as they are: nothing of them is stored
+          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + c.row0 + r) * p.d;
       }
       for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
@@ -548,7 +516,8 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int r = i * 16 + r_sub;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+            if (src_row[i])
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
                          ::"r"(sa + r * 128 + ((ch ^ (r & 7)) << 4)), "l"(src_row[i] + k_src), "r"(bytes)
                          : "memory");
           }
@@ -704,7 +673,6 @@ struct UmmaBuffers {
   const void* w_down = nullptr;      // packed W_down
   const void* w_rep = nullptr;       // [n_outer][2*n_rp][d] padded representative rows
   const void* x_fixed = nullptr;     // hierarchical: the layer's own outer-row copy of x
-  const void* x_perm = nullptr;      // routed rows of x in expert-contiguous order
   void *h_s = nullptr, *h_r = nullptr, *y_s = nullptr, *y_r = nullptr;
   const GroupStatic* gs_dev = nullptr;
   const float *u = nullptr, *b = nullptr;
@@ -728,8 +696,7 @@ struct UmmaPlan {
   int32_t* rt_ticket = nullptr;            // [n_sms][4], zeroed once
   bool has_s = false, has_r = false;
   PFN_encodeTiled encode = nullptr;
-  CUtensorMap x_rows, x_gather;            // x: 64 x 128 boxes for consecutive rows, 64 x 1 for gather4
-  CUtensorMap x_perm;                      // permuted copy of x
+  CUtensorMap x_rows;                      // x: 64 x 128 boxes of consecutive rows
   CUtensorMap b1_s, b1_r;                  // stacked gate+up rows, box heights bn_s / bn_r
   CUtensorMap a2_s, a2_r, b2_s, b2_r;      // H_s / H_r / shared W_down / routed W_down blocks
   CUtensorMap w_rep;                       // padded representative rows
@@ -738,7 +705,9 @@ struct UmmaPlan {
 // Neurons per gate/up tile: 128 (N = 256 MMAs, the fewest passes over the A rows) when that pads the width
 // by at most 5 %, else the multiple of 8 in [96, 128] that wastes the least of the last tile.  (Measured on
 // widths 864 / 1728 at 16384 tokens: 128 against 96, which pads nothing, is 12 % faster in the gate/up GEMM:
-// seven instead of nine passes over the gathered rows outweigh 3.7 % of padded MMA work.)
+// seven instead of nine passes over the gathered rows outweigh 3.7 % of padded MMA work.  At 130 to 2000 rows the time
+// of a k block hardly falls with the width (425 / 375 / 337 ns for 128 / 96 / 64), so narrower tiles that would even out
+// the last round lose as well.)
 inline int umma_pick_bn(int width) {
   if (width <= 0) return 128;
   if ((long long)((width + 127) / 128 * 128) * 100 <= (long long)width * 105) return 128;
@@ -779,8 +748,7 @@ inline bool umma_encode_rows(UmmaPlan* P, CUtensorMap* tm, const void* base, siz
 // struct fill, no allocation), fixed at plan creation for a hierarchical layer.
 inline bool umma_bind_x(UmmaPlan* P, const void* x_rows, int n_rows) {
   if (P->buf.x_fixed) return true;
-  return umma_encode_rows(P, &P->x_rows, x_rows, (size_t)n_rows, (size_t)P->shape.d, kUmmaBM, "x") &&
-         umma_encode_rows(P, &P->x_gather, x_rows, (size_t)n_rows, (size_t)P->shape.d, 1, "x (gather)");
+  return umma_encode_rows(P, &P->x_rows, x_rows, (size_t)n_rows, (size_t)P->shape.d, kUmmaBM, "x");
 }
 
 // 0: plan built; 1: shape not taken by this path; -5: a driver call failed (P->error).
@@ -819,7 +787,6 @@ inline int umma_plan_create(UmmaPlan* P, const UmmaShape& s, const UmmaBuffers& 
     ok = umma_encode(P, shared ? &P->b1_s : &P->b1_r, buf.w_gate_up, 3, dims, str, box, "gate/up weights");
   }
   if (ok && has_r) ok = umma_encode_rows(P, &P->a2_r, buf.h_r, s.max_routed_rows, s.m, kUmmaBM, "H routed");
-  if (ok && has_r) ok = umma_encode_rows(P, &P->x_perm, buf.x_perm, s.max_routed_rows, d, kUmmaBM, "permuted x");
   if (ok && has_s) ok = umma_encode_rows(P, &P->a2_s, buf.h_s, s.max_outer_rows, s.shared_width, kUmmaBM, "H shared");
   // W_down: shared block [d, W_s] of every outer expert; routed blocks [d, m] x N_r of every outer expert
   if (ok && has_s) {
@@ -842,8 +809,7 @@ inline int umma_plan_create(UmmaPlan* P, const UmmaShape& s, const UmmaBuffers& 
     ok = umma_encode(P, &P->w_rep, buf.w_rep, 3, dims, str, box, "representative rows");
   }
   if (ok && buf.x_fixed)
-    ok = umma_encode_rows(P, &P->x_rows, buf.x_fixed, s.max_outer_rows, d, kUmmaBM, "outer rows of x") &&
-         umma_encode_rows(P, &P->x_gather, buf.x_fixed, s.max_outer_rows, d, 1, "outer rows of x (gather)");
+    ok = umma_encode_rows(P, &P->x_rows, buf.x_fixed, s.max_outer_rows, d, kUmmaBM, "outer rows of x");
   if (!ok) return -5;
   // placeholders for absent operand classes (never dereferenced: such groups have no tiles)
   if (!has_r) { P->a2_r = P->a2_s; P->b2_r = P->b2_s; }
@@ -910,21 +876,18 @@ inline int umma_router_forward(UmmaPlan* P, int n_rows, const int32_t* outer_off
   return 1;
 }
 
-// Enqueues the gate/up and the down GEMM over all groups.  gather_mode: how routed groups get
-// their rows of x (0 permuted copy, 1 TMA gather4, 2 cp.async gather).  Requires umma_bind_x for this
-// forward.  which: bit 0 the gate/up GEMM, bit 1 the down GEMM.  Returns the number of kernels
-// launched, or -1 (P->error).
-inline int umma_forward(UmmaPlan* P, const GroupRows* gr, int gather_mode, const void* x_rows, int32_t* err_word,
-                        cudaStream_t st, cudaEvent_t mid, bool dep = false, int which = 3) {
+// Enqueues the gate/up and the down GEMM over all groups.  Requires umma_bind_x for this forward.  which: bit 0 the
+// gate/up GEMM, bit 1 the down GEMM.  Returns the number of kernels launched, or -1 (P->error).
+inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, int32_t* err_word,
+                        cudaStream_t st, cudaEvent_t mid, bool dep, int which) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
-  a.use_gather = gather_mode;
   a.x_rows_ptr = (const bf16*)x_rows;
   a.band_mt = umma_band_tiles(s.d);
   if (which & 1)
     launch_kernel(dep, umma_grouped_kernel<1>, dim3(P->n_sms), dim3(kUmmaThreads + kUmmaGatherThreads), kUmmaSmemBytes,
-                  st, P->x_rows, (gather_mode != 0 || !P->has_r) ? P->x_gather : P->x_perm, P->b1_s, P->b1_r, a);
+                  st, P->x_rows, P->x_rows, P->b1_s, P->b1_r, a);
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
