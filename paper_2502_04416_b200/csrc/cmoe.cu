@@ -455,8 +455,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                                        L->row_of, L->perm_scratch, st, po, dep);
   } else {
     mark(1);
-    plan_groups_kernel<<<1, 256, 0, st>>>(L->n_outer, n_r, n_tok, L->hier ? L->outer_off : nullptr,
-                                          L->counts, L->offsets, L->gr);
+    launch_kernel(dep && !L->hier, plan_groups_kernel, dim3(1), dim3(256), 0, st, L->n_outer, n_r, n_tok,
+                  (const int32_t*)(L->hier ? L->outer_off : nullptr), (const int32_t*)L->counts, (const int32_t*)L->offsets, L->gr);
     ++launches;
   }
   // The tensor path gathers routed rows inside the gate/up GEMM; only large SIMT tiles read a permuted copy of x.
@@ -912,13 +912,13 @@ int cmoe_profile_activations(cmoe_layer* L, const void* x, int32_t T, int32_t k_
   if (L->cfg.dtype == CMOE_BF16) {
     rc = forward_impl<bf16>(L, (const bf16*)x, T, nullptr, st, true);
     if (rc == CMOE_OK)
-      atopk_kernel<bf16><<<T, kAtopkThreads, (size_t)d_ff * sizeof(uint16_t), st>>>((const bf16*)L->h_s, d_ff, d_ff, k_a, token0, act_bits,
-                                                      words_per_neuron, act_count);
+      launch_kernel(L->chain_launches, atopk_kernel<bf16>, dim3(T), dim3(kAtopkThreads), (size_t)d_ff * sizeof(uint16_t), st,
+                    (const bf16*)L->h_s, d_ff, d_ff, k_a, token0, act_bits, words_per_neuron, act_count);
   } else {
     rc = forward_impl<float>(L, (const float*)x, T, nullptr, st, true);
     if (rc == CMOE_OK)
-      atopk_kernel<float><<<T, kAtopkThreads, (size_t)d_ff * sizeof(uint32_t), st>>>((const float*)L->h_s, d_ff, d_ff, k_a, token0, act_bits,
-                                                       words_per_neuron, act_count);
+      launch_kernel(L->chain_launches, atopk_kernel<float>, dim3(T), dim3(kAtopkThreads), (size_t)d_ff * sizeof(uint32_t), st,
+                    (const float*)L->h_s, d_ff, d_ff, k_a, token0, act_bits, words_per_neuron, act_count);
   }
   if (rc != CMOE_OK) return rc;
   L->launches += 1;

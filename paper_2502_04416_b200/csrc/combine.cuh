@@ -24,6 +24,8 @@ __global__ void plan_groups_kernel(int n_outer, int n_r, int n_tokens,
                                    const int32_t* __restrict__ outer_off /* null: plain layer */,
                                    const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets,
                                    GroupRows* __restrict__ gr) {
+  grid_dep_wait();
+  grid_dep_trigger();
   const int n_groups = n_outer + n_outer * n_r;
   for (int g = threadIdx.x; g < n_groups; g += blockDim.x) {
     GroupRows r;
