@@ -363,29 +363,45 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   cudaEvent_t* ev = (L->ev_ring && !gate_up_only) ? &L->ev[(size_t)(L->ev_count % L->ev_ring) * (CMOE_N_STAGES + 1)] : nullptr;
   auto mark = [&](int i) { if (ev) cudaEventRecord(ev[i], st); };
   mark(0);
-  // bf16 layers on the tensor path chain their kernels by programmatic dependent launch (a kernel
-  // may become resident early and waits on the device for its predecessor).  The small-batch router of a
-  // plain layer is chained to whatever precedes it in the stream, which it waits for in full (7B-shaped layer
-  // 1 / 16 / 300 rows 35.0 / 63.1 / 108.9 -> 33.6 / 61.4 / 104.8 us, even from 600 rows on); per-stage events and the prologue of a hierarchical layer (outer router, outer
-  // permutation, row copy) use ordinary launches.
+  // The kernels of a forward are chained by programmatic dependent launch (a kernel may become resident early and waits on
+  // the device for its predecessor), except while per-stage events are recorded between them.  The first kernel is chained to
+  // whatever precedes it in the stream, which it waits for in full (7B-shaped layer 1 / 16 / 300 rows 35.0 / 63.1 / 108.9
+  // -> 33.6 / 61.4 / 104.8 us, even from 600 rows on).
   const bool dep = !ev && L->chain_launches;
 
+  bool copy_in_router = false;                    // the router copies the outer rows of x in passing
   if (L->hier) {
+    bool routed = false;
     if constexpr (std::is_same<T, bf16>::value) {
-      outer_router_mma_kernel<8, 1><<<(n_tok + 15) / 16, 256, 0, st>>>(
-          x, n_tok, d, L->n_outer, L->outer_k, (const bf16*)L->w_router, L->outer_logits, L->outer_idx,
-          L->outer_w);
+      copy_in_router = n_r > 0 && R <= kRcMaxRows;
+      routed = router_cluster_fuses(n_tok, L->outer_k, L->n_outer);
+      if (routed) {
+        RouterArgs oa{};
+        oa.x = x; oa.n_rows = n_tok; oa.d = d; oa.n_r = L->n_outer; oa.n_k = L->outer_k; oa.w_rep = (const bf16*)L->w_router;
+        oa.ticket = L->router_ticket; oa.scores = L->outer_logits; oa.topk_idx = L->outer_idx; oa.topk_gate = L->outer_w;
+        oa.fuse_permute = 1; oa.n_groups = L->n_outer; oa.counts = L->outer_counts; oa.offsets = L->outer_off;
+        oa.row_token = L->outer_row_token; oa.row_of = L->outer_row_of;
+        CU_TRY(outer_router_cluster_launch(oa, dep, st));
+      } else {
+        outer_router_mma_kernel<8, 1><<<(n_tok + 15) / 16, 256, 0, st>>>(
+            x, n_tok, d, L->n_outer, L->outer_k, (const bf16*)L->w_router, L->outer_logits, L->outer_idx,
+            L->outer_w);
+      }
     } else {
       outer_router_kernel<T><<<(n_tok + 7) / 8, 256, 0, st>>>(x, n_tok, d, L->n_outer, L->outer_k,
                                                               (const T*)L->w_router, L->outer_logits,
                                                               L->outer_idx, L->outer_w);
     }
     ++launches;
-    launches += launch_token_permute(L->outer_idx, n_tok, L->outer_k, L->n_outer, L->outer_counts,
-                                     L->outer_off, L->outer_row_token, L->outer_row_of,
-                                     L->outer_scratch, st);
-    gather_rows_kernel<<<R, 256, 0, st>>>((const uint4*)x, L->outer_row_token, R, row_vec, (uint4*)L->xo);
-    ++launches;
+    if (!routed)
+      launches += launch_token_permute(L->outer_idx, n_tok, L->outer_k, L->n_outer, L->outer_counts,
+                                       L->outer_off, L->outer_row_token, L->outer_row_of,
+                                       L->outer_scratch, st, GroupPlanOut(), dep);
+    if (!copy_in_router) {
+      launch_kernel(dep, gather_rows_kernel, dim3(R), dim3(256), 0, st, (const uint4*)x, (const int32_t*)L->outer_row_token, R,
+                    row_vec, (uint4*)L->xo);
+      ++launches;
+    }
     xo = (const T*)L->xo;
   }
 
@@ -408,8 +424,10 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   const bool decode = use_umma && !gemv && !stream && R <= decode_rows;
   if (use_umma && !stream && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if ((decode || (stream && L->fp8)) && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
-  if ((decode || stream) && L->fp8 && R <= kDecMaxRows) {      // E4M3 planes of the token rows: independent of the routing
-    if (decode_split_x(&L->umma, &L->decode, R, st, dep && !L->hier) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
+  // E4M3 planes of the token rows: independent of the routing, but for the outer rows, which the router may copy
+  const bool split_x = (decode || stream) && L->fp8 && R <= kDecMaxRows;
+  if (split_x && !L->hier) {
+    if (decode_split_x(&L->umma, &L->decode, R, st, dep) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
     ++launches;
   }
   GroupPlanOut po;                                // the permutation also writes every group's row range
@@ -420,7 +438,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     const int32_t* ooff = L->hier ? L->outer_off : nullptr;
     // fp32: a warp per row while that leaves SMs idle (4 warps on each), two rows per warp beyond
 #define CMOE_ROUTER(NACC)                                                                                  \
-  launch_kernel(dep && !L->hier, R <= 592 ? router_row_kernel<T, NACC> : router_kernel<T, NACC>,           \
+  launch_kernel(dep, R <= 592 ? router_row_kernel<T, NACC> : router_kernel<T, NACC>,           \
                 dim3(R <= 592 ? (R + 3) / 4 : blocks), dim3(R <= 592 ? 128 : 256), 0, st, xo, R, d, n_r, L->n_rp, n_k,  \
                 (const T*)L->w_rep, (const float*)L->u, (const float*)L->b, ooff, L->n_outer, L->scores, L->keys,       \
                 L->topk_idx, L->topk_gate)
@@ -431,12 +449,12 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
       } else if (R <= kRcMaxRows) {
         perm_fused = router_cluster_fuses(R, n_k, G);
         RouterArgs ra{};
-        ra.x = xo; ra.n_rows = R; ra.d = d; ra.n_r = n_r; ra.n_rp = L->n_rp; ra.n_k = n_k;
+        ra.x = L->hier ? x : xo; ra.row_src = L->outer_row_token; ra.x_copy = (bf16*)L->xo; ra.n_rows = R; ra.d = d; ra.n_r = n_r; ra.n_rp = L->n_rp; ra.n_k = n_k;
         ra.w_rep = (const bf16*)L->w_rep; ra.u = L->u; ra.b = L->b; ra.outer_off = ooff; ra.n_outer = L->n_outer;
         ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
         ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
         ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
-        CU_TRY(router_cluster_launch(ra, L->hier, dep && !L->hier, stream, st));
+        CU_TRY(router_cluster_launch(ra, L->hier, dep, stream, st));
       } else {
         router_mma_kernel<8, 1><<<(R + 15) / 16, 256, 0, st>>>(
             xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->scores,
@@ -455,8 +473,12 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                                        L->row_of, L->perm_scratch, st, po, dep);
   } else {
     mark(1);
-    launch_kernel(dep && !L->hier, plan_groups_kernel, dim3(1), dim3(256), 0, st, L->n_outer, n_r, n_tok,
+    launch_kernel(dep, plan_groups_kernel, dim3(1), dim3(256), 0, st, L->n_outer, n_r, n_tok,
                   (const int32_t*)(L->hier ? L->outer_off : nullptr), (const int32_t*)L->counts, (const int32_t*)L->offsets, L->gr);
+    ++launches;
+  }
+  if (split_x && L->hier) {
+    if (decode_split_x(&L->umma, &L->decode, R, st, dep) < 0) return arg_fail(CMOE_ERR_CUDA, "split_rows launch failed");
     ++launches;
   }
   // The tensor path gathers routed rows inside the gate/up GEMM; only large SIMT tiles read a permuted copy of x.

@@ -11,11 +11,13 @@ namespace cmoe {
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ idx, int n_rows,
                    int row_vec /* 16-byte vectors per row */, uint4* __restrict__ dst) {
+  grid_dep_wait();
+  grid_dep_trigger();
   const int r = blockIdx.x;
   if (r >= n_rows) return;
-  const uint4* s = src + (size_t)__ldg(idx + r) * row_vec;
+  const uint4* s = src + (size_t)__ldcg(idx + r) * row_vec;
   uint4* o = dst + (size_t)r * row_vec;
-  for (int v = threadIdx.x; v < row_vec; v += blockDim.x) o[v] = __ldg(s + v);
+  for (int v = threadIdx.x; v < row_vec; v += blockDim.x) o[v] = ld_dep16(s + v);
 }
 
 // Row range of every group for this forward.  Groups: n_outer shared groups (rows of

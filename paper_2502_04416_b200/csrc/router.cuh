@@ -54,47 +54,6 @@ __device__ __forceinline__ void gate_row(int lane, int n_r, int n_k, float a, fl
   }
 }
 
-// The same gate logic with W lanes per row (W = 8, 16 or 32 >= n_r): a warp handles 32 / W rows at
-// once.  `sub` is the lane's position in its W-lane group; every lane of the warp must call it (the
-// shuffles name the full warp), `live_row` = false for groups that hold no row.  The arithmetic and
-// its order per row are those of gate_row with the idle lanes removed, so the results are the same bits.
-template <int W>
-__device__ __forceinline__ void gate_row_sub(int sub, bool live_row, int n_r, int n_k, float a, float v,
-                                             const float* __restrict__ u, const float* __restrict__ b,
-                                             int group_base, float* __restrict__ scores_row,
-                                             float* __restrict__ keys_row, int32_t* __restrict__ idx_row,
-                                             float* __restrict__ gates_row) {
-  const bool live = live_row && sub < n_r;
-  const float s = live ? silu_accurate(a) * v : -INFINITY;
-  float s_max = s;
-#pragma unroll
-  for (int o = W / 2; o > 0; o >>= 1) s_max = fmaxf(s_max, __shfl_xor_sync(0xffffffffu, s_max, o));
-  const float e = live ? expf(s - s_max) : 0.0f;
-  float e_sum = e;
-#pragma unroll
-  for (int o = W / 2; o > 0; o >>= 1) e_sum += __shfl_xor_sync(0xffffffffu, e_sum, o);
-  const float s_prime = e / e_sum;
-  const float key = live ? s_prime + __ldg(b + sub) : -INFINITY;
-  if (live) { scores_row[sub] = s; keys_row[sub] = key; }
-  const float gate = live ? 1.0f + s_prime * __ldg(u + sub) : 0.0f;
-  const float rank_key = (key != key) ? -INFINITY : key;
-  const int lane = threadIdx.x & 31, group0 = lane - sub;
-  bool taken = !live;
-  for (int i = 0; i < n_k; ++i) {
-    float best = taken ? -INFINITY : rank_key;
-    int who = taken ? 64 + sub : sub;
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) {
-      const float k2 = __shfl_xor_sync(0xffffffffu, best, o);
-      const int i2 = __shfl_xor_sync(0xffffffffu, who, o);
-      if (k2 > best || (k2 == best && i2 < who)) { best = k2; who = i2; }
-    }
-    const float g = __shfl_sync(0xffffffffu, gate, group0 + (who & (W - 1)));
-    if (sub == who) taken = true;
-    if (live_row && sub == 0) { idx_row[i] = group_base + who; gates_row[i] = g; }
-  }
-}
-
 // A float's bits mapped so that unsigned order is numeric order (-0 counts as +0).
 __device__ __forceinline__ uint32_t ordered_bits(float v) {
   const uint32_t b = __float_as_uint(v + 0.0f);
@@ -126,6 +85,28 @@ __device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float
     if (lane == i) { sel = group_base + who; my_gate = g; }
   }
   if (lane < n_k) { idx_row[lane] = sel; gates_row[lane] = my_gate; }
+}
+
+// Top-level selection of one row (the outer_k largest logits, ties to the lower index; weights = softmax over the
+// selected logits) by the same reduction: lane j < n_outer carries logit j.  Lane i < outer_k returns its selection.
+__device__ __forceinline__ void outer_row_redux(int lane, int n_outer, int outer_k, float logit, float* __restrict__ logits_row,
+                                                int32_t* __restrict__ idx_row, float* __restrict__ weight_row, int& sel) {
+  const bool live = lane < n_outer;
+  if (live) logits_row[lane] = logit;
+  uint32_t bits = live ? ordered_bits((logit != logit) ? -INFINITY : logit) : 0u;
+  float sel_logit = -INFINITY;
+#pragma unroll 1
+  for (int i = 0; i < outer_k; ++i) {
+    const uint32_t best = __reduce_max_sync(0xffffffffu, bits);
+    const int who = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
+    const float l = __shfl_sync(0xffffffffu, logit, who);
+    if (lane == who) bits = 0u;
+    if (lane == i) { sel = who; sel_logit = l; }
+  }
+  const float mx = warp_max(lane < outer_k ? sel_logit : -INFINITY);
+  const float e = lane < outer_k ? expf(sel_logit - mx) : 0.0f;
+  const float weight = e / warp_sum(e);
+  if (lane < outer_k) { idx_row[lane] = sel; weight_row[lane] = weight; }
 }
 
 // One row per warp, for batches that leave SMs idle otherwise (bound by latency).  The column sums meet by a reduce-scatter over the lanes (each step halves

@@ -8,6 +8,10 @@
 //     logic, one warp per row;
 //   - rank 0 collects the selections the same way and, with one row tile, permutes at once; with more, the tile that
 //     takes the last ticket permutes the batch: per group a bit mask of its rows, population counts for ranks and counts.
+// A hierarchical layer runs it twice, for the outer experts and for the inner ones; the second pass reads every outer row
+// from its token and writes the layer's copy of the rows as it goes.  Against a block per 16 tokens for the first, a permutation
+// and a copy kernel, all four unchained: 7 / 128 / 700 tokens of the 8 x 7B-shaped layer 288.8 / 512.4 / 594.2 -> 266.8 /
+// 491.7 / 575.9 us.
 // Against K slices over independent blocks (partial sums and a ticket through global memory, the last block alone
 // doing the gate logic and a block-wide scan; the permutation in kernels of its own above 128 rows), whole forwards: 7B-shaped
 // layer 1 / 16 / 64 / 128 / 512 rows 40.5 / 67.4 / 74.1 / 86.9 / 114.0 -> 35.0 / 62.1 / 69.1 / 80.0 / 109.3 us, 8B-shaped 32 /
@@ -47,13 +51,15 @@ __device__ __forceinline__ void rc_push(uint32_t addr, int v) {
 
 struct RouterArgs {
   const bf16* x;
-  int n_rows, d, n_r, n_rp, n_k;
+  const int32_t* row_src;          // hierarchical: the token of every outer row; x_copy takes the row in passing
+  bf16* x_copy;
+  int n_rows, d, n_r, n_rp, n_k;   // top-level router: n_r = outer experts, n_k = those of a token
   const bf16* w_rep;
   const float *u, *b;
   const int32_t* outer_off;        // hierarchical: row ranges of the outer experts
   int n_outer;
   int32_t* ticket;                 // zero between launches
-  float *scores, *keys;
+  float *scores, *keys;            // top-level router: scores = logits, topk_gate = weights
   int32_t* topk_idx;
   float* topk_gate;
   int fuse_permute, n_groups;
@@ -62,8 +68,9 @@ struct RouterArgs {
 };
 
 // MAXT: tiles of 8 router columns at most (2 N_r rounded up); NB: outer experts whose representative rows are held in
-// flight at once when a tile's rows belong to several (1 for a plain layer).
-template <int MAXT, int NB>
+// flight at once when a tile's rows belong to several (1 for a plain layer).  OUTER: the top-level router of a
+// hierarchical layer, one column per outer expert.
+template <int MAXT, int NB, bool OUTER = false>
 __global__ void __cluster_dims__(kRcCluster, 1, 1) __launch_bounds__(kRcThreads, MAXT * NB <= 2 ? 3 : 2)
 router_cluster_kernel(const RouterArgs p) {
   constexpr int kCols = MAXT * 8, kStride = kCols + 8;
@@ -81,7 +88,7 @@ router_cluster_kernel(const RouterArgs p) {
   const int n_rows = min(kRcRows, p.n_rows - row_base);
   rc_cluster_arrive();                                               // the peers have started: waited for before the push
   const int g = lane >> 2, t = lane & 3;
-  const int n2 = 2 * p.n_rp, n_tiles = n2 >> 3;
+  const int n2 = OUTER ? p.n_r : 2 * p.n_rp, n_tiles = (n2 + 7) >> 3;
   const int n_slices = (p.d + 31) >> 5, s0 = (int)rank * 8 + warp;
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   uint4 w[kUnr][NB][MAXT];
@@ -96,7 +103,7 @@ router_cluster_kernel(const RouterArgs p) {
         const bf16* wr = p.w_rep + ((size_t)(NB > 1 && have ? g_list[i0 + i] : 0) * n2 + g) * p.d + k;
 #pragma unroll
         for (int nt = 0; nt < MAXT; ++nt)
-          w[q][i][nt] = (have && nt < n_tiles) ? __ldg(reinterpret_cast<const uint4*>(wr + (size_t)nt * 8 * p.d)) : zero;
+          w[q][i][nt] = (have && (OUTER ? nt * 8 + g < n2 : nt < n_tiles)) ? __ldg(reinterpret_cast<const uint4*>(wr + (size_t)nt * 8 * p.d)) : zero;
       }
     }
   };
@@ -118,14 +125,14 @@ router_cluster_kernel(const RouterArgs p) {
   const bool gate_warp = warp < 2 && my_row < n_rows;
   float u_pre = 0.0f, b_pre = 0.0f;
   int go_mine = 0;
-  if (gate_warp) {
+  if (!OUTER && gate_warp) {
     if (NB > 1) go_mine = row_group[my_row];
     if (lane < p.n_r) { u_pre = __ldcg(p.u + go_mine * p.n_r + lane); b_pre = __ldcg(p.b + go_mine * p.n_r + lane); }
   }
   // ---- partial sums over this warp's k slices
   const int r_lo = min(g, n_rows - 1), r_hi = min(g + 8, n_rows - 1);
-  const bf16* x_lo = p.x + (size_t)(row_base + r_lo) * p.d + 8 * t;
-  const bf16* x_hi = p.x + (size_t)(row_base + r_hi) * p.d + 8 * t;
+  const bf16* x_lo = p.x + (size_t)(NB > 1 ? __ldcg(p.row_src + row_base + r_lo) : row_base + r_lo) * p.d + 8 * t;
+  const bf16* x_hi = p.x + (size_t)(NB > 1 ? __ldcg(p.row_src + row_base + r_hi) : row_base + r_hi) * p.d + 8 * t;
   const int nl = NB > 1 ? n_list : 1;
 #pragma unroll 1
   for (int i0 = 0; i0 < nl; i0 += NB) {
@@ -147,6 +154,16 @@ router_cluster_kernel(const RouterArgs p) {
         a_hi[q] = in ? ld_dep16(x_hi + k) : zero;
       }
       if (NB > 1 || s != s0) load_w(s, i0, nl);
+      if (NB > 1 && i0 == 0) {                                       // the outer rows, for the GEMMs
+#pragma unroll
+        for (int q = 0; q < kUnr; ++q) {
+          const int k = (s + 64 * q) * 32 + 8 * t;
+          if (k < p.d) {
+            if (g < n_rows) *reinterpret_cast<uint4*>(p.x_copy + (size_t)(row_base + g) * p.d + k) = a_lo[q];
+            if (g + 8 < n_rows) *reinterpret_cast<uint4*>(p.x_copy + (size_t)(row_base + g + 8) * p.d + k) = a_hi[q];
+          }
+        }
+      }
 #pragma unroll
       for (int q = 0; q < kUnr; ++q)
 #pragma unroll
@@ -190,10 +207,13 @@ router_cluster_kernel(const RouterArgs p) {
     float a = 0.0f, v = 0.0f;
     if (lane < p.n_r)
 #pragma unroll
-      for (int q = 0; q < kRcCluster; ++q) { a += recv[q][warp][lane]; v += recv[q][warp][p.n_rp + lane]; }
+      for (int q = 0; q < kRcCluster; ++q) { a += recv[q][warp][lane]; if (!OUTER) v += recv[q][warp][p.n_rp + lane]; }
     const size_t row = (size_t)row_base + my_row;
     int sel = 0;
-    gate_row_redux(lane, p.n_r, p.n_k, a, v, u_pre, b_pre, go_mine * p.n_r, p.scores + row * p.n_r, p.keys + row * p.n_r,
+    if (OUTER)
+      outer_row_redux(lane, p.n_r, p.n_k, a, p.scores + row * p.n_r, p.topk_idx + row * p.n_k, p.topk_gate + row * p.n_k, sel);
+    else
+      gate_row_redux(lane, p.n_r, p.n_k, a, v, u_pre, b_pre, go_mine * p.n_r, p.scores + row * p.n_r, p.keys + row * p.n_r,
                    p.topk_idx + row * p.n_k, p.topk_gate + row * p.n_k, sel);
     if (p.fuse_permute && lane < p.n_k) rc_push(rc_peer(&sel_recv[my_row * p.n_k + lane], 0), sel);
   }
@@ -234,10 +254,17 @@ inline bool router_cluster_fuses(int n_rows, int n_k, int n_groups) {
   return n_rows <= kRcMaxRows && permute_masks_fit(n_rows, n_k, n_groups);
 }
 
+// Top-level router of a hierarchical layer with its permutation (router_cluster_fuses(n_tokens, outer_k, n_outer)).
+inline cudaError_t outer_router_cluster_launch(const RouterArgs& a, bool dep, cudaStream_t st) {
+  const dim3 grid(kRcCluster, (a.n_rows + kRcRows - 1) / kRcRows), block(kRcThreads);
+  if (a.n_r <= 8) return launch_kernel(dep, router_cluster_kernel<1, 1, true>, grid, block, 0, st, a);
+  return launch_kernel(dep, router_cluster_kernel<4, 1, true>, grid, block, 0, st, a);
+}
+
 inline cudaError_t router_cluster_launch(const RouterArgs& a, bool hier, bool dep, bool all_smem, cudaStream_t st) {
   const dim3 grid(kRcCluster, (a.n_rows + kRcRows - 1) / kRcRows), block(kRcThreads);
   const int tiles = 2 * a.n_rp / 8;
-  if (hier) {
+  if (hier) {                                                         // a.row_src and a.x_copy are set
     if (tiles <= 2) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<2, 4>, grid, block, 0, st, a);
     if (tiles <= 4) return launch_kernel_smem(dep, all_smem, router_cluster_kernel<4, 2>, grid, block, 0, st, a);
     return launch_kernel_smem(dep, all_smem, router_cluster_kernel<8, 2>, grid, block, 0, st, a);

@@ -55,3 +55,19 @@ def test_router_hierarchical_tiles(n_routed, n_outer):
         st = parity.check_hier_layer(layer, inp, inp.x[:t])
         assert st["differing"] <= st["near_tie"]
     layer.destroy()
+
+
+# outer experts 1, 8 | 9, 32 (one column tile, four), d cut inside a 32-wide slice, and the 1024 outer rows up to which
+# the routers run clustered and the inner one copies the rows
+@pytest.mark.parametrize("n_outer,outer_k,d,tokens", [(1, 1, 64, (1, 17)), (8, 2, 192, (16, 512, 513)), (9, 3, 72, (15, 341, 342)),
+                                                      (32, 4, 264, (1, 33))])
+def test_router_outer_edges(n_outer, outer_k, d, tokens):
+    shape = wl.LayerShape(d, 16 * 6, 6, 2, 2, "bf16")
+    w = wl.Workload("hier_outer", shape, (max(tokens),), seed=5, n_outer=n_outer, outer_top_k=outer_k)
+    inp = wl.make_inputs(w)
+    inners = [parity.gpu_layer(lay, 8) for lay in inp.layers]
+    layer = binding.Layer.create_hier(parity.to_device(inp.w_router, "bf16"), inners, outer_k, max(tokens))
+    for t in tokens:
+        st = parity.check_hier_layer(layer, inp, inp.x[:t])
+        assert st["differing"] <= st["near_tie"]
+    layer.destroy()
