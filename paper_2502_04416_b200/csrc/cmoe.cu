@@ -22,6 +22,7 @@
 #include "profile.cuh"
 #include "router.cuh"
 #include "router_cluster.cuh"
+#include "router_tile.cuh"
 #include "router_mma.cuh"
 #include "simt_gemm.cuh"
 #include "umma2_gemm.cuh"
@@ -114,11 +115,10 @@ struct cmoe_layer {
   Umma2Plan pair;
   StreamPlan stream;
   int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
-  float* rt_part = nullptr;     // tcgen05 router: K-slice partial sums and tickets
-  int32_t* rt_ticket = nullptr;
+  uint32_t *rt_words = nullptr, *rt_words_outer = nullptr;     // tcgen05 routers: row masks per expert
   float* dec_part = nullptr;    // decode GEMMs: K-slice partial sums, tickets per (tile, epilogue warp)
   int32_t* dec_ticket = nullptr;
-  size_t n_dec_ticket = 0, n_rt_ticket = 0, n_stream_ticket = 0;    // lengths of the ticket arrays (zeroed again after a device timeout)
+  size_t n_dec_ticket = 0, n_stream_ticket = 0;    // lengths of the ticket arrays (zeroed again after a device timeout)
   float *share = nullptr, *target = nullptr;   // utilisation of the last step / bias-update targets
 
   cudaStream_t last_stream = nullptr;
@@ -270,10 +270,9 @@ void carve_workspace(cmoe_layer* L, char* base) {
     L->stream.part = a.take<float>(stream_part_floats((int)T));
   }
   if (esz == 2 && nr > 0) {
-    L->n_rt_ticket = 4 * 256;
-    L->rt_ticket = a.take<int32_t>(L->n_rt_ticket);
-    L->rt_part = a.take<float>((size_t)256 * 64 * 128);
+    L->rt_words = a.take<uint32_t>(router_tile_words((int)R, (int)nr, L->n_outer));
   }
+  if (esz == 2 && L->hier) L->rt_words_outer = a.take<uint32_t>(router_tile_words((int)T, L->n_outer, 1));
   L->ws_bytes = align_up(a.used + 256, 256);
 }
 
@@ -313,15 +312,14 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     ub.w_gate_up = L->w_gu; ub.w_down = L->wd_p; ub.w_rep = L->w_rep;
     ub.x_fixed = L->hier ? L->xo : nullptr;
     ub.h_s = L->h_s; ub.h_r = L->h_r; ub.y_s = L->y_s; ub.y_r = L->y_r;
-    ub.gs_dev = L->gs; ub.u = L->u; ub.b = L->b;
-    ub.scores = L->scores; ub.keys = L->keys; ub.topk_idx = L->topk_idx; ub.topk_gate = L->topk_gate;
+    ub.gs_dev = L->gs; ub.topk_idx = L->topk_idx; ub.topk_gate = L->topk_gate;
     ub.row_token = L->row_token;
     rc = umma_plan_create(&L->umma, s, ub, L->n_groups_total());
     if (rc == CMOE_ERR_CUDA) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     L->umma_ok = (rc == CMOE_OK);
     if (L->umma_ok && !decode_plan_create(&L->umma, &L->decode)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     L->decode.part = L->dec_part; L->decode.ticket = L->dec_ticket;
-    L->umma.rt_part = L->rt_part; L->umma.rt_ticket = L->rt_ticket;
+    if (L->umma_ok) CU_TRY(router_tile_allow());
     if (L->umma_ok && stream_shape_ok(s, L->umma.n_sms) && !stream_plan_create(&L->umma, &L->stream))
       return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     if (L->umma_ok && !umma2_plan_create(&L->umma, &L->pair)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
@@ -382,6 +380,21 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         oa.fuse_permute = 1; oa.n_groups = L->n_outer; oa.counts = L->outer_counts; oa.offsets = L->outer_off;
         oa.row_token = L->outer_row_token; oa.row_of = L->outer_row_of;
         CU_TRY(outer_router_cluster_launch(oa, dep, st));
+      } else if (use_umma) {                       // more tokens than the clustered kernel takes
+        CUtensorMap tm_x, tm_w;
+        RouterTileArgs oa{};
+        oa.n_rows = n_tok; oa.d = d; oa.n_r = L->n_outer; oa.n_k = L->outer_k; oa.n_outer = 1;
+        oa.n_cols = (L->n_outer + 15) / 16 * 16;
+        oa.scores = L->outer_logits; oa.topk_idx = L->outer_idx; oa.topk_gate = L->outer_w;
+        oa.words = L->rt_words_outer; oa.err = L->err_word;
+        if (!umma_encode_rows(&L->umma, &tm_x, x, n_tok, d, kRtTile, "x") ||
+            !router_tile_encode_outer(&L->umma, &tm_w, L->w_router, L->n_outer, d, oa.n_cols))
+          return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+        const int n = router_tile_forward<true>(tm_x, tm_w, oa, PermuteOut{n_tok, L->outer_k, L->n_outer, L->outer_counts,
+            L->outer_off, L->outer_row_token, L->outer_row_of, GroupPlanOut()}, L->outer_scratch, L->umma.n_sms, dep, st);
+        if (n < 0) return arg_fail(CMOE_ERR_CUDA, "outer router launch failed");
+        launches += n - 1;
+        routed = true;
       } else {
         outer_router_mma_kernel<8, 1><<<(n_tok + 15) / 16, 256, 0, st>>>(
             x, n_tok, d, L->n_outer, L->outer_k, (const bf16*)L->w_router, L->outer_logits, L->outer_idx,
@@ -432,7 +445,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   }
   GroupPlanOut po;                                // the permutation also writes every group's row range
   po.gr = L->gr; po.n_outer = L->n_outer; po.n_tokens = n_tok; po.outer_off = L->hier ? L->outer_off : nullptr;
-  bool perm_fused = false;                        // decode: the router's last block also permutes
+  bool perm_fused = false, marked = false;        // the router's launches include the permutation; stage 1 is recorded
   if (n_r > 0) {
     const int warps = (R + 1) / 2, blocks = (warps + 7) / 8;
     const int32_t* ooff = L->hier ? L->outer_off : nullptr;
@@ -443,9 +456,18 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
                 (const T*)L->w_rep, (const float*)L->u, (const float*)L->b, ooff, L->n_outer, L->scores, L->keys,       \
                 L->topk_idx, L->topk_gate)
     if constexpr (std::is_same<T, bf16>::value) {
-      if (use_umma && R > kRcMaxRows) {
-        if (umma_router_forward(&L->umma, R, ooff, L->err_word, st) < 0)
-          return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+      if (use_umma && router_takes_tiles(R, L->n_rp, L->hier)) {
+        CUtensorMap tm_x;
+        if (!umma_encode_rows(&L->umma, &tm_x, xo, R, d, kRtTile, "x")) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+        RouterTileArgs ra{};
+        ra.n_rows = R; ra.d = d; ra.n_r = n_r; ra.n_rp = L->n_rp; ra.n_k = n_k; ra.n_cols = 2 * L->n_rp;
+        ra.n_outer = L->n_outer; ra.outer_off = ooff; ra.u = L->u; ra.b = L->b; ra.scores = L->scores; ra.keys = L->keys;
+        ra.topk_idx = L->topk_idx; ra.topk_gate = L->topk_gate; ra.words = L->rt_words; ra.err = L->err_word;
+        const int n = router_tile_forward<false>(tm_x, L->umma.w_rep, ra, PermuteOut{R, n_k, G, L->counts, L->offsets,
+            L->row_token, L->row_of, po}, L->perm_scratch, L->umma.n_sms, dep, st, ev ? ev[1] : nullptr);
+        if (n < 0) return arg_fail(CMOE_ERR_CUDA, "router launch failed");
+        launches += n - 1;
+        perm_fused = marked = true;
       } else if (R <= kRcMaxRows) {
         perm_fused = router_cluster_fuses(R, n_k, G);
         RouterArgs ra{};
@@ -467,7 +489,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     }
 #undef CMOE_ROUTER
     ++launches;
-    mark(1);
+    if (!marked) mark(1);
     if (!perm_fused)
       launches += launch_token_permute(L->topk_idx, R, n_k, G, L->counts, L->offsets, L->row_token,
                                        L->row_of, L->perm_scratch, st, po, dep);
@@ -1119,7 +1141,6 @@ int cmoe_layer_status(cmoe_layer* L, int32_t* device_error_word) {
   CU_TRY(cudaMemsetAsync(L->router_ticket, 0, 4, st));
   if (L->dec_ticket) CU_TRY(cudaMemsetAsync(L->dec_ticket, 0, L->n_dec_ticket * 4, st));
   if (L->n_stream_ticket) CU_TRY(cudaMemsetAsync(L->stream.ticket, 0, L->n_stream_ticket * 4, st));
-  if (L->rt_ticket) CU_TRY(cudaMemsetAsync(L->rt_ticket, 0, L->n_rt_ticket * 4, st));
   CU_TRY(cudaStreamSynchronize(st));
   return CMOE_ERR_DEVICE_TIMEOUT;
 }

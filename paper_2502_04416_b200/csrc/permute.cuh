@@ -28,7 +28,7 @@ __device__ __forceinline__ void chunk_histogram(const int32_t* __restrict__ topk
 }
 
 // Exclusive scan of counts[0..n_groups) into offsets[0..n_groups]; sums[] holds
-// blockDim.x ints of shared memory.
+// an int per warp in shared memory (blockDim.x is a multiple of 32).
 __device__ __forceinline__ void block_scan_groups(const int32_t* counts, int32_t* offsets,
                                                   int n_groups, int32_t* sums) {
   const int per = (n_groups + blockDim.x - 1) / blockDim.x;
@@ -36,15 +36,18 @@ __device__ __forceinline__ void block_scan_groups(const int32_t* counts, int32_t
   const int hi = min(lo + per, n_groups);
   int s = 0;
   for (int g = lo; g < hi; ++g) s += counts[g];
-  sums[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int i = 0; i < (int)blockDim.x; ++i) { const int v = sums[i]; sums[i] = run; run += v; }
-    offsets[n_groups] = run;
+  int incl = s;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
   }
+  if (lane == 31) sums[warp] = incl;
   __syncthreads();
-  int run = sums[threadIdx.x];
+  int run = incl - s;
+  for (int w = 0; w < warp; ++w) run += sums[w];
+  if (threadIdx.x == blockDim.x - 1) offsets[n_groups] = run + s;
   for (int g = lo; g < hi; ++g) { offsets[g] = run; run += counts[g]; }
   __syncthreads();
 }

@@ -60,31 +60,67 @@ __device__ __forceinline__ uint32_t ordered_bits(float v) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// gate_row with u and b already in registers and the arg-max by one warp-wide integer reduction and a ballot (the
-// same order: larger key first, equal keys by index).  Lane i < n_k returns its selection in `sel`.
-__device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float a, float v, float u, float b, int group_base,
-                                               float* __restrict__ scores_row, float* __restrict__ keys_row,
-                                               int32_t* __restrict__ idx_row, float* __restrict__ gates_row, int& sel) {
+// gate_row for U rows at once, step by step so that the rows' chains of reductions overlap, with u and b already in
+// registers and the arg-max by one warp-wide integer reduction and a ballot (the same order: larger key first, equal keys by
+// index).  Lane i < n_k returns its selections in `sel`; rows that are not live are not stored.
+template <int U>
+__device__ __forceinline__ void gate_rows_redux(int lane, int n_r, int n_k, const float (&a)[U], const float (&v)[U], float u,
+                                                float b, int group_base, const size_t (&row)[U], const bool (&row_live)[U],
+                                                float* __restrict__ scores, float* __restrict__ keys,
+                                                int32_t* __restrict__ idx, float* __restrict__ gates, int (&sel)[U]) {
   const bool live = lane < n_r;
-  const float s = live ? silu_accurate(a) * v : -INFINITY;            // Eq. router
-  const float s_max = warp_max(s);
-  const float e = live ? expf(s - s_max) : 0.0f;
-  const float s_prime = e / warp_sum(e);                               // Softmax over all N_r
-  const float key = live ? s_prime + b : -INFINITY;
-  if (live) { scores_row[lane] = s; keys_row[lane] = key; }
-  const float gate = 1.0f + s_prime * u;                               // 1 + s'_i u_i
-  const float rank_key = (key != key) ? -INFINITY : key;               // NaN ranks last
-  uint32_t bits = live ? ordered_bits(rank_key) : 0u;                  // every live key is above 0
-  float my_gate = 0.0f;
+  float s[U], m[U], e[U], sum[U], gate[U], my_gate[U];
+  uint32_t bits[U];
+#pragma unroll
+  for (int q = 0; q < U; ++q) { s[q] = live ? silu_accurate(a[q]) * v[q] : -INFINITY; m[q] = s[q]; }   // Eq. router
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < U; ++q) m[q] = fmaxf(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
+#pragma unroll
+  for (int q = 0; q < U; ++q) { e[q] = live ? expf(s[q] - m[q]) : 0.0f; sum[q] = e[q]; }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < U; ++q) sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], o);
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+    const float s_prime = e[q] / sum[q];                               // Softmax over all N_r
+    const float key = live ? s_prime + b : -INFINITY;
+    if (live && row_live[q]) { scores[row[q] * n_r + lane] = s[q]; keys[row[q] * n_r + lane] = key; }
+    gate[q] = 1.0f + s_prime * u;                                      // 1 + s'_i u_i
+    bits[q] = live ? ordered_bits((key != key) ? -INFINITY : key) : 0u;  // NaN ranks last; every live key is above 0
+    my_gate[q] = 0.0f;
+  }
 #pragma unroll 1
   for (int i = 0; i < n_k; ++i) {
-    const uint32_t best = __reduce_max_sync(0xffffffffu, bits);
-    const int who = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
-    const float g = __shfl_sync(0xffffffffu, gate, who);
-    if (lane == who) bits = 0u;
-    if (lane == i) { sel = group_base + who; my_gate = g; }
+    uint32_t best[U];
+    int who[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) best[q] = __reduce_max_sync(0xffffffffu, bits[q]);
+#pragma unroll
+    for (int q = 0; q < U; ++q) who[q] = __ffs(__ballot_sync(0xffffffffu, bits[q] == best[q])) - 1;
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const float g = __shfl_sync(0xffffffffu, gate[q], who[q]);
+      if (lane == who[q]) bits[q] = 0u;
+      if (lane == i) { sel[q] = group_base + who[q]; my_gate[q] = g; }
+    }
   }
-  if (lane < n_k) { idx_row[lane] = sel; gates_row[lane] = my_gate; }
+  if (lane < n_k)
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (row_live[q]) { idx[row[q] * n_k + lane] = sel[q]; gates[row[q] * n_k + lane] = my_gate[q]; }
+}
+__device__ __forceinline__ void gate_row_redux(int lane, int n_r, int n_k, float a, float v, float u, float b, int group_base,
+                                               size_t row, float* __restrict__ scores, float* __restrict__ keys,
+                                               int32_t* __restrict__ idx, float* __restrict__ gates, int& sel) {
+  const float a1[1] = {a}, v1[1] = {v};
+  const size_t r1[1] = {row};
+  const bool l1[1] = {true};
+  int s1[1] = {0};
+  gate_rows_redux<1>(lane, n_r, n_k, a1, v1, u, b, group_base, r1, l1, scores, keys, idx, gates, s1);
+  sel = s1[0];
 }
 
 // Top-level selection of one row (the outer_k largest logits, ties to the lower index; weights = softmax over the
@@ -177,8 +213,7 @@ router_row_kernel(const T* __restrict__ xo, int n_rows, int d, int n_r, int n_rp
     if (cv >= 32) v = v1;
   }
   int sel = 0;
-  gate_row_redux(lane, n_r, n_k, a, v, u_pre, b_pre, go * n_r, scores + (size_t)row * n_r, keys + (size_t)row * n_r,
-                 topk_idx + (size_t)row * n_k, topk_gate + (size_t)row * n_k, sel);
+  gate_row_redux(lane, n_r, n_k, a, v, u_pre, b_pre, go * n_r, (size_t)row, scores, keys, topk_idx, topk_gate, sel);
 }
 
 template <typename T, int NACC>

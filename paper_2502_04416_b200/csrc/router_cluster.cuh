@@ -213,8 +213,7 @@ router_cluster_kernel(const RouterArgs p) {
     if (OUTER)
       outer_row_redux(lane, p.n_r, p.n_k, a, p.scores + row * p.n_r, p.topk_idx + row * p.n_k, p.topk_gate + row * p.n_k, sel);
     else
-      gate_row_redux(lane, p.n_r, p.n_k, a, v, u_pre, b_pre, go_mine * p.n_r, p.scores + row * p.n_r, p.keys + row * p.n_r,
-                   p.topk_idx + row * p.n_k, p.topk_gate + row * p.n_k, sel);
+      gate_row_redux(lane, p.n_r, p.n_k, a, v, u_pre, b_pre, go_mine * p.n_r, row, p.scores, p.keys, p.topk_idx, p.topk_gate, sel);
     if (p.fuse_permute && lane < p.n_k) rc_push(rc_peer(&sel_recv[my_row * p.n_k + lane], 0), sel);
   }
   if (!p.fuse_permute) return;

@@ -16,10 +16,6 @@
 //   MODE 2, down GEMM: Y[r, c] = sum_n H[r, n] Wd[c, n]
 //       A tile  : 128 rows of H x 64 k ;  B tile: 256 output channels of the group's W_down
 //       block x 64 k ;  D: 128 x 256 fp32 ; epilogue rounds to bf16 Y.
-//   MODE 3, router: a_j = x_r . w_gate^{R_j}, v_j = x_r . w_up^{R_j}          (Eq. router)
-//       B tile  : the (outer) layer's padded representative rows, gate block then up block;
-//       epilogue: one thread per row does Swish(a)*v, the softmax over all N_r scores, the
-//       biased top-N_k and the gates 1 + s'u                                 (Eq. final_gate).
 // All operands are K-major with the 128-byte swizzle; rows or k beyond a tensor's extent
 // are zero-filled by TMA, rows beyond a group's count are computed but never stored.
 //
@@ -224,36 +220,12 @@ struct UmmaArgs {
   int band_mt;                // row tiles per band of the tile order (see umma_decode)
   const bf16* x_rows_ptr;     // mode 1: the outer rows of x (source of the cp.async gather)
   int32_t* err;
-  // mode 3 (router)
-  int ksplit;                 // K slices per tile (>= 1): a tile's k range is cut so that more SMs take part
-  float* rt_part;             // ksplit > 1: [unit][2 n_rp columns][128 rows] fp32 partial sums
-  int32_t* rt_ticket;         // ksplit > 1: [tile][4 epilogue warps], zero between launches
-  const int32_t* outer_off;   // row ranges of the outer experts, or null (one range [0, n_rows))
-  int n_rows, n_rp, n_k;      // n_rp: N_r rounded up to 8 (rows per block of the padded W^R)
-  const float* u;
-  const float* b;
-  float* scores;
-  float* keys;
-  int32_t* topk_idx;
-  float* topk_gate;
 };
 
 struct TileCoord { int g, mt, nt, row0, count; };
 
 template <int MODE>
-__device__ __forceinline__ GroupRows umma_rows(const UmmaArgs& p, int g) {
-  if (MODE == 3) {
-    GroupRows r;
-    r.row0 = p.outer_off ? p.outer_off[g] : 0;
-    r.count = p.outer_off ? p.outer_off[g + 1] - p.outer_off[g] : p.n_rows;
-    return r;
-  }
-  return p.gr[g];
-}
-
-template <int MODE>
 __device__ __forceinline__ int umma_n_tiles(const UmmaArgs& p, int g) {
-  if (MODE == 3) return 1;
   const GroupStatic gs = p.gs[g];
   if (MODE == 1) {
     const int bn = gs.is_shared ? p.bn_s : p.bn_r;
@@ -271,7 +243,7 @@ __device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_
     if (tile_start[mid] <= t) lo = mid; else hi = mid;
   }
   const int local = t - tile_start[lo];
-  const GroupRows r = umma_rows<MODE>(p, lo);
+  const GroupRows r = p.gr[lo];
   // Order inside a group: bands of p.band_mt row tiles; inside a band the row tiles run fastest (CTAs
   // working side by side share a weight tile), then the n-tiles, then the next band.  A band's rows of A
   // (about 16 MB) stay in L2 while the n-tiles pass over them; without bands a large group's rows left L2
@@ -280,63 +252,13 @@ __device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_
   // groups that do fit (every CTA then streams a different weight tile).
   const int m_tiles = (r.count + kUmmaBM - 1) / kUmmaBM;
   const int n_tiles = umma_n_tiles<MODE>(p, lo);
-  const int band_mt = MODE == 3 ? m_tiles : max(p.band_mt, 1);
+  const int band_mt = max(p.band_mt, 1);
   const int per_band = band_mt * n_tiles;
   const int band = local / per_band, in_band = local - band * per_band;
   const int cur_mt = min(band_mt, m_tiles - band * band_mt);
   TileCoord c;
   c.g = lo; c.nt = in_band / cur_mt; c.mt = band * band_mt + in_band % cur_mt; c.row0 = r.row0; c.count = r.count;
   return c;
-}
-
-// Router epilogue for one row (Eq. router, Eq. final_gate): a[j], v[j] are the gate / up
-// pre-activations of routed expert j's representative neuron, j < n_r <= 32.
-__device__ __forceinline__ void router_row_epilogue(const float (&a)[32], const float (&v)[32], int n_r, int n_k,
-                                                    const float* __restrict__ u, const float* __restrict__ b,
-                                                    int group_base, float* __restrict__ scores_row,
-                                                    float* __restrict__ keys_row, int32_t* __restrict__ idx_row,
-                                                    float* __restrict__ gates_row) {
-  float s[32];
-  float s_max = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    s[j] = j < n_r ? silu_accurate(a[j]) * v[j] : -INFINITY;
-    s_max = fmaxf(s_max, s[j]);
-  }
-  float sum = 0.0f;
-  float e[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    e[j] = j < n_r ? expf(s[j] - s_max) : 0.0f;
-    sum += e[j];
-  }
-  float key[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    if (j < n_r) {
-      e[j] = e[j] / sum;                              // s'_j
-      const float k = e[j] + __ldg(b + j);
-      scores_row[j] = s[j];
-      keys_row[j] = k;
-      key[j] = (k != k) ? -INFINITY : k;              // NaN ranks last
-    } else {
-      key[j] = -INFINITY;
-    }
-  }
-  uint32_t taken = 0;
-  for (int i = 0; i < n_k; ++i) {
-    int who = -1;
-    float best = 0.0f, best_sp = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      if (j < n_r && !((taken >> j) & 1u) && (who < 0 || key[j] > best)) {   // ties: lower index
-        who = j; best = key[j]; best_sp = e[j];
-      }
-    }
-    taken |= 1u << who;
-    idx_row[i] = group_base + who;
-    gates_row[i] = 1.0f + best_sp * __ldg(u + who);
-  }
 }
 
 template <int MODE>
@@ -350,8 +272,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - raw);                       // generic pointer to the aligned base
-  constexpr int kStages = MODE == 3 ? 8 : kUmmaStages;             // the router's B tile is at most 8 KB
-  constexpr int kStageBytes = MODE == 3 ? kUmmaABytes + 8192 : kUmmaStageBytes;
+  constexpr int kStages = kUmmaStages, kStageBytes = kUmmaStageBytes;
   const uint32_t bars = base + kStages * kStageBytes;   // barrier block
   uint8_t* bars_gen = gen + kStages * kStageBytes;
   // barrier block: full[8] empty[8] acc_full[2] acc_empty[2] (8 B each), tmem slot, abort flag
@@ -361,7 +282,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int n_groups = MODE == 3 ? p.n_outer : p.n_groups;
+  const int n_groups = p.n_groups;
 
   if (threadIdx.x == 0) {
     // mode 1: besides the producer's expect_tx arrival, every gather thread arrives once per stage
@@ -378,7 +299,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   }
   // tiles of every group, then their exclusive prefix
   for (int g = threadIdx.x; g < n_groups; g += blockDim.x) {
-    const int m_tiles = (umma_rows<MODE>(p, g).count + kUmmaBM - 1) / kUmmaBM;
+    const int m_tiles = (p.gr[g].count + kUmmaBM - 1) / kUmmaBM;
     tile_start[g + 1] = m_tiles * umma_n_tiles<MODE>(p, g);
   }
   __syncthreads();
@@ -392,19 +313,15 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int total_tiles = tile_start[n_groups];
-  const int ksplit = MODE == 3 ? max(p.ksplit, 1) : 1;
-  const int total_units = total_tiles * ksplit;
-  const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;      // modes 1 and 3: K = d
+  const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;      // mode 1: K = d
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp)
     uint32_t it = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-      const int t = u / ksplit, kz = u - t * ksplit;
+    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
       const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
-      GroupStatic g;
-      if (MODE != 3) g = p.gs[c.g]; else { g.is_shared = 1; g.outer = c.g; g.width = 0; g.w_row0 = 0; }
+      const GroupStatic g = p.gs[c.g];
       const int row = c.row0 + c.mt * kUmmaBM;
       const bool by_threads = MODE == 1 && !g.is_shared;              // the gather warps fill A
       const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
@@ -415,17 +332,13 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
         k_blocks = k_blocks_fixed;
         b_bytes = 2 * bn * kUmmaBK * 2;
         b_row = g.w_row0 + c.nt * bn;
-      } else if (MODE == 2) {
+      } else {
         k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK;
         b_bytes = kUmmaBBytes;
         b_row = c.nt * 256;
         j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
-      } else {
-        k_blocks = k_blocks_fixed;
-        b_bytes = 2 * p.n_rp * kUmmaBK * 2;
       }
-      const int kb_lo = kz * k_blocks / ksplit, kb_hi = (kz + 1) * k_blocks / ksplit;      // this unit's k slice
-      for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
+      for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
         if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb = full0 + 8 * s;
@@ -434,7 +347,6 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
           mbar_expect_tx(fb, (by_threads ? 0 : kUmmaABytes) + b_bytes);
           if (!by_threads) tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
           if (MODE == 1) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, 0);
-          else if (MODE == 3) tma_load_3d(sb, tb, fb, kb * kUmmaBK, 0, c.g);
           else if (g.is_shared) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
           else tma_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
         }
@@ -446,25 +358,21 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
     uint32_t it = 0, tile_n = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++tile_n) {
-      const int t = u / ksplit, kz = u - t * ksplit;
+    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_n) {
       const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
       int k_blocks, n_mma;
       if (MODE == 1) {
         const GroupStatic g = p.gs[c.g];
         k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r);
-      } else if (MODE == 2) {
-        k_blocks = (p.gs[c.g].width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
       } else {
-        k_blocks = k_blocks_fixed; n_mma = 2 * p.n_rp;
+        k_blocks = (p.gs[c.g].width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
       }
       const uint32_t idesc = umma_idesc(n_mma);
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
       if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + buf * 256;
-      const int kb_lo = kz * k_blocks / ksplit, kb_hi = (kz + 1) * k_blocks / ksplit;
-      for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
+      for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
         if (!mbar_wait_warp(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
         if (MODE == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // cp.async-written rows
@@ -474,7 +382,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
 #pragma unroll
           for (int k = 0; k < kUmmaBK / 16; ++k)
             umma_bf16(d_tmem, umma_smem_desc(sa + k * 32), umma_smem_desc(sb + k * 32), idesc,
-                      (kb != kb_lo || k != 0) ? 1u : 0u);
+                      (kb != 0 || k != 0) ? 1u : 0u);
           umma_commit(empty0 + 8 * s);         // stage reusable once these MMAs have read it
         }
         __syncwarp();
@@ -533,8 +441,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
     uint32_t tile_n = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++tile_n) {
-      const int t = u / ksplit, kz = u - t * ksplit;
+    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_n) {
       const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
       if (!mbar_wait(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
@@ -574,7 +481,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
             }
           }
         }
-      } else if (MODE == 2) {
+      } else {
         const GroupStatic g = p.gs[c.g];
         const int n0 = c.nt * 256;
         const int n_valid = min(256, p.d - n0);
@@ -597,56 +504,6 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
               }
             }
           }
-        }
-      } else {
-        float a[32], v[32];
-        tmem_ld16(taddr, a);
-        tmem_ld16(taddr + p.n_rp, v);
-        if (p.n_rp > 16) {                     // warp-uniform
-          tmem_ld16(taddr + 16, a + 16);
-          tmem_ld16(taddr + p.n_rp + 16, v + 16);
-        }
-        tmem_ld_wait();
-        bool finish_row = true;
-        if (ksplit > 1) {
-          // K slice of a split tile: park this row's partial sums ([column][row]: a warp's store is one
-          // 128-byte line), take the warp's ticket for the tile; the warp that takes the last one adds
-          // the slices in ascending order (a fixed order: deterministic) and goes on to the gate logic
-          const int row128 = quad * 32 + lane;
-          float* mine = p.rt_part + ((size_t)t * ksplit + kz) * (64 * 128) + row128;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < p.n_rp) { __stcg(mine + (size_t)j * 128, a[j]); __stcg(mine + (size_t)(32 + j) * 128, v[j]); }
-          }
-          __threadfence();
-          __syncwarp();
-          int32_t* tk = p.rt_ticket + (size_t)t * 4 + quad;
-          int last = 0;
-          if (lane == 0) last = atomicAdd(tk, 1) == ksplit - 1;
-          last = __shfl_sync(0xffffffffu, last, 0);
-          finish_row = last != 0;
-          if (finish_row) {
-            __threadfence();
-            const float* all = p.rt_part + (size_t)t * ksplit * (64 * 128) + row128;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) { a[j] = 0.0f; v[j] = 0.0f; }
-            for (int z = 0; z < ksplit; ++z) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                if (j < p.n_rp) {
-                  a[j] += __ldcg(all + (size_t)z * (64 * 128) + (size_t)j * 128);
-                  v[j] += __ldcg(all + (size_t)z * (64 * 128) + (size_t)(32 + j) * 128);
-                }
-              }
-            }
-            if (lane == 0) *tk = 0;            // ready for the next launch
-          }
-        }
-        if (row_ok && finish_row) {
-          const size_t row = (size_t)(c.row0 + row_in_group);
-          router_row_epilogue(a, v, p.n_r, p.n_k, p.u + c.g * p.n_r, p.b + c.g * p.n_r, c.g * p.n_r,
-                              p.scores + row * p.n_r, p.keys + row * p.n_r, p.topk_idx + row * p.n_k,
-                              p.topk_gate + row * p.n_k);
         }
       }
       tc_fence_before();
@@ -675,9 +532,8 @@ struct UmmaBuffers {
   const void* x_fixed = nullptr;     // hierarchical: the layer's own outer-row copy of x
   void *h_s = nullptr, *h_r = nullptr, *y_s = nullptr, *y_r = nullptr;
   const GroupStatic* gs_dev = nullptr;
-  const float *u = nullptr, *b = nullptr;
-  float *scores = nullptr, *keys = nullptr, *topk_gate = nullptr;
-  int32_t* topk_idx = nullptr;
+  const float* topk_gate = nullptr;
+  const int32_t* topk_idx = nullptr;
   const int32_t* row_token = nullptr;
 };
 
@@ -692,8 +548,6 @@ struct UmmaPlan {
   UmmaShape shape;
   UmmaBuffers buf;
   int bn_s = 128, bn_r = 128, n_sms = 0, n_groups = 0;
-  float* rt_part = nullptr;                // router K-slice partials: n_sms units x 64 columns x 128 rows (caller's workspace)
-  int32_t* rt_ticket = nullptr;            // [n_sms][4], zeroed once
   bool has_s = false, has_r = false;
   PFN_encodeTiled encode = nullptr;
   CUtensorMap x_rows;                      // x: 64 x 128 boxes of consecutive rows
@@ -818,7 +672,6 @@ inline int umma_plan_create(UmmaPlan* P, const UmmaShape& s, const UmmaBuffers& 
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
   if (e != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     return -5;
@@ -844,36 +697,7 @@ inline UmmaArgs umma_base_args(const UmmaPlan* P, const GroupRows* gr, int32_t* 
   a.d = s.d; a.bn_s = P->bn_s; a.bn_r = P->bn_r; a.err = err_word;
   a.row_token = P->buf.row_token;
   a.x_rows_ptr = nullptr;
-  a.n_rp = s.n_rp; a.n_k = s.n_k; a.u = P->buf.u; a.b = P->buf.b;
-  a.scores = P->buf.scores; a.keys = P->buf.keys; a.topk_idx = P->buf.topk_idx; a.topk_gate = P->buf.topk_gate;
   return a;
-}
-
-// Router on the tensor path (mode 3).  Requires umma_bind_x for this forward.  Returns launches or -1.
-inline int umma_router_forward(UmmaPlan* P, int n_rows, const int32_t* outer_off, int32_t* err_word,
-                               cudaStream_t st) {
-  UmmaArgs a = umma_base_args(P, nullptr, err_word);
-  a.outer_off = outer_off; a.n_rows = n_rows;
-  const int tiles = (n_rows + kUmmaBM - 1) / kUmmaBM + P->shape.n_outer;     // upper bound of the tile count
-  // with few tiles, cut each tile's K range so that up to four times as many SMs stream x
-  int ksplit = 1;
-  if (P->rt_part && P->rt_ticket) {
-    const int kb = (P->shape.d + kUmmaBK - 1) / kUmmaBK;
-    ksplit = P->n_sms / tiles;
-    if (ksplit > 4) ksplit = 4;
-    if (ksplit > kb / 8) ksplit = kb / 8;
-    if (ksplit < 1) ksplit = 1;
-  }
-  a.ksplit = ksplit; a.rt_part = P->rt_part; a.rt_ticket = P->rt_ticket;
-  const int units = tiles * ksplit;
-  const int grid = units < P->n_sms ? units : P->n_sms;
-  umma_grouped_kernel<3><<<grid, kUmmaThreads, kUmmaSmemBytes, st>>>(P->x_rows, P->x_rows, P->w_rep, P->w_rep, a);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    snprintf(P->error, sizeof(P->error), "tensor-core router launch: %s", cudaGetErrorString(e));
-    return -1;
-  }
-  return 1;
 }
 
 // Enqueues the gate/up and the down GEMM over all groups.  Requires umma_bind_x for this forward.  which: bit 0 the

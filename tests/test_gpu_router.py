@@ -1,4 +1,4 @@
-"""-m gpu: the clustered small-batch router (up to 1024 rows) with its fused permutation, at the edges of
+"""-m gpu: the clustered router (up to 1024 rows) with its fused permutation and the tile router, at the edges of
 its 16-row tiles and row limit, of its 32-wide k slices and of its column tiles."""
 import numpy as np
 import pytest
@@ -64,6 +64,34 @@ def test_router_hierarchical_tiles(n_routed, n_outer):
 def test_router_outer_edges(n_outer, outer_k, d, tokens):
     shape = wl.LayerShape(d, 16 * 6, 6, 2, 2, "bf16")
     w = wl.Workload("hier_outer", shape, (max(tokens),), seed=5, n_outer=n_outer, outer_top_k=outer_k)
+    inp = wl.make_inputs(w)
+    inners = [parity.gpu_layer(lay, 8) for lay in inp.layers]
+    layer = binding.Layer.create_hier(parity.to_device(inp.w_router, "bf16"), inners, outer_k, max(tokens))
+    for t in tokens:
+        st = parity.check_hier_layer(layer, inp, inp.x[:t])
+        assert st["differing"] <= st["near_tie"]
+    layer.destroy()
+
+
+# tile routers: rows at the edges of a 64-row tile, of the line at 512 rows, and for clusters of 8, 4, 2 and 1 CTAs; k cut inside
+# a block; 32832 rows of 32 experts: more row masks than the one-launch permutation takes
+@pytest.mark.parametrize("n_experts,n_shared,top_k,d,tokens", [(20, 2, 4, 1032, (512, 513, 576, 577)), (9, 1, 2, 1032, (1025, 2400)),
+                                                               (33, 1, 8, 520, (4800,)), (12, 1, 3, 520, (9601,)),
+                                                               (33, 1, 2, 64, (32832,))])
+def test_router_tiles(n_experts, n_shared, top_k, d, tokens):
+    lay, x = _layer(n_experts, n_shared, top_k, d, max(tokens))
+    layer = parity.gpu_layer(lay, max(tokens))
+    for t in tokens:
+        st = parity.check_plain_layer(layer, lay, x[:t])
+        assert st["differing"] <= st["near_tie"]
+    layer.destroy()
+
+
+# outer rows past 1024 (tiles that begin at every expert's first row), tokens past 1024 (top-level router on tiles)
+@pytest.mark.parametrize("n_outer,outer_k,tokens", [(9, 2, (520, 1025)), (20, 4, (300, 1090)), (3, 1, (1024, 1025))])
+def test_router_tiles_hierarchical(n_outer, outer_k, tokens):
+    shape = wl.LayerShape(200, 16 * 6, 6, 2, 2, "bf16")
+    w = wl.Workload("hier_tiles", shape, (max(tokens),), seed=3, n_outer=n_outer, outer_top_k=outer_k)
     inp = wl.make_inputs(w)
     inners = [parity.gpu_layer(lay, 8) for lay in inp.layers]
     layer = binding.Layer.create_hier(parity.to_device(inp.w_router, "bf16"), inners, outer_k, max(tokens))
