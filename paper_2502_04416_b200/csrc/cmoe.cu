@@ -476,7 +476,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
         ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
         ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
-        CU_TRY(router_cluster_launch(ra, L->hier, dep, stream, st));
+        CU_TRY(router_cluster_launch(ra, L->hier, dep, use_umma && !gemv && !L->hier, st));
       } else {
         router_mma_kernel<8, 1><<<(R + 15) / 16, 256, 0, st>>>(
             xo, R, d, n_r, L->n_rp, n_k, (const bf16*)L->w_rep, L->u, L->b, ooff, L->n_outer, L->scores,
@@ -567,8 +567,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
       for (int bit = 1; bit <= 2 && n >= 0; bit <<= 1) {          // gate/up, then down, each on its chosen tile shape
         if (!(todo & bit)) continue;
         const int k = (pair_mask & bit)
-            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit)
-            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit);
+            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R)
+            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R);
         n = k < 0 ? -1 : n + k;
       }
     }

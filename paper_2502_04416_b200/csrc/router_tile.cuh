@@ -275,8 +275,8 @@ permute_words_kernel(const uint32_t* __restrict__ words, const int32_t* __restri
   const int c0 = blockIdx.x * 8, c = c0 + warp;
 #pragma unroll 1
   for (int g = threadIdx.x; g < 2 * p.n_groups; g += 256) sm[g] = 0;
+  grid_dep_trigger();                          // the gate/up GEMM may start on what needs no permutation
   grid_dep_wait();
-  grid_dep_trigger();
   int row0, count, total_tiles;
   const int first = outer_tile_prefix(outer_off, n_outer, p.n_rows, lane, row0, count, total_tiles);
   if (c0 >= total_tiles * 2 && blockIdx.x != 0) return;

@@ -38,7 +38,8 @@ constexpr int kU2Stages = 6;
 constexpr int kU2ABytes = kUmmaBM * kUmmaBK * 2;        // 16 KB: this CTA's 128 rows
 constexpr int kU2BBytes = 128 * kUmmaBK * 2;            // 16 KB: this CTA's half of B
 constexpr int kU2StageBytes = kU2ABytes + kU2BBytes;
-constexpr int kU2SmemBytes = 1024 + kU2Stages * kU2StageBytes + 256 + (kUmmaMaxGroups + 1) * 4;
+constexpr int kU2SmemBytes = 1024 + kU2Stages * kU2StageBytes + 256 + (kUmmaMaxGroups + 1) * 4 + kUmmaMaxGroups * 8;
+inline int umma2_smem_bytes(int n_groups) { return kU2SmemBytes - (kUmmaMaxGroups - n_groups) * 12; }
 constexpr int kU2Threads1 = kUmmaThreads + kUmmaGatherThreads + 32;   // gate/up: + 4 gather warps + 1 relay warp
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -116,31 +117,27 @@ __device__ __forceinline__ uint32_t umma2_idesc(int n) {     // M = 256 across t
 
 struct Pair2Coord { int g, mp, nt, row0, count; };
 
-template <int MODE>
-__device__ __forceinline__ int umma2_pairs(const UmmaArgs& p, int g) {
-  const int m_tiles = (p.gr[g].count + kUmmaBM - 1) / kUmmaBM;
-  return ((m_tiles + 1) >> 1) * umma_n_tiles<MODE>(p, g);
-}
-
-template <int MODE>
-__device__ __forceinline__ Pair2Coord umma2_decode(const UmmaArgs& p, const int32_t* tile_start, int t) {
-  int lo = 0, hi = p.n_groups;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (tile_start[mid] <= t) lo = mid; else hi = mid;
-  }
-  const int local = t - tile_start[lo];
-  const GroupRows r = p.gr[lo];
+// Tile pair `local` of group g.
+__device__ __forceinline__ Pair2Coord umma2_tile_in(const UmmaArgs& p, int g, const GroupRows r, int n_tiles, int local) {
   // bands of row-tile pairs, row tiles fastest inside a band, then n-tiles (see umma_decode)
   const int m_pairs = ((r.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
-  const int n_tiles = umma_n_tiles<MODE>(p, lo);
   const int band_mp = max(p.band_mt >> 1, 1);
   const int per_band = band_mp * n_tiles;
   const int band = local / per_band, in_band = local - band * per_band;
   const int cur_mp = min(band_mp, m_pairs - band * band_mp);
   Pair2Coord c;
-  c.g = lo; c.nt = in_band / cur_mp; c.mp = band * band_mp + in_band % cur_mp; c.row0 = r.row0; c.count = r.count;
+  c.g = g; c.nt = in_band / cur_mp; c.mp = band * band_mp + in_band % cur_mp; c.row0 = r.row0; c.count = r.count;
   return c;
+}
+
+template <int MODE>
+__device__ __forceinline__ Pair2Coord umma2_decode(const UmmaArgs& p, const int32_t* tile_start, const GroupRows* rows, int t) {
+  int lo = 0, hi = p.n_groups;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (tile_start[mid] <= t) lo = mid; else hi = mid;
+  }
+  return umma2_tile_in(p, lo, rows[lo], umma_n_tiles<MODE>(p, lo), t - tile_start[lo]);
 }
 
 template <int MODE>
@@ -148,8 +145,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MODE == 1 ? kU2Threa
 umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_constant__ CUtensorMap tm_a_r,
                      const __grid_constant__ CUtensorMap tm_b_s, const __grid_constant__ CUtensorMap tm_b_r,
                      const UmmaArgs p) {
-  grid_dep_wait();
-  grid_dep_trigger();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -157,10 +152,11 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
   const uint32_t bars = base + kU2Stages * kU2StageBytes;
   uint8_t* bars_gen = gen + kU2Stages * kU2StageBytes;
   // barrier block: full[8] empty[8] acc_full[2] acc_empty[2], tmem slot, abort flag
-  const uint32_t full0 = bars, empty0 = bars + 64, accf0 = bars + 128, acce0 = bars + 144, afull0 = bars + 192;
+  const uint32_t full0 = bars, empty0 = bars + 64, accf0 = bars + 128, acce0 = bars + 144, tbl_bar = bars + 168, afull0 = bars + 192;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars_gen + 160);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 164);
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);
+  GroupRows* rows = reinterpret_cast<GroupRows*>(tile_start + p.n_groups + 1);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
@@ -173,16 +169,10 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
       mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); mbar_init(afull0 + 8 * s, kUmmaGatherThreads);
     }
     for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 8); }
+    mbar_init(tbl_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  for (int g = threadIdx.x; g < p.n_groups; g += blockDim.x) tile_start[g + 1] = umma2_pairs<MODE>(p, g);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    tile_start[0] = 0;
-    for (int g = 0; g < p.n_groups; ++g) { run += tile_start[g + 1]; tile_start[g + 1] = run; }
   }
   cluster_sync_all();                         // both CTAs' barriers exist before any remote use
   if (warp == 1) {
@@ -193,16 +183,54 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int total_tiles = tile_start[p.n_groups];
   const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;
+  // table and tiles that need none: as in umma_grouped_kernel
+  const int early_tiles = MODE == 1 && p.early_rows > 0
+      ? ((p.early_rows + kUmmaBM - 1) / kUmmaBM + 1) / 2 * ((p.ld_out_s + p.bn_s - 1) / p.bn_s) : 0;
+  if (warp == 2) {
+    for (int g = lane; g < p.n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<MODE>(p, g);
+    if (MODE == 1) grid_dep_wait();
+    grid_dep_trigger();
+    for (int g = lane; g < p.n_groups; g += 32) {
+      const GroupRows gr = p.gr[g];
+      rows[g] = gr;
+      tile_start[g + 1] *= ((gr.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
+    }
+    __syncwarp();
+    warp_prefix(tile_start, p.n_groups, lane);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(tbl_bar);
+  }
+  bool seen = false;
+  auto tile_at = [&](int t, Pair2Coord& c, GroupStatic& g, bool whole_warp, bool& ok) {
+    if (MODE == 1 && t < early_tiles) {
+      GroupRows all; all.row0 = 0; all.count = p.early_rows;
+      c = umma2_tile_in(p, 0, all, (p.ld_out_s + p.bn_s - 1) / p.bn_s, t);
+      g.w_row0 = 0; g.width = p.ld_out_s; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
+      return true;
+    }
+    if (!seen) {
+      ok = mbar_wait(tbl_bar, 0, abort_flag, p.err, kErrWaitFull);
+      if (whole_warp) ok = __all_sync(0xffffffffu, ok);
+      if (!ok) return false;
+      if (MODE == 1) grid_dep_wait();
+      seen = true;
+    }
+    if (t >= tile_start[p.n_groups]) return false;
+    c = umma2_decode<MODE>(p, tile_start, rows, t);
+    g = p.gs[c.g];
+    return true;
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
-    uint32_t it = 0;
+    uint32_t it = 0, n_ahead = 0;
+    bool waited = false;
     bool ok = true;
-    for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
-      const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
-      const GroupStatic g = p.gs[c.g];
+    for (int t = pair_id; ok; t += n_pairs) {
+      Pair2Coord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, true, ok)) break;
       const int row = c.row0 + (2 * c.mp + (int)rank) * kUmmaBM;     // this CTA's m-tile
       const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
       const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
@@ -219,6 +247,23 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
         b_row = c.nt * 256 + (int)rank * 128;
         j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
       }
+      auto load_b = [&](int kb, uint32_t sb, uint32_t fb) {
+        if (MODE == 1) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, (int)rank);   // plane 0 gate, 1 up
+        else if (g.is_shared) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
+        else tma2_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
+      };
+      if (MODE == 2 && it == 0 && !waited) {
+        n_ahead = min(kU2Stages, k_blocks);
+        for (uint32_t i = 0; i < n_ahead; ++i) {
+          if (elect_one()) {
+            if (leader) mbar_expect_tx(full0 + 8 * i, 2 * (kU2ABytes + b_half));
+            load_b(i, base + i * kU2StageBytes + kU2ABytes, mapa_shared(full0 + 8 * i, 0));
+          }
+          __syncwarp();
+        }
+        grid_dep_wait();
+        waited = true;
+      }
       for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const uint32_t s = it % kU2Stages, n = it / kU2Stages;
         if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
@@ -226,11 +271,11 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
         const uint32_t fb = mapa_shared(fb_local, 0);               // the leader's barrier
         const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
         if (elect_one()) {
-          if (leader) mbar_expect_tx(fb_local, 2 * ((by_threads ? 0 : kU2ABytes) + b_half));
+          if (MODE == 1 || it >= n_ahead) {
+            if (leader) mbar_expect_tx(fb_local, 2 * ((by_threads ? 0 : kU2ABytes) + b_half));
+            load_b(kb, sb, fb);
+          }
           if (!by_threads) tma2_load_2d(sa, ta, fb, kb * kUmmaBK, row);
-          if (MODE == 1) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, (int)rank);   // plane 0 gate, 1 up
-          else if (g.is_shared) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
-          else tma2_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
         }
         __syncwarp();
       }
@@ -241,9 +286,10 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
     if (leader) {
       uint32_t it = 0, tile_n = 0;
       bool ok = true;
-      for (int t = pair_id; t < total_tiles && ok; t += n_pairs, ++tile_n) {
-        const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
-        const GroupStatic g = p.gs[c.g];
+      for (int t = pair_id; ok; t += n_pairs, ++tile_n) {
+        Pair2Coord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, true, ok)) break;
         int k_blocks, n_mma;
         if (MODE == 1) { k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r); }
         else { k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK; n_mma = 256; }
@@ -278,7 +324,10 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
+      for (int t = pair_id; ok; t += n_pairs) {
+        Pair2Coord c;
+        GroupStatic g;
+        if (!tile_at(t, c, g, false, ok)) break;
         for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
           const uint32_t s = it % kU2Stages, n = it / kU2Stages;
           if (!mbar_wait(afull0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
@@ -296,9 +345,10 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
     const int ch = gt & 7, r_sub = gt >> 3;
     uint32_t it = 0;
     bool ok = true;
-    for (int t = pair_id; t < total_tiles && ok; t += n_pairs) {
-      const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
-      const GroupStatic g = p.gs[c.g];
+    for (int t = pair_id; ok; t += n_pairs) {
+      Pair2Coord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, false, ok)) break;
       const bool mine = !g.is_shared;
       const bf16* src_row[8];
 #pragma unroll
@@ -337,9 +387,10 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
     const int quad = warp & 3;
     uint32_t tile_n = 0;
     bool ok = true;
-    for (int t = pair_id; t < total_tiles && ok; t += n_pairs, ++tile_n) {
-      const Pair2Coord c = umma2_decode<MODE>(p, tile_start, t);
-      const GroupStatic g = p.gs[c.g];
+    for (int t = pair_id; ok; t += n_pairs, ++tile_n) {
+      Pair2Coord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, false, ok)) break;
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
       if (!mbar_wait(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
       tc_fence_after();
@@ -466,21 +517,22 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
 // `D` supplies the 128-channel W_down maps (shared with the decode path).  Requires
 // umma_bind_x for this forward.  which: bit 0 the gate/up GEMM, bit 1 the down GEMM.  Returns launches or -1.
 inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRows* gr, const void* x_rows, int32_t* err_word, cudaStream_t st, cudaEvent_t mid, bool dep,
-                         int which) {
+                         int which, int early_rows) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   const int grid = Q->grid;
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
   a.x_rows_ptr = (const bf16*)x_rows;
   a.band_mt = umma_band_tiles(s.d);
+  a.early_rows = early_rows;
   if (which & 1)
-    launch_kernel(dep, umma2_grouped_kernel<1>, dim3(grid), dim3(kU2Threads1), kU2SmemBytes, st,
+    launch_kernel(dep, umma2_grouped_kernel<1>, dim3(grid), dim3(kU2Threads1), umma2_smem_bytes(P->n_groups), st,
                   P->x_rows, P->x_rows, Q->b1_s, Q->b1_r, a);
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
   if (which & 2)
-    launch_kernel(dep, umma2_grouped_kernel<2>, dim3(grid), dim3(kUmmaThreads), kU2SmemBytes, st, P->a2_s, P->a2_r,
+    launch_kernel(dep, umma2_grouped_kernel<2>, dim3(grid), dim3(kUmmaThreads), umma2_smem_bytes(P->n_groups), st, P->a2_s, P->a2_r,
                   D->wd_s, D->wd_r, a);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -43,7 +43,9 @@ constexpr int kUmmaThreads = 192;     // warp 0 TMA, warp 1 MMA, warps 2..5 epil
 constexpr int kUmmaGatherThreads = 128;   // mode 1 only: warps 6..9, one thread per A-tile row
 constexpr int kUmmaTmemCols = 512;    // two accumulator buffers of 256 columns
 constexpr int kUmmaSmemBytes = 1024 /*alignment slack*/ + kUmmaStages * kUmmaStageBytes +
-                               256 /*barriers*/ + (kUmmaMaxGroups + 1) * 4;
+                               256 /*barriers*/ + (kUmmaMaxGroups + 1) * 4 + kUmmaMaxGroups * 8 /*group rows*/;
+// A layer asks for its own groups only: a small router then fits on the SM beside the gate/up GEMM.
+inline int umma_smem_bytes(int n_groups) { return kUmmaSmemBytes - (kUmmaMaxGroups - n_groups) * 12; }
 constexpr long long kUmmaWaitCycles = 2000000000LL;   // ~1 s at SM clock
 
 enum { kErrWaitFull = 1, kErrWaitEmpty = 2, kErrWaitAccFull = 3, kErrWaitAccEmpty = 4 };
@@ -220,7 +222,24 @@ struct UmmaArgs {
   int band_mt;                // row tiles per band of the tile order (see umma_decode)
   const bf16* x_rows_ptr;     // mode 1: the outer rows of x (source of the cp.async gather)
   int32_t* err;
+  int early_rows;             // mode 1: rows of group 0 where the host knows them (the shared experts of a plain layer), else 0
 };
+
+// tile_start[g + 1] holds the tiles of group g; turns them into the prefix sums, tile_start[0] = 0 (one warp).
+__device__ __forceinline__ void warp_prefix(int32_t* tile_start, int n_groups, int lane) {
+  const int each = (n_groups + 31) / 32, lo = lane * each, hi = min(lo + each, n_groups);
+  int sum = 0;
+  for (int g = lo; g < hi; ++g) sum += tile_start[g + 1];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  int run = incl - sum;
+  for (int g = lo; g < hi; ++g) { run += tile_start[g + 1]; tile_start[g + 1] = run; }
+  if (lane == 0) tile_start[0] = 0;
+}
 
 struct TileCoord { int g, mt, nt, row0, count; };
 
@@ -234,16 +253,9 @@ __device__ __forceinline__ int umma_n_tiles(const UmmaArgs& p, int g) {
   return gs.width > 0 ? (p.d + 255) / 256 : 0;
 }
 
+// Tile `local` of group g.
 template <int MODE>
-__device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_t* tile_start, int n_groups,
-                                                 int t) {
-  int lo = 0, hi = n_groups;                 // last g with tile_start[g] <= t
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (tile_start[mid] <= t) lo = mid; else hi = mid;
-  }
-  const int local = t - tile_start[lo];
-  const GroupRows r = p.gr[lo];
+__device__ __forceinline__ TileCoord umma_tile_in(const UmmaArgs& p, int g, const GroupRows r, int n_tiles, int local) {
   // Order inside a group: bands of p.band_mt row tiles; inside a band the row tiles run fastest (CTAs
   // working side by side share a weight tile), then the n-tiles, then the next band.  A band's rows of A
   // (about 16 MB) stay in L2 while the n-tiles pass over them; without bands a large group's rows left L2
@@ -251,14 +263,24 @@ __device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_
   // GEMM of the 16384-token workload), while letting the n-tiles run fastest everywhere was slower for the
   // groups that do fit (every CTA then streams a different weight tile).
   const int m_tiles = (r.count + kUmmaBM - 1) / kUmmaBM;
-  const int n_tiles = umma_n_tiles<MODE>(p, lo);
   const int band_mt = max(p.band_mt, 1);
   const int per_band = band_mt * n_tiles;
   const int band = local / per_band, in_band = local - band * per_band;
   const int cur_mt = min(band_mt, m_tiles - band * band_mt);
   TileCoord c;
-  c.g = lo; c.nt = in_band / cur_mt; c.mt = band * band_mt + in_band % cur_mt; c.row0 = r.row0; c.count = r.count;
+  c.g = g; c.nt = in_band / cur_mt; c.mt = band * band_mt + in_band % cur_mt; c.row0 = r.row0; c.count = r.count;
   return c;
+}
+
+template <int MODE>
+__device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_t* tile_start, const GroupRows* rows,
+                                                 int n_groups, int t) {
+  int lo = 0, hi = n_groups;                 // last g with tile_start[g] <= t
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (tile_start[mid] <= t) lo = mid; else hi = mid;
+  }
+  return umma_tile_in<MODE>(p, lo, rows[lo], umma_n_tiles<MODE>(p, lo), t - tile_start[lo]);
 }
 
 template <int MODE>
@@ -266,8 +288,6 @@ __global__ void __launch_bounds__(MODE == 1 ? kUmmaThreads + kUmmaGatherThreads 
 umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_constant__ CUtensorMap tm_a_r,
                     const __grid_constant__ CUtensorMap tm_b_s, const __grid_constant__ CUtensorMap tm_b_r,
                     const UmmaArgs p) {
-  grid_dep_wait();
-  grid_dep_trigger();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -276,10 +296,11 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   const uint32_t bars = base + kStages * kStageBytes;   // barrier block
   uint8_t* bars_gen = gen + kStages * kStageBytes;
   // barrier block: full[8] empty[8] acc_full[2] acc_empty[2] (8 B each), tmem slot, abort flag
-  const uint32_t full0 = bars, empty0 = bars + 64, accf0 = bars + 128, acce0 = bars + 144;
+  const uint32_t full0 = bars, empty0 = bars + 64, accf0 = bars + 128, acce0 = bars + 144, tbl_bar = bars + 168;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars_gen + 160);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + 164);
   int32_t* tile_start = reinterpret_cast<int32_t*>(bars_gen + 256);
+  GroupRows* rows = reinterpret_cast<GroupRows*>(tile_start + p.n_groups + 1);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int n_groups = p.n_groups;
@@ -289,6 +310,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     const uint32_t full_count = MODE == 1 ? 1 + kUmmaGatherThreads : 1;
     for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 4); }
+    mbar_init(tbl_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -297,31 +319,64 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     tmem_alloc(smem_u32(tmem_slot), kUmmaTmemCols);
     tmem_relinquish();
   }
-  // tiles of every group, then their exclusive prefix
-  for (int g = threadIdx.x; g < n_groups; g += blockDim.x) {
-    const int m_tiles = (p.gr[g].count + kUmmaBM - 1) / kUmmaBM;
-    tile_start[g + 1] = m_tiles * umma_n_tiles<MODE>(p, g);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    tile_start[0] = 0;
-    for (int g = 0; g < n_groups; ++g) { run += tile_start[g + 1]; tile_start[g + 1] = run; }
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int total_tiles = tile_start[n_groups];
   const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;      // mode 1: K = d
+  // Warp 2 counts the tiles of every group and publishes the table on a barrier; in mode 1 it waits for the router and the
+  // permutation first, in mode 2 the preceding kernel has read the same rows already.  Tiles that need no table, those of the shared
+  // experts of a plain layer (group 0, all rows of x), run at once, under the routing and this kernel's own start-up.
+  // Mode 2 fetches the weights of its first stages under the end of the gate/up GEMM.  Against a wait at the top and a table that all
+  // threads count and one sums (3.7 us from the permutation's end to the first operands of a tile, 3.3 from the gate/up GEMM's): 8B-shaped 300 / 500 / 700 /
+  // 2048 rows 102.0 / 112.5 / 125.1 / 231 -> 94.4 / 107.9 / 112.6 / 213 us, 7B-shaped 200 / 300 / 500 rows 75.5 / 79.2 / 109.5 -> 71.4 /
+  // 75.5 / 102.7, 13B-shaped 300 / 600 rows 128.0 / 171.4 -> 113.2 / 162.0.
+  const int early_tiles = MODE == 1 && p.early_rows > 0
+      ? (p.early_rows + kUmmaBM - 1) / kUmmaBM * ((p.ld_out_s + p.bn_s - 1) / p.bn_s) : 0;
+  if (warp == 2) {
+    for (int g = lane; g < n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<MODE>(p, g);
+    if (MODE == 1) grid_dep_wait();
+    grid_dep_trigger();
+    for (int g = lane; g < n_groups; g += 32) {
+      const GroupRows gr = p.gr[g];
+      rows[g] = gr;
+      tile_start[g + 1] *= (gr.count + kUmmaBM - 1) / kUmmaBM;
+    }
+    __syncwarp();
+    warp_prefix(tile_start, n_groups, lane);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(tbl_bar);
+  }
+  bool seen = false;                             // this thread has waited for the table
+  auto tile_at = [&](int t, TileCoord& c, GroupStatic& g, bool whole_warp, bool& ok) {   // false: no tile t, or a wait gave up
+    if (MODE == 1 && t < early_tiles) {
+      GroupRows all; all.row0 = 0; all.count = p.early_rows;
+      c = umma_tile_in<MODE>(p, 0, all, (p.ld_out_s + p.bn_s - 1) / p.bn_s, t);
+      g.w_row0 = 0; g.width = p.ld_out_s; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
+      return true;
+    }
+    if (!seen) {
+      ok = mbar_wait(tbl_bar, 0, abort_flag, p.err, kErrWaitFull);
+      if (whole_warp) ok = __all_sync(0xffffffffu, ok);
+      if (!ok) return false;
+      if (MODE == 1) grid_dep_wait();
+      seen = true;
+    }
+    if (t >= tile_start[n_groups]) return false;
+    c = umma_decode<MODE>(p, tile_start, rows, n_groups, t);
+    g = p.gs[c.g];
+    return true;
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp)
-    uint32_t it = 0;
+    uint32_t it = 0, n_ahead = 0;
+    bool waited = false;
     bool ok = true;
-    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-      const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
-      const GroupStatic g = p.gs[c.g];
+    for (int t = blockIdx.x; ok; t += gridDim.x) {
+      TileCoord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, true, ok)) break;
       const int row = c.row0 + c.mt * kUmmaBM;
       const bool by_threads = MODE == 1 && !g.is_shared;              // the gather warps fill A
       const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
@@ -338,17 +393,34 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
         b_row = c.nt * 256;
         j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
       }
+      auto load_b = [&](int kb, uint32_t sb, uint32_t fb) {
+        if (MODE == 1) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, 0);
+        else if (g.is_shared) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
+        else tma_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
+      };
+      if (MODE == 2 && it == 0 && !waited) {         // weights of the first stages ahead of the wait for the gate/up GEMM
+        n_ahead = min(kStages, k_blocks);
+        for (uint32_t i = 0; i < n_ahead; ++i) {
+          if (elect_one()) {
+            mbar_expect_tx(full0 + 8 * i, kUmmaABytes + b_bytes);
+            load_b(i, base + i * kStageBytes + kUmmaABytes, full0 + 8 * i);
+          }
+          __syncwarp();
+        }
+        grid_dep_wait();
+        waited = true;
+      }
       for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;
         if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb = full0 + 8 * s;
         const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
         if (elect_one()) {
-          mbar_expect_tx(fb, (by_threads ? 0 : kUmmaABytes) + b_bytes);
+          if (MODE == 1 || it >= n_ahead) {
+            mbar_expect_tx(fb, (by_threads ? 0 : kUmmaABytes) + b_bytes);
+            load_b(kb, sb, fb);
+          }
           if (!by_threads) tma_load_2d(sa, ta, fb, kb * kUmmaBK, row);
-          if (MODE == 1) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, 0);
-          else if (g.is_shared) tma_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
-          else tma_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
         }
         __syncwarp();
       }
@@ -358,14 +430,15 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
     uint32_t it = 0, tile_n = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_n) {
-      const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
+    for (int t = blockIdx.x; ok; t += gridDim.x, ++tile_n) {
+      TileCoord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, true, ok)) break;
       int k_blocks, n_mma;
       if (MODE == 1) {
-        const GroupStatic g = p.gs[c.g];
         k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r);
       } else {
-        k_blocks = (p.gs[c.g].width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
+        k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK; n_mma = 256;
       }
       const uint32_t idesc = umma_idesc(n_mma);
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
@@ -400,9 +473,10 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     const int ch = gt & 7, r_sub = gt >> 3;
     uint32_t it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-      const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
-      const GroupStatic g = p.gs[c.g];
+    for (int t = blockIdx.x; ok; t += gridDim.x) {
+      TileCoord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, false, ok)) break;
       const bool mine = !g.is_shared;
       const bf16* src_row[8];
 #pragma unroll
@@ -441,8 +515,10 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
     uint32_t tile_n = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_n) {
-      const TileCoord c = umma_decode<MODE>(p, tile_start, n_groups, t);
+    for (int t = blockIdx.x; ok; t += gridDim.x, ++tile_n) {
+      TileCoord c;
+      GroupStatic g;
+      if (!tile_at(t, c, g, false, ok)) break;
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
       if (!mbar_wait(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
       tc_fence_after();
@@ -450,7 +526,6 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
       const bool row_ok = row_in_group < c.count;
       const uint32_t taddr = tmem_base + buf * 256 + ((uint32_t)(quad * 32) << 16);
       if (MODE == 1) {
-        const GroupStatic g = p.gs[c.g];
         const int bn = g.is_shared ? p.bn_s : p.bn_r;
         const int ld = g.is_shared ? p.ld_out_s : p.ld_out_r;
         const int n0 = c.nt * bn;
@@ -482,7 +557,6 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
           }
         }
       } else {
-        const GroupStatic g = p.gs[c.g];
         const int n0 = c.nt * 256;
         const int n_valid = min(256, p.d - n0);
         bf16* dst = (g.is_shared ? p.out_s : p.out_r) + (size_t)(c.row0 + row_in_group) * p.d + n0;
@@ -701,22 +775,23 @@ inline UmmaArgs umma_base_args(const UmmaPlan* P, const GroupRows* gr, int32_t* 
 }
 
 // Enqueues the gate/up and the down GEMM over all groups.  Requires umma_bind_x for this forward.  which: bit 0 the
-// gate/up GEMM, bit 1 the down GEMM.  Returns the number of kernels launched, or -1 (P->error).
+// gate/up GEMM, bit 1 the down GEMM.  early_rows: rows of the shared experts where the host knows them (plain layer).  Returns the number of kernels launched, or -1 (P->error).
 inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, int32_t* err_word,
-                        cudaStream_t st, cudaEvent_t mid, bool dep, int which) {
+                        cudaStream_t st, cudaEvent_t mid, bool dep, int which, int early_rows) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
   a.x_rows_ptr = (const bf16*)x_rows;
   a.band_mt = umma_band_tiles(s.d);
+  a.early_rows = early_rows;
   if (which & 1)
-    launch_kernel(dep, umma_grouped_kernel<1>, dim3(P->n_sms), dim3(kUmmaThreads + kUmmaGatherThreads), kUmmaSmemBytes,
+    launch_kernel(dep, umma_grouped_kernel<1>, dim3(P->n_sms), dim3(kUmmaThreads + kUmmaGatherThreads), umma_smem_bytes(P->n_groups),
                   st, P->x_rows, P->x_rows, P->b1_s, P->b1_r, a);
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
   if (which & 2)
-    launch_kernel(dep, umma_grouped_kernel<2>, dim3(P->n_sms), dim3(kUmmaThreads), kUmmaSmemBytes, st, P->a2_s,
+    launch_kernel(dep, umma_grouped_kernel<2>, dim3(P->n_sms), dim3(kUmmaThreads), umma_smem_bytes(P->n_groups), st, P->a2_s,
                   P->a2_r, P->b2_s, P->b2_r, a);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

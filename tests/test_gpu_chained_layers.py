@@ -10,8 +10,8 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 
 
-def _stack(dtype, fp8, tokens, n_layers=3, d=512, m=176):
-    shape = wl.LayerShape(d, m * 8, 8, 2, 2, dtype)
+def _stack(dtype, fp8, tokens, n_layers=3, d=512, m=176, n=8, n_shared=2, top_k=2):
+    shape = wl.LayerShape(d, m * n, n, n_shared, top_k, dtype)
     rng = np.random.Generator(np.random.PCG64(3))
     layers = []
     for _ in range(n_layers):
@@ -27,8 +27,19 @@ def _stack(dtype, fp8, tokens, n_layers=3, d=512, m=176):
 @pytest.mark.parametrize("dtype,fp8,tokens", [("bf16", False, t) for t in (1, 2, 16, 64, 100, 300, 1100)] +
                          [("bf16", True, t) for t in (1, 16, 64)] + [("fp32", False, t) for t in (1, 64, 700)])
 def test_layer_stack_matches_synchronised_calls(dtype, fp8, tokens):
+    _check_stack(*_stack(dtype, fp8, tokens), dtype)
+
+
+# the shared experts' tiles run ahead of the routing: more of them than CTAs (single CTAs and pairs), none, only them, and a router
+# too large to share an SM with the GEMM
+@pytest.mark.parametrize("n,n_shared,top_k,m,tokens", [(8, 6, 2, 512, 1030), (8, 6, 2, 512, 2100), (8, 0, 2, 176, 300), (4, 4, 0, 176, 300),
+                                                       (32, 4, 4, 48, 300), (32, 4, 4, 48, 700)])
+def test_layer_stack_shared_tiles(n, n_shared, top_k, m, tokens):
+    _check_stack(*_stack("bf16", False, tokens, m=m, n=n, n_shared=n_shared, top_k=top_k), "bf16")
+
+
+def _check_stack(layers, x, dtype):
     import torch
-    layers, x = _stack(dtype, fp8, tokens)
     xs = [parity.to_device(x, dtype)]
     xs += [torch.roll(xs[0], k, 1).contiguous() for k in (1, 2, 3)]
     bufs = [torch.empty_like(xs[0]) for _ in range(3)]
