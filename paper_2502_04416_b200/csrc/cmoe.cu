@@ -313,7 +313,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     ub.x_fixed = L->hier ? L->xo : nullptr;
     ub.h_s = L->h_s; ub.h_r = L->h_r; ub.y_s = L->y_s; ub.y_r = L->y_r;
     ub.gs_dev = L->gs; ub.topk_idx = L->topk_idx; ub.topk_gate = L->topk_gate;
-    ub.row_token = L->row_token;
+    ub.row_token = L->row_token; ub.row_of = L->row_of;
     rc = umma_plan_create(&L->umma, s, ub, L->n_groups_total());
     if (rc == CMOE_ERR_CUDA) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     L->umma_ok = (rc == CMOE_OK);
@@ -559,21 +559,34 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   } else if (use_umma) {
     cudaEvent_t mid = ev ? ev[3] : nullptr;
     int n;
+    bf16* fold_out = nullptr;                         // the down GEMM of the shared experts also combines
     if (decode) {
       n = decode_forward(&L->umma, &L->decode, L->gr, R, L->err_word, st, mid, dep, gate_up_only);
     } else {
       const int todo = gate_up_only ? 1 : 3;
+      if constexpr (std::is_same<T, bf16>::value)
+        if (!gate_up_only && !L->hier && umma_folds_combine(&L->umma, R, n_k, d)) fold_out = out;
       n = 0;
       for (int bit = 1; bit <= 2 && n >= 0; bit <<= 1) {          // gate/up, then down, each on its chosen tile shape
         if (!(todo & bit)) continue;
         const int k = (pair_mask & bit)
-            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R)
-            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R);
+            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R, fold_out != nullptr)
+            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R, fold_out != nullptr);
         n = k < 0 ? -1 : n + k;
       }
     }
     if (n < 0) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     launches += n;
+    if (fold_out) {
+      if (umma_fold_forward(&L->umma, L->gr, R, fold_out, L->err_word, st, dep) < 0) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+      ++launches;
+      mark(4);
+      mark(5);
+      if (ev) ++L->ev_count;
+      CU_TRY(cudaGetLastError());
+      L->launches = launches;
+      return CMOE_OK;
+    }
   } else {
     SimtGemmArgs<T> a;
     a.gs = L->gs; a.gr = L->gr; a.d = d;

@@ -98,6 +98,15 @@ __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
   v[4] = __uint_as_float(b.x); v[5] = __uint_as_float(b.y); v[6] = __uint_as_float(b.z); v[7] = __uint_as_float(b.w);
 }
 
+// Sixteen bf16 elements with one 32-byte access that is not kept in L1.
+__device__ __forceinline__ void ld256_stream(const bf16* p, uint32_t (&w)[8]) {
+  // volatile + memory clobber: the load must stay below griddepcontrol.wait (its source is written
+  // by the preceding kernel of a chained launch)
+  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+               : "l"(p) : "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);

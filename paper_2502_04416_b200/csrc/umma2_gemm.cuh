@@ -185,28 +185,28 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
   const uint32_t tmem_base = *tmem_slot;
   const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;
   // table and tiles that need none: as in umma_grouped_kernel
-  const int early_tiles = MODE == 1 && p.early_rows > 0
-      ? ((p.early_rows + kUmmaBM - 1) / kUmmaBM + 1) / 2 * ((p.ld_out_s + p.bn_s - 1) / p.bn_s) : 0;
+  const int early_n = MODE == 1 && p.early_rows > 0 ? (p.shared_width + p.bn_s - 1) / p.bn_s : 0;
+  const int early_tiles = (((p.early_rows + kUmmaBM - 1) / kUmmaBM + 1) / 2) * early_n;
   if (warp == 2) {
     for (int g = lane; g < p.n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<MODE>(p, g);
-    if (MODE == 1) grid_dep_wait();
-    grid_dep_trigger();
+    if (MODE == 1) { grid_dep_wait(); grid_dep_trigger(); }
     for (int g = lane; g < p.n_groups; g += 32) {
       const GroupRows gr = p.gr[g];
       rows[g] = gr;
-      tile_start[g + 1] *= ((gr.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
+      tile_start[g + 1] *= MODE == 2 && g < p.skip_groups ? 0 : ((gr.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
     }
     __syncwarp();
     warp_prefix(tile_start, p.n_groups, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(tbl_bar);
+    if (MODE == 2) { grid_dep_wait(); grid_dep_trigger(); }     // what follows may count on the gate/up GEMM
   }
   bool seen = false;
   auto tile_at = [&](int t, Pair2Coord& c, GroupStatic& g, bool whole_warp, bool& ok) {
     if (MODE == 1 && t < early_tiles) {
       GroupRows all; all.row0 = 0; all.count = p.early_rows;
-      c = umma2_tile_in(p, 0, all, (p.ld_out_s + p.bn_s - 1) / p.bn_s, t);
-      g.w_row0 = 0; g.width = p.ld_out_s; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
+      c = umma2_tile_in(p, 0, all, early_n, t);
+      g.w_row0 = 0; g.width = p.shared_width; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
       return true;
     }
     if (!seen) {
@@ -517,7 +517,7 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
 // `D` supplies the 128-channel W_down maps (shared with the decode path).  Requires
 // umma_bind_x for this forward.  which: bit 0 the gate/up GEMM, bit 1 the down GEMM.  Returns launches or -1.
 inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRows* gr, const void* x_rows, int32_t* err_word, cudaStream_t st, cudaEvent_t mid, bool dep,
-                         int which, int early_rows) {
+                         int which, int early_rows, bool skip_shared = false) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   const int grid = Q->grid;
@@ -531,6 +531,7 @@ inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRo
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
+  a.skip_groups = skip_shared ? s.n_outer : 0;
   if (which & 2)
     launch_kernel(dep, umma2_grouped_kernel<2>, dim3(grid), dim3(kUmmaThreads), umma2_smem_bytes(P->n_groups), st, P->a2_s, P->a2_r,
                   D->wd_s, D->wd_r, a);

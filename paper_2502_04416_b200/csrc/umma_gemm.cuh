@@ -13,6 +13,8 @@
 //                 layer 200 / 256 rows 94.2 / 106.2 us against 78.2 / 78.1.
 //       B tile  : bn gate rows + bn up rows of the group's neurons x 64 k (one 3-D TMA box)
 //       D (TMEM): 128 lanes x 2*bn fp32 columns; epilogue fuses SiLU(gate)*up -> bf16 H
+//   MODE 3, down GEMM of the shared experts of a plain layer with the combine in its epilogue (umma_folds_combine), after mode 2 for
+//       the routed experts.
 //   MODE 2, down GEMM: Y[r, c] = sum_n H[r, n] Wd[c, n]
 //       A tile  : 128 rows of H x 64 k ;  B tile: 256 output channels of the group's W_down
 //       block x 64 k ;  D: 128 x 256 fp32 ; epilogue rounds to bf16 Y.
@@ -222,7 +224,13 @@ struct UmmaArgs {
   int band_mt;                // row tiles per band of the tile order (see umma_decode)
   const bf16* x_rows_ptr;     // mode 1: the outer rows of x (source of the cp.async gather)
   int32_t* err;
-  int early_rows;             // mode 1: rows of group 0 where the host knows them (the shared experts of a plain layer), else 0
+  int shared_width;           // neurons of the shared experts
+  int skip_groups;            // mode 2: this many groups ahead are left out (the shared experts, which mode 3 does)
+  const bf16* y_r;            // mode 3: routed rows, their places and gates
+  const int32_t* row_of;
+  const float* topk_gate;
+  int n_k;
+  int early_rows;             // modes 1, 3: rows of group 0 where the host knows them (the shared experts of a plain layer), else 0
 };
 
 // tile_start[g + 1] holds the tiles of group g; turns them into the prefix sums, tile_start[0] = 0 (one warp).
@@ -331,30 +339,33 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   // threads count and one sums (3.7 us from the permutation's end to the first operands of a tile, 3.3 from the gate/up GEMM's): 8B-shaped 300 / 500 / 700 /
   // 2048 rows 102.0 / 112.5 / 125.1 / 231 -> 94.4 / 107.9 / 112.6 / 213 us, 7B-shaped 200 / 300 / 500 rows 75.5 / 79.2 / 109.5 -> 71.4 /
   // 75.5 / 102.7, 13B-shaped 300 / 600 rows 128.0 / 171.4 -> 113.2 / 162.0.
-  const int early_tiles = MODE == 1 && p.early_rows > 0
-      ? (p.early_rows + kUmmaBM - 1) / kUmmaBM * ((p.ld_out_s + p.bn_s - 1) / p.bn_s) : 0;
-  if (warp == 2) {
+  const int early_n = MODE == 3 ? (p.d + 255) / 256 : MODE == 1 && p.early_rows > 0 ? (p.shared_width + p.bn_s - 1) / p.bn_s : 0;
+  const int early_tiles = (p.early_rows + kUmmaBM - 1) / kUmmaBM * early_n;
+  if (MODE == 3) {
+    if (warp == 2) { grid_dep_wait(); grid_dep_trigger(); }     // as an epilogue warp it waits all the same
+  } else if (warp == 2) {
     for (int g = lane; g < n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<MODE>(p, g);
-    if (MODE == 1) grid_dep_wait();
-    grid_dep_trigger();
+    if (MODE == 1) { grid_dep_wait(); grid_dep_trigger(); }
     for (int g = lane; g < n_groups; g += 32) {
       const GroupRows gr = p.gr[g];
       rows[g] = gr;
-      tile_start[g + 1] *= (gr.count + kUmmaBM - 1) / kUmmaBM;
+      tile_start[g + 1] *= MODE == 2 && g < p.skip_groups ? 0 : (gr.count + kUmmaBM - 1) / kUmmaBM;
     }
     __syncwarp();
     warp_prefix(tile_start, n_groups, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(tbl_bar);
+    if (MODE == 2) { grid_dep_wait(); grid_dep_trigger(); }     // what follows may count on the gate/up GEMM
   }
   bool seen = false;                             // this thread has waited for the table
   auto tile_at = [&](int t, TileCoord& c, GroupStatic& g, bool whole_warp, bool& ok) {   // false: no tile t, or a wait gave up
-    if (MODE == 1 && t < early_tiles) {
+    if (MODE != 2 && t < early_tiles) {
       GroupRows all; all.row0 = 0; all.count = p.early_rows;
-      c = umma_tile_in<MODE>(p, 0, all, (p.ld_out_s + p.bn_s - 1) / p.bn_s, t);
-      g.w_row0 = 0; g.width = p.ld_out_s; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
+      c = umma_tile_in<MODE>(p, 0, all, early_n, t);
+      g.w_row0 = 0; g.width = p.shared_width; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
       return true;
     }
+    if (MODE == 3) return false;
     if (!seen) {
       ok = mbar_wait(tbl_bar, 0, abort_flag, p.err, kErrWaitFull);
       if (whole_warp) ok = __all_sync(0xffffffffu, ok);
@@ -416,7 +427,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
         const uint32_t fb = full0 + 8 * s;
         const uint32_t sa = base + s * kStageBytes, sb = sa + kUmmaABytes;
         if (elect_one()) {
-          if (MODE == 1 || it >= n_ahead) {
+          if (MODE != 2 || it >= n_ahead) {
             mbar_expect_tx(fb, (by_threads ? 0 : kUmmaABytes) + b_bytes);
             load_b(kb, sb, fb);
           }
@@ -519,6 +530,18 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
       TileCoord c;
       GroupStatic g;
       if (!tile_at(t, c, g, false, ok)) break;
+      int pos[4];
+      float gate[4];
+      if (MODE == 3) {                             // this row's routing, under the multiplies
+        const size_t tok = (size_t)(c.row0 + (c.mt * kUmmaBM + quad * 32 + lane));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool on = j < p.n_k && (c.mt * kUmmaBM + quad * 32 + lane) < c.count;
+          pos[j] = on ? __ldcg(p.row_of + tok * p.n_k + j) : 0;
+          gate[j] = on ? __ldcg(p.topk_gate + tok * p.n_k + j) : 0.0f;
+        }
+        if (tile_n == 0) grid_dep_wait();          // the routed experts' rows are complete
+      }
       const uint32_t buf = tile_n & 1, use = tile_n >> 1;
       if (!mbar_wait(accf0 + 8 * buf, use & 1, abort_flag, p.err, kErrWaitAccFull)) { ok = false; break; }
       tc_fence_after();
@@ -554,6 +577,42 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
                 }
               }
             }
+          }
+        }
+      } else if (MODE == 3) {
+        // out = Y_s + sum_j g_j Y_r[row_of_j], with the rounding and the order of combine_plain_bf16_kernel: the same bits.
+        // 32 columns at a time: all loads of the routed rows before any arithmetic.
+        const int n0 = c.nt * 256;
+        const int n_valid = min(256, p.d - n0);                      // a multiple of 16
+        const size_t tok = (size_t)(c.row0 + row_in_group);
+        const bf16* yr[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) yr[j] = p.y_r + (size_t)pos[j] * p.d + n0;
+        bf16* dst = p.out_s + tok * p.d + n0;
+        for (int c0 = 0; c0 < n_valid; c0 += 32) {
+          const bool two = c0 + 16 < n_valid;
+          uint32_t w[4][16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < p.n_k && row_ok) {
+              ld256_stream(yr[j] + c0, *reinterpret_cast<uint32_t(*)[8]>(&w[j][0]));
+              if (two) ld256_stream(yr[j] + c0 + 16, *reinterpret_cast<uint32_t(*)[8]>(&w[j][8]));
+            }
+          float acc[32];
+          tmem_ld16(taddr + c0, acc);
+          if (two) tmem_ld16(taddr + c0 + 16, acc + 16);
+          tmem_ld_wait();
+          if (row_ok) {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+              float y = __bfloat162float(__float2bfloat16_rn(acc[q]));
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (j < p.n_k) y = fmaf(gate[j], __uint_as_float((q & 1) ? (w[j][q >> 1] & 0xffff0000u) : (w[j][q >> 1] << 16)), y);
+              acc[q] = y;
+            }
+            store16(dst + c0, acc);
+            if (two) store16(dst + c0 + 16, acc + 16);
           }
         }
       } else {
@@ -608,7 +667,7 @@ struct UmmaBuffers {
   const GroupStatic* gs_dev = nullptr;
   const float* topk_gate = nullptr;
   const int32_t* topk_idx = nullptr;
-  const int32_t* row_token = nullptr;
+  const int32_t *row_token = nullptr, *row_of = nullptr;
 };
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -746,6 +805,7 @@ inline int umma_plan_create(UmmaPlan* P, const UmmaShape& s, const UmmaBuffers& 
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_grouped_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmemBytes);
   if (e != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     return -5;
@@ -770,14 +830,32 @@ inline UmmaArgs umma_base_args(const UmmaPlan* P, const GroupRows* gr, int32_t* 
   a.gs = P->buf.gs_dev; a.gr = gr; a.n_groups = P->n_groups; a.n_outer = s.n_outer; a.n_r = s.n_r;
   a.d = s.d; a.bn_s = P->bn_s; a.bn_r = P->bn_r; a.err = err_word;
   a.row_token = P->buf.row_token;
+  a.shared_width = s.shared_width;
+  a.row_of = P->buf.row_of; a.topk_gate = P->buf.topk_gate; a.n_k = s.n_k; a.y_r = (const bf16*)P->buf.y_r;
   a.x_rows_ptr = nullptr;
   return a;
+}
+
+// Whether the down GEMM of the shared experts runs after that of the routed ones and combines in its epilogue: Y_s is neither
+// written nor read back, and the routed rows are read under its multiplies.  Bound by the epilogue's gathers (a thread reads
+// 32-byte pieces of n_k rows), which a tile's multiplies must cover, and by the last round of tiles, which no routed tiles fill up any
+// more: taken when the SMs' idle time in that round (425 ns per 64-wide k block) is at most a third of the combine's own time (3 us and
+// the rows at 5.5 TB/s).  Without / with: 8B-shaped 700 rows 100.5 / 106.4 us and 1400 rows 155.6 / 159.1 (not taken), 1000 / 2048 / 8192
+// rows 136.3 / 208.5 / 693 against 131.3 / 204.3 / 644, 7B-shaped 300 / 2500 rows 74.0 / 293 against 78.4 / 300 (not taken), 4000 / 8000 rows 445 /
+// 889 against 443 / 857, 13B-shaped 4096 / 16384 rows 568 / 2295 against 562 / 2286.  Fetching the routed rows of the next columns ahead
+// (233 registers) is slower: 8B-shaped 2048 / 8192 rows 213 / 667.
+inline bool umma_folds_combine(const UmmaPlan* P, int R, int n_k, int d) {
+  if (!P->has_s || !P->has_r || n_k < 1 || n_k > 4 || d % 16 != 0) return false;
+  const int tiles = (R + kUmmaBM - 1) / kUmmaBM * ((d + 255) / 256), over = tiles % P->n_sms;
+  const double idle = over ? (1.0 - (double)over / P->n_sms) * 0.425 * ((P->shape.shared_width + kUmmaBK - 1) / kUmmaBK) : 0.0;
+  return 3.0 * idle <= 3.0 + (double)R * d * 2 * (n_k + 3) / 5.5e6;
 }
 
 // Enqueues the gate/up and the down GEMM over all groups.  Requires umma_bind_x for this forward.  which: bit 0 the
 // gate/up GEMM, bit 1 the down GEMM.  early_rows: rows of the shared experts where the host knows them (plain layer).  Returns the number of kernels launched, or -1 (P->error).
 inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, int32_t* err_word,
-                        cudaStream_t st, cudaEvent_t mid, bool dep, int which, int early_rows) {
+                        cudaStream_t st, cudaEvent_t mid, bool dep, int which, int early_rows,
+                        bool skip_shared = false) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
@@ -790,6 +868,7 @@ inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, in
   if (mid && (which & 1)) cudaEventRecord(mid, st);
   a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
   a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
+  a.skip_groups = skip_shared ? s.n_outer : 0;
   if (which & 2)
     launch_kernel(dep, umma_grouped_kernel<2>, dim3(P->n_sms), dim3(kUmmaThreads), umma_smem_bytes(P->n_groups), st, P->a2_s,
                   P->a2_r, P->b2_s, P->b2_r, a);
@@ -799,6 +878,20 @@ inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, in
     return -1;
   }
   return (which & 1) + ((which >> 1) & 1);
+}
+
+// Down GEMM of the shared experts with the combine, after the routed experts' (umma_forward or umma2_forward with skip_shared).
+inline int umma_fold_forward(UmmaPlan* P, const GroupRows* gr, int n_rows, bf16* out, int32_t* err_word, cudaStream_t st, bool dep) {
+  const UmmaShape& s = P->shape;
+  UmmaArgs a = umma_base_args(P, gr, err_word);
+  a.out_s = out; a.ld_out_s = s.d; a.early_rows = n_rows;
+  a.band_mt = umma_band_tiles(s.shared_width);
+  if (launch_kernel(dep, umma_grouped_kernel<3>, dim3(P->n_sms), dim3(kUmmaThreads), umma_smem_bytes(P->n_groups), st, P->a2_s, P->a2_s,
+                    P->b2_s, P->b2_s, a) != cudaSuccess) {
+    snprintf(P->error, sizeof(P->error), "shared down GEMM launch failed");
+    return -1;
+  }
+  return 1;
 }
 
 }  // namespace cmoe

@@ -63,3 +63,17 @@ def _check_stack(layers, x, dtype):
     for layer in layers:
         assert layer.status() == 0
         layer.destroy()
+
+
+# the shared experts' down GEMM combines (a narrow shared block always qualifies): columns cut inside a tile and a 32-column step,
+# rows inside a tile, one to four selections, five (combined by its own kernel), and rows past one tile per CTA
+@pytest.mark.parametrize("d,top_k,tokens", [(272, 1, 129), (512, 2, 300), (304, 3, 257), (1040, 4, 700), (272, 5, 300), (2064, 4, 2600)])
+def test_combine_in_the_down_gemm(d, top_k, tokens):
+    shape = wl.LayerShape(d, 16 * 8, 8, 2, top_k, "bf16")
+    inp = wl.make_inputs(wl.Workload("fold", shape, (tokens,), seed=9))
+    layer = parity.gpu_layer(inp.layers[0], tokens)
+    for _ in range(2):
+        st = parity.check_plain_layer(layer, inp.layers[0], inp.x)
+        assert st["differing"] <= st["near_tie"]
+    assert layer.status() == 0
+    layer.destroy()
