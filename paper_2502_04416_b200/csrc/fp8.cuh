@@ -23,20 +23,6 @@ __device__ __forceinline__ float2 e4m3x2_to_f32x2(uint16_t v) {
   return __half22float2(*reinterpret_cast<const __half2*>(&h2));
 }
 
-// Four E4M3 codes (one 32-bit word, lowest byte first) -> four bf16 values as two packed words.
-// A code's magnitude bits, shifted into a bf16's exponent / mantissa fields, read as
-// 2^-120 times the code's value (also for subnormal codes, which become bf16 subnormals), so
-// one exact multiplication by 2^120 finishes the conversion without a case distinction.
-__device__ __forceinline__ void e4m3x4_to_bf16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
-  const uint32_t a = __byte_perm(w, 0u, 0x1404);          // halfwords b0 << 8, b1 << 8
-  const uint32_t b = __byte_perm(w, 0u, 0x3424);          // halfwords b2 << 8, b3 << 8
-  const uint32_t ma = ((a >> 4) & 0x07F007F0u) | (a & 0x80008000u);
-  const uint32_t mb = ((b >> 4) & 0x07F007F0u) | (b & 0x80008000u);
-  const uint32_t two120 = 0x7B807B80u;                    // bf16 2^120, twice
-  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(lo) : "r"(ma), "r"(two120));
-  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(hi) : "r"(mb), "r"(two120));
-}
-
 // Smallest e with amax * 2^-e <= 448 = 0.875 * 2^9 (0 for amax == 0).
 __device__ __forceinline__ int pow2_scale_exponent(float amax) {
   if (!(amax > 0.0f)) return 0;

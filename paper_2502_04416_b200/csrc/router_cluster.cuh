@@ -15,10 +15,7 @@
 // Against K slices over independent blocks (partial sums and a ticket through global memory, the last block alone
 // doing the gate logic and a block-wide scan; the permutation in kernels of its own above 128 rows), whole forwards: 7B-shaped
 // layer 1 / 16 / 64 / 128 / 512 rows 40.5 / 67.4 / 74.1 / 86.9 / 114.0 -> 35.0 / 62.1 / 69.1 / 80.0 / 109.3 us, 8B-shaped 32 /
-// 256 / 512 rows 88.2 / 112.3 / 140.9 -> 80.7 / 102.0 / 121.8, hierarchical 7 rows 295 -> 278.  Against the 128-row
-// tensor-core tiles of umma_grouped_kernel<3>: 8B-shaped 700 / 1000 / 2048 rows 143.7 / 181.4 / 237.6 -> 129.5 / 170.3 /
-// 240.7, 7B-shaped 600 / 1000 / 2048 rows 121.0 / 186.8 / 257.9 -> 117.9 / 179.3 / 269.3: every tile re-reads the
-// representative rows, so the line is drawn at 1024 rows.
+// 256 / 512 rows 88.2 / 112.3 / 140.9 -> 80.7 / 102.0 / 121.8, hierarchical 7 rows 295 -> 278.  Where tensor-core tiles take over: router_takes_tiles.
 #pragma once
 
 #include "common.cuh"
