@@ -474,7 +474,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         ra.x = L->hier ? x : xo; ra.row_src = L->outer_row_token; ra.x_copy = (bf16*)L->xo; ra.n_rows = R; ra.d = d; ra.n_r = n_r; ra.n_rp = L->n_rp; ra.n_k = n_k;
         ra.w_rep = (const bf16*)L->w_rep; ra.u = L->u; ra.b = L->b; ra.outer_off = ooff; ra.n_outer = L->n_outer;
         ra.ticket = L->router_ticket; ra.scores = L->scores; ra.keys = L->keys; ra.topk_idx = L->topk_idx;
-        ra.topk_gate = L->topk_gate; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
+        ra.topk_gate = L->topk_gate; ra.late_wait = split_x && !L->hier; ra.fuse_permute = perm_fused; ra.n_groups = G; ra.counts = L->counts;
         ra.offsets = L->offsets; ra.row_token = L->row_token; ra.row_of = L->row_of; ra.po = po;
         CU_TRY(router_cluster_launch(ra, L->hier, dep, use_umma && !gemv && !L->hier, st));
       } else {

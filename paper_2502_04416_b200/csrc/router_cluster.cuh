@@ -59,6 +59,7 @@ struct RouterArgs {
   float *scores, *keys;            // top-level router: scores = logits, topk_gate = weights
   int32_t* topk_idx;
   float* topk_gate;
+  int late_wait;                   // the preceding kernel of the forward is the split of the token rows, which this one does not read
   int fuse_permute, n_groups;
   int32_t *counts, *offsets, *row_token, *row_of;
   GroupPlanOut po;
@@ -105,8 +106,10 @@ router_cluster_kernel(const RouterArgs p) {
     }
   };
   if (NB == 1) load_w(s0, 0, 1);          // the layer's own rows: fetched while the preceding kernel of the stream drains
-  grid_dep_wait();
-  grid_dep_trigger();
+  // The split lets this kernel start after its own wait, so x is final; what follows reads the planes and starts after it.
+  // FP8 layers, waiting first / late: 8B-shaped 4 rows 42.7 / 40.0 us, 7B-shaped 2 rows 38.2 / 37.3, even from 16 rows on.
+  const bool late = NB == 1 && !OUTER && p.late_wait;
+  if (!late) { grid_dep_wait(); grid_dep_trigger(); }
   if (NB > 1 && warp == 0) {
     const int go = (p.outer_off && lane < kRcRows) ? find_outer(p.outer_off, p.n_outer, row_base + min(lane, n_rows - 1)) : 0;
     const int prev = __shfl_up_sync(0xffffffffu, go, 1);
@@ -187,6 +190,7 @@ router_cluster_kernel(const RouterArgs p) {
         }
     }
   }
+  if (late) { grid_dep_wait(); grid_dep_trigger(); }
   __syncthreads();
   rc_cluster_wait();
 #pragma unroll 1
