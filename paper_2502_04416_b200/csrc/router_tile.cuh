@@ -2,8 +2,8 @@
 // 64 rows, and the permutation that follows them.
 //
 // The contraction [rows, d] x [d, at most 64] is bound by reading x once; a tile per CTA left most SMs idle and every tile a
-// chain of 64 k blocks, partial sums and a ticket through global memory, and a gate stage of one thread per row (unrolled over
-// 32 experts: more time in instruction fetch than in arithmetic).  Here a cluster of 1, 2, 4 or 8 CTAs owns a tile:
+// chain of 64 k blocks, partial sums and a ticket through global memory, and a gate stage of one thread per row (a serial
+// chain over up to 32 experts).  Here a cluster of 1, 2, 4 or 8 CTAs owns a tile:
 //   - every CTA multiplies its slice of k (TMA, tcgen05.mma, sums in tensor memory) and lays its sums out in its shared memory;
 //   - after one cluster barrier it adds the slices of its share of the tile's rows in rank order (deterministic) straight
 //     from its peers' shared memory and runs their gate logic, one warp per row;
@@ -22,7 +22,7 @@
 
 namespace cmoe {
 
-constexpr int kRtThreads = 256;                // warp 0 TMA, warp 1 MMA, warps 4..7 read tensor memory, all eight gate
+constexpr int kRtThreads = 256;                // warp 0 TMA, warp 1 MMA, warps 4 and 5 read tensor memory, all eight gate
 constexpr int kRtTile = 64;                    // rows of a tile (the multiply takes 128; the upper half is not read back)
 constexpr int kRtStages = 6;                   // two CTAs on an SM: alone on theirs, clusters of 8 found no place at once
 constexpr int kRtABytes = kRtTile * kUmmaBK * 2;
@@ -40,7 +40,7 @@ struct RouterTileArgs {
   int32_t* err;
 };
 
-// Tiles (of `rows` rows) of every outer expert's row range, one expert per lane: lane o < n_outer returns its exclusive
+// Tiles of every outer expert's row range, one expert per lane: lane o < n_outer returns its exclusive
 // prefix and the range; `total` takes the sum.
 __device__ __forceinline__ int outer_tile_prefix(const int32_t* outer_off, int n_outer, int n_rows, int lane, int& row0, int& count,
                                                  int& total) {
