@@ -292,7 +292,7 @@ __device__ __forceinline__ TileCoord umma_decode(const UmmaArgs& p, const int32_
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(MODE == 1 ? kUmmaThreads + kUmmaGatherThreads : kUmmaThreads, 1)
+__global__ void __launch_bounds__(MODE == 2 ? kUmmaThreads : kUmmaThreads + 128, 1)
 umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_constant__ CUtensorMap tm_a_r,
                     const __grid_constant__ CUtensorMap tm_b_s, const __grid_constant__ CUtensorMap tm_b_r,
                     const UmmaArgs p) {
@@ -317,7 +317,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     // mode 1: besides the producer's expect_tx arrival, every gather thread arrives once per stage
     const uint32_t full_count = MODE == 1 ? 1 + kUmmaGatherThreads : 1;
     for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, MODE == 3 ? 8 : 4); }
     mbar_init(tbl_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -522,7 +522,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
     }
     if (!ok) asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2..5)
+    // ------------------------------------------------------------ epilogue (warps 2..5, mode 3: 2..9)
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
     uint32_t tile_n = 0;
     bool ok = true;
@@ -589,8 +589,9 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
 #pragma unroll
         for (int j = 0; j < 4; ++j) yr[j] = p.y_r + (size_t)pos[j] * p.d + n0;
         bf16* dst = p.out_s + tok * p.d + n0;
-        for (int c0 = 0; c0 < n_valid; c0 += 32) {
-          const bool two = c0 + 16 < n_valid;
+        const int c_end = min(n_valid, warp < 6 ? 128 : 256);         // warps 2..5 the left half, 6..9 the right
+        for (int c0 = warp < 6 ? 0 : 128; c0 < c_end; c0 += 32) {
+          const bool two = c0 + 16 < c_end;
           uint32_t w[4][16];
 #pragma unroll
           for (int j = 0; j < 4; ++j)
@@ -843,7 +844,8 @@ inline UmmaArgs umma_base_args(const UmmaPlan* P, const GroupRows* gr, int32_t* 
 // the rows at 5.5 TB/s).  Without / with: 8B-shaped 700 rows 100.5 / 106.4 us and 1400 rows 155.6 / 159.1 (not taken), 1000 / 2048 / 8192
 // rows 136.3 / 208.5 / 693 against 131.3 / 204.3 / 644, 7B-shaped 300 / 2500 rows 74.0 / 293 against 78.4 / 300 (not taken), 4000 / 8000 rows 445 /
 // 889 against 443 / 857, 13B-shaped 4096 / 16384 rows 568 / 2295 against 562 / 2286.  Fetching the routed rows of the next columns ahead
-// (233 registers) is slower: 8B-shaped 2048 / 8192 rows 213 / 667.
+// (233 registers) is slower: 8B-shaped 2048 / 8192 rows 213 / 667.  Eight epilogue warps instead of four, each with half of the columns: 8B-shaped
+// 2048 rows 205.5 / 198.7, 7B-shaped 2048 rows 229.4 / 227.4, 13B-shaped 16384 rows 2269 / 2252, even at 8192.
 inline bool umma_folds_combine(const UmmaPlan* P, int R, int n_k, int d) {
   if (!P->has_s || !P->has_r || n_k < 1 || n_k > 4 || d % 16 != 0) return false;
   const int tiles = (R + kUmmaBM - 1) / kUmmaBM * ((d + 255) / 256), over = tiles % P->n_sms;
@@ -886,7 +888,7 @@ inline int umma_fold_forward(UmmaPlan* P, const GroupRows* gr, int n_rows, bf16*
   UmmaArgs a = umma_base_args(P, gr, err_word);
   a.out_s = out; a.ld_out_s = s.d; a.early_rows = n_rows;
   a.band_mt = umma_band_tiles(s.shared_width);
-  if (launch_kernel(dep, umma_grouped_kernel<3>, dim3(P->n_sms), dim3(kUmmaThreads), umma_smem_bytes(P->n_groups), st, P->a2_s, P->a2_s,
+  if (launch_kernel(dep, umma_grouped_kernel<3>, dim3(P->n_sms), dim3(kUmmaThreads + 128), umma_smem_bytes(P->n_groups), st, P->a2_s, P->a2_s,
                     P->b2_s, P->b2_s, a) != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "shared down GEMM launch failed");
     return -1;
