@@ -305,7 +305,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
   if (L->cfg.dtype == CMOE_BF16) {
     UmmaShape s;
     s.d = L->cfg.d_model; s.m = L->m; s.shared_width = L->shared_width(); s.d_ff = L->cfg.d_ff;
-    s.n_outer = L->n_outer; s.n_r = L->n_r; s.n_rp = L->n_rp; s.n_k = L->cfg.top_k;
+    s.n_outer = L->n_outer; s.n_r = L->n_r; s.n_rp = L->n_rp; s.n_k = L->cfg.top_k; s.plain = !L->hier;
     s.max_outer_rows = (size_t)L->cfg.max_tokens * (L->hier ? L->outer_k : 1);
     s.max_routed_rows = s.max_outer_rows * L->cfg.top_k;
     UmmaBuffers ub;

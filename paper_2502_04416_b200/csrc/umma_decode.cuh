@@ -757,7 +757,7 @@ inline int decode_forward(UmmaPlan* P, DecodePlan* D, const GroupRows* gr, int n
   a.tok_box_rows = 16 << bi;
   // plain layer: group 0 is the shared expert and its rows are the whole batch, known here
   a.tile_rows_s = trs; a.tile_rows_r = trr;
-  a.early_units = (s.n_outer == 1 && P->has_s) ? (s.shared_width + trs - 1) / trs : 0;
+  a.early_units = (s.plain && P->has_s) ? (s.shared_width + trs - 1) / trs : 0;
   a.n_rows_plain = n_rows;
   a.scale_gu = D->scale_gu; a.scale_d = D->scale_d; a.rows_w = (long long)s.n_outer * s.d_ff;
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;

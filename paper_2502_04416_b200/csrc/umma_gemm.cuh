@@ -656,6 +656,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
 // ----------------------------------------------------------------------------- host
 struct UmmaShape {
   int d = 0, m = 0, shared_width = 0, d_ff = 0, n_outer = 1, n_r = 0, n_rp = 0, n_k = 0;
+  bool plain = true;                 // no top-level router (a hierarchical layer may have one outer expert as well)
   size_t max_outer_rows = 0, max_routed_rows = 0;
 };
 
