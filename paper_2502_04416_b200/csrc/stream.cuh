@@ -674,7 +674,7 @@ template <int NT> inline cudaError_t stream_allow_smem() {
 
 // Shapes this path takes: plain layers whose k blocks can be numbered in 31 bits.
 inline bool stream_shape_ok(const UmmaShape& s, int n_sms) {
-  return s.n_outer == 1 && s.n_r <= kMaxRouted && n_sms <= kStreamMaxGrid && s.d_ff >= 128 &&
+  return s.plain && s.n_r <= kMaxRouted && n_sms <= kStreamMaxGrid && s.d_ff >= 128 &&
          (long long)((s.d + 127) / 128) * (s.d_ff / 64 + 40) < (1ll << 30);
 }
 

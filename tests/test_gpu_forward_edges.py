@@ -8,8 +8,9 @@ from tests.test_gpu_fp8 import _quantised
 pytestmark = pytest.mark.gpu
 
 
-# A top-level router over one outer expert is no plain layer: the layer's copy of the rows is written by its own launches.
-@pytest.mark.parametrize("m,fp8", [(16, False), (16, True)])
+# A top-level router over one outer expert is no plain layer: the layer's copy of the rows is written by its own launches, and
+# the weight streamers (experts of at least 128 neurons in all) have no buffers there.
+@pytest.mark.parametrize("m,fp8", [(16, False), (16, True), (176, False), (176, True)])
 def test_one_outer_expert(m, fp8):
     shape = wl.LayerShape(256, m * 6, 6, 2, 2, "bf16")
     inp = wl.make_inputs(wl.Workload("one_outer", shape, (300,), seed=8, n_outer=1, outer_top_k=1))
