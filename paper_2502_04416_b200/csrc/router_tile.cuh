@@ -30,6 +30,7 @@ constexpr int kRtRows = 4;                     // rows whose gate logic a warp r
 
 struct RouterTileArgs {
   int n_rows, d, n_r, n_rp, n_k, n_cols;       // n_cols: columns of a tile, a multiple of 16; top-level: n_r = outer experts
+  int ks;                                      // CTAs of a tile's cluster; the grid's one extent is ks x tiles (2^31 - 1 at most)
   int n_outer;
   const int32_t* outer_off;                    // row ranges of the outer experts, or null (one range [0, n_rows))
   const float *u, *b;
@@ -80,7 +81,7 @@ router_tile_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   volatile int* abort_flag = &abort_mem;
   const uint32_t full0 = smem_u32(bar_mem), empty0 = full0 + 8 * kRtStages, accf = full0 + 16 * kRtStages;
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int ks = gridDim.x, rank = blockIdx.x, tile = blockIdx.y;    // the grid's x extent is one cluster
+  const int ks = p.ks, tile = blockIdx.x / ks, rank = blockIdx.x - tile * ks;
   const uint32_t b_bytes = (uint32_t)p.n_cols * kUmmaBK * 2, stage_bytes = kRtABytes + b_bytes;
   const uint32_t tmem_cols = p.n_cols <= 32 ? 32 : 64;
   const int k_blocks = (p.d + kUmmaBK - 1) / kUmmaBK;
@@ -388,7 +389,8 @@ inline int router_tile_forward(const CUtensorMap& tm_x, const CUtensorMap& tm_w,
   int ks = 8;
   while (ks > 1 && (tiles * ks > 2 * n_sms || 2 * ks > kb)) ks >>= 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ks, tiles); cfg.blockDim = dim3(kRtThreads); cfg.stream = st;
+  a.ks = ks;
+  cfg.gridDim = dim3(ks * tiles); cfg.blockDim = dim3(kRtThreads); cfg.stream = st;
   cfg.dynamicSmemBytes = 1024 + (size_t)kRtStages * (kRtABytes + a.n_cols * kUmmaBK * 2) + kRtABytes /* read past the last A */;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;

@@ -1,6 +1,7 @@
 """-m gpu: forwards at the edges of what the entry points take."""
 import pytest
 
+from oracle import cmoe_oracle as oracle
 from paper_2502_04416_b200 import workloads as wl
 from tests import parity
 from tests.test_gpu_fp8 import _quantised
@@ -23,4 +24,24 @@ def test_one_outer_expert(m, fp8):
         for x in (inp.x[-t:], inp.x[:t]):           # other rows in the copy than the forward before left there
             st = parity.check_hier_layer(layer, inp, x, expert_weights=weights)
             assert st["differing"] <= st["near_tie"]
+    layer.destroy()
+
+
+# 65535 row tiles of 64 and one more: past what a grid's second dimension can hold
+def test_more_rows_than_a_grid_dimension_of_tiles():
+    import torch
+    tokens, ends = 65535 * 64 + 70, 300
+    shape = wl.LayerShape(64, 16 * 2, 2, 1, 1, "bf16")      # one routed expert: nothing to tie
+    inp = wl.make_inputs(wl.Workload("many_rows", shape, (2 * ends,), seed=6))
+    lay = inp.layers[0]
+    layer = parity.gpu_layer(lay, tokens)
+    x = torch.zeros(tokens, 64, dtype=torch.bfloat16, device="cuda")
+    edge = parity.to_device(inp.x, "bf16")
+    x[:ends], x[-ends:] = edge[:ends], edge[ends:]
+    out = layer.forward(x)
+    torch.cuda.synchronize()
+    assert layer.status() == 0
+    got = parity.to_host(torch.cat([out[:ends], out[-ends:]]))
+    parity.check_output(got, oracle.cmoe_layer_forward(inp.x, **parity.oracle_kwargs(lay))[0])
+    assert torch.count_nonzero(out[ends:-ends]) == 0
     layer.destroy()
