@@ -251,7 +251,8 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
  * padding of the expert groups to 256-row tiles is expected to stay small; batches of 65 to 128 rows stream the bf16 weights through the
  * decode-shaped kernels, weights on the MMA's M side; 2 to 64 rows of a plain layer
  * run on two weight streamers with the gates folded into the hidden activations (rounded to bf16 once, after the
- * gate) and the sum over the experts inside the down projection; a single row of a plain layer
+ * gate) and the sum over the experts inside the down projection (a layer with an Inf or NaN in a routed expert's W_down
+ * stays on the decode-shaped kernels there, where such a weight reaches only the tokens that selected the expert); a single row of a plain layer
  * runs on the CUDA cores with plain-load weight streams, down projection and combine in one
  * launch), 1 = always SIMT, 2 = tensor-core with
  * single-CTA token-major tiles only (decode-shaped kernels up to 64 rows), 3 = tensor-core on CTA

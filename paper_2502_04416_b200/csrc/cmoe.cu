@@ -78,6 +78,7 @@ struct cmoe_layer {
   int gemm_path = 0;
   bool chain_launches = true;
   bool umma_ok = false;
+  bool down_finite = true;  // no Inf or NaN in the routed experts' W_down (see stream_shape_ok)
 
   // packed weights
   void* w_gu = nullptr;     // one allocation [2][n_outer*d_ff, d]: gate plane, then up plane
@@ -167,7 +168,7 @@ void free_layer(cmoe_layer* L) {
 
 template <typename T>
 __global__ void pack_down_kernel(const T* __restrict__ w_down, const int32_t* __restrict__ perm, int d,
-                                 int d_ff, int m, int shared_w, T* __restrict__ dst) {
+                                 int d_ff, int m, int shared_w, T* __restrict__ dst, int32_t* __restrict__ non_finite) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;   // packed neuron position
   const int c = blockIdx.y;
   if (n >= d_ff) return;
@@ -178,6 +179,7 @@ __global__ void pack_down_kernel(const T* __restrict__ w_down, const int32_t* __
   } else {
     const int j = (n - shared_w) / m, k = (n - shared_w) % m;
     o = (size_t)shared_w * d + (size_t)j * m * d + (size_t)c * m + k;
+    if (!isfinite(to_float(v))) *non_finite = 1;
   }
   dst[o] = v;
 }
@@ -320,7 +322,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     if (L->umma_ok && !decode_plan_create(&L->umma, &L->decode)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     L->decode.part = L->dec_part; L->decode.ticket = L->dec_ticket;
     if (L->umma_ok) CU_TRY(router_tile_allow());
-    if (L->umma_ok && stream_shape_ok(s, L->umma.n_sms) && !stream_plan_create(&L->umma, &L->stream))
+    if (L->umma_ok && L->down_finite && stream_shape_ok(s, L->umma.n_sms) && !stream_plan_create(&L->umma, &L->stream))
       return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     if (L->umma_ok && !umma2_plan_create(&L->umma, &L->pair)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   }
@@ -330,7 +332,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
 
 template <typename T>
 int pack_weights(cmoe_layer* L, const void* w_gate, const void* w_up, const void* w_down,
-                 const int32_t* perm_dev, const int32_t* rep_dev, cudaStream_t st) {
+                 const int32_t* perm_dev, const int32_t* rep_dev, int32_t* non_finite_dev, cudaStream_t st) {
   const int d = L->cfg.d_model, d_ff = L->cfg.d_ff;
   const int row_vec = d * (int)sizeof(T) / 16;
   gather_rows_kernel<<<d_ff, 256, 0, st>>>((const uint4*)w_gate, perm_dev, d_ff, row_vec, (uint4*)L->wg_p);
@@ -343,7 +345,7 @@ int pack_weights(cmoe_layer* L, const void* w_gate, const void* w_up, const void
   }
   dim3 grid((d_ff + 255) / 256, d);
   pack_down_kernel<T><<<grid, 256, 0, st>>>((const T*)w_down, perm_dev, d, d_ff, L->m, L->shared_width(),
-                                            (T*)L->wd_p);
+                                            (T*)L->wd_p, non_finite_dev);
   CU_TRY(cudaGetLastError());
   return CMOE_OK;
 }
@@ -683,7 +685,8 @@ int cmoe_layer_create(const cmoe_config* cfg, const void* w_gate, const void* w_
   L->esz = cfg->dtype == CMOE_BF16 ? 2 : 4;
   cudaGetDevice(&L->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int32_t *perm_dev = nullptr, *rep_dev = nullptr;
+  int32_t *perm_dev = nullptr, *rep_dev = nullptr;       // rep_dev: one word more, set if W_down is not finite
+  int32_t non_finite = 0;
   auto fail = [&](int code) { cudaFree(perm_dev); cudaFree(rep_dev); free_layer(L); return code; };
 #define TRY_OR_FAIL(expr)                                                 \
   do {                                                                    \
@@ -700,15 +703,19 @@ int cmoe_layer_create(const cmoe_config* cfg, const void* w_gate, const void* w_
   TRY_OR_FAIL(cudaMalloc(&L->u, (size_t)(n_r ? n_r : 1) * sizeof(float)));
   TRY_OR_FAIL(cudaMalloc(&L->b, (size_t)(n_r ? n_r : 1) * sizeof(float)));
   TRY_OR_FAIL(cudaMalloc(&perm_dev, (size_t)d_ff * sizeof(int32_t)));
-  TRY_OR_FAIL(cudaMalloc(&rep_dev, (size_t)(n_r ? n_r : 1) * sizeof(int32_t)));
+  TRY_OR_FAIL(cudaMalloc(&rep_dev, (size_t)(n_r + 1) * sizeof(int32_t)));
+  TRY_OR_FAIL(cudaMemsetAsync(rep_dev + n_r, 0, sizeof(int32_t), st));
   TRY_OR_FAIL(cudaMemcpyAsync(perm_dev, neuron_perm, (size_t)d_ff * sizeof(int32_t),
                               cudaMemcpyHostToDevice, st));
   if (n_r)
     TRY_OR_FAIL(cudaMemcpyAsync(rep_dev, rep_idx, (size_t)n_r * sizeof(int32_t),
                                 cudaMemcpyHostToDevice, st));
-  rc = cfg->dtype == CMOE_BF16 ? pack_weights<bf16>(L, w_gate, w_up, w_down, perm_dev, rep_dev, st)
-                               : pack_weights<float>(L, w_gate, w_up, w_down, perm_dev, rep_dev, st);
+  rc = cfg->dtype == CMOE_BF16 ? pack_weights<bf16>(L, w_gate, w_up, w_down, perm_dev, rep_dev, rep_dev + n_r, st)
+                               : pack_weights<float>(L, w_gate, w_up, w_down, perm_dev, rep_dev, rep_dev + n_r, st);
   if (rc != CMOE_OK) return fail(rc);
+  TRY_OR_FAIL(cudaMemcpyAsync(&non_finite, rep_dev + n_r, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  TRY_OR_FAIL(cudaStreamSynchronize(st));
+  L->down_finite = non_finite == 0;
   rc = upload_gate_params(L, gate_scale_u, select_bias_b, st);
   if (rc != CMOE_OK) return fail(rc);
   rc = finish_layer(L, st);

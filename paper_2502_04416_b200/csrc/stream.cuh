@@ -672,7 +672,8 @@ template <int NT> inline cudaError_t stream_allow_smem() {
   return e;
 }
 
-// Shapes this path takes: plain layers whose k blocks can be numbered in 31 bits.
+// Shapes this path takes: plain layers whose k blocks can be numbered in 31 bits.  Their routed experts' W_down has to be finite
+// as well: a token's sum runs over all active experts, with zeros in Hd for those it did not select, and 0 x Inf is NaN.
 inline bool stream_shape_ok(const UmmaShape& s, int n_sms) {
   return s.plain && s.n_r <= kMaxRouted && n_sms <= kStreamMaxGrid && s.d_ff >= 128 &&
          (long long)((s.d + 127) / 128) * (s.d_ff / 64 + 40) < (1ll << 30);

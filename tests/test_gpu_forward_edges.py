@@ -1,4 +1,5 @@
 """-m gpu: forwards at the edges of what the entry points take."""
+import numpy as np
 import pytest
 
 from oracle import cmoe_oracle as oracle
@@ -44,4 +45,33 @@ def test_more_rows_than_a_grid_dimension_of_tiles():
     got = parity.to_host(torch.cat([out[:ends], out[-ends:]]))
     parity.check_output(got, oracle.cmoe_layer_forward(inp.x, **parity.oracle_kwargs(lay))[0])
     assert torch.count_nonzero(out[ends:-ends]) == 0
+    layer.destroy()
+
+
+# An expert's weights reach only the tokens that selected it, whatever they hold: 0 x Inf is NaN, so a sum over all active
+# experts would carry a single Inf of W_down to every token of the batch.
+@pytest.mark.parametrize("fp8,value", [(False, np.inf), (False, np.nan), (True, np.nan)])
+def test_non_finite_down_weight_stays_with_its_expert(fp8, value):
+    import torch
+    shape = wl.LayerShape(256, 176 * 8, 8, 2, 2, "bf16")
+    inp = wl.make_inputs(wl.Workload("non_finite", shape, (65,), seed=3))
+    lay, expert, channel = inp.layers[0], 3, 5
+    clean = lay.w_down.copy()
+    lay.w_down[channel, lay.neuron_perm[(shape.n_shared + expert) * shape.m + 7]] = value
+    layer = parity.gpu_layer(lay, 65)
+    lay.w_down = clean
+    if fp8:
+        layer.quantise_fp8()
+    ew = _quantised(lay) if fp8 else dict(w_gate=lay.w_gate, w_up=lay.w_up, w_down=clean)
+    for t in (1, 2, 16, 33, 64, 65):
+        out = layer.forward(parity.to_device(inp.x[:t], "bf16"))
+        torch.cuda.synchronize()
+        got, r = parity.to_host(out), layer.routing(t, shape.n_routed)
+        hit = (r["topk_idx"] == expert).any(axis=1)
+        want = oracle.moe_forward(inp.x[:t], ew["w_gate"], ew["w_up"], ew["w_down"], lay.neuron_perm, shape.n_experts,
+                                  shape.n_shared, r["topk_idx"].astype(np.int32), r["topk_gate"].astype(np.float64))
+        assert not np.isfinite(got[hit, channel]).any()
+        got[hit, channel] = want[hit, channel] = 0.0
+        parity.check_output(got, want)
+        assert t < 16 or 0 < hit.sum() < t
     layer.destroy()
