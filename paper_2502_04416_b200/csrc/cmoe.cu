@@ -933,7 +933,7 @@ int cmoe_layer_quantise_fp8(cmoe_layer* L, void* stream) {
       f.hr_scale = a.take<float>(f.hr_rows);
       if (!L->hier) {
         hq = a.take<uint8_t>(2 * (size_t)kStreamMaxRows * L->cfg.d_ff);
-        hq_scale = a.take<float>(kStreamMaxRows);
+        hq_scale = a.take<float>((size_t)(1 + L->n_r) * kStreamMaxRows);
       }
     };
     carve(nullptr);

@@ -22,8 +22,8 @@
 //
 // W8 = true streams FP8 (E4M3) codes, half the bytes, into kind::f8f6f4 MMAs.  The token rows are E4M3 planes hi and lo (see
 // split_rows_e4m3_kernel), both multiplied by one MMA (N = 2 x token rows); the planes of x are written ahead of the router,
-// those of Hd by a split launch between the two kernels.  The scale of a down weight row differs from expert to expert, so the
-// down kernel accumulates one group at a time and its epilogue adds them up in registers.
+// those of Hd by a split launch between the two kernels.  The scales of a down weight row and of a token's Hd differ from expert
+// to expert, so the down kernel accumulates one group at a time and its epilogue adds them up in registers.
 //
 // Registers and shared memory are sized so that the router, the up and the down kernel fit one SM
 // pairwise: otherwise the successor's CTAs start when the predecessor's end, and the streams pause in between.  Loops
@@ -70,8 +70,8 @@ struct StreamArgs {
   float* part;                 // down: [2 * CTAs] slots of 128 x NT fp32
   int32_t* ticket;             // down: [tiles][8], zero between launches
   int32_t* err;
-  // FP8 weights: per-row power-of-two scales of the token planes (up: x rows; down: Hd rows) and of the weight rows
-  const float* tok_scale;
+  // FP8 weights: power-of-two scales of the token planes and of the weight rows
+  const float* tok_scale;      // up: [rows] of x; down: [1 + n_r][kStreamMaxRows] of Hd
   const float* scale_gu;       // [2][rows_w]: gate plane, then up plane, packed neuron order
   const float* scale_d;        // [1 + n_r][d]: per group and output channel
   long long rows_w;
@@ -384,7 +384,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 172);
   int* n_active = reinterpret_cast<int*>(tail + 176);
   int* active = reinterpret_cast<int*>(tail + 192);             // [32]
-  const uint32_t ring = base + 1024;
+  const uint32_t ring = base + (W8 ? 2048 : 1024);              // W8: [8 warps][32] token scales in between
   const int stages = p.stages;
   constexpr uint32_t kWBytes = 128 * 128;
   const uint32_t stage_bytes = kWBytes + (W8 ? 2 : 1) * p.tok_rows * 128;
@@ -502,10 +502,8 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
     const int quad = warp & 3, half = (warp - 2) >> 2;              // 8-column chunks half, half + 2, ...
     const int slot_q = quad * 32 + lane;
     constexpr int kCh = NT / 16;                                    // this warp's chunks: columns 16 i + 8 half
+    float* tok_sc = reinterpret_cast<float*>(tail + 1024) + 32 * (warp - 2);
     grid_dep_wait();                                                // also orders this kernel's stores to `out`
-    float ts_lo = 1.0f, ts_hi = 1.0f;                               // W8: this lane's token scales
-    if (W8 && lane < p.n_rows) ts_lo = __ldcg(p.tok_scale + lane);
-    if (W8 && lane + 32 < p.n_rows) ts_hi = __ldcg(p.tok_scale + lane + 32);
     bool ok = true;
     uint32_t seg = 0;
 #pragma unroll 1
@@ -526,6 +524,10 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
           const int kb = b - tile_b0;
           const int g = kb < run.kb_s ? 0 : 1 + active[(kb - run.kb_s) / run.kb_m];
           if (ch < p.d) sc = __ldg(p.scale_d + (size_t)g * p.d + ch);
+          const int tok = 16 * (lane >> 3) + 8 * half + (lane & 7);  // the tokens' scales, in the order of v
+          __syncwarp();
+          if (tok < p.n_rows) tok_sc[lane] = __ldcg(p.tok_scale + g * kStreamMaxRows + tok);
+          __syncwarp();
         }
         b = W8 ? min(end, run.group_end(tile_b0, b)) : end;
         const uint32_t buf = seg & 1, use = seg >> 1;
@@ -542,7 +544,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
               tmem_ld8(taddr + p.tok_rows + 16 * i, l);
               tmem_ld_wait();
 #pragma unroll
-              for (int q = 0; q < 8; ++q) v[i][q] = fmaf(fmaf(l[q], 0.0625f, t[q]), sc, v[i][q]);
+              for (int q = 0; q < 8; ++q) v[i][q] = fmaf(fmaf(l[q], 0.0625f, t[q]) * sc, tok_sc[8 * i + q], v[i][q]);
             } else {
               tmem_ld_wait();
 #pragma unroll
@@ -557,9 +559,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
       auto store8 = [&](int c0, const float (&r)[8]) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          float y = r[q];
-          if (W8) y *= __shfl_sync(0xffffffffu, c0 < 32 ? ts_lo : ts_hi, (c0 + q) & 31);
-          if (ch < p.d && c0 + q < p.n_rows) p.out[(size_t)(c0 + q) * p.d + ch] = __float2bfloat16_rn(y);
+          if (ch < p.d && c0 + q < p.n_rows) p.out[(size_t)(c0 + q) * p.d + ch] = __float2bfloat16_rn(r[q]);
         }
       };
       if (whole) {
@@ -635,7 +635,7 @@ struct StreamPlan {
   // FP8 weights (stream_plan_attach_fp8): codes of the gate/up rows, boxes of 128 k; E4M3 planes of x and of Hd
   CUtensorMap w_gu8[16], xq[4], hq_s[4], hq_r[4];
   uint8_t* hq = nullptr;            // [2][kStreamMaxRows][d_ff]
-  float* hq_scale = nullptr;        // [kStreamMaxRows]
+  float* hq_scale = nullptr;        // [1 + n_r][kStreamMaxRows]
   const float *x_scale = nullptr, *scale_gu = nullptr, *scale_d = nullptr;
 };
 
@@ -662,7 +662,7 @@ inline int stream_down_stages(int tok) {
   const int n = 98 * 1024 / (16384 + tok);
   return n > 8 ? 8 : n;
 }
-inline int stream_down_smem(int tok) { return 2048 + stream_down_stages(tok) * (16384 + tok); }
+inline int stream_down_smem(int tok, bool w8) { return 2048 + (w8 ? 1024 : 0) + stream_down_stages(tok) * (16384 + tok); }
 
 template <int NT> inline cudaError_t stream_allow_smem() {
   cudaError_t e = allow_smem(stream_up_kernel<NT, false>, 227 * 1024);
@@ -719,7 +719,7 @@ inline bool stream_plan_create(UmmaPlan* P, StreamPlan* S) {
 }
 
 // FP8 codes and token planes of a quantised layer, all owned by the caller: w_gu8 [2][d_ff][d], xq [2][kStreamMaxRows][d],
-// hq [2][kStreamMaxRows][d_ff]; d, m and the shared width are multiples of 16.
+// hq [2][kStreamMaxRows][d_ff], hq_scale [1 + n_r][kStreamMaxRows]; d, m and the shared width are multiples of 16.
 inline bool stream_plan_attach_fp8(UmmaPlan* P, StreamPlan* S, const void* w_gu8, const uint8_t* xq, const float* x_scale,
                                    uint8_t* hq, float* hq_scale, const float* scale_gu, const float* scale_d) {
   const UmmaShape& s = P->shape;
@@ -816,12 +816,12 @@ inline void stream_launch(const UmmaPlan* P, const StreamPlan* S, const CUtensor
   if (mid) cudaEventRecord(mid, st);
   if (gate_up_only) return;
   if (W8) {                                       // E4M3 planes of Hd
-    const SplitSegment hd{S->h, a.n_rows, a.ld_h, (long long)a.ld_h, S->hq, (long long)kStreamMaxRows, S->hq_scale};
-    launch_kernel(dep, split_rows_e4m3_kernel, dim3(a.n_rows), dim3(kSplitThreads), 0, st, hd, SplitSegment{});
+    const SplitGroups hd{S->h, S->hq, S->hq_scale, a.has_s ? a.shared_w : 0, a.m, a.ld_h, kStreamMaxRows};
+    launch_kernel(dep, split_groups_e4m3_kernel, dim3(a.n_rows, 1 + a.n_r), dim3(kSplitGroupThreads), 0, st, hd);
     a.tok_scale = S->hq_scale;
   }
   a.stages = stream_down_stages(tok);
-  launch_kernel(dep, stream_down_kernel<NT, W8>, dim3(P->n_sms), dim3(kStreamThreads), stream_down_smem(tok), st, wd_s, wd_r,
+  launch_kernel(dep, stream_down_kernel<NT, W8>, dim3(P->n_sms), dim3(kStreamThreads), stream_down_smem(tok, W8), st, wd_s, wd_r,
                 W8 ? S->hq_s[bi] : S->h_s[bi], W8 ? S->hq_r[bi] : S->h_r[bi], a);
 }
 

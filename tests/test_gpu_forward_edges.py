@@ -75,3 +75,20 @@ def test_non_finite_down_weight_stays_with_its_expert(fp8, value):
         parity.check_output(got, want)
         assert t < 16 or 0 < hit.sum() < t
     layer.destroy()
+
+
+# The hidden activations of the shared experts 2^20 times those of the routed ones, their down rows smaller by as much: both
+# contribute alike, and every expert's channels have scales of their own.
+@pytest.mark.parametrize("n_experts,n_shared,top_k", [(8, 2, 2), (32, 4, 4)])
+def test_fp8_experts_of_different_magnitude(n_experts, n_shared, top_k):
+    shape = wl.LayerShape(256, 176 * n_experts, n_experts, n_shared, top_k, "bf16")
+    inp = wl.make_inputs(wl.Workload("fp8_magnitudes", shape, (64,), seed=4))
+    lay = inp.layers[0]
+    shared = lay.neuron_perm[:n_shared * shape.m]
+    lay.w_up[shared] *= 2.0 ** 20
+    lay.w_down[:, shared] *= 2.0 ** -20
+    layer = parity.gpu_layer(lay, 64)
+    layer.quantise_fp8()
+    for t in (1, 2, 16, 17, 48, 64):
+        parity.check_plain_layer(layer, lay, inp.x[:t], expert_weights=_quantised(lay))
+    layer.destroy()
