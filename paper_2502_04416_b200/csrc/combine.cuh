@@ -32,11 +32,11 @@ __global__ void plan_groups_kernel(int n_outer, int n_r, int n_tokens,
   for (int g = threadIdx.x; g < n_groups; g += blockDim.x) {
     GroupRows r;
     if (g < n_outer) {
-      r.row0 = outer_off ? outer_off[g] : 0;
-      r.count = outer_off ? outer_off[g + 1] - outer_off[g] : n_tokens;
+      r.row0 = outer_off ? __ldcg(outer_off + g) : 0;
+      r.count = outer_off ? __ldcg(outer_off + g + 1) - r.row0 : n_tokens;
     } else {
-      r.row0 = offsets[g - n_outer];
-      r.count = counts[g - n_outer];
+      r.row0 = __ldcg(offsets + g - n_outer);
+      r.count = __ldcg(counts + g - n_outer);
     }
     gr[g] = r;
   }
@@ -47,7 +47,8 @@ __global__ void plan_groups_kernel(int n_outer, int n_r, int n_tokens,
 // added in the order of the selection (descending key), a fixed order, so results are
 // reproducible run to run; fp32 accumulation, one rounding to the output type.  Every
 // thread reads the token's few routing words itself (same addresses across the block, so
-// they broadcast from L1) and then streams its 16 (bf16) or 8 columns of every row.
+// they broadcast from L1; the down GEMM lets this kernel start when they are long complete) and
+// then streams its 16 (bf16) or 8 columns of every row.
 template <typename T>
 __global__ void __launch_bounds__(256)
 combine_kernel(const T* __restrict__ y_s, const T* __restrict__ y_r,

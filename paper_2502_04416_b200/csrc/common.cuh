@@ -74,6 +74,10 @@ template <typename T> __device__ __forceinline__ T from_float(float v);
 template <> __device__ __forceinline__ float from_float<float>(float v) { return v; }
 template <> __device__ __forceinline__ bf16 from_float<bf16>(float v) { return __float2bfloat16_rn(v); }
 
+// Read-only loads (__ldg, ld.global.nc, a subscript of a const __restrict__ pointer) are for data that no kernel writes while this
+// one is resident: the layer's own weights, and what was complete before the predecessor let this kernel start.  Everything that
+// the predecessor itself may write is read by __ldcg or the loads below.
+//
 // 16 bytes of data that a preceding kernel of the stream may have written: a volatile load stays below grid_dep_wait(),
 // and it is not a read-only (.nc) one, whose cache lines need not be dropped while the kernel runs.
 __device__ __forceinline__ uint4 ld_dep16(const void* p) {
@@ -102,7 +106,7 @@ __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
 __device__ __forceinline__ void ld256_stream(const bf16* p, uint32_t (&w)[8]) {
   // volatile + memory clobber: the load must stay below griddepcontrol.wait (its source is written
   // by the preceding kernel of a chained launch)
-  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                : "l"(p) : "memory");
 }
@@ -135,9 +139,9 @@ __device__ __forceinline__ void store16(bf16* p, const float* v) {
 }
 __device__ __forceinline__ void load16(const bf16* p, float* v) {
   uint32_t w[8];
-  asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-               : "l"(p));
+               : "l"(p) : "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     v[2 * i] = __uint_as_float(w[i] << 16);

@@ -21,7 +21,7 @@ __device__ __forceinline__ void chunk_histogram(const int32_t* __restrict__ topk
   __syncthreads();
   if (row < n_rows)
     for (int j = 0; j < n_k; ++j) {
-      const int e = topk_idx[(size_t)row * n_k + j];
+      const int e = __ldcg(topk_idx + (size_t)row * n_k + j);
       if ((unsigned)e < (unsigned)n_groups) atomicAdd(&hist[e], 1);   // out-of-range entries are ignored
     }
   __syncthreads();
@@ -63,7 +63,7 @@ __device__ __forceinline__ void chunk_scatter(const int32_t* __restrict__ topk_i
   int sel[kMaxTopK], rank[kMaxTopK];
 #pragma unroll
   for (int j = 0; j < kMaxTopK; ++j) {
-    sel[j] = (row < n_rows && j < n_k) ? topk_idx[(size_t)row * n_k + j] : -1;
+    sel[j] = (row < n_rows && j < n_k) ? __ldcg(topk_idx + (size_t)row * n_k + j) : -1;
     if ((unsigned)sel[j] >= (unsigned)n_groups) sel[j] = -1;
     rank[j] = 0;
   }
@@ -104,8 +104,8 @@ __device__ __forceinline__ void write_group_rows(const GroupPlanOut& po, int n_g
   for (int g = threadIdx.x; g < po.n_outer + n_groups; g += blockDim.x) {
     GroupRows r;
     if (g < po.n_outer) {
-      r.row0 = po.outer_off ? po.outer_off[g] : 0;
-      r.count = po.outer_off ? po.outer_off[g + 1] - po.outer_off[g] : po.n_tokens;
+      r.row0 = po.outer_off ? __ldcg(po.outer_off + g) : 0;
+      r.count = po.outer_off ? __ldcg(po.outer_off + g + 1) - r.row0 : po.n_tokens;
     } else {
       r.row0 = offsets[g - po.n_outer];
       r.count = counts[g - po.n_outer];
@@ -193,8 +193,8 @@ __device__ __forceinline__ void permute_by_masks(const PermuteOut& p, uint8_t* s
 #pragma unroll 1
     for (int g = threadIdx.x - 32; g < p.po.n_outer; g += kMaskThreads - 32) {
       GroupRows r;
-      r.row0 = p.po.outer_off ? p.po.outer_off[g] : 0;
-      r.count = p.po.outer_off ? p.po.outer_off[g + 1] - r.row0 : p.po.n_tokens;
+      r.row0 = p.po.outer_off ? __ldcg(p.po.outer_off + g) : 0;
+      r.count = p.po.outer_off ? __ldcg(p.po.outer_off + g + 1) - r.row0 : p.po.n_tokens;
       p.po.gr[g] = r;
     }
   }
@@ -309,7 +309,7 @@ permute_scatter_kernel(const int32_t* __restrict__ topk_idx, int n_rows, int n_k
   int32_t* base = sm;                      // [n_groups]
   int32_t* warp_cnt = base + n_groups;     // [8][n_groups]
   for (int g = threadIdx.x; g < n_groups; g += blockDim.x)
-    base[g] = offsets[g] + chunk_cnt[(size_t)blockIdx.x * n_groups + g];
+    base[g] = __ldcg(offsets + g) + __ldcg(chunk_cnt + (size_t)blockIdx.x * n_groups + g);
   __syncthreads();
   const int row = blockIdx.x * kPermChunk + threadIdx.x;
   chunk_scatter(topk_idx, n_rows, n_k, n_groups, row, base, warp_cnt, row_token, row_of);
@@ -339,7 +339,7 @@ permute_scan_scatter_kernel(const int32_t* __restrict__ topk_idx, int n_rows, in
   for (int g = threadIdx.x; g < n_groups; g += blockDim.x) {
     int before = 0, all = 0;
     for (int cc = 0; cc < n_chunks; ++cc) {
-      const int v = __ldg(chunk_cnt + (size_t)cc * n_groups + g);
+      const int v = __ldcg(chunk_cnt + (size_t)cc * n_groups + g);
       before += cc < c ? v : 0;
       all += v;
     }

@@ -116,7 +116,7 @@ atopk_kernel(const T* __restrict__ h, int ld, int d_h, int k_a, int token0, uint
       for (int q = 0; q < kVec; ++q) f(k[q], v * kVec + q);
     }
 #pragma unroll 1
-    for (int i = tail + tid; i < d_h; i += kAtopkThreads) f((uint32_t)KeyOf<T>::make(row[i]), i);
+    for (int i = tail + tid; i < d_h; i += kAtopkThreads) f((uint32_t)KeyOf<T>::make(__ldcg(row + i)), i);
   };
   uint32_t my_max = 0;
   for_keys([&](uint32_t k, int) { my_max = max(my_max, k); });

@@ -12,7 +12,7 @@ namespace cmoe {
 __device__ __forceinline__ int find_outer(const int32_t* __restrict__ off, int n_outer, int r) {
   int g = 0;
 #pragma unroll 4
-  for (int i = 1; i < n_outer; ++i) g += (__ldg(off + i) <= r) ? 1 : 0;
+  for (int i = 1; i < n_outer; ++i) g += (__ldcg(off + i) <= r) ? 1 : 0;
   return g;
 }
 
@@ -39,9 +39,9 @@ __device__ __forceinline__ void gate_row(int lane, int n_r, int n_k, float a, fl
   const float s_max = warp_max(s);
   const float e = live ? expf(s - s_max) : 0.0f;
   const float s_prime = e / warp_sum(e);                               // Softmax over all N_r
-  const float key = live ? s_prime + __ldg(b + lane) : -INFINITY;
+  const float key = live ? s_prime + __ldcg(b + lane) : -INFINITY;
   if (live) { scores_row[lane] = s; keys_row[lane] = key; }
-  const float gate = live ? 1.0f + s_prime * __ldg(u + lane) : 0.0f;   // 1 + s'_i u_i
+  const float gate = live ? 1.0f + s_prime * __ldcg(u + lane) : 0.0f;   // 1 + s'_i u_i
   const float rank_key = (key != key) ? -INFINITY : key;               // NaN ranks last
   bool taken = !live;
   for (int i = 0; i < n_k; ++i) {

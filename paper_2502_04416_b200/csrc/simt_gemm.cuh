@@ -28,7 +28,7 @@ __device__ __forceinline__ void load_seg(const T* row_ptr, int k, int K, bool ve
     load8(row_ptr + k, v);
   } else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = (k + q < K) ? to_float(row_ptr[k + q]) : 0.0f;
+    for (int q = 0; q < 8; ++q) v[q] = (k + q < K) ? to_float(__ldcg(row_ptr + k + q)) : 0.0f;
   }
 }
 
@@ -103,7 +103,7 @@ __device__ __forceinline__ float4 load_quad(const T* row_ptr, int k, int K, bool
   if (vec && k + 4 <= K) return load4f(row_ptr + k);
   float v[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) v[q] = k + q < K ? to_float(row_ptr[k + q]) : 0.0f;
+  for (int q = 0; q < 4; ++q) v[q] = k + q < K ? to_float(__ldcg(row_ptr + k + q)) : 0.0f;
   return make_float4(v[0], v[1], v[2], v[3]);
 }
 

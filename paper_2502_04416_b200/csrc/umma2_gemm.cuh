@@ -356,7 +356,7 @@ umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_co
         src_row[i] = nullptr;
         const int r = (2 * c.mp + (int)rank) * kUmmaBM + i * 16 + r_sub;
         if (mine && r < c.count)                      // rows past the group are left as they are: nothing of them is stored
-          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + c.row0 + r) * p.d;
+          src_row[i] = p.x_rows_ptr + (size_t)__ldcg(p.row_token + c.row0 + r) * p.d;
       }
       for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
         const uint32_t s = it % kU2Stages, n = it / kU2Stages;

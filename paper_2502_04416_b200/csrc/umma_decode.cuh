@@ -412,7 +412,7 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
 #pragma unroll
         for (int c = 0; c < NT; c += 32) if (c + lane < NT) inv[c + lane] = -1;
         __syncwarp();
-        for (int c = lane; c < r.count; c += 32) inv[__ldg(p.row_token + r.row0 + c) - rs.row0] = c;
+        for (int c = lane; c < r.count; c += 32) inv[__ldcg(p.row_token + r.row0 + c) - rs.row0] = c;
         __syncwarp();
       }
       const bool row_live = quad * 32 + lane < tr && wr < span;
@@ -431,7 +431,7 @@ umma_decode_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
         if (row_live && c < n_cols) {
           const int pos = lookup ? inv[c] : c;
           if (pos >= 0) {
-            if constexpr (W8) { const float ts = __ldg(tok_scale + c); a *= sc_a * ts; b *= sc_b * ts; }
+            if constexpr (W8) { const float ts = __ldcg(tok_scale + c); a *= sc_a * ts; b *= sc_b * ts; }
             const float v = MODE == 4 ? swiglu_fast(a, b) : a;
             dst[(size_t)pos * ld] = __float2bfloat16_rn(v);
           }

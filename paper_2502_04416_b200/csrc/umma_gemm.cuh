@@ -495,7 +495,7 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
         src_row[i] = nullptr;
         const int r = c.mt * kUmmaBM + i * 16 + r_sub;
         if (mine && r < c.count)                      // rows past the group are left as they are: nothing of them is stored
-          src_row[i] = p.x_rows_ptr + (size_t)__ldg(p.row_token + c.row0 + r) * p.d;
+          src_row[i] = p.x_rows_ptr + (size_t)__ldcg(p.row_token + c.row0 + r) * p.d;
       }
       for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
         const uint32_t s = it % kStages, n = it / kStages;

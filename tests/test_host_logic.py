@@ -87,6 +87,30 @@ def test_null_layer_calls(lib):
     assert lib.cmoe_layer_get_gate_params(None, None, None, None) == -1
 
 
+# ------------------------------------------------------------------ sources
+def test_read_only_loads_are_of_data_no_predecessor_writes():
+    """A chained kernel is resident while its predecessor runs, so what that one writes may not be read through the
+    read-only path (__ldg, ld.global.nc): only the layer's weights, or data that is complete before the kernel may start."""
+    allowed = {
+        "gemv.cuh": [r"L1::no_allocate\.v[24]\.u32", r"p\.scale_(gu|d)\b"],           # weight streams, scales of weight rows
+        "router_cluster.cuh": [r"\bwr \+"],                                          # representative rows
+        "stream.cuh": [r"p\.scale_(gu|d)\b"],
+        "umma_decode.cuh": [r"p\.scale_(gu|d)\b"],
+        "combine.cuh": [r"\b(outer_row_of|outer_w|row_of|topk_gate) \+"],            # complete before the gate/up GEMM ends
+        "router_mma.cuh": [r"."], "cluster.cuh": [r"."],                             # launched the ordinary way
+        "profile.cuh": [r"\bact_count \+"],                                          # select_shared_kernel: the ordinary way
+    }
+    csrc = os.path.join(ROOT, "paper_2502_04416_b200", "csrc")
+    bad = []
+    for name in sorted(os.listdir(csrc)):
+        for n, line in enumerate(open(os.path.join(csrc, name)), 1):
+            code = line.split("//")[0]
+            for load in re.findall(r"(?:__ldg\(|ld\.global\.nc).*?(?=__ldg\(|ld\.global\.nc|$)", code.rstrip("\n")):
+                if not any(re.search(a, load) for a in allowed.get(name, [])):
+                    bad.append(f"{name}:{n}: {line.strip()}")
+    assert not bad, "\n".join(bad)
+
+
 # ------------------------------------------------------------------ workloads
 def test_bf16_rounding_is_nearest_even():
     import torch
