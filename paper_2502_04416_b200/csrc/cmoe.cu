@@ -73,7 +73,7 @@ struct cmoe_layer {
   cmoe_config cfg{};
   int m = 0, n_r = 0, n_rp = 0, n_outer = 1, outer_k = 1;   // n_rp: N_r rounded up to 8
   bool hier = false;
-  int device = 0;
+  int device = 0, n_sms = 0;
   size_t esz = 2;
   int gemm_path = 0;
   bool chain_launches = true;
@@ -199,10 +199,11 @@ int check_config(const cmoe_config& c) {
   return CMOE_OK;
 }
 
-int check_device() {
-  int dev = 0, major = 0;
-  CU_TRY(cudaGetDevice(&dev));
-  CU_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+int check_device(int* dev, int* n_sms) {
+  int major = 0;
+  CU_TRY(cudaGetDevice(dev));
+  CU_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, *dev));
+  CU_TRY(cudaDeviceGetAttribute(n_sms, cudaDevAttrMultiProcessorCount, *dev));
   if (major != 10) return arg_fail(CMOE_ERR_UNSUPPORTED, "device is not compute capability 10.x");
   return CMOE_OK;
 }
@@ -451,10 +452,11 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   if (n_r > 0) {
     const int warps = (R + 1) / 2, blocks = (warps + 7) / 8;
     const int32_t* ooff = L->hier ? L->outer_off : nullptr;
-    // fp32: a warp per row while that leaves SMs idle (4 warps on each), two rows per warp beyond
+    // fp32: a warp per row while an SM has at most four of them, two rows per warp beyond
+    const bool row_warps = R <= 4 * L->n_sms;
 #define CMOE_ROUTER(NACC)                                                                                  \
-  launch_kernel(dep, R <= 592 ? router_row_kernel<T, NACC> : router_kernel<T, NACC>,           \
-                dim3(R <= 592 ? (R + 3) / 4 : blocks), dim3(R <= 592 ? 128 : 256), 0, st, xo, R, d, n_r, L->n_rp, n_k,  \
+  launch_kernel(dep, row_warps ? router_row_kernel<T, NACC> : router_kernel<T, NACC>,           \
+                dim3(row_warps ? (R + 3) / 4 : blocks), dim3(row_warps ? 128 : 256), 0, st, xo, R, d, n_r, L->n_rp, n_k,  \
                 (const T*)L->w_rep, (const float*)L->u, (const float*)L->b, ooff, L->n_outer, L->scores, L->keys,       \
                 L->topk_idx, L->topk_gate)
     if constexpr (std::is_same<T, bf16>::value) {
@@ -511,7 +513,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   // SIMT path: small tiles (which gather their rows themselves) while 64 x 64 tiles would not give every SM a few
   const long long simt_tiles = (long long)((R + kSimtTile - 1) / kSimtTile) * ((L->shared_width() + kSimtTile - 1) / kSimtTile) +
                                ((long long)P / kSimtTile + G) * ((L->m + kSimtTile - 1) / kSimtTile);
-  const bool simt_small = !use_umma && simt_tiles <= 4 * 148;
+  const bool simt_small = !use_umma && simt_tiles <= 4 * L->n_sms;
   if (P > 0 && !use_umma && !simt_small) {
     gather_rows_kernel<<<P, 256, 0, st>>>((const uint4*)xo, L->row_token, P, row_vec, (uint4*)L->x_perm);
     ++launches;
@@ -621,8 +623,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     const int th = (d / 16 + 31) / 32 * 32;
     if (!L->hier && d % 16 == 0 && th <= 1024 && n_k <= 4 && n_tok > 64) {
       fast_combine = true;
-      const int sms = L->umma.n_sms > 0 ? L->umma.n_sms : 148;
-      const int grid = std::min(n_tok, sms * std::max(1, 1024 / th) * 2);
+      const int grid = std::min(n_tok, L->n_sms * std::max(1, 1024 / th) * 2);
       const bf16* ys = L->cfg.n_shared > 0 ? (const bf16*)L->y_s : nullptr;
       if (n_k <= 1)
         launch_kernel(dep, combine_plain_bf16_kernel<1>, dim3(grid), dim3(th), 0, st, ys, (const bf16*)L->y_r, L->topk_gate, L->row_of, n_tok, n_k, d, (bf16*)out);
@@ -676,14 +677,15 @@ int cmoe_layer_create(const cmoe_config* cfg, const void* w_gate, const void* w_
         return arg_fail(CMOE_ERR_BAD_REP, "representative outside its routed expert's slice");
     }
   }
-  rc = check_device();
+  int dev = 0, n_sms = 0;
+  rc = check_device(&dev, &n_sms);
   if (rc != CMOE_OK) return rc;
 
   cmoe_layer* L = new (std::nothrow) cmoe_layer();
   if (!L) return arg_fail(CMOE_ERR_INVALID_ARG, "out of host memory");
   L->cfg = *cfg; L->m = m; L->n_r = n_r; L->n_rp = (n_r + 7) / 8 * 8; L->n_outer = 1; L->outer_k = 1; L->hier = false;
   L->esz = cfg->dtype == CMOE_BF16 ? 2 : 4;
-  cudaGetDevice(&L->device);
+  L->device = dev; L->n_sms = n_sms;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int32_t *perm_dev = nullptr, *rep_dev = nullptr;       // rep_dev: one word more, set if W_down is not finite
   int32_t non_finite = 0;
@@ -744,14 +746,15 @@ int cmoe_hier_create(int32_t n_outer, int32_t outer_top_k, const void* w_router,
     for (int k = 0; k < i; ++k)
       if (inner[k] == inner[i]) return arg_fail(CMOE_ERR_INVALID_ARG, "inner layer listed twice");
   }
-  int rc = check_device();
+  int dev = 0, n_sms = 0;
+  int rc = check_device(&dev, &n_sms);
   if (rc != CMOE_OK) return rc;
   cmoe_layer* L = new (std::nothrow) cmoe_layer();
   if (!L) return arg_fail(CMOE_ERR_INVALID_ARG, "out of host memory");
   L->cfg = inner[0]->cfg; L->cfg.max_tokens = max_tokens;
   L->m = inner[0]->m; L->n_r = inner[0]->n_r; L->n_rp = inner[0]->n_rp; L->esz = inner[0]->esz;
   L->n_outer = n_outer; L->outer_k = outer_top_k; L->hier = true;
-  cudaGetDevice(&L->device);
+  L->device = dev; L->n_sms = n_sms;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t d = L->cfg.d_model, d_ff = L->cfg.d_ff, nr = L->n_r, esz = L->esz;
   const size_t wbytes = d_ff * d * esz, rep_bytes = 2 * (size_t)L->n_rp * d * esz;
