@@ -4,7 +4,7 @@ resident while the preceding layer's last kernel still runs."""
 import numpy as np
 import pytest
 
-from paper_2502_04416_b200 import workloads as wl
+from paper_2502_04416_b200 import binding, workloads as wl
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -36,6 +36,49 @@ def test_layer_stack_matches_synchronised_calls(dtype, fp8, tokens):
                                                        (32, 4, 4, 48, 300), (32, 4, 4, 48, 700)])
 def test_layer_stack_shared_tiles(n, n_shared, top_k, m, tokens):
     _check_stack(*_stack("bf16", False, tokens, m=m, n=n, n_shared=n_shared, top_k=top_k), "bf16")
+
+
+# under a top-level router: rows copied by the inner router (up to 1024 outer rows), by a launch of their own, both routers on
+# tiles; FP8 planes made from the copied rows
+@pytest.mark.parametrize("fp8,tokens", [(False, 7), (False, 300), (False, 700), (False, 1100), (True, 7), (True, 30)])
+def test_hierarchical_stack(fp8, tokens):
+    shape = wl.LayerShape(512, 176 * 8, 8, 2, 2, "bf16")
+    rng = np.random.Generator(np.random.PCG64(5))
+    layers = []
+    for _ in range(3):
+        inners = []
+        for _ in range(4):
+            lay = wl.draw_layer(rng, shape)
+            for w in (lay.w_gate, lay.w_up, lay.w_down):
+                w *= 2.0
+            inners.append(parity.gpu_layer(lay, 8))
+        w_router = wl.round_to_storage(rng.normal(scale=0.02, size=(4, 512)).astype(np.float32), "bf16")
+        layers.append(binding.Layer.create_hier(parity.to_device(w_router, "bf16"), inners, 2, tokens))
+        if fp8:
+            layers[-1].quantise_fp8()
+    _check_stack(layers, wl.draw_tokens(rng, tokens, shape), "bf16")
+
+
+# batches of all kinds in turn on one layer: the streamers' down kernel, which lets its successor start at once, followed by kernels
+# that allocate tensor memory ahead of their wait, and the other way round
+@pytest.mark.parametrize("fp8", [False, True])
+def test_mixed_batches_back_to_back(fp8):
+    import torch
+    (layer,), x = _stack("bf16", fp8, 2300, n_layers=1)
+    xd = parity.to_device(x, "bf16")
+    sizes = (64, 1100, 16, 2300, 64, 300, 48, 700, 1, 1100, 33, 100, 64, 2300)
+    starts = [(97 * i) % (2300 - t + 1) for i, t in enumerate(sizes)]
+    want = []
+    for t, a in zip(sizes, starts):
+        want.append(layer.forward(xd[a:a + t]).clone())
+        torch.cuda.synchronize()
+    for _ in range(5):
+        got = [layer.forward(xd[a:a + t]) for t, a in zip(sizes, starts)]
+        torch.cuda.synchronize()
+        for g, w in zip(got, want):
+            assert torch.equal(g, w)
+    assert layer.status() == 0
+    layer.destroy()
 
 
 def _check_stack(layers, x, dtype):

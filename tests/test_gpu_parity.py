@@ -179,25 +179,31 @@ def test_call_contract():
 
 
 def test_forward_host_matches_device_forward():
-    """cmoe_ffn_forward_host (chunked, copies overlapped on side streams) against the device-buffer
-    call: a token's result does not depend on what else is in its batch (Eq. moe_output is per x), so
-    chunks processed by the same kernel family give the same bits; a ragged last chunk, a single
-    chunk and pageable host memory are covered."""
+    """cmoe_ffn_forward_host (chunked, copies overlapped on side streams) against the device-buffer call on each chunk:
+    the same kernels on the same rows, so the same bits; a ragged last chunk, a single chunk and pageable host memory
+    are covered.  (A batch and its chunks may take different router forms, whose sums differ in the last bit.)"""
     import torch
     inp = _inputs("c2_llama2_7b", d_model=256, tokens=(2900,), m=160)
     lay = inp.layers[0]
     layer = parity.gpu_layer(lay, 2900)
     x = parity.to_device(inp.x, "bf16")
-    ref = layer.forward(x).cpu()
-    torch.cuda.synchronize()
+
+    def chunks(rows, n):
+        ref = torch.cat([layer.forward(x[t:min(t + n, rows)]) for t in range(0, rows, n)]).cpu()
+        torch.cuda.synchronize()
+        return ref
+
     x_pin = x.cpu().pin_memory()
     out_pin = torch.empty_like(x_pin).pin_memory()
-    for chunk in (1024, 700, 0, 2900, 5000):
+    for chunk, rows in ((1024, 1024), (700, 700), (0, 512), (2900, 2900), (5000, 2900)):
+        ref = chunks(2900, rows)
         out_pin.zero_()
         layer.forward_host(x_pin, out_pin, chunk)
         torch.cuda.synchronize()
         assert layer.status() == 0
         assert torch.equal(out_pin.view(torch.int16), ref.view(torch.int16)), chunk
+        parity.check_output(parity.to_host(out_pin), oracle.cmoe_layer_forward(inp.x, **parity.oracle_kwargs(lay))[0])
+    ref = chunks(2900, 1024)
     for _ in range(3):                                  # back-to-back calls reuse the staging buffers
         layer.forward_host(x_pin, out_pin, 1024)
     torch.cuda.synchronize()
@@ -205,8 +211,7 @@ def test_forward_host_matches_device_forward():
     x_page, out_page = x.cpu(), torch.zeros_like(ref)   # pageable memory: serial copies, same result
     layer.forward_host(x_page[:1500], out_page[:1500], 600)
     torch.cuda.synchronize()
-    assert torch.equal(out_page[:1500].view(torch.int16), ref[:1500].view(torch.int16))
-    parity.check_output(parity.to_host(out_pin), oracle.cmoe_layer_forward(inp.x, **parity.oracle_kwargs(lay))[0])
+    assert torch.equal(out_page[:1500].view(torch.int16), chunks(1500, 600).view(torch.int16))
     layer.destroy()
 
 
@@ -276,13 +281,14 @@ def test_launch_chaining_is_bit_identical():
 
 
 def test_launch_chaining_hierarchical_is_bit_identical():
-    """The same for a layer under a top-level router (Section 4.4): the kernels after the expert router are chained."""
+    """The same for a layer under a top-level router (Section 4.4), whose kernels are all chained: rows copied by the inner
+    router, by a launch of their own (over 1024 outer rows), and both routers on tiles (over 1024 tokens)."""
     import torch
-    inp = _inputs("c4_hier_8x7b", d_model=256, tokens=(300,), m=224)
+    inp = _inputs("c4_hier_8x7b", d_model=256, tokens=(1100,), m=224)
     inners = [parity.gpu_layer(lay, 8) for lay in inp.layers]
-    layer = binding.Layer.create_hier(parity.to_device(inp.w_router, "bf16"), inners, 2, 300)
+    layer = binding.Layer.create_hier(parity.to_device(inp.w_router, "bf16"), inners, 2, 1100)
     x = parity.to_device(inp.x, "bf16")
-    for t in (3, 20, 50, 100, 300):
+    for t in (3, 20, 50, 100, 300, 700, 1100):
         layer.set_launch_chaining(False)
         ref = layer.forward(x[:t]).clone()
         layer.set_launch_chaining(True)
