@@ -260,15 +260,14 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
  * 2 and 3 return CMOE_ERR_INVALID_ARG if the layer cannot take the tensor-core path. */
 int cmoe_layer_set_gemm_path(cmoe_layer* layer, int32_t path);
 
-/* Launch chaining (on by default): on the bf16 tensor-core path every kernel of a forward
- * (of a plain layer: from the expert router on for up to 1024 rows, after it for more; of a
- * hierarchical one: after it) is launched as a programmatic dependent of its predecessor, so it
- * may become resident (and fetch what does not depend on the predecessor) while the
- * predecessor drains, and waits on the device before touching anything the predecessor
- * produces.  Results are bit-identical either way; 0 restores ordinary stream-ordered
- * launches.  Has no effect while per-stage timing is enabled, and the
- * prologue of a hierarchical layer (top-level router, its permutation, the row copy) always
- * uses ordinary launches.  Error: INVALID_ARG (null layer). */
+/* Launch chaining (on by default): the kernels of a forward, the first one and the prologue of a hierarchical
+ * layer (top-level router, its permutation, the row copy) included, are launched as programmatic dependents of
+ * their predecessors in the stream: a kernel may become resident (and fetch the layer's own weights, or what an
+ * earlier kernel has completed) while its predecessor drains, and waits on the device before touching anything
+ * the predecessor produces.  Ordinary launches remain for the top-level router of fp32 layers and, on the
+ * SIMT path, for the bf16 routers of batches above 1024 rows and for the row gather of large tiles.
+ * Results are bit-identical either way; 0 restores ordinary stream-ordered launches throughout.  Has no
+ * effect while per-stage timing is enabled.  Error: INVALID_ARG (null layer). */
 int cmoe_layer_set_launch_chaining(cmoe_layer* layer, int32_t on);
 
 /* Sizes a caller needs to read the routing state back.  n_outer / outer_top_k

@@ -430,7 +430,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
            gemv_plan((int)R, L->n_outer, L->n_groups_total(), n_k, n_r, d, L->shared_width(), L->m, L->cfg.n_shared > 0,
                      L->fp8, &gemv_ring);
   // Two to 64 rows of a plain bf16 layer: the weight streamers that end in the layer's output (automatic path only).  From 65
-  // rows on a token's bits do not depend on the batch size, which the folded gates of the streamers would break.
+  // rows on the expert GEMMs and the combine give a token the same bits in every batch for equal gates, which the folded gates
+  // of the streamers would break.  (The router forms add their sums in different orders: gates may differ in the last bit.)
   const bool stream = use_umma && !gemv && L->gemm_path == 0 && L->stream.built && L->fp8 == L->stream.fp8 &&
                       R <= kStreamMaxRows;
   // Weights-on-M streaming kernels: up to 64 rows; the wide form takes up to 128 rows, on the bf16 weights also where the
