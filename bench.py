@@ -164,18 +164,15 @@ def prepare_inputs(name: str):
     return inputs
 
 
-# DRAM bytes (read + write) per forward of the dominant kernels (the two expert GEMMs), from the ncu
+# DRAM bytes (read + write) per forward of the dominant kernels (the expert GEMMs), from the ncu
 # captures summarised under profiles/; an entry is only valid for the kernel version it was taken on,
 # so the table is emptied whenever those kernels change and refilled from a new capture.
 NCU_TRAFFIC = {
-    ("c5_skew_13b", 16384): {"bytes": (1586.5 + 162.8 + 363.8 + 795.8) * 1e6,
-                             "source": "profiles/umma2_pair_gemm_c5_skew_13b.md"},
-    ("c2_llama2_7b", 4096): {"bytes": (282.2 + 34.5 + 138.5 + 68.2) * 1e6,
-                             "source": "profiles/launch_lists_c2_c3_c4_prefill_and_mid_size.md"},
-    ("c3_llama3_8b", 8192): {"bytes": (517.0 + 52.0 + 182.0 + 281.5) * 1e6,
-                             "source": "profiles/launch_lists_c2_c3_c4_prefill_and_mid_size.md"},
-    ("c4_hier_8x7b", 4096): {"bytes": (2038.5 + 111.7 + 1064.4 + 184.3) * 1e6,
-                             "source": "profiles/launch_lists_c2_c3_c4_prefill_and_mid_size.md"},
+    ("c5_skew_13b", 16384): {"bytes": (1585.1 + 164.5 + 249.1 + 628.4 + 884.5 + 151.9) * 1e6,
+                             "source": "profiles/launch_lists.md"},
+    ("c2_llama2_7b", 4096): {"bytes": (280.4 + 36.0 + 90.2 + 34.2 + 126.3 + 15.8) * 1e6, "source": "profiles/launch_lists.md"},
+    ("c3_llama3_8b", 8192): {"bytes": (509.3 + 52.7 + 132.2 + 214.5 + 357.7 + 50.9) * 1e6, "source": "profiles/launch_lists.md"},
+    ("c4_hier_8x7b", 4096): {"bytes": (2038.8 + 112.6 + 1060.0 + 184.3) * 1e6, "source": "profiles/launch_lists.md"},
 }
 
 # Every (workload, T) point the metric is quoted on; the last one (the largest single-GPU
@@ -188,6 +185,22 @@ SWEEP_POINTS_FP8 = [("c2_llama2_7b", 1), ("c2_llama2_7b", 16), ("c2_llama2_7b", 
 # between the decode and the prefill regime (not points of the metric: reported beside the sweep)
 MID_POINTS = [("c2_llama2_7b", 128), ("c2_llama2_7b", 256), ("c2_llama2_7b", 1024),
               ("c3_llama3_8b", 128), ("c3_llama3_8b", 256), ("c3_llama3_8b", 512), ("c3_llama3_8b", 1024)]
+
+
+def rounded(o):
+    """Floats to six significant digits: the line stays short enough to be kept whole by whoever reads its tail."""
+    if isinstance(o, float):
+        return float(f"{o:.6g}")
+    if isinstance(o, dict):
+        return {k: rounded(v) for k, v in o.items()}
+    return [rounded(v) for v in o] if isinstance(o, list) else o
+
+
+def point_summary(recs):
+    """One entry per measured point: [ms per step, fraction of its roofline, speedup over the dense FFN or null]."""
+    return {f"{r['workload'].split('_')[0]}{'_fp8' if r['expert_weights'].startswith('fp8') else ''}:{r['tokens']}":
+            [float(f"{r['ms_per_step']:.4g}"), round(r["roofline"]["whole_step_frac"], 3),
+             round(r["speedup_vs_dense"], 2) if r.get("speedup_vs_dense") else None] for r in recs}
 
 
 def traffic_note(name, tokens, use_graph):
@@ -349,8 +362,7 @@ def roofline_record(peaks, w, T, touched, step_ms, first_ms, gemm_ms, stage_ms, 
                 "frac": ach / peaks["hbm_gbs"]}
         t_roof, t_sus = t_hbm, t_hbm
     roof.update({
-        "kernel": ("expert GEMMs (gate/up + SwiGLU, down), timed by per-stage events in a separate short loop"
-                   if not use_graph else "whole forward, all kernels (CUDA graph replay; no per-stage events)"),
+        "kernel": "expert GEMMs (stage events)" if not use_graph else "whole forward (graph replay)",
         "kernel_ms": gemm_ms, "peak_source": peaks["source"], "traffic": traffic_note(w.name, T, use_graph),
         "algorithmic_flops": flops, "algorithmic_bytes": alg_bytes,
         "whole_step_frac": t_roof / (step_ms * 1e-3),                    # median block, against the burst peak
@@ -549,23 +561,24 @@ def run_gpu(args):
                    "tokens_per_step": T, "parallelism": "replicas only" if world > 1 else "single GPU",
                    "l2": "weights (%.0f MB) exceed the 126 MB L2" % (w_bytes / 1e6),
                    "launch": head["launch"],
-                   "timing": "the K-step block is repeated until the timed region reaches %.1f s; ms_per_step is "
-                             "the median block / K, first_block_ms_per_step the first" % args.min_region_s},
+                   "timing": "median of K-step blocks over at least %.1f s" % args.min_region_s},
         "first_block_ms_per_step": head["first_block_ms_per_step"], "blocks": head["blocks"],
         "timed_region_s": head["timed_region_s"],
         "e2e": {"value": world * T / (e2e_ms * 1e-3), "unit": UNIT,
                 "h2d_bytes_per_step": io_bytes, "d2h_bytes_per_step": io_bytes,
-                "call": "cmoe_ffn_forward_host: pinned host x and out, chunks double-buffered on two copy streams",
+                "call": "cmoe_ffn_forward_host, pinned buffers",
                 "chunk_tokens": args.e2e_chunk or "auto", "ms_per_step": e2e_ms,
                 "bit_identical_to_device_call": same},
-        "gpu_launches": launches, "clocks": head["clocks"], "roofline": roof, "cpu_baseline": cpu,
+        "gpu_launches": launches, "clocks": head["clocks"], "cpu_baseline": cpu,
+        "roofline": {k: v for k, v in roof.items() if k not in ("other_bound_frac", "algorithmic_flops", "algorithmic_bytes")},
         "dense_cublas": head["dense_cublas"], "speedup_vs_dense": head.get("speedup_vs_dense"),
     }
     if sweep is not None:
-        line["sweep"] = sweep
-        line["mid_size"] = mid
+        # every point in full on stderr; the line itself carries one short entry per point
+        print(json.dumps({"points": rounded(sweep + mid)}), file=sys.stderr)
+        line["points"] = point_summary(sweep + mid)
     rig.close()
-    return line
+    return rounded(line)
 
 
 def run_ranks(args):
@@ -834,8 +847,8 @@ def main():
                     help="expert-GEMM implementation (cmoe_layer_set_gemm_path); 0 = the library's choice")
     ap.add_argument("--fp8", action="store_true", help="quantise the expert weights to FP8 (cmoe_layer_quantise_fp8) first")
     ap.add_argument("--sweep", choices=["auto", "on", "off"], default="auto",
-                    help="add one record per (workload, T) point of the metric to the JSON line "
-                         "(auto: on for the default single-GPU headline run)")
+                    help="measure every (workload, T) point of the metric as well: a short entry each in the JSON "
+                         "line, the full records on stderr (auto: on for the default single-GPU headline run)")
     ap.add_argument("--min-region-s", type=float, default=1.0,
                     help="the K-step block is repeated until the timed region is at least this long")
     ap.add_argument("--sweep-region-s", type=float, default=0.4)
