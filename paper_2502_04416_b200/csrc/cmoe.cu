@@ -435,8 +435,9 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   const bool stream = use_umma && !gemv && L->gemm_path == 0 && L->stream.built && L->fp8 == L->stream.fp8 &&
                       R <= kStreamMaxRows;
   // Weights-on-M streaming kernels: up to 64 rows; the wide form takes up to 128 rows, on the bf16 weights also where the
-  // layer holds FP8 codes (their token planes stop at 64 rows; 7B-shaped layer with FP8 weights, 100 rows: 83.2 ->
-  // 75.6 us against token-major tiles, 13B-shaped 138.8 -> 101.8).  Path 2 keeps token-major tiles from 65 rows.
+  // layer holds FP8 codes (their token planes stop at 64 rows).  Path 2 keeps token-major tiles from 65 rows, which run nearly as
+  // fast since their shared tiles need no routing: 7B-shaped 65 / 100 / 128 rows 70.6 / 72.4 / 75.0 against 74.3 / 73.7 / 74.2 us, 13B-shaped
+  // 100 / 128 rows 98.7 / 102.2 against 98.5 / 98.4, 8B-shaped 128 rows 93.0 against 86.6, hierarchical 33 tokens 415 against 424.
   const int decode_rows = L->gemm_path != 2 ? kDecWideRows : kDecMaxRows;
   const bool decode = use_umma && !gemv && !stream && R <= decode_rows;
   if (use_umma && !stream && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);

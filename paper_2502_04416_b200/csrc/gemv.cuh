@@ -15,10 +15,9 @@
 //       are one launch and Y never reaches memory.
 // FP8 = true streams the E4M3 codes of a quantised layer (one byte per weight) and multiplies the
 // sums by the per-row power-of-two scales; the token rows stay bf16.
-// The kernels are written for TT rows and instantiated for one: measured on 7B-, 8B- and 13B-shaped
-// layers, two rows already run faster on the tensor-core streamers (61 vs 64, 55 vs 60, 64 vs 80 us),
-// one row is faster here (40.4 vs 54.3, 37.8 vs 45.3, 50.7 vs 59.6 us per forward; with FP8 weights
-// 35.0 vs 43.2, 35.0 vs 43.2, 45.6 vs 48.1).
+// The kernels are written for TT rows and instantiated for one: two rows already run faster on the tensor-core
+// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 34.0 vs 41.9,
+// 28.4 vs 30.5, 43.8 vs 48.5 us per forward; with FP8 weights 25.3 vs 28.7, 24.7 vs 30.1, 36.4 vs 34.9).
 #pragma once
 
 #include "common.cuh"

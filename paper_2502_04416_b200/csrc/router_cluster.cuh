@@ -9,13 +9,11 @@
 //   - rank 0 collects the selections the same way and, with one row tile, permutes at once; with more, the tile that
 //     takes the last ticket permutes the batch: per group a bit mask of its rows, population counts for ranks and counts.
 // A hierarchical layer runs it twice, for the outer experts and for the inner ones; the second pass reads every outer row
-// from its token and writes the layer's copy of the rows as it goes.  Against a block per 16 tokens for the first, a permutation
-// and a copy kernel, all four unchained: 7 / 128 / 700 tokens of the 8 x 7B-shaped layer 288.8 / 512.4 / 594.2 -> 266.8 /
-// 491.7 / 575.9 us.
-// Against K slices over independent blocks (partial sums and a ticket through global memory, the last block alone
-// doing the gate logic and a block-wide scan; the permutation in kernels of its own above 128 rows), whole forwards: 7B-shaped
-// layer 1 / 16 / 64 / 128 / 512 rows 40.5 / 67.4 / 74.1 / 86.9 / 114.0 -> 35.0 / 62.1 / 69.1 / 80.0 / 109.3 us, 8B-shaped 32 /
-// 256 / 512 rows 88.2 / 112.3 / 140.9 -> 80.7 / 102.0 / 121.8, hierarchical 7 rows 295 -> 278.  Where tensor-core tiles take over: router_takes_tiles.
+// from its token and writes the layer's copy of the rows as it goes (8 x 7B-shaped layer, 7 / 128 / 700 tokens, against a block per 16
+// tokens, a permutation and a copy kernel: 288.8 / 512.4 / 594.2 -> 266.8 / 491.7 / 575.9 us).  Against K slices over independent blocks
+// that met in global memory, the last block alone doing the gate logic: 7B-shaped layer 1 / 16 / 64 rows 40.5 / 67.4 / 74.1 -> 35.0 /
+// 62.1 / 69.1 us.  Alone and with cold caches a launch takes 9 us at 16 and 11 at 300 rows.  Where tensor-core tiles take over:
+// router_takes_tiles.
 #pragma once
 
 #include "common.cuh"

@@ -9,10 +9,9 @@
 //     from its peers' shared memory and runs their gate logic, one warp per row;
 //   - with the selections it writes, per 32 rows and expert, the bit mask of the rows that chose the expert.
 // The permutation is then one launch over those masks (population counts; the whole batch's masks are a few ten KB).
-// Whole forwards against tiles of 128 rows by one to four CTAs with partial sums and tickets in global memory, a gate stage of one
-// thread per row and a permutation in two launches: 8B-shaped 2048 / 4000 rows 241.8 / 376.8 -> 217.8 / 366.8 us, 7B-shaped 2048
-// rows 269.3 -> 261.3, 8 x 7B-shaped hierarchical layer 1500 / 4096 tokens 745.5 / 1450 -> 696.5 / 1425 us.  Of the 18.5 us from the
-// start to the GEMM at 2048 rows (32 before), the contraction takes 5, the sums of the cluster 3, the gates 3, the permutation 5.
+// Against 128-row tiles of one to four CTAs with partial sums and tickets in global memory, a gate stage of one thread per row and a
+// permutation in two launches: 8B-shaped 2048 rows 241.8 -> 217.8 us, 7B-shaped 269.3 -> 261.3.  Of the 18.5 us from the start to the
+// GEMM at 2048 rows of the 8B-shaped layer the contraction takes 5, the sums of the cluster 3, the gates 3, the permutation 5.
 #pragma once
 
 #include "permute.cuh"
@@ -360,10 +359,10 @@ permute_words_kernel(const uint32_t* __restrict__ words, const int32_t* __restri
 }
 
 // ----------------------------------------------------------------------------- host
-// Rows from which this router is the better one (below: router_cluster_kernel, whose 16-row tiles each read all
-// representative rows).  More than 16 columns, cluster / tile: 8B-shaped 500 / 600 / 700 / 850 rows 110.9 / 126.6 / 126.5 / 132.8
-// against 111.9 / 120.2 / 121.7 / 127.3 us, 13B-shaped 600 / 1024 rows 174.2 / 221.6 against 169.3 / 216.6; 16 columns: 7B-shaped 500 / 700
-// / 850 / 1000 rows 102.6 / 115.3 / 142.2 / 164.4 against 106.6 / 121.9 / 148.9 / 156.9.  Outer rows: the clustered router copies them as well.
+// Rows from which this router is the better one (below: router_cluster_kernel, whose 16-row tiles each read all representative
+// rows).  Whole forwards with either router, cluster / tiles: more than 16 columns, 8B-shaped 500 / 600 / 700 / 850 rows 103 / 115 / 111 /
+// 129 against 103 / 108 / 103 / 119 us, 13B-shaped 600 rows 154 against 149; 16 columns, 7B-shaped 500 / 700 / 850 / 1000 rows 91 / 108 / 133 / 158
+// against 89 / 108 / 135 / 147: even up to 850.  Outer rows: the clustered router copies them as well.
 inline bool router_takes_tiles(int n_rows, int n_rp, bool hier) { return n_rows > (!hier && n_rp > 8 ? 512 : kRcMaxRows); }
 
 inline cudaError_t router_tile_allow() {

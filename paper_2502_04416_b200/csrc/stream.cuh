@@ -30,14 +30,14 @@
 // whose trip count is not fixed are not unrolled: the weight streams push the code out of L2 between two forwards, and
 // every line of it that a short kernel needs is a miss to DRAM.
 //
-// Measured against the kernels of umma_decode.cuh followed by the combine kernel (chained forwards): 7B-shaped layer 2 / 8 /
-// 16 / 32 / 64 rows 51.4 / 58.4 / 60.6 / 63.4 / 67.7 -> 48.2 / 52.6 / 53.3 / 56.6 / 62.1 us, 8B-shaped 4 / 32 / 64 rows 52.3 /
-// 77.8 / 82.6 -> 48.6 / 71.0 / 77.9, 13B-shaped 16 / 64 rows 79.4 / 97.4 -> 72.9 / 87.6.  In a forward of 16 rows (270 MB of
-// weights, 41 us at the copy rate) the up kernel streams for 31 us from its start under the router, its slowest CTA and the
-// hand-over cost 4, the down kernel streams for 13 and its sums take 4.  A single row stays on the CUDA-core kernels of
-// gemv.cuh (33.7 us against 46).  FP8 weights: 7B-shaped 2 / 16 / 48 / 64 rows 44.4 / 48.6 / 56.0 / 58.1 -> 38.0 / 39.2 / 46.9 /
-// 49.8 us, 8B-shaped 8 / 32 / 64 rows 52.1 / 62.6 / 68.6 -> 47.8 / 50.2 / 56.5, 13B-shaped 16 / 48 rows 61.9 / 75.1 -> 49.6 / 58.5.  Fetching the down kernel's weights into L2 at the end of the up kernel was slower (it
-// delays the up kernel's last CTAs), equal runs of k blocks instead of tiles in the up kernel as well (the partial sums).
+// Against the kernels of umma_decode.cuh followed by the combine kernel (cmoe_layer_set_gemm_path 0 / 2, chained forwards): 7B-shaped layer
+// 2 / 16 / 64 rows 50.8 / 53.9 / 63.1 against 52.1 / 58.4 / 64.8 us, 8B-shaped 4 / 32 / 64 rows 48.5 / 69.5 / 75.3 against 51.8 / 78.7 / 81.5,
+// 13B-shaped 16 / 64 rows 76.5 / 88.8 against 87.2 / 94.3; FP8 weights, 7B-shaped 2 / 16 / 48 rows 36.8 / 38.8 / 47.0 against 37.8 / 45.6 /
+// 58.6, 8B-shaped 8 / 32 / 64 rows 44.2 / 50.6 / 58.9 against 50.0 / 69.2 / 83.0, 13B-shaped 16 / 48 rows 52.5 / 60.7 against 64.4 / 83.2.
+// In a forward of 16 rows of the 7B-shaped layer (270 MB of weights, 42 us at the copy rate) the up kernel streams for 31 us from its start
+// under the router, its slowest CTA and the hand-over cost 4, the down kernel streams for 13 and its sums take 4.  A single row stays on the
+// CUDA-core kernels of gemv.cuh (34 us against 46).  Fetching the down kernel's weights into L2 at the end of the up kernel was slower
+// (it delays the up kernel's last CTAs), equal runs of k blocks instead of tiles in the up kernel as well (the partial sums).
 #pragma once
 
 #include <cmath>

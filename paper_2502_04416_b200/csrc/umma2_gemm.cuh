@@ -571,12 +571,13 @@ inline double umma_busiest(int n_s, double c_s, int n_r, double c_r, int n_slots
 // n_routed groups (even load assumed).  Both are persistent kernels whose tiles are dealt round-robin.
 //   Below kPairLargeRows: a few rounds, so what counts for gate/up is the busiest SM.  Per 64-wide k block a 128 x 256 tile
 // takes 425 ns on a single CTA (the operands' round trip through four stages) and a 256 x 256 tile 320 ns on a pair
-// (on-device timelines, 7B-shaped layer, 512 rows).  Single against pairs: 7B-shaped 300 / 512 / 1000 rows 78 / 124 / 173
-// against 98 / 110 / 159 us, 8B-shaped 300 / 700 / 1000 rows 116 / 132 / 171 against 104 / 141 / 164.  The load is taken
-// once as expected and once with a fifth more tiles, for skewed routing.  The down GEMM stays on single CTAs (8B-shaped
-// 300 rows 104 against 118 us, hierarchical 300 rows 545 against 614, 7B-shaped 512 rows 110 against 108).
+// (on-device timelines, 7B-shaped layer, 512 rows).  The load is taken once as expected and once with a fifth more tiles, for skewed
+// routing.  The down GEMM stays on single CTAs.  Whole forwards with both GEMMs on single CTAs / on pairs / as chosen here
+// (cmoe_layer_set_gemm_path 2 / 3 / 0): 7B-shaped 300 / 512 / 1000 rows 79 / 108 / 164, 88 / 98 / 167, 80 / 102 / 162 us, 8B-shaped 300 / 700 /
+// 1000 rows 105 / 111 / 155, 111 / 133 / 149, 103 / 112 / 144, 13B-shaped 600 rows 163, 145, 153, hierarchical 300 tokens 530, 650, 530.
 //   From there on the part runs at its power limit and padding costs energy: pairs when rounding the groups up to an
-// even number of 128-row tiles adds at most 3 % (gate/up) or 8 % (down, not for K extents of a few k blocks).
+// even number of 128-row tiles adds at most 3 % (gate/up) or 8 % (down, not for K extents of a few k blocks).  7B-shaped 2048 / 4096 rows
+// 280 / 503, 259 / 489, 268 / 499, 8B-shaped 8192 rows 762, 718, 720, 13B-shaped 4096 / 16384 rows 682 / 2633, 627 / 2336, 626 / 2355 us.
 constexpr int kPairLargeRows = 2048;
 inline int umma_pick_pairs(const UmmaPlan* P, int pair_grid, int R, int n_sel, int n_routed, int gemm_path) {
   if (gemm_path == 2 || R < kPairMinRows) return 0;

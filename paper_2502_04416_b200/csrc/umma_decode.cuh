@@ -1,4 +1,4 @@
-// Decode-shaped expert GEMMs (at most 64 rows per group): the contraction is turned
+// Decode-shaped expert GEMMs (at most 64 rows per group, 128 in the wide bf16 form): the contraction is turned
 // around so that the WEIGHTS sit on the 128-row M side of the tcgen05 MMA and the few
 // tokens on the N side (N = row count rounded up to 16).  The tensor-core time per
 // 64-wide k block is then a few dozen cycles instead of the 512 a 128-row token tile
@@ -30,8 +30,8 @@
 // lo = 16 x the remainder, after a per-row power-of-two scale; a bf16 number has 8 significant
 // bits and each plane carries 4, so hi + lo/16 is the value itself (exactly, down to 2^-13 of the
 // row's largest magnitude).  A stage covers 128 k (128 bytes per weight row, the same TMA box
-// geometry as the bf16 tiles), each k step issues one MMA per (weight plane, token plane) into
-// its own accumulator columns, and the epilogue forms (hi + lo/16) x row scale x token scale.
+// geometry as the bf16 tiles), each k step issues one MMA per weight plane over both token planes
+// (side by side in the accumulator), and the epilogue forms (hi + lo/16) x row scale x token scale.
 #pragma once
 
 #include "fp8.cuh"

@@ -335,10 +335,9 @@ umma_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_con
   // Warp 2 counts the tiles of every group and publishes the table on a barrier; in mode 1 it waits for the router and the
   // permutation first, in mode 2 the preceding kernel has read the same rows already.  Tiles that need no table, those of the shared
   // experts of a plain layer (group 0, all rows of x), run at once, under the routing and this kernel's own start-up.
-  // Mode 2 fetches the weights of its first stages under the end of the gate/up GEMM.  Against a wait at the top and a table that all
-  // threads count and one sums (3.7 us from the permutation's end to the first operands of a tile, 3.3 from the gate/up GEMM's): 8B-shaped 300 / 500 / 700 /
-  // 2048 rows 102.0 / 112.5 / 125.1 / 231 -> 94.4 / 107.9 / 112.6 / 213 us, 7B-shaped 200 / 300 / 500 rows 75.5 / 79.2 / 109.5 -> 71.4 /
-  // 75.5 / 102.7, 13B-shaped 300 / 600 rows 128.0 / 171.4 -> 113.2 / 162.0.
+  // Mode 2 fetches the weights of its first stages under the end of the gate/up GEMM.  (With a wait at the top and a table that all
+  // threads count and one sums, 3.7 us passed from the permutation's end to the first operands of a tile, 3.3 from the gate/up GEMM's:
+  // 8B-shaped 300 / 2048 rows 102.0 / 231 -> 94.4 / 213 us, 7B-shaped 300 rows 79.2 -> 75.5, 13B-shaped 128.0 -> 113.2.)
   const int early_n = MODE == 3 ? (p.d + 255) / 256 : MODE == 1 && p.early_rows > 0 ? (p.shared_width + p.bn_s - 1) / p.bn_s : 0;
   const int early_tiles = (p.early_rows + kUmmaBM - 1) / kUmmaBM * early_n;
   if (MODE == 3) {
@@ -842,11 +841,11 @@ inline UmmaArgs umma_base_args(const UmmaPlan* P, const GroupRows* gr, int32_t* 
 // written nor read back, and the routed rows are read under its multiplies.  Bound by the epilogue's gathers (a thread reads
 // 32-byte pieces of n_k rows), which a tile's multiplies must cover, and by the last round of tiles, which no routed tiles fill up any
 // more: taken when the SMs' idle time in that round (425 ns per 64-wide k block) is at most a third of the combine's own time (3 us and
-// the rows at 5.5 TB/s).  Without / with: 8B-shaped 700 rows 100.5 / 106.4 us and 1400 rows 155.6 / 159.1 (not taken), 1000 / 2048 / 8192
-// rows 136.3 / 208.5 / 693 against 131.3 / 204.3 / 644, 7B-shaped 300 / 2500 rows 74.0 / 293 against 78.4 / 300 (not taken), 4000 / 8000 rows 445 /
-// 889 against 443 / 857, 13B-shaped 4096 / 16384 rows 568 / 2295 against 562 / 2286.  Fetching the routed rows of the next columns ahead
-// (233 registers) is slower: 8B-shaped 2048 / 8192 rows 213 / 667.  Eight epilogue warps instead of four, each with half of the columns: 8B-shaped
-// 2048 rows 205.5 / 198.7, 7B-shaped 2048 rows 229.4 / 227.4, 13B-shaped 16384 rows 2269 / 2252, even at 8192.
+// the rows at 5.5 TB/s).  With / without, both forced: 8B-shaped 700 rows 106 / 101 us, 7B-shaped 300 rows 79.0 / 76.4, 13B-shaped 300 rows
+// 105 / 99 (not taken), 8B-shaped 1400 and 7B-shaped 2500 rows even (not taken), 8B-shaped 1000 / 2048 / 8192 rows 131 / 221 / 716 against
+// 143 / 229 / 738, 7B-shaped 4000 / 8000 rows 500 / 946 against 513 / 979, 13B-shaped 4096 / 16384 rows 615 / 2310 against 640 / 2397.
+// Eight epilogue warps, each with half of the columns, keep twice the gathers of four in flight (8B-shaped 2048 rows 205.5 -> 198.7 us);
+// fetching the routed rows of the next columns ahead as well (233 registers) was slower.
 inline bool umma_folds_combine(const UmmaPlan* P, int R, int n_k, int d) {
   if (!P->has_s || !P->has_r || n_k < 1 || n_k > 4 || d % 16 != 0) return false;
   const int tiles = (R + kUmmaBM - 1) / kUmmaBM * ((d + 255) / 256), over = tiles % P->n_sms;
