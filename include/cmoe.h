@@ -246,9 +246,8 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
 
 /* Choose the expert-GEMM implementation: 0 = automatic (tensor-core path when the
  * dtype is bf16 and the shape allows, else the plain SIMT path; for batches of at least 256
- * rows each of the two GEMMs may run on CTA pairs: the gate/up GEMM below 2048 rows when the expected tiles
- * keep the busiest SM for less time that way, both from 2048 rows on when the
- * padding of the expert groups to 256-row tiles is expected to stay small; batches of 65 to 128 rows stream the bf16 weights through the
+ * rows each of the two GEMMs may run on CTA pairs, where that is expected to take less time or, from 2048 rows on, to multiply
+ * less padding; batches of 65 to 128 rows stream the bf16 weights through the
  * decode-shaped kernels, weights on the MMA's M side; 2 to 64 rows of a plain layer
  * run on two weight streamers with the gates folded into the hidden activations (rounded to bf16 once, after the
  * gate) and the sum over the experts inside the down projection (a layer with an Inf or NaN in a routed expert's W_down

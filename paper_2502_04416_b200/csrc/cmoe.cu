@@ -26,6 +26,7 @@
 #include "router_mma.cuh"
 #include "simt_gemm.cuh"
 #include "umma2_gemm.cuh"
+#include "umma2t_gemm.cuh"
 #include "umma_decode.cuh"
 #include "gemv.cuh"
 #include "stream.cuh"
@@ -114,6 +115,7 @@ struct cmoe_layer {
   UmmaPlan umma;
   DecodePlan decode;
   Umma2Plan pair;
+  Umma2tPlan turned;
   StreamPlan stream;
   int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
   uint32_t *rt_words = nullptr, *rt_words_outer = nullptr;     // tcgen05 routers: row masks per expert
@@ -326,6 +328,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
     if (L->umma_ok && L->down_finite && stream_shape_ok(s, L->umma.n_sms) && !stream_plan_create(&L->umma, &L->stream))
       return arg_fail(CMOE_ERR_CUDA, L->umma.error);
     if (L->umma_ok && !umma2_plan_create(&L->umma, &L->pair)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
+    if (L->umma_ok && !umma2t_plan_create(&L->umma, &L->turned)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   }
   CU_TRY(cudaStreamSynchronize(st));
   return CMOE_OK;
@@ -510,8 +513,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     ++launches;
   }
   // The tensor path gathers routed rows inside the gate/up GEMM; only large SIMT tiles read a permuted copy of x.
-  const int pair_mask = use_umma && !gemv && !stream && !decode
-      ? umma_pick_pairs(&L->umma, L->pair.grid, R, P, G, L->gemm_path) : 0;
+  const GemmForms forms = use_umma && !gemv && !stream && !decode
+      ? umma_pick_forms(&L->umma, L->pair.grid, R, P, G, L->gemm_path) : GemmForms();
   // SIMT path: small tiles (which gather their rows themselves) while 64 x 64 tiles would not give every SM a few
   const long long simt_tiles = (long long)((R + kSimtTile - 1) / kSimtTile) * ((L->shared_width() + kSimtTile - 1) / kSimtTile) +
                                ((long long)P / kSimtTile + G) * ((L->m + kSimtTile - 1) / kSimtTile);
@@ -575,9 +578,12 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
       n = 0;
       for (int bit = 1; bit <= 2 && n >= 0; bit <<= 1) {          // gate/up, then down, each on its chosen tile shape
         if (!(todo & bit)) continue;
-        const int k = (pair_mask & bit)
-            ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R, fold_out != nullptr)
-            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, L->hier ? 0 : R, fold_out != nullptr);
+        const GemmForm form = bit == 1 ? forms.gate_up : forms.down;
+        const int early = L->hier ? 0 : R;
+        const int k = form == GemmForm::kTurned
+            ? umma2t_forward(&L->umma, &L->turned, L->pair.grid, &L->decode, L->gr, xo, R, L->err_word, st, mid, dep, bit, early, fold_out != nullptr)
+            : form == GemmForm::kPair ? umma2_forward(&L->umma, &L->pair, L->gr, xo, L->err_word, st, mid, dep, early)
+            : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, early, fold_out != nullptr);
         n = k < 0 ? -1 : n + k;
       }
     }

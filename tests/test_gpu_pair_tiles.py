@@ -1,0 +1,51 @@
+"""-m gpu: expert GEMMs on CTA pairs with weights on M and tokens on N, at the edges of their tiles."""
+import numpy as np
+import pytest
+
+from paper_2502_04416_b200 import binding, workloads as wl
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+# token tiles: one group below, at and above 256 rows, equal tiles with a shorter last one; columns in steps of 32.  Neurons: fewer than
+# one tile, halves of 8 and 56 neurons per CTA, a last tile that ends early; d: k and output channels that fill no block.
+CASES = [
+    (256, 24, (256, 257, 300, 511, 513)),
+    (328, 200, (287, 1030)),
+    (1032, 448, (1000,)),
+    (512, 384, (2049, 4100)),
+]
+
+
+@pytest.mark.parametrize("skew", [0.0, 1.0], ids=["even", "skewed"])
+@pytest.mark.parametrize("d,m,tokens", CASES, ids=[f"d{c[0]}-m{c[1]}" for c in CASES])
+def test_pair_tiles(d, m, tokens, skew):
+    shape = wl.LayerShape(d, m * 8, 8, 2, 2, "bf16")
+    inp = wl.make_inputs(wl.Workload("pair_tiles", shape, tokens, seed=11))
+    lay = inp.layers[0]
+    # skewed: one expert takes every row, others a handful or none
+    lay.select_bias_b = (skew * np.array([2.0, 0.3, 0.0, -0.3, -2.0, 0.1])).astype(np.float32)
+    lay.gate_scale_u = np.random.default_rng(2).normal(scale=0.5, size=6).astype(np.float32)
+    layer = parity.gpu_layer(lay, max(tokens))
+    layer.set_gemm_path(binding.GEMM_TENSOR_PAIRS)
+    for t in tokens:
+        st = parity.check_plain_layer(layer, lay, inp.x[:t])
+        assert st["differing"] <= st["near_tie"]
+    assert layer.status() == 0
+    layer.destroy()
+
+
+# The tiles change which rows are multiplied together, not the sums of one output: same bits as single-CTA tiles.
+@pytest.mark.parametrize("tokens", [256, 700, 1111])
+def test_pair_tiles_have_the_bits_of_single_tiles(tokens):
+    import torch
+    shape = wl.LayerShape(512, 200 * 8, 8, 2, 2, "bf16")
+    inp = wl.make_inputs(wl.Workload("pair_bits", shape, (tokens,), seed=5))
+    layer = parity.gpu_layer(inp.layers[0], tokens)
+    x = parity.to_device(inp.x, "bf16")
+    got = []
+    for path in (binding.GEMM_TENSOR, binding.GEMM_TENSOR_PAIRS):
+        layer.set_gemm_path(path)
+        got.append(layer.forward(x).view(torch.int16).clone())
+    assert torch.equal(*got)
+    layer.destroy()
