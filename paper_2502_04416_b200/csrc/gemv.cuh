@@ -12,11 +12,14 @@
 //       (Eq. moe_output) one warp per pair of output channels, over all active groups in group
 //       order, each group's products times its row's gate (lane-level sums, one warp reduction per
 //       channel at the end); fp32, one rounding: the down projection and the gate-weighted combine
-//       are one launch and Y never reaches memory.
+//       are one launch and Y never reaches memory.  Up to 4736 channels (148 SMs) two warps share a pair: with one, 4096 channels
+//       are 256 blocks, two on some SMs and one on others, and 57 KB in flight per SM.  The shared expert's rows are fetched into L2
+//       while the gate/up kernel's last blocks run (its blocks fill the register files, so these come in one by one as they end).
+//       Both together: 7B-shaped layer 33.75 -> 30.83 us.
 // FP8 = true streams the E4M3 codes of a quantised layer (one byte per weight) and multiplies the
 // sums by the per-row power-of-two scales; the token rows stay bf16.
 // The kernels are written for TT rows and instantiated for one: two rows already run faster on the tensor-core
-// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 34.0 vs 41.9,
+// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 30.8 vs 41.9,
 // 28.4 vs 30.5, 43.8 vs 48.5 us per forward; with FP8 weights 25.3 vs 28.7, 24.7 vs 30.1, 36.4 vs 34.9).
 #pragma once
 
@@ -244,19 +247,27 @@ gemv_gate_up_kernel(const GemvArgs p) {
   }
 }
 
-template <int TT, bool FP8>
+// KS: warps that share a pair of channels, each with every KS-th run of 32 chunks of every group; their sums meet in shared memory.
+template <int TT, bool FP8, int KS>
 __global__ void __launch_bounds__(kGemvThreads, 4)
 gemv_down_combine_kernel(const GemvArgs p) {
-  constexpr int CH = kGemvCH, esz = FP8 ? 1 : 2;
+  constexpr int CH = kGemvCH, esz = FP8 ? 1 : 2, kTeams = kGemvWarps / KS;
   __shared__ GemvGroups<TT> L;
+  __shared__ float part[KS > 1 ? kTeams : 1][KS][CH][TT];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ks = warp % KS, team = warp / KS;
+  const int n_warps = gridDim.x * kTeams, gw = blockIdx.x * kTeams + team;
+  // The shared expert's weights of the first channels need nothing from the gate/up kernel: into L2, while its last blocks run.
+  const GroupStatic g0 = p.gs[0];
+  if (ks == 0 && lane == 0 && g0.is_shared && g0.width > 0 && gw * CH < p.d)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                 ::"l"((const char*)p.w_down + ((size_t)g0.wd_offset + (size_t)gw * CH * g0.width) * esz), "r"(CH * g0.width * esz));
   grid_dep_wait();
   grid_dep_trigger();
   gemv_list_groups(p, L);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_warps = gridDim.x * kGemvWarps, gw = blockIdx.x * kGemvWarps + warp;
   // One pass = CH output channels; per active group one partial dot product per (channel, row), reduced over
   // the warp and added, times the row's gate, to its token's sum.
-  for (int c0 = gw * CH; c0 < p.d; c0 += n_warps * CH) {
+  for (int c0 = gw * CH; KS > 1 ? c0 == gw * CH : c0 < p.d; c0 += n_warps * CH) {
     float out_acc[CH][TT];
 #pragma unroll
     for (int h = 0; h < CH; ++h)
@@ -279,7 +290,7 @@ gemv_down_combine_kernel(const GemvArgs p) {
 #pragma unroll
         for (int j = 0; j < TT; ++j) acc[h][j] = 0.0f;
 #pragma unroll 4
-      for (int c = lane; c < chunks; c += 32) {
+      for (int c = lane + 32 * ks; c < chunks; c += 32 * KS) {
         GemvChunk<FP8> cw[CH];
 #pragma unroll
         for (int h = 0; h < CH; ++h) cw[h].load(w0 + (size_t)h * width * esz, c);    // rows c0 + h (d is even)
@@ -314,8 +325,19 @@ gemv_down_combine_kernel(const GemvArgs p) {
 #pragma unroll
       for (int tt = 0; tt < TT; ++tt) {
         const float y = warp_sum(out_acc[h][tt]);
-        if (lane == 0 && tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
+        if (KS > 1) { if (lane == 0) part[team][ks][h][tt] = y; }
+        else if (lane == 0 && tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
       }
+    if constexpr (KS > 1) {                     // d % 8 = 0: the grid's teams are exactly the pairs of channels, one pass each
+      __syncthreads();
+      if (ks == 0 && lane < CH * TT) {
+        const int h = lane / TT, tt = lane % TT;
+        float y = part[team][0][h][tt];
+#pragma unroll
+        for (int q = 1; q < KS; ++q) y += part[team][q][h][tt];
+        if (tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
+      }
+    }
   }
 }
 
@@ -339,12 +361,14 @@ inline int gemv_forward(const GemvArgs& a, const GemvPlan& plan, bool fp8, int n
   // down + combine: a warp takes kGemvCH channels per pass; as many passes as four blocks per SM need, evenly filled
   const int warps = 4 * n_sms * kGemvWarps, pairs = a.d / kGemvCH;
   const int passes = (pairs + warps - 1) / warps;
-  const dim3 grid2(((pairs + passes - 1) / passes + kGemvWarps - 1) / kGemvWarps);
+  const bool two = 2 * pairs <= warps;               // two warps per pair of channels
+  const dim3 grid2(two ? 2 * pairs / kGemvWarps : ((pairs + passes - 1) / passes + kGemvWarps - 1) / kGemvWarps);
 #define CMOE_GEMV(TT, F8)                                                                                          \
   do {                                                                                                             \
     launch_kernel(dep, gemv_gate_up_kernel<TT, F8>, grid1, block, 0, st, a);                                       \
     if (mid) cudaEventRecord(mid, st);                                                                             \
-    if (!gate_up_only) launch_kernel(dep, gemv_down_combine_kernel<TT, F8>, grid2, block, 0, st, a);               \
+    if (!gate_up_only)                                                                                             \
+      launch_kernel(dep, two ? gemv_down_combine_kernel<TT, F8, 2> : gemv_down_combine_kernel<TT, F8, 1>, grid2, block, 0, st, a); \
   } while (0)
   if (fp8) CMOE_GEMV(1, true); else CMOE_GEMV(1, false);
 #undef CMOE_GEMV
