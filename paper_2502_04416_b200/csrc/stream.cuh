@@ -35,7 +35,9 @@
 // 13B-shaped 16 / 64 rows 76.5 / 88.8 against 87.2 / 94.3; FP8 weights, 7B-shaped 2 / 16 / 48 rows 36.8 / 38.8 / 47.0 against 37.8 / 45.6 /
 // 58.6, 8B-shaped 8 / 32 / 64 rows 44.2 / 50.6 / 58.9 against 50.0 / 69.2 / 83.0, 13B-shaped 16 / 48 rows 52.5 / 60.7 against 64.4 / 83.2.
 // In a forward of 16 rows of the 7B-shaped layer (270 MB of weights, 42 us at the copy rate) the up kernel streams for 31 us from its start
-// under the router, its slowest CTA and the hand-over cost 4, the down kernel streams for 13 and its sums take 4.  A single row stays on the
+// under the router, its slowest CTA and the hand-over cost 4, the down kernel streams for 13 and its sums take 3.  (The sums are one chain of latencies: stores,
+// release, ticket, loads.  With a fence per lane beside lane 0's release and six of seven contributions in flight 16 rows took 56.1
+// instead of 55.4 us, 8B-shaped 32 rows 69.8 instead of 69.3.)  A single row stays on the
 // CUDA-core kernels of gemv.cuh (34 us against 46).  Fetching the down kernel's weights into L2 at the end of the up kernel was slower
 // (it delays the up kernel's last CTAs), equal runs of k blocks instead of tiles in the up kernel as well (the partial sums).
 #pragma once
@@ -502,6 +504,7 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
     const int quad = warp & 3, half = (warp - 2) >> 2;              // 8-column chunks half, half + 2, ...
     const int slot_q = quad * 32 + lane;
     constexpr int kCh = NT / 16;                                    // this warp's chunks: columns 16 i + 8 half
+    constexpr int kSum = W8 && NT == 64 ? 6 : 7;                    // contributions in flight: 4096 channels on 148 SMs have 6 or 7 (registers)
     float* tok_sc = reinterpret_cast<float*>(tail + 1024) + 32 * (warp - 2);
     grid_dep_wait();                                                // also orders this kernel's stores to `out`
     bool ok = true;
@@ -581,30 +584,29 @@ stream_down_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_cons
           __stcg(mine + (size_t)(4 * i) * 128, make_float4(v[i][0], v[i][1], v[i][2], v[i][3]));
           __stcg(mine + (size_t)(4 * i + 1) * 128, make_float4(v[i][4], v[i][5], v[i][6], v[i][7]));
         }
-      __threadfence();
-      __syncwarp();
+      __syncwarp();                                                 // the lanes' stores are ordered before lane 0's release
       int taken = 0;
       if (lane == 0) taken = atom_inc_acq_rel(tk);
       taken = __shfl_sync(0xffffffffu, taken, 0);
       if (taken != nz - 1) continue;
-      __threadfence();                                              // every contribution is in: add them in CTA order
+      __syncwarp();                                                 // lane 0's acquire for all: every contribution is in, add them in CTA order
 #pragma unroll 1
       for (int c0 = 8 * half; c0 < p.n_rows; c0 += 16) {
         float r[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) r[q] = 0.0f;
 #pragma unroll 1
-        for (int z0 = 0; z0 < nz; z0 += 6) {                        // six in flight
-          float4 t[6][2];
+        for (int z0 = 0; z0 < nz; z0 += kSum) {
+          float4 t[kSum][2];
 #pragma unroll
-          for (int z = 0; z < 6; ++z)
+          for (int z = 0; z < kSum; ++z)
             if (z0 + z < nz) {
               const float4* sl = slot(z0 + z) + (size_t)(c0 / 4) * 128;
               t[z][0] = __ldcg(sl);
               t[z][1] = __ldcg(sl + 128);
             }
 #pragma unroll
-          for (int z = 0; z < 6; ++z)
+          for (int z = 0; z < kSum; ++z)
             if (z0 + z < nz) {
               r[0] += t[z][0].x; r[1] += t[z][0].y; r[2] += t[z][0].z; r[3] += t[z][0].w;
               r[4] += t[z][1].x; r[5] += t[z][1].y; r[6] += t[z][1].z; r[7] += t[z][1].w;
