@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -25,6 +26,7 @@
 #include "router_tile.cuh"
 #include "router_mma.cuh"
 #include "simt_gemm.cuh"
+#include "small_fp32.cuh"
 #include "umma2_gemm.cuh"
 #include "umma2t_gemm.cuh"
 #include "umma_decode.cuh"
@@ -117,6 +119,7 @@ struct cmoe_layer {
   Umma2Plan pair;
   Umma2tPlan turned;
   StreamPlan stream;
+  float* small_h = nullptr;            // fp32 layers of a few rows: H of all experts
   int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
   uint32_t *rt_words = nullptr, *rt_words_outer = nullptr;     // tcgen05 routers: row masks per expert
   float* dec_part = nullptr;    // decode GEMMs: K-slice partial sums, tickets per (tile, epilogue warp)
@@ -274,6 +277,10 @@ void carve_workspace(cmoe_layer* L, char* base) {
     L->stream.h = a.take<bf16>((size_t)kStreamMaxRows * L->cfg.d_ff);
     L->stream.part = a.take<float>(stream_part_floats((int)T));
   }
+  if (esz == 4 && !L->hier) {
+    const int rows = small_fp32_rows((int)std::min<size_t>(T, kSmMaxRows), (int)d, L->cfg.d_ff, L->shared_width(), L->m, L->n_r, L->cfg.top_k);
+    if (rows > 0) L->small_h = a.take<float>((size_t)rows * L->cfg.d_ff);
+  }
   if (esz == 2 && nr > 0) {
     L->rt_words = a.take<uint32_t>(router_tile_words((int)R, (int)nr, L->n_outer));
   }
@@ -306,6 +313,7 @@ int finish_layer(cmoe_layer* L, cudaStream_t st) {
                          cudaMemcpyHostToDevice, st));
   int rc = alloc_workspace(L);
   if (rc != CMOE_OK) return rc;
+  if (L->small_h) CU_TRY(small_fp32_allow());
   L->umma_ok = false;
   if (L->cfg.dtype == CMOE_BF16) {
     UmmaShape s;
@@ -499,6 +507,21 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
 #undef CMOE_ROUTER
     ++launches;
     if (!marked) mark(1);
+    if constexpr (std::is_same<T, float>::value)
+      if (L->small_h && R <= small_fp32_rows(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k)) {
+        SmallArgs a{};
+        a.x = xo; a.w_gate = (const float*)L->wg_p; a.w_up = (const float*)L->wu_p; a.w_down = (const float*)L->wd_p;
+        a.h = L->small_h; a.out = out; a.topk_idx = L->topk_idx; a.topk_gate = L->topk_gate;
+        a.n_rows = R; a.d = d; a.d_ff = L->cfg.d_ff; a.shared_w = L->shared_width(); a.m = L->m; a.n_r = n_r; a.n_k = n_k;
+        a.perm = PermuteOut{R, n_k, G, L->counts, L->offsets, L->row_token, L->row_of, po};
+        mark(2);
+        CU_TRY(small_fp32_forward(a, dep, st, ev ? ev[3] : nullptr));
+        mark(4);
+        mark(5);
+        if (ev) ++L->ev_count;
+        L->launches = launches + 2;
+        return CMOE_OK;
+      }
     if (!perm_fused)
       launches += launch_token_permute(L->topk_idx, R, n_k, G, L->counts, L->offsets, L->row_token,
                                        L->row_of, L->perm_scratch, st, po, dep);

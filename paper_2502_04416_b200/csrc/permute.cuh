@@ -216,11 +216,7 @@ __device__ __forceinline__ void permute_by_masks(const PermuteOut& p, uint8_t* s
 
 
 // The same for selections that have been written already.
-__global__ void __launch_bounds__(kMaskThreads)
-permute_masks_kernel(const int32_t* __restrict__ topk_idx, const PermuteOut p) {
-  grid_dep_wait();
-  grid_dep_trigger();
-  __shared__ __align__(16) uint8_t scratch[kMaskBytes];
+__device__ __forceinline__ void permute_from_selections(const int32_t* topk_idx, const PermuteOut& p, uint8_t* scratch) {
   const int pairs = p.n_rows * p.n_k;
 #pragma unroll 1
   for (int i0 = threadIdx.x; i0 < pairs; i0 += 4 * kMaskThreads) {
@@ -234,6 +230,13 @@ permute_masks_kernel(const int32_t* __restrict__ topk_idx, const PermuteOut p) {
   }
   __syncthreads();
   permute_by_masks(p, scratch);
+}
+__global__ void __launch_bounds__(kMaskThreads)
+permute_masks_kernel(const int32_t* __restrict__ topk_idx, const PermuteOut p) {
+  grid_dep_wait();
+  grid_dep_trigger();
+  __shared__ __align__(16) uint8_t scratch[kMaskBytes];
+  permute_from_selections(topk_idx, p, scratch);
 }
 
 // n_rows <= kPermChunk: histogram, scan and scatter in one block.
