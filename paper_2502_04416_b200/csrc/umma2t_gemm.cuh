@@ -263,7 +263,7 @@ umma2t_grouped_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_c
       }
     }
   } else if (MODE == 1 && warp == 10) {
-    // ------------------------------------------------------------ relay (gate/up, both CTAs): see umma2_grouped_kernel
+    // ------------------------------------------------------------ relay (gate/up, both CTAs): see umma2_gate_up_kernel
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
