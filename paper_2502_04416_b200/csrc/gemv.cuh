@@ -9,18 +9,20 @@
 //       one warp per neuron of an active group, both weight rows at once; the rows r are the
 //       group's rows (shared group: every token; routed group: the tokens that selected it).
 //   gemv_down_combine_kernel:  out[t, c] = Y_s[t, c] + sum_j g[t, j] Y_{e_j}[t, c],  Y_e[t, c] = W_down^e[c] . H_e[t]
-//       (Eq. moe_output) one warp per pair of output channels, over all active groups in group
-//       order, each group's products times its row's gate (lane-level sums, one warp reduction per
-//       channel at the end); fp32, one rounding: the down projection and the gate-weighted combine
-//       are one launch and Y never reaches memory.  Up to 4736 channels (148 SMs) two warps share a pair: with one, 4096 channels
-//       are 256 blocks, two on some SMs and one on others, and 57 KB in flight per SM.  The shared expert's rows are fetched into L2
-//       while the gate/up kernel's last blocks run (its blocks fill the register files, so these come in one by one as they end).
-//       Both together: 7B-shaped layer 33.75 -> 30.83 us.
+//       (Eq. moe_output) one warp per output channel, over all active groups in group order, each group's products times its
+//       row's gate (lane-level sums, one warp reduction per channel at the end); fp32, one rounding: the down projection and
+//       the gate-weighted combine are one launch and Y never reaches memory.  A warp takes two channels where there are more
+//       channels than warps fit on the chip (4736 on 148 SMs); with two everywhere, 4096 channels are 256 blocks, two on some
+//       SMs and one on others.  Bound by the latency of its rounds of loads: with the loads of a round issued together, the
+//       last, partly filled ones too, instead of an unrolled loop with a serial remainder, one row of the 7B- / 8B- / 13B-shaped layer
+//       takes 30.7 / 26.9 / 37.7 us (two channels per warp, serial remainder: 33.2 / 29.5 / 43.0), with FP8 weights 25.2 / 24.3 / 31.8
+//       (26.9 / 27.1 / 37.7).  Two to six loads per lane and round: 31.9 / 30.6 / 30.7 / 30.8 us for 2 / 3 / 4 / 6 (7B-shaped), 34.7 / 34.8 /
+//       33.1 / 35.3 (4608 channels).  The rows of the shared expert fetched into L2 ahead of the wait: even (+-0.3 us).
 // FP8 = true streams the E4M3 codes of a quantised layer (one byte per weight) and multiplies the
 // sums by the per-row power-of-two scales; the token rows stay bf16.
 // The kernels are written for TT rows and instantiated for one: two rows already run faster on the tensor-core
-// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 30.8 vs 41.9,
-// 28.4 vs 30.5, 43.8 vs 48.5 us per forward; with FP8 weights 25.3 vs 28.7, 24.7 vs 30.1, 36.4 vs 34.9).
+// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 30.7 vs 41.9,
+// 26.9 vs 30.5, 37.7 vs 48.5 us per forward; with FP8 weights 25.2 vs 28.7, 24.3 vs 30.1, 31.8 vs 34.9).
 #pragma once
 
 #include "common.cuh"
@@ -32,7 +34,8 @@ constexpr int kGemvMaxRows = 1;
 constexpr int kGemvThreads = 256;
 constexpr int kGemvWarps = kGemvThreads / 32;
 constexpr int kGemvMaxGroups = 64;         // group tables in shared memory
-constexpr int kGemvCH = 2;                 // output channels per warp pass of the down kernel
+constexpr int kGemvCH = 2;                 // output channels per warp pass of the down kernel where there are too many for a warp each
+constexpr int kGemvDepth = 4;              // 16-byte (8-byte: codes) loads per lane, channel and round of the down kernel
 
 struct GemvArgs {
   const GroupStatic* gs;
@@ -64,19 +67,24 @@ __device__ __forceinline__ uint2 ld_stream8(const void* p) {
   return r;
 }
 
+// Eight bf16 values as floats.
+__device__ __forceinline__ void unpack8(const uint4& raw, float (&v)[8]) {
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { v[2 * i] = __uint_as_float(w[i] << 16); v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+}
+
 // Eight weights of one row chunk: bf16 (16 bytes) or E4M3 codes (8 bytes); as floats after unpack.
 template <bool FP8> struct GemvChunk;
 template <> struct GemvChunk<false> {
   uint4 raw;
+  __device__ __forceinline__ void clear() { raw = make_uint4(0u, 0u, 0u, 0u); }
   __device__ __forceinline__ void load(const void* chunk0, int chunk) { raw = ld_stream16((const uint4*)chunk0 + chunk); }
-  __device__ __forceinline__ void unpack(float (&w)[8]) const {
-    const uint32_t v[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { w[2 * i] = __uint_as_float(v[i] << 16); w[2 * i + 1] = __uint_as_float(v[i] & 0xffff0000u); }
-  }
+  __device__ __forceinline__ void unpack(float (&w)[8]) const { unpack8(raw, w); }
 };
 template <> struct GemvChunk<true> {
   uint2 raw;
+  __device__ __forceinline__ void clear() { raw = make_uint2(0u, 0u); }
   __device__ __forceinline__ void load(const void* chunk0, int chunk) { raw = ld_stream8((const uint2*)chunk0 + chunk); }
   __device__ __forceinline__ void unpack(float (&w)[8]) const {
     const uint32_t v[2] = {raw.x, raw.y};
@@ -247,27 +255,21 @@ gemv_gate_up_kernel(const GemvArgs p) {
   }
 }
 
-// KS: warps that share a pair of channels, each with every KS-th run of 32 chunks of every group; their sums meet in shared memory.
-template <int TT, bool FP8, int KS>
+// CH: output channels per warp pass.  A channel's products are added by one warp in one order whatever CH is, so a layer's width does
+// not show in the bits.
+template <int TT, bool FP8, int CH>
 __global__ void __launch_bounds__(kGemvThreads, 4)
 gemv_down_combine_kernel(const GemvArgs p) {
-  constexpr int CH = kGemvCH, esz = FP8 ? 1 : 2, kTeams = kGemvWarps / KS;
+  constexpr int esz = FP8 ? 1 : 2;
   __shared__ GemvGroups<TT> L;
-  __shared__ float part[KS > 1 ? kTeams : 1][KS][CH][TT];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ks = warp % KS, team = warp / KS;
-  const int n_warps = gridDim.x * kTeams, gw = blockIdx.x * kTeams + team;
-  // The shared expert's weights of the first channels need nothing from the gate/up kernel: into L2, while its last blocks run.
-  const GroupStatic g0 = p.gs[0];
-  if (ks == 0 && lane == 0 && g0.is_shared && g0.width > 0 && gw * CH < p.d)
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
-                 ::"l"((const char*)p.w_down + ((size_t)g0.wd_offset + (size_t)gw * CH * g0.width) * esz), "r"(CH * g0.width * esz));
+  const int n_warps = gridDim.x * kGemvWarps, gw = blockIdx.x * kGemvWarps + warp;
   grid_dep_wait();
   grid_dep_trigger();
   gemv_list_groups(p, L);
   // One pass = CH output channels; per active group one partial dot product per (channel, row), reduced over
   // the warp and added, times the row's gate, to its token's sum.
-  for (int c0 = gw * CH; KS > 1 ? c0 == gw * CH : c0 < p.d; c0 += n_warps * CH) {
+  for (int c0 = gw * CH; c0 < p.d; c0 += n_warps * CH) {
     float out_acc[CH][TT];
 #pragma unroll
     for (int h = 0; h < CH; ++h)
@@ -289,22 +291,41 @@ gemv_down_combine_kernel(const GemvArgs p) {
       for (int h = 0; h < CH; ++h)
 #pragma unroll
         for (int j = 0; j < TT; ++j) acc[h][j] = 0.0f;
-#pragma unroll 4
-      for (int c = lane + 32 * ks; c < chunks; c += 32 * KS) {
-        GemvChunk<FP8> cw[CH];
+#pragma unroll 1
+      for (int k0 = 0; k0 < chunks; k0 += 32 * kGemvDepth) {
+        // every load of a round is on its way before the first product: past the end of the row zeros, whose products change no sum
+        GemvChunk<FP8> cw[kGemvDepth][CH];
+        uint4 hv[kGemvDepth][TT];
 #pragma unroll
-        for (int h = 0; h < CH; ++h) cw[h].load(w0 + (size_t)h * width * esz, c);    // rows c0 + h (d is even)
-        float hv[TT][8];
+        for (int i = 0; i < kGemvDepth; ++i) {
+          const int c = k0 + 32 * i + lane;
+          const bool in = c < chunks;
 #pragma unroll
-        for (int j = 0; j < TT; ++j) load8(hr[j] + 8 * c, hv[j]);
+          for (int h = 0; h < CH; ++h) {                       // rows c0 + h (d % CH = 0)
+            cw[i][h].clear();
+            if (in) cw[i][h].load(w0 + (size_t)h * width * esz, c);
+          }
 #pragma unroll
-        for (int h = 0; h < CH; ++h) {
-          float fw[8];
-          cw[h].unpack(fw);
+          for (int j = 0; j < TT; ++j) {
+            hv[i][j] = make_uint4(0u, 0u, 0u, 0u);
+            if (in) hv[i][j] = ld_dep16(hr[j] + 8 * c);
+          }
+        }
 #pragma unroll
-          for (int j = 0; j < TT; ++j)
+        for (int i = 0; i < kGemvDepth; ++i) {
+          if (i > 0 && k0 + 32 * i >= chunks) break;           // the whole warp
+          float hf[TT][8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[h][j] = fmaf(fw[q], hv[j][q], acc[h][j]);
+          for (int j = 0; j < TT; ++j) unpack8(hv[i][j], hf[j]);
+#pragma unroll
+          for (int h = 0; h < CH; ++h) {
+            float fw[8];
+            cw[i][h].unpack(fw);
+#pragma unroll
+            for (int j = 0; j < TT; ++j)
+#pragma unroll
+              for (int q = 0; q < 8; ++q) acc[h][j] = fmaf(fw[q], hf[j][q], acc[h][j]);
+          }
         }
       }
 #pragma unroll
@@ -325,19 +346,8 @@ gemv_down_combine_kernel(const GemvArgs p) {
 #pragma unroll
       for (int tt = 0; tt < TT; ++tt) {
         const float y = warp_sum(out_acc[h][tt]);
-        if (KS > 1) { if (lane == 0) part[team][ks][h][tt] = y; }
-        else if (lane == 0 && tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
+        if (lane == 0 && tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
       }
-    if constexpr (KS > 1) {                     // d % 8 = 0: the grid's teams are exactly the pairs of channels, one pass each
-      __syncthreads();
-      if (ks == 0 && lane < CH * TT) {
-        const int h = lane / TT, tt = lane % TT;
-        float y = part[team][0][h][tt];
-#pragma unroll
-        for (int q = 1; q < KS; ++q) y += part[team][q][h][tt];
-        if (tt < p.n_rows) p.out[(size_t)tt * p.d + c0 + h] = __float2bfloat16_rn(y);
-      }
-    }
   }
 }
 
@@ -358,17 +368,17 @@ inline int gemv_forward(const GemvArgs& a, const GemvPlan& plan, bool fp8, int n
                         bool dep, bool gate_up_only) {
   const dim3 block(kGemvThreads);
   const dim3 grid1(4 * n_sms);
-  // down + combine: a warp takes kGemvCH channels per pass; as many passes as four blocks per SM need, evenly filled
+  // down + combine: a warp takes one channel, or kGemvCH per pass; as many passes as four blocks per SM need, evenly filled
   const int warps = 4 * n_sms * kGemvWarps, pairs = a.d / kGemvCH;
   const int passes = (pairs + warps - 1) / warps;
-  const bool two = 2 * pairs <= warps;               // two warps per pair of channels
-  const dim3 grid2(two ? 2 * pairs / kGemvWarps : ((pairs + passes - 1) / passes + kGemvWarps - 1) / kGemvWarps);
+  const bool single = a.d <= warps;                  // a warp per channel
+  const dim3 grid2(((single ? a.d : (pairs + passes - 1) / passes) + kGemvWarps - 1) / kGemvWarps);
 #define CMOE_GEMV(TT, F8)                                                                                          \
   do {                                                                                                             \
     launch_kernel(dep, gemv_gate_up_kernel<TT, F8>, grid1, block, 0, st, a);                                       \
     if (mid) cudaEventRecord(mid, st);                                                                             \
     if (!gate_up_only)                                                                                             \
-      launch_kernel(dep, two ? gemv_down_combine_kernel<TT, F8, 2> : gemv_down_combine_kernel<TT, F8, 1>, grid2, block, 0, st, a); \
+      launch_kernel(dep, single ? gemv_down_combine_kernel<TT, F8, 1> : gemv_down_combine_kernel<TT, F8, kGemvCH>, grid2, block, 0, st, a); \
   } while (0)
   if (fp8) CMOE_GEMV(1, true); else CMOE_GEMV(1, false);
 #undef CMOE_GEMV
