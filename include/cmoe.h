@@ -253,7 +253,8 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
  * gate) and the sum over the experts inside the down projection (a layer with an Inf or NaN in a routed expert's W_down
  * stays on the decode-shaped kernels there, where such a weight reaches only the tokens that selected the expert); a single row of a plain layer
  * runs on the CUDA cores with plain-load weight streams, down projection and combine in one
- * launch), 1 = always SIMT, 2 = tensor-core with
+ * launch; up to 256 rows of a plain fp32 layer may run on three launches that multiply every expert, where that is expected
+ * to take less time), 1 = always SIMT, per-expert products over permuted rows, 2 = tensor-core with
  * single-CTA token-major tiles only (decode-shaped kernels up to 64 rows), 3 = tensor-core on CTA
  * pairs (cta_group::2) for batches of at least 256 rows;
  * 2 and 3 return CMOE_ERR_INVALID_ARG if the layer cannot take the tensor-core path. */

@@ -508,7 +508,8 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     ++launches;
     if (!marked) mark(1);
     if constexpr (std::is_same<T, float>::value)
-      if (L->small_h && R <= small_fp32_rows(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k)) {
+      if (L->small_h && L->gemm_path == 0 && !gate_up_only &&
+          R <= small_fp32_rows(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k)) {
         SmallArgs a{};
         a.x = xo; a.w_gate = (const float*)L->wg_p; a.w_up = (const float*)L->wu_p; a.w_down = (const float*)L->wd_p;
         a.h = L->small_h; a.out = out; a.topk_idx = L->topk_idx; a.topk_gate = L->topk_gate;

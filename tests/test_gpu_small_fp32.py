@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from paper_2502_04416_b200 import workloads as wl
+from paper_2502_04416_b200 import binding, workloads as wl
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -44,6 +44,24 @@ def test_same_rows_on_the_general_path():
     # two orders of fp32 sums over at most 1024 terms each: sqrt(1024) roundings of 6e-8
     assert ((whole - few).norm() / whole.norm()).item() < 2e-6
     assert torch.isfinite(few).all()
+    layer.destroy()
+
+
+def test_the_general_path_can_be_forced():
+    import torch
+    inp = wl.make_inputs(wl.Workload("small_fp32", wl.LayerShape(256, 1024, 8, 2, 2, "fp32"), (256,), seed=10))
+    layer = parity.gpu_layer(inp.layers[0], 256)
+    x = parity.to_device(inp.x, "fp32")
+    for t in (1, 64, 256):
+        got = []
+        for path, launches in ((binding.GEMM_AUTO, 3), (binding.GEMM_SIMT, 5)):
+            layer.set_gemm_path(path)
+            got.append(layer.forward(x[:t].contiguous()))
+            assert layer.launch_count() == launches
+        # as above: two orders of fp32 sums over at most 1024 terms each
+        assert ((got[0] - got[1]).norm() / got[1].norm()).item() < 2e-6
+    st = parity.check_plain_layer(layer, inp.layers[0], inp.x[:64])
+    assert st["differing"] == 0 and st["max_rel"] < 1e-4
     layer.destroy()
 
 
