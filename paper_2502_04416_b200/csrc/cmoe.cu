@@ -278,7 +278,7 @@ void carve_workspace(cmoe_layer* L, char* base) {
     L->stream.part = a.take<float>(stream_part_floats((int)T));
   }
   if (esz == 4 && !L->hier) {
-    const int rows = small_fp32_rows((int)std::min<size_t>(T, kSmMaxRows), (int)d, L->cfg.d_ff, L->shared_width(), L->m, L->n_r, L->cfg.top_k);
+    const int rows = small_fp32_rows((int)std::min<size_t>(T, kSmMaxRows), (int)d, L->cfg.d_ff, L->shared_width(), L->m, L->n_r, L->cfg.top_k, L->n_sms);
     if (rows > 0) L->small_h = a.take<float>((size_t)rows * L->cfg.d_ff);
   }
   if (esz == 2 && nr > 0) {
@@ -509,7 +509,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     if (!marked) mark(1);
     if constexpr (std::is_same<T, float>::value)
       if (L->small_h && L->gemm_path == 0 && !gate_up_only &&
-          R <= small_fp32_rows(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k)) {
+          small_fp32_takes(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k, L->n_sms)) {
         SmallArgs a{};
         a.x = xo; a.w_gate = (const float*)L->wg_p; a.w_up = (const float*)L->wu_p; a.w_down = (const float*)L->wd_p;
         a.h = L->small_h; a.out = out; a.topk_idx = L->topk_idx; a.topk_gate = L->topk_gate;

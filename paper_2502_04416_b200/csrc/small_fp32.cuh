@@ -11,9 +11,11 @@
 // Forward of 64 rows, d = 256, 8 x 128 neurons: 26.0 us in five launches (router, permutation, two GEMMs, combine), 14.7 in three; 1 / 128 /
 // 256 rows 22.0 / 27.8 / 38.1 -> 15.4 / 16.2 / 29.1; d = 512, 8 x 192 neurons, 8 / 64 / 128 rows 33.8 / 48.8 / 56.1 -> 15.2 / 22.0 / 43.5.
 // A warp fetches its whole 64-wide slice at once (coalesced 16-byte loads, all in flight) into its own part of shared memory: no
-// block barrier inside the sums.  Unselected experts' products are computed in vain, so the host takes this path only while that is
-// cheaper than two more launches (small_fp32_rows).
+// block barrier inside the sums.  Unselected experts' products are computed in vain, so the host takes this path only where that is
+// expected to be cheaper than two more launches (small_fp32_takes).
 #pragma once
+
+#include <cmath>
 
 #include "common.cuh"
 #include "permute.cuh"
@@ -27,6 +29,7 @@ constexpr int kSmMaxRows = 256;
 constexpr double kSmMaxWork = 400e6;                 // multiply-adds of all experts: 302 M 43.5 against 56.1 us, even on both paths at 440 to 600 M
 constexpr int kSmUpSmem = kSmUpWarps * (kSmUpM + 2 * kSmUpN) * kSmLd * 4;
 constexpr int kSmDnSmem = kSmDnWarps * (kSmDnM + kSmDnN) * kSmLd * 4;
+static_assert(kSmMaxRows <= kMaskRows && kMaxRouted <= kMaskGroups && kSmMaxRows * kMaxTopK <= kMaskPairs, "one block permutes");
 static_assert(kMaskBytes <= kSmDnSmem && kSmDnWarps * 32 == kMaskThreads, "the permutation runs in a block of the down kernel");
 
 struct SmallArgs {
@@ -222,14 +225,38 @@ __global__ void __launch_bounds__(32 * kSmDnWarps) small_down_kernel(const Small
   }
 }
 
-// How many of n_rows rows a plain fp32 layer's forward takes on this path: 16-byte rows, and no more multiply-adds than two launches
-// are worth.
-inline int small_fp32_rows(int n_rows, int d, int d_ff, int shared_w, int m, int n_r, int n_k) {
-  if (n_r < 1 || n_k < 1 || m % 4 || shared_w % 4) return 0;
-  const double most = kSmMaxWork / (3.0 * d * d_ff);
+// Whether a plain fp32 layer's forward of so many rows takes this path: 16-byte rows, and less time expected here than in the five
+// launches of the general path, which multiplies the selected experts only.  Both times (us) are fits to 40 shapes (d 64 to 4096, 2 to 34
+// experts of 32 to 1376 neurons, top-1 to 8) at 1 to 256 rows, chained forwards on one B200, good to about 17 %.
+//   Here: rounds of up blocks (four per SM) times the slices of d that a warp takes, the slices of all experts that a warp of a down block
+// takes, alone and times the down blocks per SM, and all experts' weights.
+//   There: the length of the two k loops, the down tiles' slices per SM (16 x 32 tiles of the rows that an expert is expected to get), and the
+// weights of the experts that at least one row is expected to select.
+// Choosing by them costs 0.5 % over the better path (geometric mean over these and 14 more shapes; the factor 1.05 is the best of 0.95 to
+// 1.1).  Here / there, us: 8 x 128 neurons, d = 256, top-2 64 rows 12.4 / 25.8, 256 rows 29.4 / 37.4; 34 x 128 neurons, d = 256, 1 / 64 / 96
+// rows 26 / 43 / 50 against 28 / 38 / 40; 34 x 256 neurons, d = 128, 16 rows 57 / 34; d = 2048, 34 x 256 neurons, one row 210 / 130; d = 2048,
+// 8 x 688 neurons, one row 98 / 166.
+inline bool small_fp32_takes(int rows, int d, int d_ff, int shared_w, int m, int n_r, int n_k, int n_sms) {
+  if (rows < 1 || rows > kSmMaxRows || n_r < 1 || n_k < 1 || m % 4 || shared_w % 4) return false;
+  if ((double)rows * 3.0 * d * d_ff > kSmMaxWork) return false;
+  auto cut = [](double v, double by) { return ceil(v / by); };
+  const double mb = 12e-6 * d * d_ff;                                            // all experts' weights
+  const double slices = cut(shared_w, kSmKC) + n_r * cut(m, kSmKC), per_warp = cut(slices, kSmDnWarps);
+  const double up_rounds = cut(cut(d_ff, kSmUpN) * cut(rows, kSmUpM), 4 * n_sms), down_blocks = cut(d, kSmDnN) * cut(rows, kSmDnM);
+  const double here = 4.5 + 3.6 * up_rounds * cut(d, kSmUpWarps * kSmKC) + 1.6 * per_warp + 1.5 * per_warp * down_blocks / n_sms + 0.38 * mb;
+  const double hit = n_r * (1.0 - pow(1.0 - (double)n_k / n_r, rows));           // experts with rows
+  const double each = (double)rows * n_k / n_r > 1.0 ? (double)rows * n_k / n_r : 1.0;
+  const double touched = mb * (shared_w + hit * m) / d_ff;
+  const double tiles = cut(d, 32) * (cut(rows, 16) * cut(shared_w, 64) + hit * cut(each, 16) * cut(m, 64));
+  const double there = 11.0 + 2.7 * d / 64 + (shared_w > m ? shared_w : m) / 64.0 + 1.4 * tiles / n_sms + 0.43 * touched;
+  if (mb > 30.0 && mb > 3.0 * touched) return false;                             // weights from DRAM: not three times as many
+  return here < 1.05 * there;
+}
+
+// The most rows (of at most n_rows) that take it.
+inline int small_fp32_rows(int n_rows, int d, int d_ff, int shared_w, int m, int n_r, int n_k, int n_sms) {
   int rows = n_rows < kSmMaxRows ? n_rows : kSmMaxRows;
-  if (rows > most) rows = (int)most;
-  while (rows > 0 && !permute_masks_fit(rows, n_k, n_r)) --rows;
+  while (rows > 0 && !small_fp32_takes(rows, d, d_ff, shared_w, m, n_r, n_k, n_sms)) --rows;
   return rows;
 }
 

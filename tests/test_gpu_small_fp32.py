@@ -65,6 +65,20 @@ def test_the_general_path_can_be_forced():
     layer.destroy()
 
 
+# many unselected experts: their slices (one row), their slices and tiles, rows, weights; beside each a batch that gains by the path
+@pytest.mark.parametrize("d,m,n,k,general,three", [(128, 256, 34, 2, 16, None), (2048, 256, 34, 2, 1, 6), (256, 64, 34, 1, 192, 16),
+                                                   (384, 96, 18, 2, 192, 24), (64, 512, 12, 2, 128, 16)])
+def test_layers_of_many_unselected_experts_take_the_general_path(d, m, n, k, general, three):
+    inp = wl.make_inputs(wl.Workload("small_fp32", wl.LayerShape(d, m * n, n, 2, k, "fp32"), (256,), seed=14))
+    layer = parity.gpu_layer(inp.layers[0], 256)
+    for t, launches in ((general, 5), (three, 3)):
+        if t:
+            st = parity.check_plain_layer(layer, inp.layers[0], inp.x[:t])
+            assert st["differing"] <= st["near_tie"] and st["max_rel"] < 1e-4
+            assert layer.launch_count() == launches
+    layer.destroy()
+
+
 @pytest.mark.parametrize("value", [np.inf, np.nan])
 def test_non_finite_weight_stays_with_its_expert(value):
     import torch
