@@ -312,6 +312,16 @@ int cmoe_layer_selftest_wait_timeout(cmoe_layer* layer, int64_t limit_cycles, vo
 /* Number of this library's kernels the last forward launched. */
 int cmoe_layer_launch_count(const cmoe_layer* layer, int32_t* n_launches);
 
+/* Tile forms that a forward of n_tokens tokens takes for its gate/up and its down GEMM under the current gemm path:
+ * tiles of a single CTA, of a CTA pair with the tokens on the MMA's M side, of a CTA pair with the weights there, or
+ * OTHER for batches that run on kernels without such a choice.  Host arithmetic only; launches nothing.
+ * Errors: INVALID_ARG, CAPACITY. */
+#define CMOE_GEMM_FORM_OTHER 0
+#define CMOE_GEMM_FORM_SINGLE 1
+#define CMOE_GEMM_FORM_PAIR 2
+#define CMOE_GEMM_FORM_TURNED_PAIR 3
+int cmoe_layer_gemm_forms(const cmoe_layer* layer, int32_t n_tokens, int32_t* gate_up, int32_t* down);
+
 /* Per-stage device timing with CUDA events on the forward's stream.  ring_steps > 0
  * creates a ring of events covering that many forwards (0 switches timing off);
  * while on, every forward records CMOE_N_STAGES+1 events and allocates nothing.

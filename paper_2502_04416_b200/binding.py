@@ -14,6 +14,7 @@ LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libcmoe.so"
 
 CMOE_BF16, CMOE_FP32 = 0, 1
 GEMM_AUTO, GEMM_SIMT, GEMM_TENSOR, GEMM_TENSOR_PAIRS = 0, 1, 2, 3
+GEMM_FORMS = ["other", "single", "pair", "turned"]
 N_STAGES = 5
 STAGE_NAMES = ["route", "permute", "gemm1_swiglu", "gemm2_down", "combine"]
 
@@ -23,7 +24,7 @@ EXPORTS = [
     "cmoe_layer_get_gate_params", "cmoe_layer_update_bias", "cmoe_profile_activations", "cmoe_select_shared",
     "cmoe_cluster_update", "cmoe_cluster_distances", "cmoe_cluster_representatives", "cmoe_layer_set_gemm_path", "cmoe_layer_set_launch_chaining",
     "cmoe_layer_dims", "cmoe_get_routing", "cmoe_layer_status", "cmoe_layer_selftest_wait_timeout",
-    "cmoe_layer_launch_count", "cmoe_layer_enable_stage_timing", "cmoe_layer_stage_times",
+    "cmoe_layer_launch_count", "cmoe_layer_gemm_forms", "cmoe_layer_enable_stage_timing", "cmoe_layer_stage_times",
     "cmoe_layer_destroy", "cmoe_token_permute_scratch_bytes",
     "cmoe_token_permute", "cmoe_token_permute_static", "cmoe_status_string", "cmoe_last_error",
 ]
@@ -76,6 +77,7 @@ def load() -> C.CDLL:
     lib.cmoe_layer_status.argtypes = [vp, C.POINTER(i32)]
     lib.cmoe_layer_selftest_wait_timeout.argtypes = [vp, i64, vp]
     lib.cmoe_layer_launch_count.argtypes = [vp, C.POINTER(i32)]
+    lib.cmoe_layer_gemm_forms.argtypes = [vp, i32, C.POINTER(i32), C.POINTER(i32)]
     lib.cmoe_layer_destroy.argtypes = [vp]
     lib.cmoe_layer_enable_stage_timing.argtypes = [vp, i32]
     lib.cmoe_layer_stage_times.argtypes = [vp, C.POINTER(C.c_float), C.POINTER(i32)]
@@ -273,6 +275,12 @@ class Layer:
         w = C.c_int32()
         _check(load().cmoe_layer_launch_count(self._h, C.byref(w)), "cmoe_layer_launch_count")
         return w.value
+
+    def gemm_forms(self, n_tokens: int):
+        """cmoe_layer_gemm_forms: names (of GEMM_FORMS) of the gate/up and the down GEMM's tiles."""
+        gu, dn = C.c_int32(), C.c_int32()
+        _check(load().cmoe_layer_gemm_forms(self._h, n_tokens, C.byref(gu), C.byref(dn)), "cmoe_layer_gemm_forms")
+        return GEMM_FORMS[gu.value], GEMM_FORMS[dn.value]
 
     def enable_stage_timing(self, ring_steps: int) -> None:
         _check(load().cmoe_layer_enable_stage_timing(self._h, ring_steps),

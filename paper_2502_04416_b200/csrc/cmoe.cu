@@ -362,6 +362,9 @@ int pack_weights(cmoe_layer* L, const void* w_gate, const void* w_up, const void
   return CMOE_OK;
 }
 
+// Outer rows up to which the weights-on-M streaming kernels run (see forward_impl).
+int decode_rows(const cmoe_layer* L) { return L->gemm_path != 2 ? kDecWideRows : kDecMaxRows; }
+
 template <typename T>
 int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, bool gate_up_only = false) {
   const int d = L->cfg.d_model, n_r = L->n_r, n_k = L->cfg.top_k;
@@ -449,8 +452,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
   // layer holds FP8 codes (their token planes stop at 64 rows).  Path 2 keeps token-major tiles from 65 rows, which run nearly as
   // fast since their shared tiles need no routing: 7B-shaped 65 / 100 / 128 rows 70.6 / 72.4 / 75.0 against 74.3 / 73.7 / 74.2 us, 13B-shaped
   // 100 / 128 rows 98.7 / 102.2 against 98.5 / 98.4, 8B-shaped 128 rows 93.0 against 86.6, hierarchical 33 tokens 415 against 424.
-  const int decode_rows = L->gemm_path != 2 ? kDecWideRows : kDecMaxRows;
-  const bool decode = use_umma && !gemv && !stream && R <= decode_rows;
+  const bool decode = use_umma && !gemv && !stream && R <= decode_rows(L);
   if (use_umma && !stream && !umma_bind_x(&L->umma, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   if ((decode || (stream && L->fp8)) && !decode_bind_x(&L->umma, &L->decode, xo, R)) return arg_fail(CMOE_ERR_CUDA, L->umma.error);
   // E4M3 planes of the token rows: independent of the routing, but for the outer rows, which the router may copy
@@ -1214,6 +1216,21 @@ int cmoe_layer_selftest_wait_timeout(cmoe_layer* L, int64_t limit_cycles, void* 
 int cmoe_layer_launch_count(const cmoe_layer* L, int32_t* n_launches) {
   if (!L || !n_launches) return arg_fail(CMOE_ERR_INVALID_ARG, "null argument");
   *n_launches = L->launches;
+  return CMOE_OK;
+}
+
+int cmoe_layer_gemm_forms(const cmoe_layer* L, int32_t n_tokens, int32_t* gate_up, int32_t* down) {
+  if (!L || !gate_up || !down || n_tokens < 0) return arg_fail(CMOE_ERR_INVALID_ARG, "null argument / negative token count");
+  if (n_tokens > L->cfg.max_tokens) return arg_fail(CMOE_ERR_CAPACITY, "n_tokens exceeds max_tokens");
+  *gate_up = *down = CMOE_GEMM_FORM_OTHER;
+  const int R = n_tokens * (L->hier ? L->outer_k : 1);
+  if (!L->umma_ok || L->gemm_path == 1 || R <= decode_rows(L)) return CMOE_OK;
+  const GemmForms f = umma_pick_forms(&L->umma, L->pair.grid, R, R * L->cfg.top_k, L->n_outer * L->n_r, L->gemm_path);
+  auto code = [](GemmForm g) {
+    return g == GemmForm::kTurned ? CMOE_GEMM_FORM_TURNED_PAIR : g == GemmForm::kPair ? CMOE_GEMM_FORM_PAIR : CMOE_GEMM_FORM_SINGLE;
+  };
+  *gate_up = code(f.gate_up);
+  *down = code(f.down);
   return CMOE_OK;
 }
 

@@ -530,7 +530,9 @@ inline int umma2t_columns(int rows) {
 // stages), a turned tile of N tokens 60 + 1.15 N ns on a pair (190 at least).  The load is taken once as expected and once with a
 // fifth more tiles, for skewed routing, and pairs have to win by an eighth.
 //   From there on the part runs at its power limit and every padded multiply costs energy: the form with the fewest, single
-// tiles counted 5 % dearer for the operands that both of a pair's CTAs would have shared.
+// tiles counted 8 % dearer for the operands that both of a pair's CTAs would have shared (over 70 measured sizes from 2048 rows on the choice is 1.0 %
+// above the best form, geometric mean; 1.3 % with 5 %, 1.9 % where pairs had to win by another 3 %: 8B-shaped 3200 / 14592 / 16384 rows
+// 307 / 1314 / 1475 on pairs, 322 / 1448 / 1633 on single CTAs).
 //   Down: turned tiles where an expert has more than 128 rows (a single tile's height) and K is more than a few k blocks.
 // Whole forwards, single / turned gate/up / both turned (alternating, us): 7B-shaped 300 / 400 / 512 / 1000 / 2048 rows 82 / 108 / 113 / 166 / 295,
 // 82 / 96 / 103 / 153 / 276, 83 / 89 / 98 / 151 / 278; 13B-shaped 300 / 600 / 1000 / 4096 rows 125 / 168 / 222 / 738, 115 / 156 / 211 / 652, 117 / 153 / 198 / 631;
@@ -556,8 +558,7 @@ inline GemmForms umma_pick_forms(const UmmaPlan* P, int pair_grid, int R, int n_
     return f;
   }
   if (R >= kPairLargeRows) {
-    const double single = 1.05 * work(up(rows_s, 128), P->bn_s, up(rows_r, 128), P->bn_r);
-    if ((turned < pair ? turned : pair) < 0.97 * single) f.gate_up = on_pairs;
+    if ((turned < pair ? turned : pair) < 1.08 * work(up(rows_s, 128), P->bn_s, up(rows_r, 128), P->bn_r)) f.gate_up = on_pairs;
   } else {
     const double dev = mean > 0 ? sqrt(mean * (1.0 - (mean < rows_s ? mean / rows_s : 1.0))) : 0.0;
     const double dev_s = s.n_outer > 1 ? sqrt((double)rows_s) : 0.0;
