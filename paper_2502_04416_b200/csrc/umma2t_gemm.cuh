@@ -506,11 +506,13 @@ inline double umma_expected_tiles(double mean, double dev, int rows) {
   return n;
 }
 
-// Busiest CTA (or pair) of n_slots when n_s tiles of cost c_s and then n_r tiles of cost c_r are dealt round-robin.
+// Busiest CTA (or pair) of n_slots when n_s tiles of cost c_s and then n_r tiles of cost c_r are dealt round-robin.  The load changes
+// with the slot only where one of the two runs of tiles ends.
 inline double umma_busiest(int n_s, double c_s, int n_r, double c_r, int n_slots) {
+  const int ends_s = n_s % n_slots, ends_all = (n_s + n_r) % n_slots;
   double worst = 0.0;
-  for (int i = 0; i < n_slots; ++i) {
-    const int s = n_s > i ? (n_s - 1 - i) / n_slots + 1 : 0, all = n_s + n_r > i ? (n_s + n_r - 1 - i) / n_slots + 1 : 0;
+  for (int i : {0, ends_s, ends_all}) {
+    const int s = n_s / n_slots + (i < ends_s), all = (n_s + n_r) / n_slots + (i < ends_all);
     const double load = s * c_s + (all - s) * c_r;
     worst = load > worst ? load : worst;
   }
@@ -527,17 +529,26 @@ inline int umma2t_columns(int rows) {
 // persistent kernels whose tiles are dealt round-robin.
 //   Below kPairLargeRows: a few rounds, so what counts for gate/up is the busiest SM, or the weights' way from DRAM (5.8 TB/s) where
 // that takes longer.  Per 64-wide k block a 128 x 256 tile takes 425 ns on a single CTA (the operands' round trip through four
-// stages), a turned tile of N tokens 60 + 1.15 N ns on a pair (190 at least).  The load is taken once as expected and once with a
-// fifth more tiles, for skewed routing, and pairs have to win by an eighth.
+// stages), a token-major tile 350 on a pair, a turned tile of N tokens 120 + 0.95 N (240 at least); pairs have to win by 9 %.  The load is
+// taken as expected and, with a third of the weight, with a fifth more routed tiles, for skewed routing.  The constants are those that choose
+// best over 251 measured sizes (7B-, 8B- and 13B-shaped, hierarchical and 28 random shapes): 1.6 % above the fastest form (geometric mean, the
+// runs themselves differ by about 1 %), 4.4 % with single CTAs and token-major pairs only.
 //   From there on the part runs at its power limit and every padded multiply costs energy: the form with the fewest, single
 // tiles counted 8 % dearer for the operands that both of a pair's CTAs would have shared (over 70 measured sizes from 2048 rows on the choice is 1.0 %
 // above the best form, geometric mean; 1.3 % with 5 %, 1.9 % where pairs had to win by another 3 %: 8B-shaped 3200 / 14592 / 16384 rows
 // 307 / 1314 / 1475 on pairs, 322 / 1448 / 1633 on single CTAs).
-//   Down: turned tiles where an expert has more than 128 rows (a single tile's height) and K is more than a few k blocks.
-// Whole forwards, single / turned gate/up / both turned (alternating, us): 7B-shaped 300 / 400 / 512 / 1000 / 2048 rows 82 / 108 / 113 / 166 / 295,
-// 82 / 96 / 103 / 153 / 276, 83 / 89 / 98 / 151 / 278; 13B-shaped 300 / 600 / 1000 / 4096 rows 125 / 168 / 222 / 738, 115 / 156 / 211 / 652, 117 / 153 / 198 / 631;
-// 8B-shaped (448 neurons: turned tiles pad them by 14 %) 300 / 1000 / 1400 rows 107 / 166 / 183, 95 / 147 / 173, 100 / 152 / 175, 8192 rows
-// token-major pairs 728 against 749; hierarchical 700 / 2000 / 4096 tokens 587 / 974 / 1560, 603 / 884 / 1539, 664 / 871 / 1521.
+//   Down: turned tiles where an expert has more than 128 rows (a single tile's height) and K is more than seven k blocks (448 neurons even
+// or 2 % slower, 496 neurons 4696 rows 445 against 484).
+// Whole forwards, gate/up on single CTAs / token-major pairs / turned pairs, each with single and turned down tiles (alternating, us):
+//   7B-shaped   300 rows  79 79 / 85 86 / 80 80      512  108 104 / 102 96 / 100 95     710  119 117 / 112 110 / 114 112
+//              1000      161 160 / 157 157 / 153 154  1470 212 211 / 208 202 / 208 206   2047 285 271 / 275 268 / 283 268
+//   13B-shaped  600      162 150 / 151 142 / 147 137  1000 217 210 / 230 231 / 222 217   4096 687 664 / 666 640 / 651 636
+//   8B-shaped (448 neurons: turned tiles pad them by 14 %)
+//               300       99 101 / 98 100 / 97 95    1000 150 151 / 141 142 / 140 139    1500 182 182 / 171 172 / 178 178
+//              8192      783 771 / 730 732 / 745 750
+//   hierarchical 700 tokens 569 564 / 599 622 / 595 589   2048 986 936 / 956 866 / 892 858   4096 1531 1509 / 1602 1626 / 1506 1478
+// A token-major down GEMM on pairs was even with the turned one at large sizes (13B-shaped 12288 / 16384 rows 1754 / 2332 against 1756 / 2336,
+// 7B-shaped 8192 rows 932 / 935) and slower below.
 inline GemmForms umma_pick_forms(const UmmaPlan* P, int pair_grid, int R, int n_sel, int n_routed, int gemm_path) {
   GemmForms f;
   if (gemm_path == 2 || R < kPairMinRows) return f;
@@ -564,27 +575,33 @@ inline GemmForms umma_pick_forms(const UmmaPlan* P, int pair_grid, int R, int n_
     const double dev_s = s.n_outer > 1 ? sqrt((double)rows_s) : 0.0;
     const int w_s = P->has_s ? (s.shared_width + 127) / 128 : 0, w_r = P->has_r ? (s.m + 127) / 128 : 0;
     const double dram = (s.n_outer * w_s + n_routed * w_r) * 32768.0 / 5800.0;
-    auto cost = [&](bool turn) {
-      const int rows = turn ? kUtMaxTok : kUmmaBM;
+    auto cost = [&](GemmForm form) {
+      const int rows = form == GemmForm::kSingle ? kUmmaBM : 256;            // of a full tile
       auto tile = [&](double r) {                      // a tile of a group with r rows
-        if (!turn) return 425.0;
-        const double t = 60.0 + 1.15 * TokenCut((int)ceil(r)).width;
-        return t > 190.0 ? t : 190.0;
+        if (form != GemmForm::kTurned) return form == GemmForm::kSingle ? 425.0 : 350.0;
+        const double t = 120.0 + 0.95 * TokenCut((int)ceil(r)).width;
+        return t > 240.0 ? t : 240.0;
       };
+      const bool turn = form == GemmForm::kTurned;
       const int per_s = turn || !P->has_s ? w_s : (s.shared_width + P->bn_s - 1) / P->bn_s;
       const int per_r = turn || !P->has_r ? w_r : (s.m + P->bn_r - 1) / P->bn_r;
       const int n_s = (int)(s.n_outer * umma_expected_tiles(rows_s, dev_s, rows) * per_s + 0.5);
       const double n_r = n_routed * umma_expected_tiles(mean, dev, rows) * per_r, c_s = tile(rows_s + dev_s / 2), c_r = tile(mean + dev / 2);
       double sum = 0.0;
-      for (int i = 0; i < 2; ++i) {
-        const double b = umma_busiest(n_s, c_s, (int)((i ? 1.2 : 1.0) * n_r + 0.5), c_r, turn ? pair_grid / 2 : P->n_sms);
-        sum += b > dram ? b : dram;
+      for (int skewed = 0; skewed < 2; ++skewed) {
+        const double b = umma_busiest(n_s, c_s, (int)((skewed ? 1.2 : 1.0) * n_r + 0.5), c_r,
+                                      form == GemmForm::kSingle ? P->n_sms : pair_grid / 2);
+        sum += (b > dram ? b : dram) * (skewed ? 1.0 : 2.0) / 3.0;
       }
       return sum;
     };
-    if (cost(true) < 0.88 * cost(false)) f.gate_up = GemmForm::kTurned;
+    double best = cost(GemmForm::kSingle);
+    for (GemmForm form : {GemmForm::kTurned, GemmForm::kPair}) {
+      const double c = 1.09 * cost(form);
+      if (c < best) { best = c; f.gate_up = form; }
+    }
   }
-  if (s.m >= 512 && (mean > kUmmaBM || !P->has_r)) f.down = GemmForm::kTurned;
+  if (s.m > 448 && (mean > kUmmaBM || !P->has_r)) f.down = GemmForm::kTurned;
   return f;
 }
 

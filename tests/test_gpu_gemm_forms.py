@@ -8,8 +8,16 @@ from paper_2502_04416_b200 import binding, workloads as wl
 pytestmark = pytest.mark.gpu
 
 # rows -> forms within 2 % of the fastest forward (single CTAs / token-major pairs / turned pairs, us, at the first size of each
-# line: 8B-shaped 3200 rows 322 / 307 / 311)
+# line: 7B-shaped 1000 rows 160 / 157 / 154, 512 rows 104 / 96 / 95, 1400 rows 201 / 195 / 199, 300 rows 79 / 86 / 80, 8B-shaped 1500 rows
+# 182 / 171 / 178, 700 rows 109 / 117 / 114, 3200 rows 322 / 307 / 311, 13B-shaped 600 rows 150 / 142 / 137)
 SIZES = [
+    ("c2_llama2_7b", (1000, 1024), ("turned",)),
+    ("c2_llama2_7b", (512, 400, 600, 850, 1300, 1600), ("turned",)),
+    ("c2_llama2_7b", (1400, 1470), ("pair",)),
+    ("c2_llama2_7b", (300, 256), ("single",)),
+    ("c3_llama3_8b", (1500, 1400), ("pair",)),
+    ("c3_llama3_8b", (700, 600, 768, 820), ("single",)),
+    ("c5_skew_13b", (600, 400, 512, 1000, 1500), ("turned",)),
     ("c3_llama3_8b", (3200, 14592, 16384), ("pair",)),
 ]
 
