@@ -1,4 +1,4 @@
-"""-m gpu: expert GEMMs on CTA pairs with weights on M and tokens on N, at the edges of their tiles."""
+"""-m gpu: expert GEMMs on CTA pairs, with weights on M and tokens on N (turned) or, for gate/up, token-major, at the edges of their tiles."""
 import numpy as np
 import pytest
 
@@ -8,8 +8,9 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 
 # token tiles: one group below, at and above 256 rows, equal tiles with a shorter last one; columns in steps of 32.  Neurons: fewer than
-# one tile, halves of 8 and 56 neurons per CTA, a last tile that ends early; d: k and output channels that fill no block.
+# one tile, halves of 8, 16 and 56 neurons per CTA, a last tile that ends early; d: k and output channels that fill no block.
 CASES = [
+    (256, 16, (257, 300, 400)),
     (256, 24, (256, 257, 300, 511, 513)),
     (328, 200, (287, 1030)),
     (1032, 448, (1000,)),
@@ -35,7 +36,8 @@ def test_pair_tiles(d, m, tokens, skew):
     layer.destroy()
 
 
-# The tiles change which rows are multiplied together, not the sums of one output: same bits as single-CTA tiles.
+# The tiles change which rows are multiplied together, not the sums of one output: same bits as single-CTA tiles, whatever form the
+# forced pairs take (see below for each form by itself).
 @pytest.mark.parametrize("tokens", [256, 700, 1111])
 def test_pair_tiles_have_the_bits_of_single_tiles(tokens):
     import torch
@@ -49,3 +51,43 @@ def test_pair_tiles_have_the_bits_of_single_tiles(tokens):
         got.append(layer.forward(x).view(torch.int16).clone())
     assert torch.equal(*got)
     layer.destroy()
+
+
+def _bits_on_single_tiles_and_pairs(lay, x, forms):
+    import torch
+    layer = parity.gpu_layer(lay, len(x))
+    xd = parity.to_device(x, "bf16")
+    layer.set_gemm_path(binding.GEMM_TENSOR)
+    want = layer.forward(xd).view(torch.int16).clone()
+    layer.set_gemm_path(binding.GEMM_TENSOR_PAIRS)
+    assert layer.gemm_forms(len(x)) == forms
+    assert torch.equal(layer.forward(xd).view(torch.int16), want)
+    st = parity.check_plain_layer(layer, lay, x)
+    assert st["differing"] <= st["near_tie"]
+    counts = layer.routing(len(x), lay.shape.n_routed)["counts"]
+    assert layer.status() == 0
+    layer.destroy()
+    return counts
+
+
+# turned gate/up tiles: one, two (both whole), three and five per group, the last one shorter; neurons that end inside the second tile,
+# and halves of 8 per CTA
+@pytest.mark.parametrize("m,tokens", [(248, 257), (248, 512), (248, 520), (248, 600), (248, 700), (248, 1111), (16, 257), (16, 300)])
+def test_turned_gate_up_has_the_bits_of_single_tiles(m, tokens):
+    shape = wl.LayerShape(328, m * 8, 8, 2, 2, "bf16")
+    inp = wl.make_inputs(wl.Workload("turned_bits", shape, (tokens,), seed=5))
+    _bits_on_single_tiles_and_pairs(inp.layers[0], inp.x, ("turned", "turned"))
+
+
+# token-major gate/up: the forced choice is made for even loads, so skewed ones bring groups with odd and even numbers of 128-row
+# tiles, a single one and none; m as neurons that fill their tiles and end inside them
+@pytest.mark.parametrize("m", [200, 448, 864])
+@pytest.mark.parametrize("tokens", [1000, 1024, 2048])
+def test_token_major_gate_up_has_the_bits_of_single_tiles(tokens, m):
+    shape = wl.LayerShape(264, m * 8, 8, 2, 3, "bf16")
+    inp = wl.make_inputs(wl.Workload("token_major_bits", shape, (tokens,), seed=8))
+    lay = inp.layers[0]
+    lay.select_bias_b = np.array([0.5, 0.01, 0.0, -0.01, -0.02, -0.5], np.float32)
+    counts = _bits_on_single_tiles_and_pairs(lay, inp.x, ("pair", "turned"))
+    tiles = (counts + 127) // 128
+    assert counts[5] == 0 and (tiles % 2 == 1).any() and ((tiles % 2 == 0) & (tiles > 0)).any(), counts

@@ -95,10 +95,13 @@ def test_non_finite_weight_stays_with_its_expert(value):
     layer.destroy()
 
 
-def test_small_fp32_stack_is_the_same_chained_or_not():
+@pytest.mark.parametrize("path", [binding.GEMM_AUTO, binding.GEMM_SIMT], ids=["three_launches", "general"])
+def test_small_fp32_stack_is_the_same_chained_or_not(path):
     import torch
     inp = wl.make_inputs(wl.Workload("small_fp32", wl.LayerShape(256, 512, 8, 2, 2, "fp32"), (64,), seed=7))
     layers = [parity.gpu_layer(inp.layers[0], 64) for _ in range(3)]
+    for layer in layers:
+        layer.set_gemm_path(path)
     x = parity.to_device(inp.x, "fp32")
 
     def run(chain):
