@@ -608,7 +608,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         const int early = L->hier ? 0 : R;
         const int k = form == GemmForm::kTurned
             ? umma2t_forward(&L->umma, &L->turned, L->pair.grid, &L->decode, L->gr, xo, R, L->err_word, st, mid, dep, bit, early, fold_out != nullptr)
-            : form == GemmForm::kPair ? umma2_forward(&L->umma, &L->pair, L->gr, xo, L->err_word, st, mid, dep, early)
+            : form == GemmForm::kPair ? umma2_forward(&L->umma, &L->pair, &L->decode, L->gr, xo, L->err_word, st, mid, dep, bit, early, fold_out != nullptr)
             : umma_forward(&L->umma, L->gr, xo, L->err_word, st, mid, dep, bit, early, fold_out != nullptr);
         n = k < 0 ? -1 : n + k;
       }

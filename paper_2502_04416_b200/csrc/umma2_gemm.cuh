@@ -1,16 +1,19 @@
-// Token-major gate/up GEMM on CTA pairs (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster, on
+// Expert GEMMs on CTA pairs (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster, on
 // neighbouring SMs, compute one 256 x N tile.  Each CTA stages its own 128 rows of A and
 // only HALF of the B tile (the MMA reads the other half from the peer's shared memory),
 // so a stage is 16 KB + 16 KB instead of 16 KB + 32 KB: six stages fit instead of four,
 // and the L2 -> SM traffic for the weights halves.  The leader CTA (cluster rank 0) issues
 // every MMA for the pair; accumulators sit in both CTAs' TMEM (128 lanes each).
 //
-// The leader stages the bn gate rows, the peer the bn up rows, so the accumulator columns are [gate | up] exactly as in the
-// single-CTA kernel.  For large batches of experts whose width the 128-neuron tiles of umma2t_gemm.cuh would pad
-// (448: 14 %); everything else that runs on pairs runs there.
+//   MODE 1, gate/up: the leader stages the bn gate rows, the peer the bn up rows, so the
+//           accumulator columns are [gate | up] exactly as in the single-CTA kernel.
+//   MODE 2, down:    each CTA stages 128 of the tile's 256 output channels.
+// Taken where the turned tiles of umma2t_gemm.cuh would multiply as much or more (umma_pick_forms): gate/up of widths that their 128 neurons
+// pad (448: 14 %), large batches whose groups fill their 256-row tiles; the down GEMM in the latter case alone.  There the epilogue's 32-byte
+// stores of whole rows beat 4-byte stores of two channels (13B-shaped 16384 / 12000 rows, the launch alone 436 / 318 us against 450 / 331 turned).
 // The two 128-row halves are two m-tiles of the same group and n-tile; a group with an odd
 // number of m-tiles leaves one half computing rows that are never stored.
-// Routed groups gather their A rows straight from x (no permuted copy):
+// Routed groups of the gate/up GEMM gather their A rows straight from x (no permuted copy):
 // four extra warps per CTA copy the CTA's 128 rows of each k block with 16-byte cp.async into the
 // swizzled layout and arrive, copy-completion-bound, on a barrier of their own CTA; a relay
 // thread per CTA forwards each completed block to the leader's full barrier.  (Waiting for the
@@ -19,14 +22,15 @@
 //
 // Synchronisation (all waits bounded):
 //   full[s]      leader's barrier; the leader's producer arrives with the byte count of BOTH
-//                CTAs' TMA copies, which complete on it; each CTA's relay
+//                CTAs' TMA copies, which complete on it; in the gate/up kernel each CTA's relay
 //                thread arrives on it as well (2 more arrivals).
-//   afull[s]     one per CTA: its 128 gather threads, then its relay waits on it.
+//   afull[s]     gate/up only, one per CTA: its 128 gather threads, then its relay waits on it.
 //   empty[s]     one per CTA; the leader's tcgen05.commit is multicast to both.
 //   acc_full[b]  one per CTA, multicast commit;  acc_empty[b]: leader's, 8 arrivals (the
 //                four epilogue warps of each CTA, the peer's arriving remotely).
 #pragma once
 
+#include "umma_decode.cuh"
 #include "umma_gemm.cuh"
 
 namespace cmoe {
@@ -127,17 +131,19 @@ __device__ __forceinline__ Pair2Coord umma2_tile_in(const UmmaArgs& p, int g, co
   return c;
 }
 
+template <int MODE>
 __device__ __forceinline__ Pair2Coord umma2_decode(const UmmaArgs& p, const int32_t* tile_start, const GroupRows* rows, int t) {
   int lo = 0, hi = p.n_groups;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (tile_start[mid] <= t) lo = mid; else hi = mid;
   }
-  return umma2_tile_in(p, lo, rows[lo], umma_n_tiles<1>(p, lo), t - tile_start[lo]);
+  return umma2_tile_in(p, lo, rows[lo], umma_n_tiles<MODE>(p, lo), t - tile_start[lo]);
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kU2Threads1, 1)
-umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
+template <int MODE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MODE == 1 ? kU2Threads1 : kUmmaThreads, 1)
+umma2_grouped_kernel(const __grid_constant__ CUtensorMap tm_a_s, const __grid_constant__ CUtensorMap tm_a_r,
                      const __grid_constant__ CUtensorMap tm_b_s, const __grid_constant__ CUtensorMap tm_b_r,
                      const UmmaArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -159,8 +165,9 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
   const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
+    const uint32_t full_count = MODE == 1 ? 3 : 1;      // gate/up: plus one relay arrival per CTA
     for (int s = 0; s < kU2Stages; ++s) {
-      mbar_init(full0 + 8 * s, 3); mbar_init(empty0 + 8 * s, 1); mbar_init(afull0 + 8 * s, kUmmaGatherThreads);
+      mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); mbar_init(afull0 + 8 * s, kUmmaGatherThreads);
     }
     for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 8); }
     mbar_init(tbl_bar, 1);
@@ -179,25 +186,25 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
   const uint32_t tmem_base = *tmem_slot;
   const int k_blocks_fixed = (p.d + kUmmaBK - 1) / kUmmaBK;
   // table and tiles that need none: as in umma_grouped_kernel
-  const int early_n = p.early_rows > 0 ? (p.shared_width + p.bn_s - 1) / p.bn_s : 0;
+  const int early_n = MODE == 1 && p.early_rows > 0 ? (p.shared_width + p.bn_s - 1) / p.bn_s : 0;
   const int early_tiles = (((p.early_rows + kUmmaBM - 1) / kUmmaBM + 1) / 2) * early_n;
   if (warp == 2) {
-    for (int g = lane; g < p.n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<1>(p, g);
-    grid_dep_wait();
-    grid_dep_trigger();
+    for (int g = lane; g < p.n_groups; g += 32) tile_start[g + 1] = umma_n_tiles<MODE>(p, g);
+    if (MODE == 1) { grid_dep_wait(); grid_dep_trigger(); }
     for (int g = lane; g < p.n_groups; g += 32) {
       const GroupRows gr = p.gr[g];
       rows[g] = gr;
-      tile_start[g + 1] *= ((gr.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
+      tile_start[g + 1] *= MODE == 2 && g < p.skip_groups ? 0 : ((gr.count + kUmmaBM - 1) / kUmmaBM + 1) >> 1;
     }
     __syncwarp();
     warp_prefix(tile_start, p.n_groups, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(tbl_bar);
+    if (MODE == 2) { grid_dep_wait(); grid_dep_trigger(); }     // what follows may count on the gate/up GEMM
   }
   bool seen = false;
   auto tile_at = [&](int t, Pair2Coord& c, GroupStatic& g, bool whole_warp, bool& ok) {
-    if (t < early_tiles) {
+    if (MODE == 1 && t < early_tiles) {
       GroupRows all; all.row0 = 0; all.count = p.early_rows;
       c = umma2_tile_in(p, 0, all, early_n, t);
       g.w_row0 = 0; g.width = p.shared_width; g.wd_offset = 0; g.is_shared = 1; g.outer = 0;
@@ -207,38 +214,69 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
       ok = mbar_wait(tbl_bar, 0, abort_flag, p.err, kErrWaitFull);
       if (whole_warp) ok = __all_sync(0xffffffffu, ok);
       if (!ok) return false;
-      grid_dep_wait();
+      if (MODE == 1) grid_dep_wait();
       seen = true;
     }
     if (t >= tile_start[p.n_groups]) return false;
-    c = umma2_decode(p, tile_start, rows, t);
+    c = umma2_decode<MODE>(p, tile_start, rows, t);
     g = p.gs[c.g];
     return true;
   };
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
-    uint32_t it = 0;
+    uint32_t it = 0, n_ahead = 0;
+    bool waited = false;
     bool ok = true;
     for (int t = pair_id; ok; t += n_pairs) {
       Pair2Coord c;
       GroupStatic g;
       if (!tile_at(t, c, g, true, ok)) break;
       const int row = c.row0 + (2 * c.mp + (int)rank) * kUmmaBM;     // this CTA's m-tile
+      const CUtensorMap* ta = g.is_shared ? &tm_a_s : &tm_a_r;
       const CUtensorMap* tb = g.is_shared ? &tm_b_s : &tm_b_r;
-      const bool by_threads = !g.is_shared;                          // the gather warps fill A
-      const int bn = g.is_shared ? p.bn_s : p.bn_r;
-      const int b_half = bn * kUmmaBK * 2, b_row = g.w_row0 + c.nt * bn;
-      for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
+      const bool by_threads = MODE == 1 && !g.is_shared;   // the gather warps fill A
+      int k_blocks, b_half, b_row, j = 0;
+      if (MODE == 1) {
+        const int bn = g.is_shared ? p.bn_s : p.bn_r;
+        k_blocks = k_blocks_fixed;
+        b_half = bn * kUmmaBK * 2;
+        b_row = g.w_row0 + c.nt * bn;
+      } else {
+        k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK;
+        b_half = kU2BBytes;
+        b_row = c.nt * 256 + (int)rank * 128;
+        j = g.is_shared ? 0 : (c.g - p.n_outer) - g.outer * p.n_r;
+      }
+      auto load_b = [&](int kb, uint32_t sb, uint32_t fb) {
+        if (MODE == 1) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, (int)rank);   // plane 0 gate, 1 up
+        else if (g.is_shared) tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, g.outer);
+        else tma2_load_4d(sb, tb, fb, kb * kUmmaBK, b_row, j, g.outer);
+      };
+      if (MODE == 2 && it == 0 && !waited) {
+        n_ahead = min(kU2Stages, k_blocks);
+        for (uint32_t i = 0; i < n_ahead; ++i) {
+          if (elect_one()) {
+            if (leader) mbar_expect_tx(full0 + 8 * i, 2 * (kU2ABytes + b_half));
+            load_b(i, base + i * kU2StageBytes + kU2ABytes, mapa_shared(full0 + 8 * i, 0));
+          }
+          __syncwarp();
+        }
+        grid_dep_wait();
+        waited = true;
+      }
+      for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const uint32_t s = it % kU2Stages, n = it / kU2Stages;
         if (!mbar_wait_warp(empty0 + 8 * s, (n & 1) ^ 1, abort_flag, p.err, kErrWaitEmpty)) { ok = false; break; }
         const uint32_t fb_local = full0 + 8 * s;
         const uint32_t fb = mapa_shared(fb_local, 0);               // the leader's barrier
         const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
         if (elect_one()) {
-          if (leader) mbar_expect_tx(fb_local, 2 * ((by_threads ? 0 : kU2ABytes) + b_half));
-          tma2_load_3d(sb, tb, fb, kb * kUmmaBK, b_row, (int)rank);   // plane 0 gate, 1 up
-          if (!by_threads) tma2_load_2d(sa, &tm_a_s, fb, kb * kUmmaBK, row);
+          if (MODE == 1 || it >= n_ahead) {
+            if (leader) mbar_expect_tx(fb_local, 2 * ((by_threads ? 0 : kU2ABytes) + b_half));
+            load_b(kb, sb, fb);
+          }
+          if (!by_threads) tma2_load_2d(sa, ta, fb, kb * kUmmaBK, row);
         }
         __syncwarp();
       }
@@ -251,17 +289,20 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
       bool ok = true;
       for (int t = pair_id; ok; t += n_pairs, ++tile_n) {
         Pair2Coord c;
-        GroupStatic g;
-        if (!tile_at(t, c, g, true, ok)) break;
-        const uint32_t idesc = umma2_idesc(2 * (g.is_shared ? p.bn_s : p.bn_r));
+      GroupStatic g;
+      if (!tile_at(t, c, g, true, ok)) break;
+        int k_blocks, n_mma;
+        if (MODE == 1) { k_blocks = k_blocks_fixed; n_mma = 2 * (g.is_shared ? p.bn_s : p.bn_r); }
+        else { k_blocks = (g.width + kUmmaBK - 1) / kUmmaBK; n_mma = 256; }
+        const uint32_t idesc = umma2_idesc(n_mma);
         const uint32_t buf = tile_n & 1, use = tile_n >> 1;
         if (!mbar_wait_warp(acce0 + 8 * buf, (use & 1) ^ 1, abort_flag, p.err, kErrWaitAccEmpty)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * 256;
-        for (int kb = 0; kb < k_blocks_fixed; ++kb, ++it) {
+        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const uint32_t s = it % kU2Stages, n = it / kU2Stages;
           if (!mbar_wait_warp(full0 + 8 * s, n & 1, abort_flag, p.err, kErrWaitFull)) { ok = false; break; }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          if (MODE == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_after();
           const uint32_t sa = base + s * kU2StageBytes, sb = sa + kU2ABytes;
           if (elect_one()) {
@@ -277,8 +318,8 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
         __syncwarp();
       }
     }
-  } else if (warp == 10) {
-    // ------------------------------------------------------------ relay (warp 10, both CTAs)
+  } else if (MODE == 1 && warp == 10) {
+    // ------------------------------------------------------------ relay (gate/up, warp 10, both CTAs)
     // Waits until this CTA's 128 gather threads have landed a k block (local barrier), fences
     // those generic-proxy writes towards the async proxy and arrives on the leader's full barrier.
     if (lane == 0) {
@@ -296,8 +337,8 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
         }
       }
     }
-  } else if (warp >= 6) {
-    // ------------------------------------------------------------ A-row gather (warps 6..9, both CTAs)
+  } else if (MODE == 1 && warp >= 6) {
+    // ------------------------------------------------------------ A-row gather (gate/up, warps 6..9, both CTAs)
     // Eight consecutive threads cover one 128-byte row segment, 16 rows per pass, 8 passes; 16-byte
     // chunk c of row r goes to the swizzled chunk c ^ (r & 7).  Each thread's arrival on the CTA's
     // local barrier is tied to the completion of its copies (cp.async.mbarrier.arrive.noinc).
@@ -357,30 +398,55 @@ umma2_gate_up_kernel(const __grid_constant__ CUtensorMap tm_a_s,
       const int row_in_group = (2 * c.mp + (int)rank) * kUmmaBM + quad * 32 + lane;
       const bool row_ok = row_in_group < c.count;
       const uint32_t taddr = tmem_base + buf * 256 + ((uint32_t)(quad * 32) << 16);
-      const int bn = g.is_shared ? p.bn_s : p.bn_r;
-      const int ld = g.is_shared ? p.ld_out_s : p.ld_out_r;
-      const int n0 = c.nt * bn;
-      const int n_valid = min(bn, g.width - n0);
-      bf16* dst = (g.is_shared ? p.out_s : p.out_r) + (size_t)(c.row0 + row_in_group) * ld + n0;
-      const bool wide = ((ld | n0) & 15) == 0;
-      for (int c0 = 0; c0 < n_valid; c0 += 16) {
-        float gt[16], up[16];
-        tmem_ld16(taddr + c0, gt);
-        tmem_ld16(taddr + bn + c0, up);
-        tmem_ld_wait();
-        if (row_ok) {
-          float h16[16];
+      if (MODE == 1) {
+        const int bn = g.is_shared ? p.bn_s : p.bn_r;
+        const int ld = g.is_shared ? p.ld_out_s : p.ld_out_r;
+        const int n0 = c.nt * bn;
+        const int n_valid = min(bn, g.width - n0);
+        bf16* dst = (g.is_shared ? p.out_s : p.out_r) + (size_t)(c.row0 + row_in_group) * ld + n0;
+        const bool wide = ((ld | n0) & 15) == 0;
+        for (int c0 = 0; c0 < n_valid; c0 += 16) {
+          float gt[16], up[16];
+          tmem_ld16(taddr + c0, gt);
+          tmem_ld16(taddr + bn + c0, up);
+          tmem_ld_wait();
+          if (row_ok) {
+            float h16[16];
 #pragma unroll
-          for (int q = 0; q < 16; ++q) h16[q] = swiglu_fast(gt[q], up[q]);
-          if (wide && c0 + 16 <= n_valid) {
-            store16(dst + c0, h16);
-          } else {
+            for (int q = 0; q < 16; ++q) h16[q] = swiglu_fast(gt[q], up[q]);
+            if (wide && c0 + 16 <= n_valid) {
+              store16(dst + c0, h16);
+            } else {
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                if (c0 + h * 8 < n_valid) {
+                  float v[8];
+#pragma unroll
+                  for (int q = 0; q < 8; ++q) v[q] = h16[h * 8 + q];
+                  store8(dst + c0 + h * 8, v);
+                }
+              }
+            }
+          }
+        }
+      } else {
+        const int n0 = c.nt * 256;
+        const int n_valid = min(256, p.d - n0);
+        bf16* dst = (g.is_shared ? p.out_s : p.out_r) + (size_t)(c.row0 + row_in_group) * p.d + n0;
+        const bool wide = (p.d & 15) == 0;
+        for (int c0 = 0; c0 < n_valid; c0 += 16) {
+          float acc[16];
+          tmem_ld16(taddr + c0, acc);
+          tmem_ld_wait();
+          if (row_ok && wide && c0 + 16 <= n_valid) {
+            store16(dst + c0, acc);
+          } else if (row_ok) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               if (c0 + h * 8 < n_valid) {
                 float v[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) v[q] = h16[h * 8 + q];
+                for (int q = 0; q < 8; ++q) v[q] = acc[h * 8 + q];
                 store8(dst + c0 + h * 8, v);
               }
             }
@@ -420,7 +486,10 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
                      "gate/up weights (CTA pair)");
   }
   if (!ok) return false;
-  cudaError_t e = cudaFuncSetAttribute(umma2_gate_up_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kU2SmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(umma2_grouped_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kU2SmemBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(umma2_grouped_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kU2SmemBytes);
   if (e != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "cudaFuncSetAttribute (CTA pair): %s", cudaGetErrorString(e));
     return false;
@@ -435,7 +504,7 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   int n_clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&n_clusters, umma2_gate_up_kernel, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&n_clusters, umma2_grouped_kernel<1>, &cfg);
   if (e != cudaSuccess || n_clusters <= 0) {
     snprintf(P->error, sizeof(P->error), "cudaOccupancyMaxActiveClusters: %s", cudaGetErrorString(e));
     return false;
@@ -445,23 +514,34 @@ inline bool umma2_plan_create(UmmaPlan* P, Umma2Plan* Q) {
   return true;
 }
 
-// Gate/up GEMM; routed rows are gathered from x_rows.  Requires umma_bind_x for this forward.  Returns launches or -1.
-inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, const GroupRows* gr, const void* x_rows, int32_t* err_word, cudaStream_t st,
-                         cudaEvent_t mid, bool dep, int early_rows) {
+// Gate/up and down GEMM on CTA pairs; routed rows are gathered from x_rows inside the gate/up kernel.
+// `D` supplies the 128-channel W_down maps (shared with the decode path).  Requires
+// umma_bind_x for this forward.  which: bit 0 the gate/up GEMM, bit 1 the down GEMM.  Returns launches or -1.
+inline int umma2_forward(UmmaPlan* P, Umma2Plan* Q, DecodePlan* D, const GroupRows* gr, const void* x_rows, int32_t* err_word, cudaStream_t st, cudaEvent_t mid, bool dep,
+                         int which, int early_rows, bool skip_shared = false) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);
+  const int grid = Q->grid;
   a.out_s = (bf16*)P->buf.h_s; a.out_r = (bf16*)P->buf.h_r; a.ld_out_s = s.shared_width; a.ld_out_r = s.m;
   a.x_rows_ptr = (const bf16*)x_rows;
   a.band_mt = umma_band_tiles(s.d);
   a.early_rows = early_rows;
-  const cudaError_t e = launch_kernel(dep, umma2_gate_up_kernel, dim3(Q->grid), dim3(kU2Threads1), umma2_smem_bytes(P->n_groups), st,
-                                      P->x_rows, Q->b1_s, Q->b1_r, a);
-  if (mid) cudaEventRecord(mid, st);
+  if (which & 1)
+    launch_kernel(dep, umma2_grouped_kernel<1>, dim3(grid), dim3(kU2Threads1), umma2_smem_bytes(P->n_groups), st,
+                  P->x_rows, P->x_rows, Q->b1_s, Q->b1_r, a);
+  if (mid && (which & 1)) cudaEventRecord(mid, st);
+  a.out_s = (bf16*)P->buf.y_s; a.out_r = (bf16*)P->buf.y_r; a.ld_out_s = s.d; a.ld_out_r = s.d;
+  a.band_mt = umma_band_tiles(s.shared_width > s.m ? s.shared_width : s.m);
+  a.skip_groups = skip_shared ? s.n_outer : 0;
+  if (which & 2)
+    launch_kernel(dep, umma2_grouped_kernel<2>, dim3(grid), dim3(kUmmaThreads), umma2_smem_bytes(P->n_groups), st, P->a2_s, P->a2_r,
+                  D->wd_s, D->wd_r, a);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(P->error, sizeof(P->error), "CTA-pair GEMM launch: %s", cudaGetErrorString(e));
     return -1;
   }
-  return 1;
+  return (which & 1) + ((which >> 1) & 1);
 }
 
 }  // namespace cmoe

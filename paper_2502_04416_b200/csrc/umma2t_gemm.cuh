@@ -263,7 +263,7 @@ umma2t_grouped_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_c
       }
     }
   } else if (MODE == 1 && warp == 10) {
-    // ------------------------------------------------------------ relay (gate/up, both CTAs): see umma2_gate_up_kernel
+    // ------------------------------------------------------------ relay (gate/up, both CTAs): see umma2_grouped_kernel
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
@@ -493,7 +493,7 @@ inline int umma2t_forward(UmmaPlan* P, Umma2tPlan* Q, int grid, DecodePlan* D, c
 constexpr int kPairMinRows = 256;        // outer rows from which the expert GEMMs may run on CTA pairs
 constexpr int kPairLargeRows = 2048;     // outer rows from which the part runs at its power limit for the whole forward
 
-enum class GemmForm { kSingle, kPair, kTurned };     // umma_gemm.cuh, umma2_gemm.cuh (gate/up only), this file
+enum class GemmForm { kSingle, kPair, kTurned };     // umma_gemm.cuh, umma2_gemm.cuh, this file
 struct GemmForms { GemmForm gate_up = GemmForm::kSingle, down = GemmForm::kSingle; };
 
 // Expected number of `rows`-row tiles of a group whose rows are binomial with this mean and deviation.
@@ -547,8 +547,8 @@ inline int umma2t_columns(int rows) {
 //               300       99 101 / 98 100 / 97 95    1000 150 151 / 141 142 / 140 139    1500 182 182 / 171 172 / 178 178
 //              8192      783 771 / 730 732 / 745 750
 //   hierarchical 700 tokens 569 564 / 599 622 / 595 589   2048 986 936 / 956 866 / 892 858   4096 1531 1509 / 1602 1626 / 1506 1478
-// A token-major down GEMM on pairs was even with the turned one at large sizes (13B-shaped 12288 / 16384 rows 1754 / 2332 against 1756 / 2336,
-// 7B-shaped 8192 rows 932 / 935) and slower below.
+// Down, turned / token-major on pairs (from kPairLargeRows on, where the turned tiles pad as much): 13B-shaped 16384 rows 2426 / 2380, 12288 even;
+// 7B-shaped 8192 rows even; where they pad less, 7B-shaped 4096 rows (1376 columns against 1536) 497 / 505.
 inline GemmForms umma_pick_forms(const UmmaPlan* P, int pair_grid, int R, int n_sel, int n_routed, int gemm_path) {
   GemmForms f;
   if (gemm_path == 2 || R < kPairMinRows) return f;
@@ -601,7 +601,12 @@ inline GemmForms umma_pick_forms(const UmmaPlan* P, int pair_grid, int R, int n_
       if (c < best) { best = c; f.gate_up = form; }
     }
   }
-  if (s.m > 448 && (mean > kUmmaBM || !P->has_r)) f.down = GemmForm::kTurned;
+  if (s.m > 448 && (mean > kUmmaBM || !P->has_r)) {
+    // K x token columns, padded
+    const double down_pair = (double)s.n_outer * s.shared_width * up(rows_s, 256) + (double)n_routed * s.m * up(rows_r, 256);
+    const double down_turned = (double)s.n_outer * s.shared_width * umma2t_columns(rows_s) + (double)n_routed * s.m * umma2t_columns(rows_r);
+    f.down = R >= kPairLargeRows && down_turned >= 0.97 * down_pair ? GemmForm::kPair : GemmForm::kTurned;
+  }
   return f;
 }
 

@@ -882,7 +882,7 @@ inline int umma_forward(UmmaPlan* P, const GroupRows* gr, const void* x_rows, in
   return (which & 1) + ((which >> 1) & 1);
 }
 
-// Down GEMM of the shared experts with the combine, after the routed experts' (umma_forward or umma2_forward with skip_shared).
+// Down GEMM of the shared experts with the combine, after the routed experts' (the other forms' down GEMM with skip_shared).
 inline int umma_fold_forward(UmmaPlan* P, const GroupRows* gr, int n_rows, bf16* out, int32_t* err_word, cudaStream_t st, bool dep) {
   const UmmaShape& s = P->shape;
   UmmaArgs a = umma_base_args(P, gr, err_word);

@@ -47,6 +47,15 @@ def test_chosen_forms(name, rows, forms):
     layer.destroy()
 
 
+# 13B-shaped 16384 rows 2380 / 2426 us with token-major / turned down tiles, 7B-shaped 4096 rows 505 / 497 (1365 rows per expert: 1536 / 1376 columns),
+# 448 neurons are too few k blocks for either
+@pytest.mark.parametrize("name,rows,form", [("c5_skew_13b", 16384, "pair"), ("c2_llama2_7b", 4096, "turned"), ("c3_llama3_8b", 8192, "single")])
+def test_chosen_down_form(name, rows, form):
+    _, layer = _layer(name, rows)
+    assert layer.gemm_forms(rows)[1] == form
+    layer.destroy()
+
+
 def test_small_batches_have_no_tile_form():
     _, layer = _layer("c2_llama2_7b", 200)
     assert layer.gemm_forms(64) == layer.gemm_forms(128) == ("other", "other")

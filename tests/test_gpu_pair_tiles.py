@@ -53,13 +53,13 @@ def test_pair_tiles_have_the_bits_of_single_tiles(tokens):
     layer.destroy()
 
 
-def _bits_on_single_tiles_and_pairs(lay, x, forms):
+def _bits_on_single_tiles_and_pairs(lay, x, forms, path=binding.GEMM_TENSOR_PAIRS):
     import torch
     layer = parity.gpu_layer(lay, len(x))
     xd = parity.to_device(x, "bf16")
     layer.set_gemm_path(binding.GEMM_TENSOR)
     want = layer.forward(xd).view(torch.int16).clone()
-    layer.set_gemm_path(binding.GEMM_TENSOR_PAIRS)
+    layer.set_gemm_path(path)
     assert layer.gemm_forms(len(x)) == forms
     assert torch.equal(layer.forward(xd).view(torch.int16), want)
     st = parity.check_plain_layer(layer, lay, x)
@@ -91,3 +91,16 @@ def test_token_major_gate_up_has_the_bits_of_single_tiles(tokens, m):
     counts = _bits_on_single_tiles_and_pairs(lay, inp.x, ("pair", "turned"))
     tiles = (counts + 127) // 128
     assert counts[5] == 0 and (tiles % 2 == 1).any() and ((tiles % 2 == 0) & (tiles > 0)).any(), counts
+
+
+# the down GEMM too: large batches whose groups are expected to fill 256-row tiles; K that ends inside a block, channels inside a tile
+@pytest.mark.parametrize("skewed", [False, True])
+@pytest.mark.parametrize("tokens,m", [(2304, 512), (2300, 520), (3071, 576)])
+def test_token_major_down_has_the_bits_of_single_tiles(tokens, m, skewed):
+    shape = wl.LayerShape(264, m * 8, 8, 2, 2, "bf16")
+    inp = wl.make_inputs(wl.Workload("token_major_down_bits", shape, (tokens,), seed=13))
+    lay = inp.layers[0]
+    if skewed:
+        lay.select_bias_b = np.array([0.5, 0.01, 0.0, -0.01, -0.02, -0.5], np.float32)
+    counts = _bits_on_single_tiles_and_pairs(lay, inp.x, ("pair", "pair"), binding.GEMM_AUTO)
+    assert not skewed or counts[5] == 0
