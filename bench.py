@@ -170,9 +170,9 @@ def prepare_inputs(name: str):
 NCU_TRAFFIC = {
     ("c5_skew_13b", 16384): {"bytes": (1585.1 + 164.5 + 249.1 + 628.4 + 884.5 + 151.9) * 1e6,
                              "source": "profiles/launch_lists.md"},
-    ("c2_llama2_7b", 4096): {"bytes": (280.4 + 36.0 + 90.2 + 34.2 + 126.3 + 15.8) * 1e6, "source": "profiles/launch_lists.md"},
+    ("c2_llama2_7b", 4096): {"bytes": (298.5 + 37.3 + 90.2 + 34.7 + 126.5 + 16.2) * 1e6, "source": "profiles/launch_lists.md"},
     ("c3_llama3_8b", 8192): {"bytes": (509.3 + 52.7 + 132.2 + 214.5 + 357.7 + 50.9) * 1e6, "source": "profiles/launch_lists.md"},
-    ("c4_hier_8x7b", 4096): {"bytes": (2038.8 + 112.6 + 1060.0 + 184.3) * 1e6, "source": "profiles/launch_lists.md"},
+    ("c4_hier_8x7b", 4096): {"bytes": (2404.0 + 114.5 + 1086.2 + 187.2) * 1e6, "source": "profiles/launch_lists.md"},
 }
 
 # Every (workload, T) point the metric is quoted on; the last one (the largest single-GPU

@@ -256,7 +256,7 @@ int cmoe_cluster_representatives(const int64_t* scaled_sq_dist, const int32_t* n
  * launch; up to 256 rows of a plain fp32 layer may run on three launches that multiply every expert, where that is expected
  * to take less time), 1 = always SIMT, per-expert products over permuted rows, 2 = tensor-core with
  * single-CTA token-major tiles only (decode-shaped kernels up to 64 rows), 3 = tensor-core on CTA
- * pairs (cta_group::2) for batches of at least 256 rows;
+ * pairs (cta_group::2) for batches of at least 256 rows, gate/up on the form of pairs that pads less (cmoe_layer_gemm_forms);
  * 2 and 3 return CMOE_ERR_INVALID_ARG if the layer cannot take the tensor-core path. */
 int cmoe_layer_set_gemm_path(cmoe_layer* layer, int32_t path);
 

@@ -21,8 +21,8 @@
 // FP8 = true streams the E4M3 codes of a quantised layer (one byte per weight) and multiplies the
 // sums by the per-row power-of-two scales; the token rows stay bf16.
 // The kernels are written for TT rows and instantiated for one: two rows already run faster on the tensor-core
-// streamers, one row is faster here (cmoe_layer_set_gemm_path 0 / 2 on 7B-, 8B- and 13B-shaped layers: 30.7 vs 41.9,
-// 26.9 vs 30.5, 37.7 vs 48.5 us per forward; with FP8 weights 25.2 vs 28.7, 24.3 vs 30.1, 31.8 vs 34.9).
+// streamers, one row is faster here (these kernels / the streamers, one row of the 7B-, 8B- and 13B-shaped layer: 30.6 / 42.3,
+// 26.8 / 39.3, 37.9 / 48.7 us per forward; with FP8 weights 25.4 / 34.7, 24.3 / 33.1, 31.7 / 39.2).
 #pragma once
 
 #include "common.cuh"

@@ -8,7 +8,7 @@
 //       selected the expert (a select, not a zero gate: an unselected expert's Inf or NaN goes no further), and meet in shared memory in
 //       warp order.  The first weights are fetched ahead of the wait.  One more block writes the permutation, which only
 //       cmoe_get_routing and the utilisation read.
-// Forward of 64 rows, d = 256, 8 x 128 neurons: 26.0 us in five launches (router, permutation, two GEMMs, combine), 14.7 in three; 1 / 128 /
+// Forwards back to back, 64 rows, d = 256, 8 x 128 neurons: 26.0 us in five launches (router, permutation, two GEMMs, combine), 14.7 in three; 1 / 128 /
 // 256 rows 22.0 / 27.8 / 38.1 -> 15.4 / 16.2 / 29.1; d = 512, 8 x 192 neurons, 8 / 64 / 128 rows 33.8 / 48.8 / 56.1 -> 15.2 / 22.0 / 43.5.
 // A warp fetches its whole 64-wide slice at once (coalesced 16-byte loads, all in flight) into its own part of shared memory: no
 // block barrier inside the sums.  Unselected experts' products are computed in vain, so the host takes this path only where that is

@@ -38,7 +38,7 @@
 // under the router, its slowest CTA and the hand-over cost 4, the down kernel streams for 13 and its sums take 3.  (The sums are one chain of latencies: stores,
 // release, ticket, loads.  With a fence per lane beside lane 0's release and six of seven contributions in flight 16 rows took 56.1
 // instead of 55.4 us, 8B-shaped 32 rows 69.8 instead of 69.3.)  A single row stays on the
-// CUDA-core kernels of gemv.cuh (34 us against 46).  Fetching the down kernel's weights into L2 at the end of the up kernel was slower
+// CUDA-core kernels of gemv.cuh (30.6 us against 42.3).  Fetching the down kernel's weights into L2 at the end of the up kernel was slower
 // (it delays the up kernel's last CTAs), equal runs of k blocks instead of tiles in the up kernel as well (the partial sums).
 #pragma once
 

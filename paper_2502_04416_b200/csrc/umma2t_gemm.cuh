@@ -13,8 +13,9 @@
 // Roles, barriers and the gather of routed rows are those of umma2_gemm.cuh; eight epilogue warps per CTA, each with 32 of every 64
 // columns (four: 6.4 us from a 256-column tile's last MMA to its last store, eight: 4.2).
 //
-// Chained forwards before / after (one side's runs differ by 0.3-1 %): hierarchical 4096 tokens 1569 / 1489 us, 8B-shaped 1000 rows 145.4 / 142.0;
-// 7B-shaped 400 / 512 / 1000 rows 100 / 89 / 162 -> 89 / 98 / 151, 13B-shaped 600 / 1000 rows 165 / 213 -> 153 / 198 (see umma_pick_forms).
+// Chained forwards with single CTAs and token-major gate/up pairs alone / as umma_pick_forms chooses now (one side's runs differ by 0.3-3 %):
+// hierarchical 2000 / 4096 tokens 928 / 1570 -> 878 / 1491 us, 8B-shaped 1000 rows 146.2 -> 142.7, 7B-shaped 400 / 512 / 1000 rows 101.9 / 105.3 /
+// 161.3 -> 88.7 / 98.8 / 156.8, 13B-shaped 600 / 1000 rows 171.5 / 220.4 -> 151.8 / 205.4.
 // Not taken: the k blocks of a tile started at another place per pair (even), the routed experts' first weights fetched into L2 under the
 // shared experts' tiles (8B-shaped 1000 rows +0 to +6 us: it delays those tiles by what it saves later), shared and routed tiles on
 // separate pairs at the same time (+3 to +20 us).
@@ -325,7 +326,7 @@ umma2t_grouped_kernel(const __grid_constant__ CUtensorMap tm_w_s, const __grid_c
     }
     if (!ok) asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2..5, both CTAs)
+    // ------------------------------------------------------------ epilogue (eight warps, both CTAs: 2..5, then 11..14 or 6..9)
     const int quad = warp & 3, first = warp < 6 ? 0 : 32;             // columns first, first + 64, ..., 32 at a time
     uint32_t tile_n = 0;
     bool ok = true;
