@@ -41,6 +41,7 @@ namespace {
 thread_local char g_last_error[512] = "";
 
 int cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();                                  // reported here: not left for the next call to find
   snprintf(g_last_error, sizeof(g_last_error), "%s: %s", what, cudaGetErrorString(e));
   return CMOE_ERR_CUDA;
 }
@@ -519,6 +520,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
         a.perm = PermuteOut{R, n_k, G, L->counts, L->offsets, L->row_token, L->row_of, po};
         mark(2);
         CU_TRY(small_fp32_forward(a, dep, st, ev ? ev[3] : nullptr));
+        CU_TRY(cudaGetLastError());                    // the router's launch
         mark(4);
         mark(5);
         if (ev) ++L->ev_count;
