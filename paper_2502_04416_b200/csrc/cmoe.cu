@@ -121,6 +121,7 @@ struct cmoe_layer {
   Umma2tPlan turned;
   StreamPlan stream;
   float* small_h = nullptr;            // fp32 layers of a few rows: H of all experts
+  bool small_takes[kSmMaxRows + 1] = {};               // by rows: small_fp32_takes
   int32_t* router_ticket = nullptr;    // row tiles of the small-batch router that are done
   uint32_t *rt_words = nullptr, *rt_words_outer = nullptr;     // tcgen05 routers: row masks per expert
   float* dec_part = nullptr;    // decode GEMMs: K-slice partial sums, tickets per (tile, epilogue warp)
@@ -279,8 +280,12 @@ void carve_workspace(cmoe_layer* L, char* base) {
     L->stream.part = a.take<float>(stream_part_floats((int)T));
   }
   if (esz == 4 && !L->hier) {
-    const int rows = small_fp32_rows((int)std::min<size_t>(T, kSmMaxRows), (int)d, L->cfg.d_ff, L->shared_width(), L->m, L->n_r, L->cfg.top_k, L->n_sms);
-    if (rows > 0) L->small_h = a.take<float>((size_t)rows * L->cfg.d_ff);
+    int most = 0;                                      // rows of the largest batch that takes the path
+    for (int rows = 1; rows <= (int)std::min<size_t>(T, kSmMaxRows); ++rows) {
+      L->small_takes[rows] = small_fp32_takes(rows, (int)d, L->cfg.d_ff, L->shared_width(), L->m, L->n_r, L->cfg.top_k, L->n_sms);
+      if (L->small_takes[rows]) most = rows;
+    }
+    if (most > 0) L->small_h = a.take<float>((size_t)most * L->cfg.d_ff);
   }
   if (esz == 2 && nr > 0) {
     L->rt_words = a.take<uint32_t>(router_tile_words((int)R, (int)nr, L->n_outer));
@@ -511,8 +516,7 @@ int forward_impl(cmoe_layer* L, const T* x, int n_tok, T* out, cudaStream_t st, 
     ++launches;
     if (!marked) mark(1);
     if constexpr (std::is_same<T, float>::value)
-      if (L->small_h && L->gemm_path == 0 && !gate_up_only &&
-          small_fp32_takes(R, d, L->cfg.d_ff, L->shared_width(), L->m, n_r, n_k, L->n_sms)) {
+      if (L->gemm_path == 0 && !gate_up_only && R <= kSmMaxRows && L->small_takes[R]) {
         SmallArgs a{};
         a.x = xo; a.w_gate = (const float*)L->wg_p; a.w_up = (const float*)L->wu_p; a.w_down = (const float*)L->wd_p;
         a.h = L->small_h; a.out = out; a.topk_idx = L->topk_idx; a.topk_gate = L->topk_gate;

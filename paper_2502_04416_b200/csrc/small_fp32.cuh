@@ -253,13 +253,6 @@ inline bool small_fp32_takes(int rows, int d, int d_ff, int shared_w, int m, int
   return here < 1.05 * there;
 }
 
-// The most rows (of at most n_rows) that take it.
-inline int small_fp32_rows(int n_rows, int d, int d_ff, int shared_w, int m, int n_r, int n_k, int n_sms) {
-  int rows = n_rows < kSmMaxRows ? n_rows : kSmMaxRows;
-  while (rows > 0 && !small_fp32_takes(rows, d, d_ff, shared_w, m, n_r, n_k, n_sms)) --rows;
-  return rows;
-}
-
 inline cudaError_t small_fp32_allow() {
   const cudaError_t e = allow_smem(small_up_kernel, kSmUpSmem);
   return e == cudaSuccess ? allow_smem(small_down_kernel, kSmDnSmem) : e;
